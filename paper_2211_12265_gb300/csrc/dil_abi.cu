@@ -18,9 +18,10 @@ struct dil_ctx {
     void *ws = nullptr;       // device scratch
     size_t ws_bytes = 0;
     int max_iter = 0;         // 0 = nonce cap
-    // plain-kernel launch shape per operation (keygen / sign / verify) and level (2 / 3 / 5)
-    int warps[3][3] = {{8, 8, 8}, {8, 8, 8}, {8, 8, 8}};   // warps per CTA
-    int wpt[3][3] = {{2, 2, 2}, {2, 2, 2}, {2, 2, 2}};     // warps per task
+    // launch shape per operation (keygen / sign / verify) and level (2 / 3 / 5)
+    // as set by dil_set_tuning; 0: not set
+    int warps[3][3] = {};   // warps per CTA
+    int wpt[3][3] = {};     // warps per task
     // host-form staging (device memory)
     void *stage = nullptr;
     size_t stage_bytes = 0;
@@ -46,6 +47,10 @@ struct dil_ctx {
 namespace {
 
 constexpr size_t POLY_BYTES = 256 * sizeof(int32_t);
+
+// Up to this many tasks the batch forms' arithmetic runs four warps per task:
+// a task's latency is what counts while the SMs are not full.
+constexpr size_t BATCH_WIDE_TASKS = 600;
 
 // NVTX range over one API call (a no-op unless a profiler is attached), so
 // traces show which entry point issued which launches.
@@ -93,13 +98,44 @@ int ensure_ws(dil_ctx *c, size_t bytes) {
     return DIL_OK;
 }
 
-// Largest number of tasks per launch whose scratch fits the budget.
-size_t chunk_tasks(dil_ctx *c, int op, int level, size_t n) {
-    size_t per = dil::scratch_polys(op, level) * POLY_BYTES;
-    if (per == 0) return n;
-    size_t fit = c->budget / per;
-    size_t lim = std::min<size_t>(n, std::min<size_t>(fit, (size_t)1 << 30));
-    return lim;
+// Largest number of tasks per launch whose scratch (`per` bytes each) fits the budget.
+size_t chunk_tasks(const dil_ctx *c, size_t per, size_t n) {
+    return std::min<size_t>(n, std::min<size_t>(c->budget / per, (size_t)1 << 30));
+}
+size_t chunk_tasks(const dil_ctx *c, int op, int level, size_t n) {
+    return chunk_tasks(c, dil::scratch_polys(op, level) * POLY_BYTES, n);
+}
+
+// Launch shape of one call.  The fused forms run when the caller asked for two
+// or four warps per task, and where the budget holds the scratch of a fused
+// task but not that of the batch form (`per` bytes a task).
+struct Shape {
+    bool fused;
+    int warps, p;
+};
+
+Shape shape_of(const dil_ctx *c, int op, int level, size_t n, size_t per) {
+    const int w = c->warps[op][lidx(level)], p = c->wpt[op][lidx(level)];
+    if (p > 1) return {true, w, p};
+    if (c->budget < per) return {true, 8, 2};
+    if (n <= BATCH_WIDE_TASKS) return {false, 4, 4};
+    return {false, w ? w : 4, 1};
+}
+
+// The fused kernels' launch shape where a caller set none.
+int fused_warps(const dil_ctx *c, int op, int level) { const int w = c->warps[op][lidx(level)]; return w ? w : 8; }
+int fused_wpt(const dil_ctx *c, int op, int level) { const int p = c->wpt[op][lidx(level)]; return p ? p : 2; }
+
+size_t verify_task_bytes(size_t polys) { return polys * POLY_BYTES + dil::VERIFY_AUX_BYTES; }
+
+// Carves m tasks of a Verify batch out of a workspace of m verify_task_bytes.
+void carve_verify(dil::VerifyBatch &b, void *ws, size_t m, size_t polys) {
+    uint8_t *aux = static_cast<uint8_t *>(ws) + m * polys * POLY_BYTES;
+    b.n = (int)m;
+    b.scratch = static_cast<int32_t *>(ws);
+    b.mu = reinterpret_cast<uint32_t *>(aux);
+    b.tr = reinterpret_cast<uint32_t *>(aux + 64 * m);
+    b.next = reinterpret_cast<int *>(aux + 96 * m);
 }
 
 void sizes_of(int level, size_t &pk, size_t &sk, size_t &sig) { dil_sizes(level, &pk, &sk, &sig); }
@@ -200,14 +236,17 @@ int dil_keygen(dil_ctx *c, int level, size_t n, const uint8_t *seeds, uint8_t *p
     DeviceGuard g(c->device);
     size_t pkb, skb, sigb;
     sizes_of(level, pkb, skb, sigb);
-    size_t chunk = chunk_tasks(c, dil::OP_KEYGEN, level, n);
+    const size_t per = dil::scratch_polys(dil::OP_KEYGEN, level) * POLY_BYTES;
+    size_t chunk = chunk_tasks(c, per, n);
     if (chunk == 0) return DIL_ENOMEM;
-    int rc = ensure_ws(c, chunk * dil::scratch_polys(dil::OP_KEYGEN, level) * POLY_BYTES);
+    int rc = ensure_ws(c, chunk * per);
     if (rc) return rc;
     for (size_t s0 = 0; s0 < n; s0 += chunk) {
         int m = (int)std::min(chunk, n - s0);
-        cudaError_t e = dil::launch_keygen(level, m, seeds + 32 * s0, pk + pkb * s0, sk + skb * s0,
-                                           (int32_t *)c->ws, c->warps[0][lidx(level)], c->wpt[0][lidx(level)], (cudaStream_t)stream);
+        const Shape sh = shape_of(c, 0, level, m, per);
+        cudaError_t e = (sh.fused ? dil::launch_keygen : dil::launch_keygen_batch)(
+            level, m, seeds + 32 * s0, pk + pkb * s0, sk + skb * s0, (int32_t *)c->ws, sh.warps, sh.p,
+            (cudaStream_t)stream);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     return DIL_OK;
@@ -235,7 +274,7 @@ int dil_sign_ex(dil_ctx *c, int level, size_t n, const uint8_t *sk, const uint8_
         cudaError_t e = dil::launch_sign(level, m, sk + skb * s0, msg, msg_off + s0, sig + sigb * s0,
                                          task_status ? task_status + s0 : nullptr,
                                          iterations ? iterations + s0 : nullptr, (int32_t *)c->ws, max_iter,
-                                         c->warps[1][lidx(level)], c->wpt[1][lidx(level)], (cudaStream_t)stream);
+                                         fused_warps(c, 1, level), fused_wpt(c, 1, level), (cudaStream_t)stream);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     return DIL_OK;
@@ -256,15 +295,29 @@ int dil_verify(dil_ctx *c, int level, size_t n, const uint8_t *pk, const uint8_t
     DeviceGuard g(c->device);
     size_t pkb, skb, sigb;
     sizes_of(level, pkb, skb, sigb);
-    size_t chunk = chunk_tasks(c, dil::OP_VERIFY, level, n);
+    const size_t polys = dil::scratch_polys(dil::OP_VERIFY, level);
+    const Shape sh = shape_of(c, 2, level, n, verify_task_bytes(polys));
+    const size_t per = sh.fused ? polys * POLY_BYTES : verify_task_bytes(polys);
+    size_t chunk = chunk_tasks(c, per, n);
     if (chunk == 0) return DIL_ENOMEM;
-    int rc = ensure_ws(c, chunk * dil::scratch_polys(dil::OP_VERIFY, level) * POLY_BYTES);
+    int rc = ensure_ws(c, chunk * per);
     if (rc) return rc;
     for (size_t s0 = 0; s0 < n; s0 += chunk) {
         int m = (int)std::min(chunk, n - s0);
-        cudaError_t e = dil::launch_verify(level, m, pk + pkb * s0, msg, msg_off + s0, sig + sigb * s0, ok + s0,
-                                           (int32_t *)c->ws, c->warps[2][lidx(level)], c->wpt[2][lidx(level)],
-                                           (cudaStream_t)stream);
+        cudaError_t e;
+        if (sh.fused) {
+            e = dil::launch_verify(level, m, pk + pkb * s0, msg, msg_off + s0, sig + sigb * s0, ok + s0,
+                                   (int32_t *)c->ws, sh.warps, sh.p, (cudaStream_t)stream);
+        } else {
+            dil::VerifyBatch b{};
+            carve_verify(b, c->ws, m, polys);
+            b.pk = pk + pkb * s0;
+            b.msg = msg;
+            b.off = msg_off + s0;
+            b.sig = sig + sigb * s0;
+            b.ok = ok + s0;
+            e = dil::launch_verify_batch(level, dil::VERIFY_PLAIN, b, sh.warps, sh.p, (cudaStream_t)stream);
+        }
         if (e != cudaSuccess) return cuda_fail(e);
     }
     return DIL_OK;
@@ -290,7 +343,7 @@ int dil_expand_a(dil_ctx *c, int level, size_t n, const uint8_t *rho, size_t rho
     // one warp per key, in the CTA size of Verify's tuning (the other kernel
     // whose first step is ExpandA); the output needs no workspace
     cudaError_t e = dil::launch_expand_a(level, (int)n, rho, rho_stride, reinterpret_cast<int32_t *>(ahat),
-                                         c->warps[2][lidx(level)], (cudaStream_t)stream);
+                                         fused_warps(c, 2, level), (cudaStream_t)stream);
     return e != cudaSuccess ? cuda_fail(e) : DIL_OK;
 }
 
@@ -318,7 +371,7 @@ int dil_sign_a(dil_ctx *c, int level, size_t n, const uint8_t *sk, const uint8_t
         cudaError_t e = dil::launch_sign_a(level, m, sk + skb * s0, msg, msg_off + s0, a + ahat_words(level) * s0,
                                            sig + sigb * s0, task_status ? task_status + s0 : nullptr,
                                            iterations ? iterations + s0 : nullptr, (int32_t *)c->ws, max_iter,
-                                           c->warps[1][lidx(level)], (cudaStream_t)stream);
+                                           fused_warps(c, 1, level), (cudaStream_t)stream);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     return DIL_OK;
@@ -335,16 +388,27 @@ int dil_verify_a(dil_ctx *c, int level, size_t n, const uint8_t *pk, const uint8
     DeviceGuard g(c->device);
     size_t pkb, skb, sigb;
     sizes_of(level, pkb, skb, sigb);
-    const size_t chunk = chunk_tasks(c, dil::OP_VERIFY, level, n);
+    // z^ and what a task's hashes leave, less than dil_verify's scratch
+    const size_t polys = dil::keyed_verify_polys(level), per = verify_task_bytes(polys);
+    const size_t chunk = chunk_tasks(c, per, n);
     if (chunk == 0) return DIL_ENOMEM;
-    int rc = ensure_ws(c, chunk * dil::scratch_polys(dil::OP_VERIFY, level) * POLY_BYTES);
+    int rc = ensure_ws(c, chunk * per);
     if (rc) return rc;
     const int32_t *a = reinterpret_cast<const int32_t *>(ahat);
     for (size_t s0 = 0; s0 < n; s0 += chunk) {
         const int m = (int)std::min(chunk, n - s0);
-        cudaError_t e = dil::launch_verify_a(level, m, pk + pkb * s0, msg, msg_off + s0, sig + sigb * s0,
-                                             a + ahat_words(level) * s0, ok + s0, (int32_t *)c->ws,
-                                             c->warps[2][lidx(level)], (cudaStream_t)stream);
+        dil::VerifyBatch b{};
+        carve_verify(b, c->ws, m, polys);
+        b.pk = pk + pkb * s0;
+        b.msg = msg;
+        b.off = msg_off + s0;
+        b.sig = sig + sigb * s0;
+        b.ok = ok + s0;
+        b.ahat = a + ahat_words(level) * s0;
+        const int w = c->warps[2][lidx(level)];
+        const bool wide = (size_t)m <= BATCH_WIDE_TASKS;
+        cudaError_t e = dil::launch_verify_batch(level, dil::VERIFY_AHAT, b, wide ? 4 : w ? w : 4, wide ? 4 : 1,
+                                                 (cudaStream_t)stream);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     return DIL_OK;
@@ -565,7 +629,7 @@ int dil_sign_keyed(dil_ctx *c, const dil_keystore *ks, size_t n, const int32_t *
         cudaError_t e = dil::launch_sign_keyed(ks->level, m, (int)ks->n, key_idx + s0, ks->sk, ks->keys, msg,
                                                msg_off + s0, sig + sigb * s0,
                                                task_status ? task_status + s0 : nullptr, nullptr, (int32_t *)c->ws,
-                                               max_iter, c->warps[1][lidx(ks->level)], c->wpt[1][lidx(ks->level)],
+                                               max_iter, fused_warps(c, 1, ks->level), fused_wpt(c, 1, ks->level),
                                                (cudaStream_t)stream);
         if (e != cudaSuccess) return cuda_fail(e);
     }
@@ -582,17 +646,34 @@ int dil_verify_keyed(dil_ctx *c, const dil_keystore *ks, size_t n, const int32_t
     DeviceGuard g(c->device);
     size_t pkb, skb, sigb;
     sizes_of(ks->level, pkb, skb, sigb);
-    const size_t per = dil::keyed_verify_polys(ks->level) * POLY_BYTES;
-    size_t chunk = std::min<size_t>(n, c->budget / per);
+    const size_t polys = dil::keyed_verify_polys(ks->level);
+    const Shape sh = shape_of(c, 2, ks->level, n, verify_task_bytes(polys));
+    const size_t per = sh.fused ? polys * POLY_BYTES : verify_task_bytes(polys);
+    size_t chunk = chunk_tasks(c, per, n);
     if (chunk == 0) return DIL_ENOMEM;
     int rc = ensure_ws(c, chunk * per);
     if (rc) return rc;
     for (size_t s0 = 0; s0 < n; s0 += chunk) {
         int m = (int)std::min(chunk, n - s0);
-        cudaError_t e = dil::launch_verify_keyed(ks->level, m, (int)ks->n, key_idx + s0, ks->pk, ks->keys, ks->tr,
-                                                 msg, msg_off + s0, sig + sigb * s0, ok + s0, (int32_t *)c->ws,
-                                                 c->warps[2][lidx(ks->level)], c->wpt[2][lidx(ks->level)],
-                                                 (cudaStream_t)stream);
+        cudaError_t e;
+        if (sh.fused) {
+            e = dil::launch_verify_keyed(ks->level, m, (int)ks->n, key_idx + s0, ks->pk, ks->keys, ks->tr, msg,
+                                         msg_off + s0, sig + sigb * s0, ok + s0, (int32_t *)c->ws, sh.warps, sh.p,
+                                         (cudaStream_t)stream);
+        } else {
+            dil::VerifyBatch b{};
+            carve_verify(b, c->ws, m, polys);
+            b.pk = ks->pk;
+            b.msg = msg;
+            b.off = msg_off + s0;
+            b.sig = sig + sigb * s0;
+            b.ok = ok + s0;
+            b.keys = ks->keys;
+            b.key_idx = key_idx + s0;
+            b.key_tr = ks->tr;
+            b.n_keys = (int)ks->n;
+            e = dil::launch_verify_batch(ks->level, dil::VERIFY_KEYED, b, sh.warps, sh.p, (cudaStream_t)stream);
+        }
         if (e != cudaSuccess) return cuda_fail(e);
     }
     return DIL_OK;
@@ -713,13 +794,15 @@ int dil_keygen_host(dil_ctx *c, int level, size_t n, const uint8_t *seeds, uint8
     int rc = ensure_stage(c, al(32 * n) + al(pkb * n) + al(skb * n));
     if (rc) return rc;
     uint8_t *d_seed = (uint8_t *)c->stage, *d_pk = d_seed + al(32 * n), *d_sk = d_pk + al(pkb * n);
-    const int w = c->warps[0][lidx(level)], p = c->wpt[0][lidx(level)];
-    return run_pipeline(c, n, dil::scratch_polys(dil::OP_KEYGEN, level) * POLY_BYTES, (cudaStream_t)stream,
+    const size_t per = dil::scratch_polys(dil::OP_KEYGEN, level) * POLY_BYTES;
+    const Shape sh = shape_of(c, 0, level, n, per);
+    return run_pipeline(c, n, per, (cudaStream_t)stream,
                         [&](size_t c0, size_t c1, cudaStream_t s, int32_t *scratch) -> int {
                             const size_t m = c1 - c0;
                             if (!h2d(d_seed + 32 * c0, seeds + 32 * c0, 32 * m, s)) return DIL_ECUDA;
-                            cudaError_t e = dil::launch_keygen(level, (int)m, d_seed + 32 * c0, d_pk + pkb * c0,
-                                                               d_sk + skb * c0, scratch, w, p, s);
+                            cudaError_t e = (sh.fused ? dil::launch_keygen : dil::launch_keygen_batch)(
+                                level, (int)m, d_seed + 32 * c0, d_pk + pkb * c0, d_sk + skb * c0, scratch, sh.warps,
+                                sh.p, s);
                             if (e != cudaSuccess) return cuda_fail(e);
                             if (!d2h(pk + pkb * c0, d_pk + pkb * c0, pkb * m, s) ||
                                 !d2h(sk + skb * c0, d_sk + skb * c0, skb * m, s))
@@ -748,7 +831,7 @@ int dil_sign_host(dil_ctx *c, int level, size_t n, const uint8_t *sk, const uint
     int32_t *d_st = (int32_t *)(d_sig + al(sigb * n));
     const int l = level == 2 ? 4 : level == 3 ? 5 : 7, cap = (65536 - l) / l + 1;
     const int max_iter = (c->max_iter > 0 && c->max_iter < cap) ? c->max_iter : cap;
-    const int w = c->warps[1][lidx(level)], p = c->wpt[1][lidx(level)];
+    const int w = fused_warps(c, 1, level), p = fused_wpt(c, 1, level);
     return run_pipeline(c, n, dil::scratch_polys(dil::OP_SIGN, level) * POLY_BYTES, (cudaStream_t)stream,
                         [&](size_t c0, size_t c1, cudaStream_t s, int32_t *scratch) -> int {
                             const size_t m = c1 - c0;
@@ -786,8 +869,9 @@ int dil_verify_host(dil_ctx *c, int level, size_t n, const uint8_t *pk, const ui
     uint64_t *d_off = (uint64_t *)(d_msg + al(mlen + 1));
     uint8_t *d_sig = (uint8_t *)d_off + al(8 * (n + 1));
     uint8_t *d_ok = d_sig + al(sigb * n);
-    const int w = c->warps[2][lidx(level)], p = c->wpt[2][lidx(level)];
-    return run_pipeline(c, n, dil::scratch_polys(dil::OP_VERIFY, level) * POLY_BYTES, (cudaStream_t)stream,
+    const size_t polys = dil::scratch_polys(dil::OP_VERIFY, level), streams = n >= PIPE_MIN_TASKS ? PIPE_STREAMS : 1;
+    const Shape sh = shape_of(c, 2, level, n, streams * verify_task_bytes(polys));
+    return run_pipeline(c, n, sh.fused ? polys * POLY_BYTES : verify_task_bytes(polys), (cudaStream_t)stream,
                         [&](size_t c0, size_t c1, cudaStream_t s, int32_t *scratch) -> int {
                             const size_t m = c1 - c0;
                             if (!h2d(d_pk + pkb * c0, pk + pkb * c0, pkb * m, s) ||
@@ -796,8 +880,20 @@ int dil_verify_host(dil_ctx *c, int level, size_t n, const uint8_t *pk, const ui
                                 !h2d(d_off + c0, msg_off + c0, 8 * (m + 1), s) ||
                                 !h2d(d_sig + sigb * c0, sig + sigb * c0, sigb * m, s))
                                 return DIL_ECUDA;
-                            cudaError_t e = dil::launch_verify(level, (int)m, d_pk + pkb * c0, d_msg, d_off + c0,
-                                                               d_sig + sigb * c0, d_ok + c0, scratch, w, p, s);
+                            cudaError_t e;
+                            if (sh.fused) {
+                                e = dil::launch_verify(level, (int)m, d_pk + pkb * c0, d_msg, d_off + c0,
+                                                       d_sig + sigb * c0, d_ok + c0, scratch, sh.warps, sh.p, s);
+                            } else {
+                                dil::VerifyBatch b{};
+                                carve_verify(b, scratch, m, polys);
+                                b.pk = d_pk + pkb * c0;
+                                b.msg = d_msg;
+                                b.off = d_off + c0;
+                                b.sig = d_sig + sigb * c0;
+                                b.ok = d_ok + c0;
+                                e = dil::launch_verify_batch(level, dil::VERIFY_PLAIN, b, sh.warps, sh.p, s);
+                            }
                             if (e != cudaSuccess) return cuda_fail(e);
                             if (!d2h(ok + c0, d_ok + c0, m, s)) return DIL_ECUDA;
                             return DIL_OK;
@@ -939,7 +1035,7 @@ int dil_test_sign_split(dil_ctx *c, int level, size_t n, const uint8_t *sk, cons
     sizes_of(level, pkb, skb, sigb);
     const int l = level == 2 ? 4 : level == 3 ? 5 : 7, cap = (65536 - l) / l + 1;
     const int max_iter = (c->max_iter > 0 && c->max_iter < cap) ? c->max_iter : cap;
-    const int p = std::min(c->wpt[1][lidx(level)], 2), w = std::max(c->warps[1][lidx(level)] / p * p, p);
+    const int p = std::min(fused_wpt(c, 1, level), 2), w = std::max(fused_warps(c, 1, level) / p * p, p);
     const size_t per = dil::scratch_polys(dil::OP_SIGN, level) * POLY_BYTES + dil::split_state_bytes();
     const size_t chunk = std::min<size_t>(n, (c->budget - 256) / per);
     if (chunk == 0) return DIL_ENOMEM;

@@ -1,8 +1,8 @@
 // Resident-A^ forms of the plain kernels: A^ = ExpandA(rho) written to a
 // caller's buffer (Alg 4; the matrix Alg 1 samples and Alg 2 / Alg 3 use in the
-// NTT domain), and Sign / Verify reading that A^ instead of sampling it.  A
-// task runs on one warp, as in the plain kernels' tuned shapes; the task
-// bodies are the plain ones (dil_procs.cuh) with the A^ source switched.
+// NTT domain), and Sign reading that A^ instead of sampling it (Verify's is a
+// source of its batch form, dil_verify.cu).  A task runs on one warp; its body
+// is the plain one (dil_procs.cuh) with the A^ source switched.
 #include "dil_kern.cuh"
 
 namespace dil {
@@ -66,30 +66,6 @@ __global__ void __launch_bounds__(256, 4) k_sign_a(int n, const uint8_t *__restr
     }
 }
 
-template <int LEVEL>
-__global__ void __launch_bounds__(256, 4) k_verify_a(int n, const uint8_t *__restrict__ pk,
-                                                     const uint8_t *__restrict__ msg,
-                                                     const uint64_t *__restrict__ off,
-                                                     const uint8_t *__restrict__ sig, const int32_t *__restrict__ ahat,
-                                                     uint8_t *ok, int32_t *scratch) {
-    extern __shared__ __align__(16) uint8_t smem[];
-    const CtaView v = cta_setup<1>(smem);
-    const int task = blockIdx.x * v.groups + v.group;
-    if (task >= n) return;
-    using V = Lv<LEVEL>;
-    uint64_t m0;
-    size_t mlen;
-    if (!message_of(off, task, m0, mlen)) {   // decreasing offsets: reject
-        if (v.lane == 0) ok[task] = 0;
-        return;
-    }
-    const int r = verify_task<LEVEL, 1, false, true>(
-        pk + (size_t)task * V::PK, msg + m0, mlen, sig + (size_t)task * V::SIG,
-        scratch + (size_t)task * Scratch<LEVEL>::VERIFY_POLYS * N, *v.gs, *v.ws, v.zt, v.izt, 0, v.bar, v.lane,
-        ahat + (size_t)task * V::K * V::L * N);
-    if (v.lane == 0) ok[task] = (uint8_t)r;
-}
-
 cudaError_t launch_expand_a(int level, int n, const uint8_t *rho, size_t rho_stride, int32_t *ahat, int warps,
                             cudaStream_t s) {
     switch (level) {
@@ -107,17 +83,6 @@ cudaError_t launch_sign_a(int level, int n, const uint8_t *sk, const uint8_t *ms
         case 2: return launch_plain(k_sign_a<2>, n, warps, 1, s, sk, msg, off, ahat, sig, status, iters, scratch, max_iter);
         case 3: return launch_plain(k_sign_a<3>, n, warps, 1, s, sk, msg, off, ahat, sig, status, iters, scratch, max_iter);
         case 5: return launch_plain(k_sign_a<5>, n, warps, 1, s, sk, msg, off, ahat, sig, status, iters, scratch, max_iter);
-    }
-    return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_verify_a(int level, int n, const uint8_t *pk, const uint8_t *msg, const uint64_t *off,
-                            const uint8_t *sig, const int32_t *ahat, uint8_t *ok, int32_t *scratch, int warps,
-                            cudaStream_t s) {
-    switch (level) {
-        case 2: return launch_plain(k_verify_a<2>, n, warps, 1, s, pk, msg, off, sig, ahat, ok, scratch);
-        case 3: return launch_plain(k_verify_a<3>, n, warps, 1, s, pk, msg, off, sig, ahat, ok, scratch);
-        case 5: return launch_plain(k_verify_a<5>, n, warps, 1, s, pk, msg, off, sig, ahat, ok, scratch);
     }
     return cudaErrorInvalidValue;
 }

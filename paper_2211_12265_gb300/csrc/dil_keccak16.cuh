@@ -70,6 +70,29 @@ __device__ __forceinline__ void k16_rho_pi(uint32_t (&b)[25], const uint32_t (&a
     if constexpr (I < 24) k16_rho_pi<I + 1>(b, a);
 }
 
+// One round on this thread's 25 state words (all 32 lanes of the warp).
+__device__ __forceinline__ void k16_round(uint32_t (&a)[25], bool high, uint64_t rc) {
+    // theta
+    uint32_t c[5], d[5];
+#pragma unroll
+    for (int x = 0; x < 5; ++x) c[x] = a[x] ^ a[x + 5] ^ a[x + 10] ^ a[x + 15] ^ a[x + 20];
+#pragma unroll
+    for (int x = 0; x < 5; ++x) d[x] = k16_rot<1>(c[x]);   // this half of rotl(C[x], 1)
+#pragma unroll
+    for (int i = 0; i < 25; ++i) a[i] ^= c[(i + 4) % 5] ^ d[(i + 1) % 5];
+    // rho + pi
+    uint32_t b[25];
+    k16_rho_pi<0>(b, a);
+    // chi
+#pragma unroll
+    for (int y = 0; y < 5; ++y)
+#pragma unroll
+        for (int x = 0; x < 5; ++x)
+            a[x + 5 * y] = b[x + 5 * y] ^ (~b[(x + 1) % 5 + 5 * y] & b[(x + 2) % 5 + 5 * y]);
+    // iota
+    a[0] ^= high ? (uint32_t)(rc >> 32) : (uint32_t)rc;
+}
+
 // Permutes the sixteen states at shared address kst (K16_WORDS words).  Called
 // by all 32 lanes of the warp.  Out of line: one copy serves every sampler.
 static __device__ __noinline__ void keccak16_permute_impl(uint32_t kst) {
@@ -80,28 +103,7 @@ static __device__ __noinline__ void keccak16_permute_impl(uint32_t kst) {
 #pragma unroll
     for (int i = 0; i < 25; ++i) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(a[i]) : "r"(base + 4 * K16_ROW * i));
 #pragma unroll 1
-    for (int round = 0; round < 24; ++round) {
-        // theta
-        uint32_t c[5], d[5];
-#pragma unroll
-        for (int x = 0; x < 5; ++x) c[x] = a[x] ^ a[x + 5] ^ a[x + 10] ^ a[x + 15] ^ a[x + 20];
-#pragma unroll
-        for (int x = 0; x < 5; ++x) d[x] = k16_rot<1>(c[x]);   // this half of rotl(C[x], 1)
-#pragma unroll
-        for (int i = 0; i < 25; ++i) a[i] ^= c[(i + 4) % 5] ^ d[(i + 1) % 5];
-        // rho + pi
-        uint32_t b[25];
-        k16_rho_pi<0>(b, a);
-        // chi
-#pragma unroll
-        for (int y = 0; y < 5; ++y)
-#pragma unroll
-            for (int x = 0; x < 5; ++x)
-                a[x + 5 * y] = b[x + 5 * y] ^ (~b[(x + 1) % 5 + 5 * y] & b[(x + 2) % 5 + 5 * y]);
-        // iota
-        const uint64_t rc = c_keccak_rc[round];
-        a[0] ^= high ? (uint32_t)(rc >> 32) : (uint32_t)rc;
-    }
+    for (int round = 0; round < 24; ++round) k16_round(a, high, c_keccak_rc[round]);
 #pragma unroll
     for (int i = 0; i < 25; ++i)
         asm volatile("st.shared.u32 [%0], %1;" ::"r"(base + 4 * K16_ROW * i), "r"(a[i]) : "memory");
@@ -115,20 +117,18 @@ __device__ __forceinline__ void keccak16_permute(uint32_t *kst) { keccak16_permu
 // tail_of(s) (the instance's nonce bytes followed by the SHAKE
 // domain/padding byte 0x1F), and the final padding bit at the last byte of
 // the rate.  Instances >= count get the same seed with tail 0 (their output is
-// never read); instances >= keep are left as they are.
+// never read).
 template <class Tail>
 __device__ __forceinline__ void keccak16_seed(uint32_t *kst, const uint32_t *seed, int seed_words, Tail tail_of,
-                                              int count, int rate, int lane, int keep = K16_STATES) {
+                                              int count, int rate, int lane) {
     const int s = lane >> 1, p = lane & 1;
     const uint32_t tail = s < count ? tail_of(s) : 0u;
-    if (s < keep) {
 #pragma unroll 1
-        for (int i = 0; i < 25; ++i) {
-            const int w = 2 * i + p;
-            uint32_t v = w < seed_words ? seed[w] : w == seed_words ? tail : 0u;
-            if (w == rate / 4 - 1) v ^= 0x80000000u;
-            kst[k16_slot(i, lane)] = v;
-        }
+    for (int i = 0; i < 25; ++i) {
+        const int w = 2 * i + p;
+        uint32_t v = w < seed_words ? seed[w] : w == seed_words ? tail : 0u;
+        if (w == rate / 4 - 1) v ^= 0x80000000u;
+        kst[k16_slot(i, lane)] = v;
     }
     __syncwarp();
 }
@@ -309,13 +309,6 @@ struct K16ChainRider {
         next = total + 1;
         __syncwarp();
     }
-};
-
-// The no-op rider of the samplers that carry none.
-struct K16NoRider {
-    static constexpr int KEEP = K16_STATES;
-    __device__ __forceinline__ void before(uint32_t *, int) {}
-    __device__ __forceinline__ void after(const uint32_t *, int) {}
 };
 
 }  // namespace dil

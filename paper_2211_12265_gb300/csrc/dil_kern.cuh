@@ -54,6 +54,27 @@ static cudaError_t launch_plain(Kern kern, int n, int warps, int p, cudaStream_t
     return cudaGetLastError();
 }
 
+// Warps that hash a batch of n tasks sixteen at a time.  One task to a pair of
+// threads while that takes at most one warp per sub-partition (608 warps);
+// beyond it two to a pair, taken as pairs come free: fewer warps then share
+// the SMs with the arithmetic, and a pair with a short message goes on to the
+// next task.
+inline int batch_hash_warps(int n) {
+    const int all = (n + 15) / 16;
+    return all <= 608 ? all : (n + 31) / 32 > 608 ? (n + 31) / 32 : 608;
+}
+
+// Launch shape of a kernel that only hashes, one task per pair of threads:
+// single-warp CTAs spread a small batch over the SMs, four-warp ones put one
+// warp on each of an SM's sub-partitions.
+struct HashGrid {
+    int blocks, threads;
+};
+inline HashGrid hash_grid(int n) {
+    const int warps = (n + 15) / 16;
+    return warps <= 152 ? HashGrid{warps, 32} : HashGrid{(warps + 3) / 4, 128};
+}
+
 // Dispatch on (level, warps per task) to kernel template K<LEVEL, P>.
 #define DIL_DISPATCH(KERN, ...)                                                                  \
     switch (level * 10 + p) {                                                                    \
@@ -64,6 +85,18 @@ static cudaError_t launch_plain(Kern kern, int n, int warps, int p, cudaStream_t
         case 32: return launch_plain(KERN<3, 2>, n, warps, p, s, __VA_ARGS__);                   \
         case 34: return launch_plain(KERN<3, 4>, n, warps, p, s, __VA_ARGS__);                   \
         case 51: return launch_plain(KERN<5, 1>, n, warps, p, s, __VA_ARGS__);                   \
+        case 52: return launch_plain(KERN<5, 2>, n, warps, p, s, __VA_ARGS__);                   \
+        case 54: return launch_plain(KERN<5, 4>, n, warps, p, s, __VA_ARGS__);                   \
+    }                                                                                            \
+    return cudaErrorInvalidValue;
+
+// As DIL_DISPATCH for kernels that exist for groups of two and four warps only.
+#define DIL_DISPATCH_GROUPS(KERN, ...)                                                           \
+    switch (level * 10 + p) {                                                                    \
+        case 22: return launch_plain(KERN<2, 2>, n, warps, p, s, __VA_ARGS__);                   \
+        case 24: return launch_plain(KERN<2, 4>, n, warps, p, s, __VA_ARGS__);                   \
+        case 32: return launch_plain(KERN<3, 2>, n, warps, p, s, __VA_ARGS__);                   \
+        case 34: return launch_plain(KERN<3, 4>, n, warps, p, s, __VA_ARGS__);                   \
         case 52: return launch_plain(KERN<5, 2>, n, warps, p, s, __VA_ARGS__);                   \
         case 54: return launch_plain(KERN<5, 4>, n, warps, p, s, __VA_ARGS__);                   \
     }                                                                                            \

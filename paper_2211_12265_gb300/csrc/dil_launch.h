@@ -25,7 +25,8 @@ size_t scratch_polys(int op, int level);
 // Dynamic shared memory of a CTA with `warps` warps.
 size_t cta_smem_bytes(int warps, int warps_per_task);
 
-// warps: warps per CTA; p: warps per task (1, 2 or 4; divides warps)
+// Fused forms, one task per group of p warps with its hashes (p: 2 or 4, for
+// Sign also 1; divides warps, the warps per CTA).
 cudaError_t launch_keygen(int level, int n, const uint8_t *seeds, uint8_t *pk, uint8_t *sk, int32_t *scratch,
                           int warps, int p, cudaStream_t s);
 cudaError_t launch_sign(int level, int n, const uint8_t *sk, const uint8_t *msg, const uint64_t *off,
@@ -33,22 +34,47 @@ cudaError_t launch_sign(int level, int n, const uint8_t *sk, const uint8_t *msg,
                         int warps, int p, cudaStream_t s);
 cudaError_t launch_verify(int level, int n, const uint8_t *pk, const uint8_t *msg, const uint64_t *off,
                           const uint8_t *sig, uint8_t *ok, int32_t *scratch, int warps, int p, cudaStream_t s);
+
+// Batch forms: the hashes of independent tasks run sixteen to a warp (dil_gen.cu,
+// dil_verify.cu); p: warps per task of the arithmetic (1 or 4; divides warps).
+cudaError_t launch_keygen_batch(int level, int n, const uint8_t *seeds, uint8_t *pk, uint8_t *sk, int32_t *scratch,
+                                int warps, int p, cudaStream_t s);
+// Where a Verify's A^ comes from: sampled, the caller's, or a resident key's.
+enum VerifySource { VERIFY_PLAIN = 0, VERIFY_AHAT = 1, VERIFY_KEYED = 2 };
+struct VerifyBatch {
+    int n;
+    const uint8_t *pk;       // task-major; VERIFY_KEYED: the store's, key-major
+    const uint8_t *msg;
+    const uint64_t *off;
+    const uint8_t *sig;
+    uint8_t *ok;
+    int32_t *scratch;        // VERIFY_PLAIN: scratch_polys(OP_VERIFY) per task, else keyed_verify_polys
+    const int32_t *ahat;     // VERIFY_AHAT
+    const int32_t *keys;     // VERIFY_KEYED: KEY_POLYS polynomials, index and tr of each key
+    const int32_t *key_idx;
+    const uint8_t *key_tr;
+    int n_keys;
+    uint32_t *mu, *tr;       // per task 16 and (not VERIFY_KEYED) 8 words
+    int *next;               // counter of the hashing warps
+    int hash_warps, hash_blocks;   // set by the launch
+};
+// Per task beside the polynomials: mu (64), tr (32) and 32 more, of which the
+// batch's counter takes the first.
+constexpr size_t VERIFY_AUX_BYTES = 128;
+cudaError_t launch_verify_batch(int level, int src, const VerifyBatch &b, int warps, int p, cudaStream_t s);
 // Loads the one-warp-per-task Sign kernel of `level` and runs it once on no
 // tasks (its code and local-memory reservation are in place afterwards).
 cudaError_t warm_sign(int level, int warps, int p, cudaStream_t s);
 
 // Resident-A^ forms (one warp per task, `warps` warps per CTA): A^ of n keys
 // from rho (task i's 32 bytes at rho + i rho_stride) into ahat (n x k l x 256
-// words, 16-byte aligned); Sign and Verify with task i's A^ at
-// ahat + i k l 256 instead of ExpandA.
+// words, 16-byte aligned); Sign with task i's A^ at ahat + i k l 256 instead of
+// ExpandA (Verify: launch_verify_batch).
 cudaError_t launch_expand_a(int level, int n, const uint8_t *rho, size_t rho_stride, int32_t *ahat, int warps,
                             cudaStream_t s);
 cudaError_t launch_sign_a(int level, int n, const uint8_t *sk, const uint8_t *msg, const uint64_t *off,
                           const int32_t *ahat, uint8_t *sig, int32_t *status, int32_t *iters, int32_t *scratch,
                           int max_iter, int warps, cudaStream_t s);
-cudaError_t launch_verify_a(int level, int n, const uint8_t *pk, const uint8_t *msg, const uint64_t *off,
-                            const uint8_t *sig, const int32_t *ahat, uint8_t *ok, int32_t *scratch, int warps,
-                            cudaStream_t s);
 
 // resident keys: per-key polynomials (A^, s^1, s^2, t^0, NTT(t1 2^d)) and
 // per-task scratch of a keyed Sign (y, y^, w, z)

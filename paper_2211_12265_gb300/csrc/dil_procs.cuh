@@ -190,21 +190,16 @@ __device__ __forceinline__ int share_lo(int g) { return g * M / P; }
 
 // A^_p (p = i l + j) for p in [lo, hi) into out + p N in index order: up to
 // sixteen sponges at a time while at least seven remain, six at a time while
-// at least three remain, then a pair or a single.  With a K16Rider the
-// sixteen-state batches take fifteen polynomials and carry the rider's hash
-// in the sixteenth instance; the hash is finished before the smaller forms
-// reuse the batches' shared memory.
-template <int LEVEL, class Rider>
-__device__ void expand_a_range(const uint8_t *rho, int lo, int hi, int32_t *out, WarpSmem &ws, int lane,
-                               Rider &rider) {
+// at least three remain, then a pair or a single.
+template <int LEVEL>
+__device__ void expand_a_range(const uint8_t *rho, int lo, int hi, int32_t *out, WarpSmem &ws, int lane) {
     constexpr int L = Lv<LEVEL>::L;
     int p = lo;
     while (hi - p >= 7) {
-        const int c = min(Rider::KEEP, hi - p);
-        expand_a_16<L>(rho, p, c, out + p * N, ws.k16, lane, rider);
+        const int c = min(K16_STATES, hi - p);
+        expand_a_16<L>(rho, p, c, out + p * N, ws.k16, lane);
         p += c;
     }
-    if constexpr (Rider::KEEP < K16_STATES) rider.finish(ws.k16, lane);
     while (hi - p >= 3) {
         const int c = min(K6_STATES, hi - p);
         expand_a_six<L>(rho, p, c, out + p * N, ws.kst, ws.kpi(), lane);
@@ -223,13 +218,6 @@ __device__ void expand_a_range(const uint8_t *rho, int lo, int hi, int32_t *out,
         store_l2(out + p * N, a, lane);
     }
     __syncwarp();
-}
-
-template <int LEVEL>
-__device__ __forceinline__ void expand_a_range(const uint8_t *rho, int lo, int hi, int32_t *out, WarpSmem &ws,
-                                               int lane) {
-    K16NoRider none;
-    expand_a_range<LEVEL>(rho, lo, hi, out, ws, lane, none);
 }
 
 // Slot of nonce u's mask polynomial y (coefficient order) in the ring.
@@ -348,8 +336,9 @@ __device__ __forceinline__ void challenge_hat(int32_t ch[8], const uint8_t *ctil
 
 // -------------------------------------------------------------------------
 // Alg 1: Gen.  seed: 32 bytes.  pk, sk: outputs.  scratch: GEN_POLYS polys.
+// SPLIT: tr = H(pk) is left to a later kernel (dil_gen.cu).
 // -------------------------------------------------------------------------
-template <int LEVEL, int P>
+template <int LEVEL, int P, bool SPLIT = false>
 __device__ void gen_task(const uint8_t *__restrict__ seed, uint8_t *pk, uint8_t *sk, int32_t *scratch,
                          GroupSmem &gs, WarpSmem &ws, const int32_t *zt, const int32_t *izt, int g, int bar,
                          int lane) {
@@ -439,41 +428,21 @@ __device__ void gen_task(const uint8_t *__restrict__ seed, uint8_t *pk, uint8_t 
         pack_seq<D>(sk + V::SK_T0 + i * V::POLYT0, t0, 1 << (D - 1), -1, lane);
     };
     constexpr int KL = V::K * V::L;
-    if constexpr (P == 1 && KL > K16_STATES) {
-        // A^ in sixteen-state batches of whole rows (R l <= 15 polynomials), the
-        // batch's rows of t computed before the next batch, and tr = H(rho || t1)
-        // riding in the batches' spare instance as far as pk is written.
-        constexpr int R = (K16_STATES - 1) / V::L;
-        K16ChainRider rider(pk, V::PK, reinterpret_cast<uint32_t *>(gs.hb), reinterpret_cast<uint32_t *>(gs.tr));
-        rider.set_ready(32);
+    // A^ = ExpandA(rho) into scratch after s^1, then the rows of t
+    expand_a_range<LEVEL>(gs.rho, share_lo<KL, P>(g), share_lo<KL, P>(g + 1), scratch + V::L * N, ws, lane);
+    group_sync<P>(bar);
 #pragma unroll 1
-        for (int i0 = 0; i0 < V::K; i0 += R) {
-            const int rows = min(R, V::K - i0);
-            expand_a_16<V::L>(gs.rho, i0 * V::L, rows * V::L, scratch + (V::L + i0 * V::L) * N, ws.k16, lane,
-                              rider);
-#pragma unroll 1
-            for (int i = i0; i < i0 + rows; ++i) row(i);
-            __syncwarp();
-            rider.set_ready(32 + (size_t)(i0 + rows) * V::POLYT1);
-        }
-        rider.finish(lane);
-        sk[64 + lane] = gs.tr[lane];
-    } else {
-        // A^ = ExpandA(rho) into scratch after s^1, then the rows of t
-        expand_a_range<LEVEL>(gs.rho, share_lo<KL, P>(g), share_lo<KL, P>(g + 1), scratch + V::L * N, ws, lane);
-        group_sync<P>(bar);
-#pragma unroll 1
-        for (int i = g; i < V::K; i += P) row(i);
-        __threadfence_block();
-        group_sync<P>(bar);
-        // tr = H(rho || t1)
-        if (g == 0) {
-            uint32_t lo = 0, hi = 0;
-            absorb_concat(lo, hi, gs.hb, 0, pk, V::PK, 136, lane);
-            if (lane < 4) {
+    for (int i = g; i < V::K; i += P) row(i);
+    if constexpr (SPLIT) return;
+    __threadfence_block();
+    group_sync<P>(bar);
+    // tr = H(rho || t1)
+    if (g == 0) {
+        uint32_t lo = 0, hi = 0;
+        absorb_concat(lo, hi, gs.hb, 0, pk, V::PK, 136, lane);
+        if (lane < 4) {
 #pragma unroll
-                for (int q = 0; q < 8; ++q) sk[64 + 8 * lane + q] = (uint8_t)((q < 4 ? lo : hi) >> (8 * (q & 3)));
-            }
+            for (int q = 0; q < 8; ++q) sk[64 + 8 * lane + q] = (uint8_t)((q < 4 ? lo : hi) >> (8 * (q & 3)));
         }
     }
 }
@@ -826,7 +795,10 @@ __device__ void sign_zero(uint8_t *sig, int g, int lane) {
 // t1 and H(pk) come from pk as in the plain form.
 // mu_in (nullable, KEYED only, global memory, 8-byte aligned): mu computed
 // beforehand.
-template <int LEVEL, int P, bool KEYED = false, bool AHAT = false>
+// SPLIT: the task's hashes run elsewhere (dil_verify.cu): nothing of msg or tr
+// is read, the packed w1' goes to the start of scratch instead of into
+// c~ = H(mu || w1'), and 1 means that only that comparison is left.
+template <int LEVEL, int P, bool KEYED = false, bool AHAT = false, bool SPLIT = false>
 __device__ int verify_task(const uint8_t *__restrict__ pk, const uint8_t *__restrict__ msg, size_t mlen,
                            const uint8_t *__restrict__ sig, int32_t *scratch, GroupSmem &gs, WarpSmem &ws,
                            const int32_t *zt, const int32_t *izt, int g, int bar, int lane,
@@ -881,23 +853,16 @@ __device__ int verify_task(const uint8_t *__restrict__ pk, const uint8_t *__rest
         ntt_fwd(r, ws.buf, zt, lane);
         store_l2(scratch + j * N, r, lane);
     }
-    // A^ = ExpandA(rho) into scratch after z^ (unless resident).  A single
-    // warp with more than one sixteen-state batch of A^ carries H(pk) in the
-    // batches' spare instance.
+    // A^ = ExpandA(rho) into scratch after z^ (unless resident)
     constexpr int KL = V::K * V::L;
-    constexpr bool RIDE = P == 1 && !KEYED && !AHAT && KL > K16_STATES;
-    if constexpr (RIDE) {
-        K16Rider rider(pk, V::PK, reinterpret_cast<uint32_t *>(gs.tr));
-        expand_a_range<LEVEL>(gs.rho, 0, KL, scratch + V::L * N, ws, lane, rider);
-    } else if (!KEYED && !AHAT) {
+    if constexpr (!KEYED && !AHAT)
         expand_a_range<LEVEL>(gs.rho, share_lo<KL, P>(g), share_lo<KL, P>(g + 1), scratch + V::L * N, ws, lane);
-    }
     // mu = H(H(rho || t1) || M), on the last warp
-    if (g == P - 1) {
+    if (!SPLIT && g == P - 1) {
         uint32_t lo = 0, hi = 0;
         if (KEYED) {
             gs.tr[lane] = __ldcg(tr + lane);
-        } else if (!RIDE) {
+        } else {
             absorb_concat(lo, hi, gs.tr, 0, pk, V::PK, 136, lane);
             squeeze_words(lo, hi, gs.tr, 4, lane);
         }
@@ -942,6 +907,11 @@ __device__ int verify_task(const uint8_t *__restrict__ pk, const uint8_t *__rest
         pack_seq<V::W1BITS>(gs.hb + HB_W1 + i * V::POLYW1, r, 0, 1, lane);
     }
     group_sync<P>(bar);
+    if constexpr (SPLIT) {   // every row has read z^ by now
+        const uint32_t *w1 = reinterpret_cast<const uint32_t *>(gs.hb + HB_W1);
+        for (int i = 32 * g + lane; i < V::K * V::POLYW1 / 4; i += 32 * P) scratch[i] = (int32_t)w1[i];
+        return 1;
+    }
     // c~ == H(mu || w1')
     if (g == 0) {
         uint32_t lo = 0, hi = 0;

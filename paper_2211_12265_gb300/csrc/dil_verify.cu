@@ -1,5 +1,15 @@
-// Plain Verify kernel (Alg 3): one task per group of P warps, A^ sampled on
-// the fly row by row (section 3.5).
+// Verify of a batch (Alg 3).
+//
+// Batch form: two kernels.  The first gives its leading blocks to the hashes
+// tr = H(pk) and mu = H(tr || M), sixteen tasks to a warp, and the others to
+// the arithmetic, one task per group of P warps up to the packed w1'; the two
+// halves of a task never wait on each other.  The second recomputes
+// c~ = H(mu || w1'), sixteen tasks to a warp, and compares.  Hashing inside
+// the task's own warp (k_verify, kept for the launch shapes a caller asks for)
+// runs the 18 blocks of a Dilithium2 task at 18.7 SM clocks per round, 8.1 k
+// of the task's 20.7 k clocks; sixteen to a warp they take 1.4 k.  10,000 tasks:
+// Dilithium2 656 -> 491 us, Dilithium5 (32 B - 4 KB) 1815 -> 1564 us.
+#include "dil_hash16.cuh"
 #include "dil_kern.cuh"
 
 namespace dil {
@@ -29,7 +39,205 @@ __global__ void __launch_bounds__(256, 4) k_verify(int n, const uint8_t *__restr
 
 cudaError_t launch_verify(int level, int n, const uint8_t *pk, const uint8_t *msg, const uint64_t *off,
                           const uint8_t *sig, uint8_t *ok, int32_t *scratch, int warps, int p, cudaStream_t s) {
-    DIL_DISPATCH(k_verify, pk, msg, off, sig, ok, scratch)
+    DIL_DISPATCH_GROUPS(k_verify, pk, msg, off, sig, ok, scratch)
+}
+
+// ---------------------------------------------------------------- batch form
+
+// Scratch polynomials of one task of the batch form.
+template <int LEVEL, int SRC>
+__host__ __device__ constexpr int verify_polys() {
+    return SRC == VERIFY_PLAIN ? Scratch<LEVEL>::VERIFY_POLYS : Scratch<LEVEL>::KEYED_VERIFY_POLYS;
+}
+
+// Task t's message (and resident key); false when the task is to be rejected.
+template <int SRC>
+__device__ __forceinline__ bool verify_input(const VerifyBatch &b, int t, int &key, uint64_t &m0, size_t &mlen) {
+    key = t;
+    if (SRC == VERIFY_KEYED) {
+        key = b.key_idx[t];
+        if (key < 0 || key >= b.n_keys) return false;
+    }
+    return message_of(b.off, t, m0, mlen);
+}
+
+static_assert(HASH16_STAGE_WORDS * sizeof(uint32_t) <= sizeof(WarpSmem), "the hashing warps' shared memory");
+
+// tr = H(pk) (not for resident keys) and mu = H(tr || M) of a pair's tasks:
+// the first by the pair's index, the next ones from the batch's counter.
+template <int LEVEL, int SRC>
+struct VerifyMuJob {
+    const VerifyBatch &b;
+    int task, lane;
+    bool first, have_tr;
+
+    __device__ VerifyMuJob(const VerifyBatch &b_, int pair, int lane_)
+        : b(b_), task(pair), lane(lane_), first(true), have_tr(false) {}
+
+    __device__ __forceinline__ bool next(HashInput &in) {
+        using V = Lv<LEVEL>;
+        uint64_t m0 = 0;
+        size_t mlen = 0;
+        int key;
+        if (!have_tr) {
+            for (;;) {
+                if (!first) {
+                    const int claimed = b.hash_warps * K16_STATES;   // one for every pair to start with
+                    if (b.n <= claimed) return false;                // (the counter is not set up either)
+                    int c = 0;
+                    if (!(lane & 1)) c = atomicAdd(b.next, 1);
+                    task = claimed + pair_bcast(c, lane);
+                }
+                first = false;
+                if (task >= b.n) return false;
+                if (verify_input<SRC>(b, task, key, m0, mlen)) break;
+            }
+            if (SRC != VERIFY_KEYED) {
+                in = {nullptr, b.pk + (size_t)task * V::PK, (size_t)V::PK, 0};
+                return true;
+            }
+        }
+        verify_input<SRC>(b, task, key, m0, mlen);
+        const uint8_t *tr = SRC == VERIFY_KEYED ? b.key_tr + (size_t)key * 32
+                                                : reinterpret_cast<const uint8_t *>(b.tr + (size_t)task * 8);
+        in = {tr, b.msg + m0, 32 + mlen, 32};
+        return true;
+    }
+
+    __device__ __forceinline__ void done(const uint32_t (&a)[25]) {
+        const int p = lane & 1;
+        if (SRC != VERIFY_KEYED && !have_tr) {   // the words this thread reads back as the prefix of mu's input
+#pragma unroll
+            for (int i = 0; i < 4; ++i) b.tr[(size_t)task * 8 + 2 * i + p] = a[i];
+            have_tr = true;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) b.mu[(size_t)task * 16 + 2 * i + p] = a[i];
+            have_tr = false;
+        }
+    }
+};
+
+template <int LEVEL, int P, int SRC>
+__global__ void __launch_bounds__(256, 4) k_verify_batch(int, const VerifyBatch b) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    using V = Lv<LEVEL>;
+    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if ((int)blockIdx.x < b.hash_blocks) {
+        const int w = blockIdx.x * warps + warp;
+        if (w >= b.hash_warps) return;
+        VerifyMuJob<LEVEL, SRC> job(b, w * K16_STATES + (lane >> 1), lane);
+        hash16_run(job, reinterpret_cast<uint32_t *>(smem) + warp * HASH16_STAGE_WORDS, lane);
+        return;
+    }
+    const CtaView v = cta_setup<P>(smem);
+    const int task = (blockIdx.x - b.hash_blocks) * v.groups + v.group;
+    if (task >= b.n) return;
+    int key;
+    uint64_t m0;
+    size_t mlen;
+    int r = 0;
+    if (verify_input<SRC>(b, task, key, m0, mlen)) {
+        const int32_t *a = SRC == VERIFY_AHAT    ? b.ahat + (size_t)task * V::K * V::L * N
+                           : SRC == VERIFY_KEYED ? b.keys + (size_t)key * Scratch<LEVEL>::KEY_POLYS * N
+                                                 : nullptr;
+        r = verify_task<LEVEL, P, SRC == VERIFY_KEYED, SRC == VERIFY_AHAT, true>(
+            b.pk + (size_t)key * V::PK, nullptr, 0, b.sig + (size_t)task * V::SIG,
+            b.scratch + (size_t)task * verify_polys<LEVEL, SRC>() * N, *v.gs, *v.ws, v.zt, v.izt, v.g, v.bar, v.lane,
+            a);
+    }
+    if (v.g == 0 && v.lane == 0) b.ok[task] = (uint8_t)r;   // 1: c~ decides (k_verify_compare)
+}
+
+// c~ = H(mu || w1') of task `pair` against the signature's.
+template <int LEVEL, int SRC>
+struct VerifyCompareJob {
+    const VerifyBatch &b;
+    int task, lane;
+    bool todo;
+
+    __device__ VerifyCompareJob(const VerifyBatch &b_, int pair, int lane_)
+        : b(b_), task(pair), lane(lane_), todo(pair < b_.n && b_.ok[pair]) {}
+
+    __device__ __forceinline__ bool next(HashInput &in) {
+        using V = Lv<LEVEL>;
+        if (!todo) return false;
+        todo = false;
+        in = {reinterpret_cast<const uint8_t *>(b.mu + (size_t)task * 16),
+              reinterpret_cast<const uint8_t *>(b.scratch + (size_t)task * verify_polys<LEVEL, SRC>() * N),
+              64 + V::K * V::POLYW1, 64};
+        return true;
+    }
+
+    __device__ __forceinline__ void done(const uint32_t (&a)[25]) {
+        const uint8_t *ct = b.sig + (size_t)task * Lv<LEVEL>::SIG + 4 * (lane & 1);
+        bool eq = true;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) eq &= ld_bytes4(ct + 8 * i, 4) == a[i];
+        const bool other = __shfl_xor_sync(3u << (lane & 30), eq, 1);
+        if (!(eq && other) && !(lane & 1)) b.ok[task] = 0;
+    }
+};
+
+template <int LEVEL, int SRC>
+__global__ void __launch_bounds__(128) k_verify_compare(const VerifyBatch b) {
+    __shared__ uint32_t stage[4][HASH16_STAGE_WORDS];
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (w * K16_STATES >= b.n) return;
+    VerifyCompareJob<LEVEL, SRC> job(b, w * K16_STATES + (lane >> 1), lane);
+    hash16_run(job, stage[threadIdx.x >> 5], lane);
+}
+
+namespace {
+
+template <int LEVEL, int P, int SRC>
+cudaError_t launch_batch(VerifyBatch b, int warps, cudaStream_t s) {
+    b.hash_warps = batch_hash_warps(b.n);
+    b.hash_blocks = (b.hash_warps + warps - 1) / warps;
+    cudaError_t e = cudaSuccess;
+    if (b.n > b.hash_warps * K16_STATES) e = cudaMemsetAsync(b.next, 0, sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    const int groups = warps / P;
+    const size_t smem = cta_bytes(warps, P);
+    e = cudaFuncSetAttribute(k_verify_batch<LEVEL, P, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_verify_batch<LEVEL, P, SRC><<<b.hash_blocks + (b.n + groups - 1) / groups, warps * 32, smem, s>>>(b.n, b);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const HashGrid h = hash_grid(b.n);
+    k_verify_compare<LEVEL, SRC><<<h.blocks, h.threads, 0, s>>>(b);
+    return cudaGetLastError();
+}
+
+template <int LEVEL, int SRC>
+cudaError_t launch_batch_p(const VerifyBatch &b, int warps, int p, cudaStream_t s) {
+    switch (p) {
+        case 1: return launch_batch<LEVEL, 1, SRC>(b, warps, s);
+        case 4: return launch_batch<LEVEL, 4, SRC>(b, warps, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+template <int LEVEL>
+cudaError_t launch_batch_src(int src, const VerifyBatch &b, int warps, int p, cudaStream_t s) {
+    switch (src) {
+        case VERIFY_PLAIN: return launch_batch_p<LEVEL, VERIFY_PLAIN>(b, warps, p, s);
+        case VERIFY_AHAT: return launch_batch_p<LEVEL, VERIFY_AHAT>(b, warps, p, s);
+        case VERIFY_KEYED: return launch_batch_p<LEVEL, VERIFY_KEYED>(b, warps, p, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+cudaError_t launch_verify_batch(int level, int src, const VerifyBatch &b, int warps, int p, cudaStream_t s) {
+    if (b.n <= 0) return cudaSuccess;
+    switch (level) {
+        case 2: return launch_batch_src<2>(src, b, warps, p, s);
+        case 3: return launch_batch_src<3>(src, b, warps, p, s);
+        case 5: return launch_batch_src<5>(src, b, warps, p, s);
+    }
+    return cudaErrorInvalidValue;
 }
 
 size_t cta_smem_bytes(int warps, int p) { return cta_bytes(warps, p); }
