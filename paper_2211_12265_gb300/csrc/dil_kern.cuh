@@ -28,7 +28,7 @@ __device__ __forceinline__ CtaView cta_setup(uint8_t *smem) {
     const int warps = blockDim.x >> 5;
     v.groups = warps / P;
     v.zt = reinterpret_cast<int32_t *>(smem);
-    v.izt = v.zt + 256;
+    v.izt = v.zt + NTT_TABLE_WORDS;
     GroupSmem *gsa = reinterpret_cast<GroupSmem *>(smem + CTA_TABLE_BYTES);
     WarpSmem *wsa = reinterpret_cast<WarpSmem *>(smem + CTA_TABLE_BYTES + v.groups * sizeof(GroupSmem));
     load_zetas(v.zt, v.izt);

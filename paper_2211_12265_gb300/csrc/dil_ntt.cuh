@@ -4,8 +4,11 @@
 // and the exchanges are padded so that no two lanes of a warp hit one bank).
 //
 // Output order (round-3 reading): index j holds f(zeta^(2 brv8(j) + 1)),
-// zeta = 1753.  Twiddles are zeta^brv8(k) (forward) and zeta^-brv8(k)
-// (inverse) in Montgomery form (times 2^32 mod q).
+// zeta = 1753.  Twiddles are z = zeta^brv8(k) (forward) and zeta^-brv8(k)
+// (inverse), centred, each with its quotient zs = round(2^32 z / q): a product
+// by a known factor is then z b - floor(zs b / 2^32) q (Shoup), one high and
+// two low multiplies with the additions of the butterfly folded in, instead of
+// a Montgomery product's two high and two low ones and three additions.
 //
 // Register layouts of the 8 values r[0..7] held by lane t:
 //   L0: coefficient t + 32 m           (natural order, coalesced loads)
@@ -20,9 +23,11 @@
 namespace dil {
 
 struct Zetas {
-    int32_t z[256];   // zeta^brv8(k) * 2^32 mod q, centred
-    int32_t iz[256];  // zeta^-brv8(k) * 2^32 mod q, centred
+    int32_t z[256], zs[256];     // zeta^brv8(k) mod q, centred, and its quotient
+    int32_t iz[256], izs[256];   // zeta^-brv8(k)
 };
+// Shared words of one direction's twiddles: z, then zs.
+constexpr int NTT_TABLE_WORDS = 512;
 
 namespace detail {
 constexpr int64_t cpow(int64_t b, int64_t e) {
@@ -48,12 +53,20 @@ constexpr int32_t centre(int64_t v) {
     if (v < 0) v += Q;
     return (int32_t)(v > (Q - 1) / 2 ? v - Q : v);
 }
+// round(2^32 z / q) for |z| <= (q - 1) / 2; |result| < 2^31
+constexpr int32_t quotient(int32_t z) {
+    const int64_t a = z < 0 ? -(int64_t)z : z;
+    const int64_t v = ((a << 32) + Q / 2) / Q;
+    return (int32_t)(z < 0 ? -v : v);
+}
 constexpr Zetas make_zetas() {
     Zetas t{};
     for (unsigned k = 0; k < 256; ++k) {
         int64_t e = cbrv8(k);
-        t.z[k] = centre(cpow(1753, e) * MONT);
-        t.iz[k] = centre(cpow(1753, 512 - e) * MONT);   // zeta^512 = 1
+        t.z[k] = centre(cpow(1753, e));
+        t.zs[k] = quotient(t.z[k]);
+        t.iz[k] = centre(cpow(1753, 512 - e));   // zeta^512 = 1
+        t.izs[k] = quotient(t.iz[k]);
     }
     return t;
 }
@@ -66,16 +79,25 @@ static __constant__ Zetas c_zetas = detail::make_zetas();
 constexpr int32_t NTT_F = detail::centre(detail::MONT * detail::MONT % Q * detail::cpow(256, Q - 2));
 constexpr int32_t NTT_G = detail::centre((int64_t)NTT_F * detail::cpow(1753, 512 - detail::cbrv8(1)) % Q);
 
-__device__ __forceinline__ void ct_bfly(int32_t &a, int32_t &b, int32_t z) {
-    int32_t t = mont_mul(z, b);
-    b = a - t;
-    a = a + t;
+// c + z b mod q, in c + [-|b| 2^-33 q, (1 + |b| 2^-33) q): the quotient's
+// rounding moves floor(zs b / 2^32) by at most |b| 2^-33 from floor(z b / q).
+// The sums are taken mod 2^32 and fit 32 bits.
+__device__ __forceinline__ int32_t mul_add_z(int32_t c, int32_t b, int32_t z, int32_t zs) {
+    return (int32_t)((uint32_t)c + (uint32_t)z * (uint32_t)b - (uint32_t)__mulhi(b, zs) * (uint32_t)Q);
 }
 
-__device__ __forceinline__ void gs_bfly(int32_t &a, int32_t &b, int32_t z) {
-    int32_t t = a;
-    a = t + b;
-    b = mont_mul(z, t - b);
+// (a, b) <- (a + z b, a - z b)
+__device__ __forceinline__ void ct_bfly(int32_t &a, int32_t &b, int32_t z, int32_t zs) {
+    const int32_t s = mul_add_z(a, b, z, zs);
+    b = (int32_t)(2u * (uint32_t)a - (uint32_t)s);
+    a = s;
+}
+
+// (a, b) <- (a + b, z (a - b))
+__device__ __forceinline__ void gs_bfly(int32_t &a, int32_t &b, int32_t z, int32_t zs) {
+    const int32_t d = a - b;
+    a = a + b;
+    b = mul_add_z(0, d, z, zs);
 }
 
 // Shared-memory accesses by 32-bit shared-window address (the out-of-line
@@ -114,8 +136,9 @@ struct Poly8 {
     int32_t v[8];
 };
 
-// Forward NTT.  In: L0, |r| < q.  Out: L2, |r| < 9q, unscaled.  buf: the
-// warp's exchange buffer (288 words), zt: the forward twiddles (shared).
+// Forward NTT.  In: L0, |r| < q.  Out: L2, |r| < 9.1q, unscaled (a level adds
+// at most 1.01q).  buf: the warp's exchange buffer (288 words), zt: the
+// forward twiddles (shared).
 // Out of line: one copy of the code serves every call site, which keeps the
 // fused kernels' instruction footprint small.
 static __device__ __noinline__ Poly8 ntt_fwd_impl(Poly8 p, uint32_t buf, uint32_t zt) {
@@ -123,20 +146,20 @@ static __device__ __noinline__ Poly8 ntt_fwd_impl(Poly8 p, uint32_t buf, uint32_
     int32_t *r = p.v;
     // level 1 (len 128): pairs (m, m+4)
     {
-        const int32_t z = c_zetas.z[1];
+        const int32_t z = c_zetas.z[1], zs = c_zetas.zs[1];
 #pragma unroll
-        for (int m = 0; m < 4; ++m) ct_bfly(r[m], r[m + 4], z);
+        for (int m = 0; m < 4; ++m) ct_bfly(r[m], r[m + 4], z, zs);
     }
     // level 2 (len 64): pairs (m, m+2), twiddle 2 + m/4
-    ct_bfly(r[0], r[2], c_zetas.z[2]);
-    ct_bfly(r[1], r[3], c_zetas.z[2]);
-    ct_bfly(r[4], r[6], c_zetas.z[3]);
-    ct_bfly(r[5], r[7], c_zetas.z[3]);
+    ct_bfly(r[0], r[2], c_zetas.z[2], c_zetas.zs[2]);
+    ct_bfly(r[1], r[3], c_zetas.z[2], c_zetas.zs[2]);
+    ct_bfly(r[4], r[6], c_zetas.z[3], c_zetas.zs[3]);
+    ct_bfly(r[5], r[7], c_zetas.z[3], c_zetas.zs[3]);
     // level 3 (len 32): pairs (m, m+1), twiddle 4 + m/2
-    ct_bfly(r[0], r[1], c_zetas.z[4]);
-    ct_bfly(r[2], r[3], c_zetas.z[5]);
-    ct_bfly(r[4], r[5], c_zetas.z[6]);
-    ct_bfly(r[6], r[7], c_zetas.z[7]);
+    ct_bfly(r[0], r[1], c_zetas.z[4], c_zetas.zs[4]);
+    ct_bfly(r[2], r[3], c_zetas.z[5], c_zetas.zs[5]);
+    ct_bfly(r[4], r[5], c_zetas.z[6], c_zetas.zs[6]);
+    ct_bfly(r[6], r[7], c_zetas.z[7], c_zetas.zs[7]);
     // exchange L0 -> L1
 #pragma unroll
     for (int m = 0; m < 8; ++m) sts32(buf + 4 * (lane + 36 * m), r[m]);
@@ -148,25 +171,25 @@ static __device__ __noinline__ Poly8 ntt_fwd_impl(Poly8 p, uint32_t buf, uint32_
     __syncwarp();
     // level 4 (len 16): pairs (m, m+4), twiddle 8 + b
     {
-        const int32_t z = ldz32(zt + 4 * (8 + b));
+        const int32_t z = ldz32(zt + 4 * (8 + b)), zs = ldz32(zt + 1024 + 4 * (8 + b));
 #pragma unroll
-        for (int m = 0; m < 4; ++m) ct_bfly(r[m], r[m + 4], z);
+        for (int m = 0; m < 4; ++m) ct_bfly(r[m], r[m + 4], z, zs);
     }
     // level 5 (len 8): pairs (m, m+2), twiddles 16 + 2b + {0, 1}
     {
-        const int2 z = ldz64(zt + 4 * (16 + 2 * b));
-        ct_bfly(r[0], r[2], z.x);
-        ct_bfly(r[1], r[3], z.x);
-        ct_bfly(r[4], r[6], z.y);
-        ct_bfly(r[5], r[7], z.y);
+        const int2 z = ldz64(zt + 4 * (16 + 2 * b)), zs = ldz64(zt + 1024 + 4 * (16 + 2 * b));
+        ct_bfly(r[0], r[2], z.x, zs.x);
+        ct_bfly(r[1], r[3], z.x, zs.x);
+        ct_bfly(r[4], r[6], z.y, zs.y);
+        ct_bfly(r[5], r[7], z.y, zs.y);
     }
     // level 6 (len 4): pairs (m, m+1), twiddles 32 + 4b + {0..3}
     {
-        const int4 z = ldz128(zt + 4 * (32 + 4 * b));
-        ct_bfly(r[0], r[1], z.x);
-        ct_bfly(r[2], r[3], z.y);
-        ct_bfly(r[4], r[5], z.z);
-        ct_bfly(r[6], r[7], z.w);
+        const int4 z = ldz128(zt + 4 * (32 + 4 * b)), zs = ldz128(zt + 1024 + 4 * (32 + 4 * b));
+        ct_bfly(r[0], r[1], z.x, zs.x);
+        ct_bfly(r[2], r[3], z.y, zs.y);
+        ct_bfly(r[4], r[5], z.z, zs.z);
+        ct_bfly(r[6], r[7], z.w, zs.w);
     }
     // exchange L1 -> L2
 #pragma unroll
@@ -178,44 +201,47 @@ static __device__ __noinline__ Poly8 ntt_fwd_impl(Poly8 p, uint32_t buf, uint32_
     // level 7 (len 2): pairs (m, m+2), twiddles 64 + 2t + {0, 1} (one 8-byte
     // load per lane: a half-warp reads 128 contiguous bytes, conflict-free)
     {
-        const int2 z = ldz64(zt + 4 * (64 + 2 * lane));
-        ct_bfly(r[0], r[2], z.x);
-        ct_bfly(r[1], r[3], z.x);
-        ct_bfly(r[4], r[6], z.y);
-        ct_bfly(r[5], r[7], z.y);
+        const int2 z = ldz64(zt + 4 * (64 + 2 * lane)), zs = ldz64(zt + 1024 + 4 * (64 + 2 * lane));
+        ct_bfly(r[0], r[2], z.x, zs.x);
+        ct_bfly(r[1], r[3], z.x, zs.x);
+        ct_bfly(r[4], r[6], z.y, zs.y);
+        ct_bfly(r[5], r[7], z.y, zs.y);
     }
     // level 8 (len 1): pairs (m, m+1), twiddles 128 + 4t + {0..3} (16-byte load)
     {
-        const int4 z = ldz128(zt + 4 * (128 + 4 * lane));
-        ct_bfly(r[0], r[1], z.x);
-        ct_bfly(r[2], r[3], z.y);
-        ct_bfly(r[4], r[5], z.z);
-        ct_bfly(r[6], r[7], z.w);
+        const int4 z = ldz128(zt + 4 * (128 + 4 * lane)), zs = ldz128(zt + 1024 + 4 * (128 + 4 * lane));
+        ct_bfly(r[0], r[1], z.x, zs.x);
+        ct_bfly(r[2], r[3], z.y, zs.y);
+        ct_bfly(r[4], r[5], z.z, zs.z);
+        ct_bfly(r[6], r[7], z.w, zs.w);
     }
     return p;
 }
 
 // Inverse NTT.  In: L2, |r| < q.  Out: L0, |r| < q, equal to INTT(in) * 2^32,
-// so it turns pointwise Montgomery products into plain coefficients.
+// so it turns pointwise Montgomery products into plain coefficients.  A sum
+// doubles per level and stays within 256 (q - 1) < 2^31 at the last; a product
+// lies in [-q/4, 5q/4), so it never exceeds the sums of its level.  The last
+// level keeps the Montgomery product, whose result is below q.
 // izt: the inverse twiddles in shared memory.
 static __device__ __noinline__ Poly8 ntt_inv_impl(Poly8 p, uint32_t buf, uint32_t izt) {
     const int lane = threadIdx.x & 31;
     int32_t *r = p.v;
     // len 1: pairs (m, m+1), twiddles 128 + 4t + {0..3}
     {
-        const int4 z = ldz128(izt + 4 * (128 + 4 * lane));
-        gs_bfly(r[0], r[1], z.x);
-        gs_bfly(r[2], r[3], z.y);
-        gs_bfly(r[4], r[5], z.z);
-        gs_bfly(r[6], r[7], z.w);
+        const int4 z = ldz128(izt + 4 * (128 + 4 * lane)), zs = ldz128(izt + 1024 + 4 * (128 + 4 * lane));
+        gs_bfly(r[0], r[1], z.x, zs.x);
+        gs_bfly(r[2], r[3], z.y, zs.y);
+        gs_bfly(r[4], r[5], z.z, zs.z);
+        gs_bfly(r[6], r[7], z.w, zs.w);
     }
     // len 2: pairs (m, m+2), twiddles 64 + 2t + {0, 1}
     {
-        const int2 z = ldz64(izt + 4 * (64 + 2 * lane));
-        gs_bfly(r[0], r[2], z.x);
-        gs_bfly(r[1], r[3], z.x);
-        gs_bfly(r[4], r[6], z.y);
-        gs_bfly(r[5], r[7], z.y);
+        const int2 z = ldz64(izt + 4 * (64 + 2 * lane)), zs = ldz64(izt + 1024 + 4 * (64 + 2 * lane));
+        gs_bfly(r[0], r[2], z.x, zs.x);
+        gs_bfly(r[1], r[3], z.x, zs.x);
+        gs_bfly(r[4], r[6], z.y, zs.y);
+        gs_bfly(r[5], r[7], z.y, zs.y);
     }
     // exchange L2 -> L1
 #pragma unroll
@@ -228,25 +254,25 @@ static __device__ __noinline__ Poly8 ntt_inv_impl(Poly8 p, uint32_t buf, uint32_
     __syncwarp();
     // len 4: pairs (m, m+1), twiddles 32 + 4b + {0..3}
     {
-        const int4 z = ldz128(izt + 4 * (32 + 4 * b));
-        gs_bfly(r[0], r[1], z.x);
-        gs_bfly(r[2], r[3], z.y);
-        gs_bfly(r[4], r[5], z.z);
-        gs_bfly(r[6], r[7], z.w);
+        const int4 z = ldz128(izt + 4 * (32 + 4 * b)), zs = ldz128(izt + 1024 + 4 * (32 + 4 * b));
+        gs_bfly(r[0], r[1], z.x, zs.x);
+        gs_bfly(r[2], r[3], z.y, zs.y);
+        gs_bfly(r[4], r[5], z.z, zs.z);
+        gs_bfly(r[6], r[7], z.w, zs.w);
     }
     // len 8: pairs (m, m+2), twiddles 16 + 2b + {0, 1}
     {
-        const int2 z = ldz64(izt + 4 * (16 + 2 * b));
-        gs_bfly(r[0], r[2], z.x);
-        gs_bfly(r[1], r[3], z.x);
-        gs_bfly(r[4], r[6], z.y);
-        gs_bfly(r[5], r[7], z.y);
+        const int2 z = ldz64(izt + 4 * (16 + 2 * b)), zs = ldz64(izt + 1024 + 4 * (16 + 2 * b));
+        gs_bfly(r[0], r[2], z.x, zs.x);
+        gs_bfly(r[1], r[3], z.x, zs.x);
+        gs_bfly(r[4], r[6], z.y, zs.y);
+        gs_bfly(r[5], r[7], z.y, zs.y);
     }
     // len 16: pairs (m, m+4), twiddle 8 + b
     {
-        const int32_t z = ldz32(izt + 4 * (8 + b));
+        const int32_t z = ldz32(izt + 4 * (8 + b)), zs = ldz32(izt + 1024 + 4 * (8 + b));
 #pragma unroll
-        for (int m = 0; m < 4; ++m) gs_bfly(r[m], r[m + 4], z);
+        for (int m = 0; m < 4; ++m) gs_bfly(r[m], r[m + 4], z, zs);
     }
     // exchange L1 -> L0
 #pragma unroll
@@ -256,15 +282,15 @@ static __device__ __noinline__ Poly8 ntt_inv_impl(Poly8 p, uint32_t buf, uint32_
     for (int m = 0; m < 8; ++m) r[m] = lds32(buf + 4 * (lane + 36 * m));
     __syncwarp();
     // len 32: pairs (m, m+1), twiddle 4 + m/2
-    gs_bfly(r[0], r[1], c_zetas.iz[4]);
-    gs_bfly(r[2], r[3], c_zetas.iz[5]);
-    gs_bfly(r[4], r[5], c_zetas.iz[6]);
-    gs_bfly(r[6], r[7], c_zetas.iz[7]);
+    gs_bfly(r[0], r[1], c_zetas.iz[4], c_zetas.izs[4]);
+    gs_bfly(r[2], r[3], c_zetas.iz[5], c_zetas.izs[5]);
+    gs_bfly(r[4], r[5], c_zetas.iz[6], c_zetas.izs[6]);
+    gs_bfly(r[6], r[7], c_zetas.iz[7], c_zetas.izs[7]);
     // len 64: pairs (m, m+2), twiddle 2 + m/4
-    gs_bfly(r[0], r[2], c_zetas.iz[2]);
-    gs_bfly(r[1], r[3], c_zetas.iz[2]);
-    gs_bfly(r[4], r[6], c_zetas.iz[3]);
-    gs_bfly(r[5], r[7], c_zetas.iz[3]);
+    gs_bfly(r[0], r[2], c_zetas.iz[2], c_zetas.izs[2]);
+    gs_bfly(r[1], r[3], c_zetas.iz[2], c_zetas.izs[2]);
+    gs_bfly(r[4], r[6], c_zetas.iz[3], c_zetas.izs[3]);
+    gs_bfly(r[5], r[7], c_zetas.iz[3], c_zetas.izs[3]);
     // len 128 with the factor 2^32/n folded in (twiddle 1)
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
@@ -295,11 +321,19 @@ __device__ __forceinline__ void ntt_inv(int32_t r[8], int32_t *buf, const int32_
     for (int m = 0; m < 8; ++m) r[m] = p.v[m];
 }
 
-// Loads the twiddle tables into shared memory (whole block participates).
-__device__ __forceinline__ void load_zetas(int32_t *zt, int32_t *izt) {
+// Loads the twiddle tables (NTT_TABLE_WORDS each) into shared memory (whole
+// block participates).
+__device__ __forceinline__ void load_zetas_fwd(int32_t *zt) {
     for (int i = threadIdx.x; i < 256; i += blockDim.x) {
         zt[i] = c_zetas.z[i];
+        zt[256 + i] = c_zetas.zs[i];
+    }
+}
+__device__ __forceinline__ void load_zetas(int32_t *zt, int32_t *izt) {
+    load_zetas_fwd(zt);
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
         izt[i] = c_zetas.iz[i];
+        izt[256 + i] = c_zetas.izs[i];
     }
 }
 

@@ -191,18 +191,18 @@ static __device__ __noinline__ Poly8 ntt_fwd_unpadded_impl(Poly8 p, uint32_t buf
     const int lane = threadIdx.x & 31;
     int32_t *r = p.v;
     {
-        const int32_t z = c_zetas.z[1];
+        const int32_t z = c_zetas.z[1], zs = c_zetas.zs[1];
 #pragma unroll
-        for (int m = 0; m < 4; ++m) ct_bfly(r[m], r[m + 4], z);
+        for (int m = 0; m < 4; ++m) ct_bfly(r[m], r[m + 4], z, zs);
     }
-    ct_bfly(r[0], r[2], c_zetas.z[2]);
-    ct_bfly(r[1], r[3], c_zetas.z[2]);
-    ct_bfly(r[4], r[6], c_zetas.z[3]);
-    ct_bfly(r[5], r[7], c_zetas.z[3]);
-    ct_bfly(r[0], r[1], c_zetas.z[4]);
-    ct_bfly(r[2], r[3], c_zetas.z[5]);
-    ct_bfly(r[4], r[5], c_zetas.z[6]);
-    ct_bfly(r[6], r[7], c_zetas.z[7]);
+    ct_bfly(r[0], r[2], c_zetas.z[2], c_zetas.zs[2]);
+    ct_bfly(r[1], r[3], c_zetas.z[2], c_zetas.zs[2]);
+    ct_bfly(r[4], r[6], c_zetas.z[3], c_zetas.zs[3]);
+    ct_bfly(r[5], r[7], c_zetas.z[3], c_zetas.zs[3]);
+    ct_bfly(r[0], r[1], c_zetas.z[4], c_zetas.zs[4]);
+    ct_bfly(r[2], r[3], c_zetas.z[5], c_zetas.zs[5]);
+    ct_bfly(r[4], r[5], c_zetas.z[6], c_zetas.zs[6]);
+    ct_bfly(r[6], r[7], c_zetas.z[7], c_zetas.zs[7]);
     // L0 -> L1: coefficient t + 32 m, read back as 32 (t >> 2) + (t & 3) + 4 m
 #pragma unroll
     for (int m = 0; m < 8; ++m) sts32(buf + 4 * (lane + 32 * m), r[m]);
@@ -213,23 +213,23 @@ static __device__ __noinline__ Poly8 ntt_fwd_unpadded_impl(Poly8 p, uint32_t buf
     for (int m = 0; m < 8; ++m) r[m] = lds32(base1 + 16 * m);
     __syncwarp();
     {
-        const int32_t z = ldz32(zt + 4 * (8 + b));
+        const int32_t z = ldz32(zt + 4 * (8 + b)), zs = ldz32(zt + 1024 + 4 * (8 + b));
 #pragma unroll
-        for (int m = 0; m < 4; ++m) ct_bfly(r[m], r[m + 4], z);
+        for (int m = 0; m < 4; ++m) ct_bfly(r[m], r[m + 4], z, zs);
     }
     {
-        const int2 z = ldz64(zt + 4 * (16 + 2 * b));
-        ct_bfly(r[0], r[2], z.x);
-        ct_bfly(r[1], r[3], z.x);
-        ct_bfly(r[4], r[6], z.y);
-        ct_bfly(r[5], r[7], z.y);
+        const int2 z = ldz64(zt + 4 * (16 + 2 * b)), zs = ldz64(zt + 1024 + 4 * (16 + 2 * b));
+        ct_bfly(r[0], r[2], z.x, zs.x);
+        ct_bfly(r[1], r[3], z.x, zs.x);
+        ct_bfly(r[4], r[6], z.y, zs.y);
+        ct_bfly(r[5], r[7], z.y, zs.y);
     }
     {
-        const int4 z = ldz128(zt + 4 * (32 + 4 * b));
-        ct_bfly(r[0], r[1], z.x);
-        ct_bfly(r[2], r[3], z.y);
-        ct_bfly(r[4], r[5], z.z);
-        ct_bfly(r[6], r[7], z.w);
+        const int4 z = ldz128(zt + 4 * (32 + 4 * b)), zs = ldz128(zt + 1024 + 4 * (32 + 4 * b));
+        ct_bfly(r[0], r[1], z.x, zs.x);
+        ct_bfly(r[2], r[3], z.y, zs.y);
+        ct_bfly(r[4], r[5], z.z, zs.z);
+        ct_bfly(r[6], r[7], z.w, zs.w);
     }
     // L1 -> L2: back to coefficient order, read as 8 t + m
 #pragma unroll
@@ -239,18 +239,18 @@ static __device__ __noinline__ Poly8 ntt_fwd_unpadded_impl(Poly8 p, uint32_t buf
     for (int m = 0; m < 8; ++m) r[m] = lds32(buf + 4 * (8 * lane + m));
     __syncwarp();
     {
-        const int2 z = ldz64(zt + 4 * (64 + 2 * lane));
-        ct_bfly(r[0], r[2], z.x);
-        ct_bfly(r[1], r[3], z.x);
-        ct_bfly(r[4], r[6], z.y);
-        ct_bfly(r[5], r[7], z.y);
+        const int2 z = ldz64(zt + 4 * (64 + 2 * lane)), zs = ldz64(zt + 1024 + 4 * (64 + 2 * lane));
+        ct_bfly(r[0], r[2], z.x, zs.x);
+        ct_bfly(r[1], r[3], z.x, zs.x);
+        ct_bfly(r[4], r[6], z.y, zs.y);
+        ct_bfly(r[5], r[7], z.y, zs.y);
     }
     {
-        const int4 z = ldz128(zt + 4 * (128 + 4 * lane));
-        ct_bfly(r[0], r[1], z.x);
-        ct_bfly(r[2], r[3], z.y);
-        ct_bfly(r[4], r[5], z.z);
-        ct_bfly(r[6], r[7], z.w);
+        const int4 z = ldz128(zt + 4 * (128 + 4 * lane)), zs = ldz128(zt + 1024 + 4 * (128 + 4 * lane));
+        ct_bfly(r[0], r[1], z.x, zs.x);
+        ct_bfly(r[2], r[3], z.y, zs.y);
+        ct_bfly(r[4], r[5], z.z, zs.z);
+        ct_bfly(r[6], r[7], z.w, zs.w);
     }
     return p;
 }

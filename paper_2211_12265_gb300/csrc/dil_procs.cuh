@@ -61,7 +61,7 @@ struct __align__(16) GroupSmem {
 };
 
 constexpr int HB_K = 0, HB_MU = 32, HB_W1 = 96;
-constexpr int CTA_TABLE_BYTES = 2 * 256 * 4;
+constexpr int CTA_TABLE_BYTES = 2 * NTT_TABLE_WORDS * 4;
 
 // Synchronises the P warps of one task group (barrier id `bar`).
 template <int P>
