@@ -126,7 +126,62 @@ Shape shape_of(const dil_ctx *c, int op, int level, size_t n, size_t per) {
 int fused_warps(const dil_ctx *c, int op, int level) { const int w = c->warps[op][lidx(level)]; return w ? w : 8; }
 int fused_wpt(const dil_ctx *c, int op, int level) { const int p = c->wpt[op][lidx(level)]; return p ? p : 2; }
 
+// Tasks and slots of one launch of Sign in rounds within `budget` bytes; tasks
+// is 0 when not even one fits.
+struct RoundSize {
+    size_t tasks, slots;
+};
+
+RoundSize round_size(int level, int src, size_t n, size_t budget) {
+    size_t m = std::min<size_t>(n, (size_t)1 << 24);
+    while (m > 0) {
+        const size_t wish = dil::sign_batch_slots(level, (int)m), least = dil::sign_batch_min_slots(level, (int)m);
+        if (dil::sign_batch_bytes(level, src, m, wish) <= budget) return {m, wish};
+        const size_t need = dil::sign_batch_bytes(level, src, m, least);
+        if (need <= budget) return {m, least};
+        m = std::min(m - 1, (size_t)((double)m * budget / need));
+    }
+    return {0, 0};
+}
+
+// The Sign form of a call: the fused kernel as for the other operations (shape_of).
+bool sign_fused(const dil_ctx *c, int level, int src) {
+    return c->wpt[1][lidx(level)] > 1 || round_size(level, src, 1, c->budget).tasks == 0;
+}
+
 size_t verify_task_bytes(size_t polys) { return polys * POLY_BYTES + dil::VERIFY_AUX_BYTES; }
+
+// Runs Sign in rounds over the n tasks of `all` (whose per-task pointers are
+// those of task 0), in as many launches as the budget asks for.
+int run_sign_batch(dil_ctx *c, int level, int src, size_t n, const dil::SignBatch &all, cudaStream_t s) {
+    const RoundSize z = round_size(level, src, n, c->budget);
+    if (z.tasks == 0) return DIL_ENOMEM;
+    const int rc = ensure_ws(c, dil::sign_batch_bytes(level, src, z.tasks, z.slots));
+    if (rc) return rc;
+    size_t pkb, skb, sigb;
+    dil_sizes(level, &pkb, &skb, &sigb);
+    const size_t k = level == 2 ? 4 : level == 3 ? 6 : 8, l = level == 2 ? 4 : level == 3 ? 5 : 7;
+    for (size_t s0 = 0; s0 < n; s0 += z.tasks) {
+        dil::SignBatch b = all;
+        b.n = (int)std::min(z.tasks, n - s0);
+        b.slots = (int)z.slots;
+        if (src != dil::SIGN_KEYED) b.sk += skb * s0;
+        if (b.ahat) b.ahat += k * l * 256 * s0;
+        if (b.key_idx) b.key_idx += s0;
+        b.off += s0;
+        b.sig += sigb * s0;
+        if (b.status) b.status += s0;
+        if (b.iters) b.iters += s0;
+        const cudaError_t e = dil::launch_sign_batch(level, src, b, c->ws, s);
+        if (e != cudaSuccess) return cuda_fail(e);
+    }
+    return DIL_OK;
+}
+
+int sign_cap(const dil_ctx *c, int level) {
+    const int l = level == 2 ? 4 : level == 3 ? 5 : 7, cap = (65536 - l) / l + 1;
+    return (c->max_iter > 0 && c->max_iter < cap) ? c->max_iter : cap;
+}
 
 // Carves m tasks of a Verify batch out of a workspace of m verify_task_bytes.
 void carve_verify(dil::VerifyBatch &b, void *ws, size_t m, size_t polys) {
@@ -262,9 +317,18 @@ int dil_sign_ex(dil_ctx *c, int level, size_t n, const uint8_t *sk, const uint8_
     DeviceGuard g(c->device);
     size_t pkb, skb, sigb;
     sizes_of(level, pkb, skb, sigb);
-    int l = level == 2 ? 4 : level == 3 ? 5 : 7;
-    int cap = (65536 - l) / l + 1;
-    int max_iter = (c->max_iter > 0 && c->max_iter < cap) ? c->max_iter : cap;
+    const int max_iter = sign_cap(c, level);
+    if (!sign_fused(c, level, dil::SIGN_PLAIN)) {
+        dil::SignBatch b{};
+        b.sk = sk;
+        b.msg = msg;
+        b.off = msg_off;
+        b.sig = sig;
+        b.status = task_status;
+        b.iters = iterations;
+        b.max_iter = max_iter;
+        return run_sign_batch(c, level, dil::SIGN_PLAIN, n, b, (cudaStream_t)stream);
+    }
     size_t chunk = chunk_tasks(c, dil::OP_SIGN, level, n);
     if (chunk == 0) return DIL_ENOMEM;
     int rc = ensure_ws(c, chunk * dil::scratch_polys(dil::OP_SIGN, level) * POLY_BYTES);
@@ -358,9 +422,20 @@ int dil_sign_a(dil_ctx *c, int level, size_t n, const uint8_t *sk, const uint8_t
     DeviceGuard g(c->device);
     size_t pkb, skb, sigb;
     sizes_of(level, pkb, skb, sigb);
-    const int l = level == 2 ? 4 : level == 3 ? 5 : 7;
-    const int cap = (65536 - l) / l + 1;
-    const int max_iter = (c->max_iter > 0 && c->max_iter < cap) ? c->max_iter : cap;
+    const int max_iter = sign_cap(c, level);
+    if (round_size(level, dil::SIGN_AHAT, 1, c->budget).tasks) {
+        dil::SignBatch b{};
+        b.sk = sk;
+        b.msg = msg;
+        b.off = msg_off;
+        b.sig = sig;
+        b.status = task_status;
+        b.iters = iterations;
+        b.ahat = reinterpret_cast<const int32_t *>(ahat);
+        b.max_iter = max_iter;
+        return run_sign_batch(c, level, dil::SIGN_AHAT, n, b, (cudaStream_t)stream);
+    }
+    // a budget for the fused kernel's scratch of a task, but not for a round's
     const size_t chunk = chunk_tasks(c, dil::OP_SIGN, level, n);
     if (chunk == 0) return DIL_ENOMEM;
     int rc = ensure_ws(c, chunk * dil::scratch_polys(dil::OP_SIGN, level) * POLY_BYTES);
@@ -616,9 +691,20 @@ int dil_sign_keyed(dil_ctx *c, const dil_keystore *ks, size_t n, const int32_t *
     DeviceGuard g(c->device);
     size_t pkb, skb, sigb;
     sizes_of(ks->level, pkb, skb, sigb);
-    const int l = ks->level == 2 ? 4 : ks->level == 3 ? 5 : 7;
-    const int cap = (65536 - l) / l + 1;
-    const int max_iter = (c->max_iter > 0 && c->max_iter < cap) ? c->max_iter : cap;
+    const int max_iter = sign_cap(c, ks->level);
+    if (!sign_fused(c, ks->level, dil::SIGN_KEYED)) {
+        dil::SignBatch b{};
+        b.sk = ks->sk;
+        b.msg = msg;
+        b.off = msg_off;
+        b.sig = sig;
+        b.status = task_status;
+        b.keys = ks->keys;
+        b.key_idx = key_idx;
+        b.n_keys = (int)ks->n;
+        b.max_iter = max_iter;
+        return run_sign_batch(c, ks->level, dil::SIGN_KEYED, n, b, (cudaStream_t)stream);
+    }
     const size_t per = dil::keyed_sign_polys(ks->level) * POLY_BYTES;
     size_t chunk = std::min<size_t>(n, c->budget / per);
     if (chunk == 0) return DIL_ENOMEM;
@@ -729,17 +815,22 @@ int ensure_aux(dil_ctx *c) {
     return DIL_OK;
 }
 
-// Runs chunk(c0, c1, stream, scratch) over the batch and waits for the
-// caller's stream.  `per_task` is the kernel scratch of one task.
+size_t pipe_streams(size_t n) { return n >= PIPE_MIN_TASKS ? PIPE_STREAMS : 1; }
+
+// Tasks of a chunk whose kernel scratch is `per_task` bytes each (0: does not fit).
+size_t pipe_tasks(const dil_ctx *c, size_t n, size_t per_task) {
+    const size_t ns = pipe_streams(n);
+    return std::min((n + ns - 1) / ns, c->budget / (ns * per_task));
+}
+
+// Runs chunk(c0, c1, stream, scratch) over the batch, `per` tasks at a time, and
+// waits for the caller's stream.  `region` is a chunk's kernel scratch in bytes.
 template <class Chunk>
-int run_pipeline(dil_ctx *c, size_t n, size_t per_task, cudaStream_t s0, Chunk chunk) {
-    const size_t ns = n >= PIPE_MIN_TASKS ? PIPE_STREAMS : 1;
-    size_t per = (n + ns - 1) / ns;
-    const size_t fit = per_task ? c->budget / (ns * per_task) : per;
-    if (fit == 0) return DIL_ENOMEM;
-    per = std::min(per, fit);
+int run_pipeline(dil_ctx *c, size_t n, size_t per, size_t region, cudaStream_t s0, Chunk chunk) {
+    const size_t ns = pipe_streams(n);
+    if (per == 0) return DIL_ENOMEM;
     const size_t k = (n + per - 1) / per;
-    int rc = ensure_ws(c, ns * per * per_task);
+    int rc = ensure_ws(c, ns * region);
     if (!rc && ns > 1) rc = ensure_aux(c);
     if (rc) return rc;
     cudaStream_t st[PIPE_STREAMS] = {s0, c->aux[0], c->aux[1], c->aux[2]};
@@ -750,7 +841,7 @@ int run_pipeline(dil_ctx *c, size_t n, size_t per_task, cudaStream_t s0, Chunk c
     }
     for (size_t i = 0; i < k && !rc; ++i) {
         const size_t c0 = i * per, c1 = std::min(n, c0 + per);
-        int32_t *scratch = (int32_t *)c->ws + (i % ns) * per * (per_task / sizeof(int32_t));
+        int32_t *scratch = (int32_t *)c->ws + (i % ns) * (region / sizeof(int32_t));
         rc = chunk(c0, c1, st[i % ns], scratch);
     }
     for (size_t j = 1; j < ns; ++j)
@@ -796,7 +887,8 @@ int dil_keygen_host(dil_ctx *c, int level, size_t n, const uint8_t *seeds, uint8
     uint8_t *d_seed = (uint8_t *)c->stage, *d_pk = d_seed + al(32 * n), *d_sk = d_pk + al(pkb * n);
     const size_t per = dil::scratch_polys(dil::OP_KEYGEN, level) * POLY_BYTES;
     const Shape sh = shape_of(c, 0, level, n, per);
-    return run_pipeline(c, n, per, (cudaStream_t)stream,
+    const size_t tasks = pipe_tasks(c, n, per);
+    return run_pipeline(c, n, tasks, tasks * per, (cudaStream_t)stream,
                         [&](size_t c0, size_t c1, cudaStream_t s, int32_t *scratch) -> int {
                             const size_t m = c1 - c0;
                             if (!h2d(d_seed + 32 * c0, seeds + 32 * c0, 32 * m, s)) return DIL_ECUDA;
@@ -829,10 +921,14 @@ int dil_sign_host(dil_ctx *c, int level, size_t n, const uint8_t *sk, const uint
     uint64_t *d_off = (uint64_t *)(d_msg + al(mlen + 1));
     uint8_t *d_sig = (uint8_t *)d_off + al(8 * (n + 1));
     int32_t *d_st = (int32_t *)(d_sig + al(sigb * n));
-    const int l = level == 2 ? 4 : level == 3 ? 5 : 7, cap = (65536 - l) / l + 1;
-    const int max_iter = (c->max_iter > 0 && c->max_iter < cap) ? c->max_iter : cap;
-    const int w = fused_warps(c, 1, level), p = fused_wpt(c, 1, level);
-    return run_pipeline(c, n, dil::scratch_polys(dil::OP_SIGN, level) * POLY_BYTES, (cudaStream_t)stream,
+    const int max_iter = sign_cap(c, level);
+    const size_t ns = pipe_streams(n);
+    const RoundSize z = c->wpt[1][lidx(level)] > 1 ? RoundSize{0, 0}
+                                                   : round_size(level, dil::SIGN_PLAIN, (n + ns - 1) / ns, c->budget / ns);
+    const size_t fused = dil::scratch_polys(dil::OP_SIGN, level) * POLY_BYTES;
+    const size_t tasks = z.tasks ? z.tasks : pipe_tasks(c, n, fused);
+    const size_t region = z.tasks ? dil::sign_batch_bytes(level, dil::SIGN_PLAIN, z.tasks, z.slots) : tasks * fused;
+    return run_pipeline(c, n, tasks, region, (cudaStream_t)stream,
                         [&](size_t c0, size_t c1, cudaStream_t s, int32_t *scratch) -> int {
                             const size_t m = c1 - c0;
                             if (!h2d(d_sk + skb * c0, sk + skb * c0, skb * m, s) ||
@@ -840,9 +936,23 @@ int dil_sign_host(dil_ctx *c, int level, size_t n, const uint8_t *sk, const uint
                                      (size_t)(msg_off[c1] - msg_off[c0]), s) ||
                                 !h2d(d_off + c0, msg_off + c0, 8 * (m + 1), s))
                                 return DIL_ECUDA;
-                            cudaError_t e = dil::launch_sign(level, (int)m, d_sk + skb * c0, d_msg, d_off + c0,
-                                                             d_sig + sigb * c0, d_st + c0, nullptr, scratch,
-                                                             max_iter, w, p, s);
+                            cudaError_t e;
+                            if (z.tasks) {
+                                dil::SignBatch b{};
+                                b.n = (int)m;
+                                b.slots = (int)z.slots;
+                                b.sk = d_sk + skb * c0;
+                                b.msg = d_msg;
+                                b.off = d_off + c0;
+                                b.sig = d_sig + sigb * c0;
+                                b.status = d_st + c0;
+                                b.max_iter = max_iter;
+                                e = dil::launch_sign_batch(level, dil::SIGN_PLAIN, b, scratch, s);
+                            } else {
+                                e = dil::launch_sign(level, (int)m, d_sk + skb * c0, d_msg, d_off + c0,
+                                                     d_sig + sigb * c0, d_st + c0, nullptr, scratch, max_iter,
+                                                     fused_warps(c, 1, level), fused_wpt(c, 1, level), s);
+                            }
                             if (e != cudaSuccess) return cuda_fail(e);
                             if (!d2h(sig + sigb * c0, d_sig + sigb * c0, sigb * m, s) ||
                                 (task_status && !d2h(task_status + c0, d_st + c0, 4 * m, s)))
@@ -869,9 +979,10 @@ int dil_verify_host(dil_ctx *c, int level, size_t n, const uint8_t *pk, const ui
     uint64_t *d_off = (uint64_t *)(d_msg + al(mlen + 1));
     uint8_t *d_sig = (uint8_t *)d_off + al(8 * (n + 1));
     uint8_t *d_ok = d_sig + al(sigb * n);
-    const size_t polys = dil::scratch_polys(dil::OP_VERIFY, level), streams = n >= PIPE_MIN_TASKS ? PIPE_STREAMS : 1;
-    const Shape sh = shape_of(c, 2, level, n, streams * verify_task_bytes(polys));
-    return run_pipeline(c, n, sh.fused ? polys * POLY_BYTES : verify_task_bytes(polys), (cudaStream_t)stream,
+    const size_t polys = dil::scratch_polys(dil::OP_VERIFY, level);
+    const Shape sh = shape_of(c, 2, level, n, pipe_streams(n) * verify_task_bytes(polys));
+    const size_t per = sh.fused ? polys * POLY_BYTES : verify_task_bytes(polys), tasks = pipe_tasks(c, n, per);
+    return run_pipeline(c, n, tasks, tasks * per, (cudaStream_t)stream,
                         [&](size_t c0, size_t c1, cudaStream_t s, int32_t *scratch) -> int {
                             const size_t m = c1 - c0;
                             if (!h2d(d_pk + pkb * c0, pk + pkb * c0, pkb * m, s) ||

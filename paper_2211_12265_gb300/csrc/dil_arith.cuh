@@ -15,6 +15,12 @@ __device__ __forceinline__ int32_t mont_mul(int32_t a, int32_t b) {
     return hi - __mulhi(u, Q);
 }
 
+// a 2^-32 mod q in (-q, q) for |a| < 2^31 q (mont_mul of a product summed in
+// 64 bits).
+__device__ __forceinline__ int32_t mont_reduce(long long a) {
+    return (int32_t)(a >> 32) - __mulhi((int32_t)a * QINV, Q);
+}
+
 // Representative of a (|a| < 2^31) with |result| <= 6291200 < q:
 // a = t 2^23 + e, |e| <= 2^22, and 2^23 - q = 8191, so a - t q = e + 8191 t.
 __device__ __forceinline__ int32_t reduce_q(int32_t a) {

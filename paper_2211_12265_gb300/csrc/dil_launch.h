@@ -62,6 +62,32 @@ struct VerifyBatch {
 // batch's counter takes the first.
 constexpr size_t VERIFY_AUX_BYTES = 128;
 cudaError_t launch_verify_batch(int level, int src, const VerifyBatch &b, int warps, int p, cudaStream_t s);
+// Sign in rounds (dil_rounds.cu).  Where a task's A^, s^1, s^2 and t^0 come from:
+// its secret key, that with the caller's A^, or a resident key.
+enum SignSource { SIGN_PLAIN = 0, SIGN_AHAT = 1, SIGN_KEYED = 2 };
+struct SignBatch {
+    int n;
+    const uint8_t *sk;       // task-major; SIGN_KEYED: the store's, key-major
+    const uint8_t *msg;
+    const uint64_t *off;
+    uint8_t *sig;
+    int32_t *status, *iters; // nullable
+    const int32_t *ahat;     // SIGN_AHAT
+    const int32_t *keys;     // SIGN_KEYED: KEY_POLYS polynomials of each key, the tasks' keys
+    const int32_t *key_idx;
+    int n_keys;
+    int max_iter;
+    int slots;               // attempts of a round, at least sign_batch_min_slots
+    // set by the launch: the workspace and the prepare kernel's blocks
+    int32_t *pre, *slot_polys;
+    uint32_t *mu, *rhop;
+    int *pending, *best, *done, *next, *count;
+    int hash_warps, hash_blocks, expand_blocks;
+};
+int sign_batch_slots(int level, int n);       // slots worth having
+int sign_batch_min_slots(int level, int n);   // slots needed
+size_t sign_batch_bytes(int level, int src, size_t n, size_t slots);   // workspace
+cudaError_t launch_sign_batch(int level, int src, const SignBatch &b, void *ws, cudaStream_t s);
 // Loads the one-warp-per-task Sign kernel of `level` and runs it once on no
 // tasks (its code and local-memory reservation are in place afterwards).
 cudaError_t warm_sign(int level, int warps, int p, cudaStream_t s);

@@ -1,0 +1,827 @@
+// Sign of a batch in rounds (Alg 2).
+//
+// A prepare kernel hashes mu and rho' of every task, sixteen tasks to a warp,
+// while its other blocks sample A^ and transform s1, s2 and t0.  Then every
+// round evaluates the next m repetitions of each unfinished task (an
+// "attempt" each, in a slot of its own), phase by phase over the whole batch:
+//   mask   y = ExpandMask: sixteen polynomials to a warp, those of whole attempts
+//   front  y^, w = INTT(A^ y^), w1: a warp per attempt
+//   hash   c~ = H(mu || w1) and SampleInBall: sixteen attempts to a warp
+//   back   z, r0 and hint checks: a warp per attempt; the warp that finishes a
+//          task's last attempt of the round writes the signature of the
+//          smallest accepting repetition, or keeps the task for the next round
+// m grows as tasks finish (slots / unfinished tasks), so the long tail of the
+// rejection loop is evaluated in parallel and a round keeps filling the GPU.
+// The host launches as many rounds as leave no task over in all but a
+// vanishing share of batches, and then a kernel that runs the plain loop on
+// whatever is left.
+//
+// Against one fused kernel with a task per warp (dil_sign.cu): every hash runs
+// at 3.2 SM clocks per round and state instead of 18.7 (c~) or with a third of
+// its output unused (masks sampled sixteen nonces ahead), each kernel's code
+// fits the instruction cache (the fused kernel's first stall is instruction
+// fetch), and no SM idles while a few tasks run 20 to 30 repetitions one after
+// the other.  Fused -> rounds: 10,000 Dilithium2 tasks 3396 -> 2021 us, 10,000
+// Dilithium3 (32 B - 4 KB) 5350 -> 3209 us, 150 Dilithium5 1580 -> 455 us, one
+// Dilithium2 task 318 -> 126 us.
+#include <climits>
+
+#include "dil_kern.cuh"
+#include "dil_sample16.cuh"
+
+namespace dil {
+
+// ---------------------------------------------------------------- slots
+// A slot holds one attempt: y (l polynomials, z replaces them), w (k), and one
+// polynomial's room for the packed w1, later c (256 bytes), the hint masks and
+// c~.
+template <int LEVEL> struct Slot {
+    using V = Lv<LEVEL>;
+    static constexpr int Y = 0, W = V::L, X = V::L + V::K, POLYS = X + 1;
+    static constexpr int XC = 0, XHINT = 256, XCT = 512;   // bytes within X, once w1 is hashed
+};
+
+constexpr int ROUND_MAX_REPS = 32;     // repetitions of one task in one round
+constexpr int ROUND_FILL = 152 * 32;   // attempts that fill the GPU with a warp each
+
+__host__ __device__ __forceinline__ int round_reps(int pending, int slots) {
+    if (pending <= 0) return 0;
+    const int m = slots / pending;
+    return m < 1 ? 1 : m > ROUND_MAX_REPS ? ROUND_MAX_REPS : m;
+}
+
+// Round r: unfinished tasks, repetitions of each, first of them.
+struct Round {
+    int p, m, base;
+};
+__device__ __forceinline__ Round round_of(const SignBatch &b, int r) {
+    Round q{b.count[r], 0, 0};
+    for (int i = 0; i < r; ++i) q.base += round_reps(b.count[i], b.slots);
+    q.m = round_reps(q.p, b.slots);
+    return q;
+}
+
+__device__ __forceinline__ const int *pending_list(const SignBatch &b, int r) {
+    return b.pending + (size_t)(r & 1) * b.n;
+}
+
+template <int LEVEL>
+__device__ __forceinline__ int32_t *slot_of(const SignBatch &b, int s) {
+    return b.slot_polys + (size_t)s * Slot<LEVEL>::POLYS * N;
+}
+
+// The precomputation (A^, s^1, s^2, t^0) of task t.
+template <int LEVEL, int SRC>
+__device__ __forceinline__ const int32_t *pre_of(const SignBatch &b, int t) {
+    if (SRC == SIGN_KEYED) return b.keys + (size_t)b.key_idx[t] * Scratch<LEVEL>::KEY_POLYS * N;
+    return b.pre + (size_t)t * Scratch<LEVEL>::PRE_POLYS * N;
+}
+
+// ---------------------------------------------------------------- prepare
+// mu = H(tr || M) and rho' = H(K || mu) of a pair's tasks: the first by the
+// pair's index, the next ones from the batch's counter.  A task with an
+// unknown key or decreasing offsets is rejected here, every other one enters
+// round 0.
+template <int LEVEL, int SRC>
+struct SignMuJob {
+    const SignBatch &b;
+    int task, lane;
+    bool first, have_mu;
+
+    __device__ SignMuJob(const SignBatch &b_, int pair, int lane_)
+        : b(b_), task(pair), lane(lane_), first(true), have_mu(false) {}
+
+    __device__ __forceinline__ bool input(int &key, uint64_t &m0, size_t &mlen) const {
+        key = task;
+        if (SRC == SIGN_KEYED) {
+            key = b.key_idx[task];
+            if (key < 0 || key >= b.n_keys) return false;
+        }
+        return message_of(b.off, task, m0, mlen);
+    }
+
+    __device__ __forceinline__ bool next(HashInput &in) {
+        using V = Lv<LEVEL>;
+        uint64_t m0 = 0;
+        size_t mlen = 0;
+        int key;
+        if (have_mu) {   // rho' = H(K || mu)
+            input(key, m0, mlen);
+            in = {b.sk + (size_t)key * V::SK + 32, reinterpret_cast<const uint8_t *>(b.mu + (size_t)task * 16), 96, 32};
+            return true;
+        }
+        for (;;) {
+            if (!first) {
+                const int claimed = b.hash_warps * K16_STATES;   // one for every pair to start with
+                if (b.n <= claimed) return false;
+                int c = 0;
+                if (!(lane & 1)) c = atomicAdd(b.next, 1);
+                task = claimed + pair_bcast(c, lane);
+            }
+            first = false;
+            if (task >= b.n) return false;
+            if (input(key, m0, mlen)) break;
+            uint8_t *sig = b.sig + (size_t)task * V::SIG;
+            for (int i = lane & 1; i < V::SIG; i += 2) sig[i] = 0;
+            if (!(lane & 1)) {
+                if (b.status) b.status[task] = DIL_EINVAL;
+                if (b.iters) b.iters[task] = 0;
+            }
+        }
+        in = {b.sk + (size_t)key * V::SK + 64, b.msg + m0, 32 + mlen, 32};
+        return true;
+    }
+
+    __device__ __forceinline__ void done(const uint32_t (&a)[25]) {
+        uint32_t *dst = (have_mu ? b.rhop : b.mu) + (size_t)task * 16 + (lane & 1);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) dst[2 * i] = a[i];
+        if (have_mu && !(lane & 1)) {
+            b.best[task] = INT_MAX;
+            b.done[task] = 0;
+            b.pending[atomicAdd(b.count, 1)] = task;
+        }
+        have_mu = !have_mu;
+    }
+};
+
+// Copies nbytes (a multiple of 4) from global memory to shared memory.
+__device__ __forceinline__ void stage_words(uint8_t *dst, const uint8_t *src, int nbytes, int lane) {
+    if ((reinterpret_cast<uintptr_t>(src) & 3) == 0) {
+        for (int i = lane; i < nbytes / 4; i += 32)
+            reinterpret_cast<uint32_t *>(dst)[i] = reinterpret_cast<const uint32_t *>(src)[i];
+    } else {
+        for (int i = lane; i < nbytes; i += 32) dst[i] = src[i];
+    }
+}
+
+// As unpack_poly_l0, with buf (a warp's exchange buffer) as staging.
+template <int BITS>
+__device__ __forceinline__ void unpack_words_l0(int32_t v[8], const uint8_t *src, int32_t off, int32_t *buf, int lane) {
+    uint8_t *sq = reinterpret_cast<uint8_t *>(buf);
+    stage_words(sq, src, N * BITS / 8, lane);
+    __syncwarp();
+#pragma unroll
+    for (int m = 0; m < 8; ++m) v[m] = off - (int32_t)get_field(sq, BITS * (lane + 32 * m), BITS);
+    __syncwarp();
+}
+
+// s^1, s^2, t^0 of one task (one warp).
+template <int LEVEL>
+__device__ __forceinline__ void sign_secrets(const uint8_t *sk, int32_t *pre, int32_t *buf, const int32_t *zt,
+                                             int lane) {
+    using V = Lv<LEVEL>;
+    using S = Scratch<LEVEL>;
+    int32_t r[8];
+#pragma unroll 1
+    for (int u = 0; u < V::L + 2 * V::K; ++u) {
+        if (u < V::L + V::K)
+            unpack_words_l0<V::ETABITS>(r, sk + V::SK_S1 + u * V::POLYETA, V::ETA, buf, lane);   // s1, then s2
+        else
+            unpack_words_l0<D>(r, sk + V::SK_T0 + (u - V::L - V::K) * V::POLYT0, 1 << (D - 1), buf, lane);
+        ntt_fwd(r, buf, zt, lane);
+        store_l2(pre + (S::S1H + u) * N, r, lane);
+    }
+}
+
+constexpr int ROUND_WARPS = 4;   // warps per CTA of every kernel here
+
+// Blocks [0, hash_blocks) hash, [.., + expand_blocks) sample A^ (SIGN_AHAT:
+// none), the rest transform the secrets (SIGN_KEYED: none), one task per warp;
+// with SIGN_AHAT they also copy the caller's A^.
+template <int LEVEL, int SRC>
+__global__ void __launch_bounds__(32 * ROUND_WARPS, 4) k_sign_prepare(const SignBatch b) {
+    extern __shared__ __align__(16) uint32_t sm[];
+    using V = Lv<LEVEL>;
+    constexpr int KL = V::K * V::L;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int blk = blockIdx.x;
+    if (blk < b.hash_blocks) {
+        const int w = blk * ROUND_WARPS + warp;
+        if (w >= b.hash_warps) return;
+        SignMuJob<LEVEL, SRC> job(b, w * K16_STATES + (lane >> 1), lane);
+        hash16_run(job, sm + warp * HASH16_STAGE_WORDS, lane);
+        return;
+    }
+    if constexpr (SRC != SIGN_KEYED) {
+        blk -= b.hash_blocks;
+        if (blk < b.expand_blocks) {
+            const long long first = (long long)(blk * ROUND_WARPS + warp) * K16_STATES;
+            expand_a_batch<LEVEL>(
+                first, (long long)b.n * KL, [&](int t) { return b.sk + (size_t)t * V::SK; },
+                [&](int t) { return b.pre + (size_t)t * Scratch<LEVEL>::PRE_POLYS * N; }, sm + warp * EXPAND16_WORDS,
+                lane);
+            return;
+        }
+        blk -= b.expand_blocks;
+        int32_t *zt = reinterpret_cast<int32_t *>(sm), *buf = zt + NTT_TABLE_WORDS + warp * 288;
+        load_zetas_fwd(zt);
+        __syncthreads();
+        const int t = blk * ROUND_WARPS + warp;
+        if (t >= b.n) return;
+        int32_t *pre = b.pre + (size_t)t * Scratch<LEVEL>::PRE_POLYS * N;
+        if (SRC == SIGN_AHAT) copy_polys(b.ahat + (size_t)t * KL * N, 0, KL, pre, lane);
+        sign_secrets<LEVEL>(b.sk + (size_t)t * V::SK, pre, buf, zt, lane);
+    }
+}
+
+// ---------------------------------------------------------------- mask
+// Words of one state's five squeezed blocks (170), spaced so that the sixteen
+// states' copies of the same word fall into sixteen different pairs of banks.
+constexpr int MASK_STRIDE = 178;
+constexpr int MASK_WORDS = K16_STATES * MASK_STRIDE;
+
+template <int LEVEL>
+__global__ void __launch_bounds__(32 * ROUND_WARPS, 4) k_sign_mask(const SignBatch b, int r) {
+    extern __shared__ __align__(16) uint32_t sm[];
+    using V = Lv<LEVEL>;
+    constexpr int G = K16_STATES / V::L;   // attempts per warp
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const Round q = round_of(b, r);
+    const int attempts = q.p * q.m, first = (blockIdx.x * ROUND_WARPS + warp) * G;
+    if (first >= attempts) return;
+    uint32_t *st = sm + warp * MASK_WORDS;
+    const int s = lane >> 1, p = lane & 1;
+    const int slot = min(first + s / V::L, attempts - 1), i = slot / q.m;
+    const int rep = q.base + slot - i * q.m;
+    const uint32_t *seed = b.rhop + (size_t)pending_list(b, r)[i] * 16;
+    uint32_t a[25];
+#pragma unroll
+    for (int w = 0; w < 25; ++w) a[w] = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) a[w] = seed[2 * w + p];
+    if (!p) a[8] = ((uint32_t)(V::L * rep + s % V::L) & 0xFFFFu) | (0x1Fu << 16);
+    if (p) a[16] = 0x80000000u;
+#pragma unroll 1
+    for (int blk = 0; blk < 5; ++blk) {
+        hash16_permute(a, p);
+#pragma unroll
+        for (int w = 0; w < 17; ++w) st[s * MASK_STRIDE + 34 * blk + 2 * w + p] = a[w];
+    }
+    __syncwarp();
+    // fields: coefficient lane + 32 m starts at bit ZBITS lane + 32 ZBITS m, so
+    // the shift is the lane's own and the word advances by ZBITS
+    const int w0 = (V::ZBITS * lane) >> 5, sh = (V::ZBITS * lane) & 31;
+#pragma unroll 1
+    for (int u = 0; u < G * V::L; ++u) {
+        const int at = first + u / V::L;
+        if (at >= attempts) break;
+        int32_t *dst = slot_of<LEVEL>(b, at) + (Slot<LEVEL>::Y + u % V::L) * N;
+        const uint32_t *src = st + u * MASK_STRIDE + w0;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            const uint32_t f = __funnelshift_r(src[V::ZBITS * m], src[V::ZBITS * m + 1], sh);
+            dst[lane + 32 * m] = V::GAMMA1 - (int32_t)(f & ((1u << V::ZBITS) - 1u));
+        }
+    }
+}
+
+// ---------------------------------------------------------------- front
+// Packs 8 consecutive w1 values of this lane at dst (2-byte aligned).
+template <int LEVEL>
+__device__ __forceinline__ void pack_w1(uint8_t *dst, const int32_t v[8], int lane) {
+    using V = Lv<LEVEL>;
+    if constexpr (V::W1BITS == 4) {
+        uint32_t x = 0;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) x |= (uint32_t)v[m] << (4 * m);
+        reinterpret_cast<uint32_t *>(dst)[lane] = x;
+    } else {
+        uint32_t lo = 0, hi = 0;   // 24 bits each
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            lo |= (uint32_t)v[m] << (6 * m);
+            hi |= (uint32_t)v[m + 4] << (6 * m);
+        }
+        uint16_t *d = reinterpret_cast<uint16_t *>(dst) + 3 * lane;
+        d[0] = (uint16_t)lo;
+        d[1] = (uint16_t)((lo >> 16) | (hi << 8));
+        d[2] = (uint16_t)(hi >> 8);
+    }
+}
+
+// Shared words of a front warp: the exchange buffer and y^ (l polynomials).
+template <int LEVEL>
+constexpr int front_warp_words() { return 288 + Lv<LEVEL>::L * N; }
+
+template <int LEVEL, int SRC>
+__global__ void __launch_bounds__(32 * ROUND_WARPS, LEVEL == 5 ? 6 : 8) k_sign_front(const SignBatch b, int r) {
+    extern __shared__ __align__(16) uint32_t sm[];
+    using V = Lv<LEVEL>;
+    using S = Scratch<LEVEL>;
+    const Round q = round_of(b, r);
+    const int attempts = q.p * q.m;
+    if ((int)blockIdx.x * ROUND_WARPS >= attempts) return;
+    int32_t *zt = reinterpret_cast<int32_t *>(sm), *izt = zt + NTT_TABLE_WORDS;
+    load_zetas(zt, izt);
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int s = blockIdx.x * ROUND_WARPS + warp;
+    if (s >= attempts) return;
+    int32_t *buf = izt + NTT_TABLE_WORDS + warp * front_warp_words<LEVEL>(), *yh = buf + 288;
+    const int32_t *pre = pre_of<LEVEL, SRC>(b, pending_list(b, r)[s / q.m]);
+    int32_t *slot = slot_of<LEVEL>(b, s);
+    int32_t v[8];
+#pragma unroll 1
+    for (int j = 0; j < V::L; ++j) {
+        load_l0(v, slot + (Slot<LEVEL>::Y + j) * N, lane);
+        ntt_fwd(v, buf, zt, lane);
+        store_l2(yh + j * N, v, lane);   // read back by the same lane
+    }
+#pragma unroll 1
+    for (int i = 0; i < V::K; ++i) {
+        // the l products of a row are summed in 64 bits (|sum| < 7 q 9q < 2^31 q) and reduced once
+        long long acc[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) acc[m] = 0;
+#pragma unroll 1
+        for (int j = 0; j < V::L; ++j) {
+            int32_t a[8], y[8];
+            load_l2(a, pre + (S::AH + i * V::L + j) * N, lane);
+            load_l2(y, yh + j * N, lane);
+#pragma unroll
+            for (int m = 0; m < 8; ++m) acc[m] += (long long)a[m] * y[m];
+        }
+#pragma unroll
+        for (int m = 0; m < 8; ++m) v[m] = mont_reduce(acc[m]);
+        ntt_inv(v, buf, izt, lane);
+        int32_t h[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            v[m] = to_canonical(v[m]);
+            h[m] = highbits<LEVEL>(v[m]);
+        }
+        store_l0(slot + (Slot<LEVEL>::W + i) * N, v, lane);
+        l0_to_seq(h, buf, lane);
+        pack_w1<LEVEL>(reinterpret_cast<uint8_t *>(slot + Slot<LEVEL>::X * N) + i * V::POLYW1, h, lane);
+    }
+}
+
+// ---------------------------------------------------------------- hash
+// c~ = H(mu || w1) of the attempt in slot `pair`.
+template <int LEVEL>
+struct SignCtJob {
+    const SignBatch &b;
+    const uint8_t *mu, *w1;
+    bool todo;
+    uint32_t ct[4];
+
+    __device__ __forceinline__ bool next(HashInput &in) {
+        if (!todo) return false;
+        todo = false;
+        in = {mu, w1, 64 + Lv<LEVEL>::K * Lv<LEVEL>::POLYW1, 64};
+        return true;
+    }
+    __device__ __forceinline__ void done(const uint32_t (&a)[25]) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ct[i] = a[i];
+    }
+};
+
+// Shared words of a hashing warp: the stage, then sixteen challenges of 256
+// bytes.
+constexpr int CHALLENGE_STRIDE = 65;   // words from one pair's challenge to the next
+constexpr int HASH_WARP_WORDS = HASH16_STAGE_WORDS + K16_STATES * CHALLENGE_STRIDE;
+
+template <int LEVEL>
+__global__ void __launch_bounds__(32 * ROUND_WARPS, 4) k_sign_hash(const SignBatch b, int r) {
+    __shared__ uint32_t sm[ROUND_WARPS][HASH_WARP_WORDS];
+    using V = Lv<LEVEL>;
+    using SL = Slot<LEVEL>;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, pair = lane >> 1, p = lane & 1;
+    const Round q = round_of(b, r);
+    const int attempts = q.p * q.m, first = (blockIdx.x * (blockDim.x >> 5) + warp) * K16_STATES;
+    if (first >= attempts) return;
+    uint32_t *stage = sm[warp];
+    uint8_t *c = reinterpret_cast<uint8_t *>(stage + HASH16_STAGE_WORDS + pair * CHALLENGE_STRIDE);
+    const int s = first + pair;
+    const bool mine = s < attempts;
+    const int task = mine ? pending_list(b, r)[s / q.m] : 0;
+    uint8_t *x = reinterpret_cast<uint8_t *>(slot_of<LEVEL>(b, mine ? s : first) + SL::X * N);
+    SignCtJob<LEVEL> job{b, reinterpret_cast<const uint8_t *>(b.mu + (size_t)task * 16), x, mine, {0, 0, 0, 0}};
+    hash16_run(job, stage, lane);
+    if (mine) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) reinterpret_cast<uint32_t *>(x + SL::XCT)[2 * i + p] = job.ct[i];
+    }
+    // c = SampleInBall(c~): the blocks go through the stage, the even thread of
+    // each pair draws and swaps (the order Alg 2 gives)
+    uint32_t a[25];
+#pragma unroll
+    for (int i = 0; i < 25; ++i) a[i] = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) a[i] = job.ct[i];
+    if (!p) a[4] = 0x1Fu;
+    if (p) a[16] = 0x80000000u;
+    for (int i = p; i < 64; i += 2) reinterpret_cast<uint32_t *>(c)[i] = 0;
+    bool more = mine;
+    int i = N - V::TAU, pos = 8;
+    uint64_t signs = 0;
+    for (int blk = 0; blk < MAX_SQUEEZE_BLOCKS && __any_sync(FULL, more); ++blk) {
+        hash16_permute(a, p);
+        __syncwarp();
+#pragma unroll
+        for (int w = 0; w < 17; ++w) stage[k16_word(pair, 2 * w + p)] = a[w];
+        __syncwarp();
+        if (more && !p) {
+            if (blk == 0)
+                signs = ((uint64_t)stage[k16_word(pair, 1)] << 32) | stage[k16_word(pair, 0)];
+            while (i < N && pos < 136) {
+                const int at = (stage[k16_word(pair, pos >> 2)] >> (8 * (pos & 3))) & 0xFF;
+                ++pos;
+                if (at > i) continue;
+                c[i] = c[at];
+                c[at] = (signs & 1) ? 0xFF : 1;
+                signs >>= 1;
+                ++i;
+            }
+            pos = 0;
+        }
+        more = more && pair_bcast(i, lane) < N;
+    }
+    __syncwarp();
+    // 256 bytes of each challenge over its slot's w1, which every pair of the
+    // warp has absorbed
+    for (int u = 0; u < K16_STATES && first + u < attempts; ++u) {
+        const uint32_t *src = stage + HASH16_STAGE_WORDS + u * CHALLENGE_STRIDE;
+        uint32_t *dst = reinterpret_cast<uint32_t *>(slot_of<LEVEL>(b, first + u) + SL::X * N);
+        dst[lane] = src[lane];
+        dst[lane + 32] = src[lane + 32];
+    }
+}
+
+// ---------------------------------------------------------------- back
+// The checks of the attempt in `slot` with challenge ch (L2 layout); z
+// replaces y, the hint masks go behind the challenge.  True when accepted.
+template <int LEVEL>
+__device__ __forceinline__ bool sign_checks(const int32_t *pre, int32_t *slot, const int32_t ch[8], int32_t *buf,
+                                            const int32_t *izt, int lane) {
+    using V = Lv<LEVEL>;
+    using S = Scratch<LEVEL>;
+    using SL = Slot<LEVEL>;
+    int32_t v[8], a[8];
+    // z = y + INTT(c^ o s^1); reject if ||z|| >= gamma1 - beta
+#pragma unroll 1
+    for (int j = 0; j < V::L; ++j) {
+        int32_t *y = slot + (SL::Y + j) * N;
+        load_l2(a, pre + (S::S1H + j) * N, lane);
+#pragma unroll
+        for (int m = 0; m < 8; ++m) v[m] = mont_mul(ch[m], a[m]);
+        load_l0(a, y, lane);
+        ntt_inv(v, buf, izt, lane);
+        bool bad = false;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            v[m] = centre_small(to_canonical(v[m]) + a[m]);
+            bad |= iabs(v[m]) >= V::GAMMA1 - V::BETA;
+        }
+        if (__any_sync(FULL, bad)) return false;
+        store_l0(y, v, lane);
+    }
+    // v_s = INTT(c^ o s^2); r0 = LowBits(w - v_s)
+#pragma unroll 1
+    for (int i = 0; i < V::K; ++i) {
+        int32_t *w = slot + (SL::W + i) * N;
+        load_l2(a, pre + (S::S2H + i) * N, lane);
+#pragma unroll
+        for (int m = 0; m < 8; ++m) v[m] = mont_mul(ch[m], a[m]);
+        load_l0(a, w, lane);
+        ntt_inv(v, buf, izt, lane);
+        bool bad = false;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            int32_t d = a[m] - v[m];                 // (-q, 2q)
+            d += (d < 0) ? Q : 0;
+            d -= (d >= Q) ? Q : 0;
+            int32_t h1, l0;
+            decompose<LEVEL>(d, h1, l0);
+            bad |= iabs(l0) >= V::GAMMA2 - V::BETA;
+            a[m] = d;
+        }
+        if (__any_sync(FULL, bad)) return false;
+        store_l0(w, a, lane);   // w - c s2, for the hint
+    }
+    // v_t = INTT(c^ o t^0); h = MakeHint(-v_t, w - v_s + v_t)
+    uint32_t *hint = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(slot + SL::X * N) + SL::XHINT);
+    int count = 0;
+#pragma unroll 1
+    for (int i = 0; i < V::K; ++i) {
+        load_l2(a, pre + (S::T0H + i) * N, lane);
+#pragma unroll
+        for (int m = 0; m < 8; ++m) v[m] = mont_mul(ch[m], a[m]);
+        load_l0(a, slot + (SL::W + i) * N, lane);
+        ntt_inv(v, buf, izt, lane);
+        bool bad = false;
+        uint32_t hbits = 0;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            int32_t vt = to_canonical(v[m]);
+            bad |= iabs(to_centred(vt)) >= V::GAMMA2;
+            int32_t rr = a[m] + vt;
+            rr -= (rr >= Q) ? Q : 0;
+            int32_t z = vt ? Q - vt : 0;
+            hbits |= (uint32_t)make_hint<LEVEL>(z, rr) << m;
+        }
+        if (__any_sync(FULL, bad)) return false;
+        uint32_t mine = 0;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            const uint32_t w = __ballot_sync(FULL, (hbits >> m) & 1u);
+            if (lane == m) mine = w;
+            count += __popc(w);
+        }
+        if (lane < 8) hint[i * 8 + lane] = mine;
+    }
+    return count <= V::OMEGA;
+}
+
+// sig = c~ || z || h of the accepted attempt in `slot` (read through L2:
+// another warp may have written it).
+template <int LEVEL>
+__device__ __forceinline__ void sign_emit(uint8_t *sig, const int32_t *slot, int lane) {
+    using V = Lv<LEVEL>;
+    using SL = Slot<LEVEL>;
+#pragma unroll 1
+    for (int j = 0; j < V::L; ++j) {
+        int32_t v[8];
+        load_l2_cg(v, slot + (SL::Y + j) * N, lane);   // 8 consecutive coefficients
+        pack_seq<V::ZBITS>(sig + V::SIG_Z + j * V::POLYZ, v, V::GAMMA1, -1, lane);
+    }
+    const uint8_t *x = reinterpret_cast<const uint8_t *>(slot + SL::X * N);
+    sig[lane] = __ldcg(x + SL::XCT + lane);
+    const uint32_t *hint = reinterpret_cast<const uint32_t *>(x + SL::XHINT);
+    uint8_t *h = sig + V::SIG_H;
+    int base = 0;
+#pragma unroll 1
+    for (int i = 0; i < V::K; ++i) {
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            const uint32_t w = __ldcg(hint + i * 8 + m);
+            if ((w >> lane) & 1u) h[base + __popc(w & lanemask_lt(lane))] = (uint8_t)(lane + 32 * m);
+            base += __popc(w);
+        }
+        if (lane == 0) h[V::OMEGA + i] = (uint8_t)base;
+    }
+    for (int p = base + lane; p < V::OMEGA; p += 32) h[p] = 0;
+}
+
+template <int LEVEL, int SRC>
+__global__ void __launch_bounds__(32 * ROUND_WARPS, 8) k_sign_back(const SignBatch b, int r) {
+    extern __shared__ __align__(16) uint32_t sm[];
+    using V = Lv<LEVEL>;
+    const Round q = round_of(b, r);
+    const int attempts = q.p * q.m;
+    if ((int)blockIdx.x * ROUND_WARPS >= attempts) return;
+    int32_t *zt = reinterpret_cast<int32_t *>(sm), *izt = zt + NTT_TABLE_WORDS;
+    load_zetas(zt, izt);
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int s = blockIdx.x * ROUND_WARPS + warp;
+    if (s >= attempts) return;
+    int32_t *buf = izt + NTT_TABLE_WORDS + warp * 288;
+    const int i = s / q.m, task = pending_list(b, r)[i], rep = q.base + s - i * q.m;
+    int32_t *slot = slot_of<LEVEL>(b, s);
+    // a repetition past the cap, or past one that has been accepted, is not looked at
+    int skip = 0;
+    if (lane == 0) skip = rep >= b.max_iter || atomicOr(&b.best[task], 0) < rep;
+    if (!__shfl_sync(FULL, skip, 0)) {
+        int32_t ch[8];
+        const int8_t *c = reinterpret_cast<const int8_t *>(slot + Slot<LEVEL>::X * N);
+#pragma unroll
+        for (int m = 0; m < 8; ++m) ch[m] = c[lane + 32 * m];
+        ntt_fwd(ch, buf, zt, lane);
+        if (sign_checks<LEVEL>(pre_of<LEVEL, SRC>(b, task), slot, ch, buf, izt, lane) && lane == 0)
+            atomicMin(&b.best[task], rep);
+    }
+    // the last of the task's attempts settles the round
+    __threadfence();
+    int arrived = 0;
+    __syncwarp();
+    if (lane == 0) arrived = atomicAdd(&b.done[task], 1);
+    if (__shfl_sync(FULL, arrived, 0) != q.m - 1) return;
+    __threadfence();
+    int best = 0;
+    if (lane == 0) best = atomicOr(&b.best[task], 0);
+    best = __shfl_sync(FULL, best, 0);
+    uint8_t *sig = b.sig + (size_t)task * V::SIG;
+    if (best != INT_MAX) {
+        sign_emit<LEVEL>(sig, slot_of<LEVEL>(b, i * q.m + best - q.base), lane);
+        if (lane == 0) {
+            if (b.status) b.status[task] = DIL_OK;
+            if (b.iters) b.iters[task] = best + 1;
+        }
+    } else if (q.base + q.m >= b.max_iter) {
+        sign_zero<LEVEL, 1>(sig, 0, lane);
+        if (lane == 0) {
+            if (b.status) b.status[task] = DIL_EITER;
+            if (b.iters) b.iters[task] = b.max_iter;
+        }
+    } else if (lane == 0) {
+        b.done[task] = 0;
+        int *list = b.pending + (size_t)((r + 1) & 1) * b.n;
+        list[atomicAdd(b.count + r + 1, 1)] = task;
+    }
+}
+
+// ---------------------------------------------------------------- what is left
+// The plain loop over the tasks still unfinished after round r - 1, from
+// round r's first repetition on, one task per warp; the slots are its scratch.
+template <int LEVEL, int SRC>
+__global__ void __launch_bounds__(256, 4) k_sign_rest(const SignBatch b, int r, int workers) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    using V = Lv<LEVEL>;
+    const Round q = round_of(b, r);
+    if (q.p <= 0) return;
+    const CtaView v = cta_setup<1>(smem);
+    const int w = blockIdx.x * v.groups + v.group;
+    if (w >= workers) return;
+    int32_t *itr = b.slot_polys + (size_t)w * Scratch<LEVEL>::ITR_POLYS * N;
+    for (int i = w; i < q.p; i += workers) {
+        const int task = pending_list(b, r)[i];
+        const int32_t *pre = pre_of<LEVEL, SRC>(b, task);
+        if (v.lane < 16) {
+            reinterpret_cast<uint32_t *>(v.gs->hb + HB_MU)[v.lane] = b.mu[(size_t)task * 16 + v.lane];
+            reinterpret_cast<uint32_t *>(v.gs->rhop)[v.lane] = b.rhop[(size_t)task * 16 + v.lane];
+        }
+        __syncwarp();
+        int it = q.base;
+        bool ok = false;
+        MaskStream ms{0, 0};
+        while (it < b.max_iter) {
+            ok = sign_attempt<LEVEL, 1>(it * V::L, pre, itr, ms, *v.gs, *v.ws, v.zt, v.izt, 0, v.bar, v.lane);
+            ++it;
+            if (ok) break;
+        }
+        uint8_t *sig = b.sig + (size_t)task * V::SIG;
+        if (ok)
+            sign_pack<LEVEL, 1>(sig, itr, *v.gs, 0, v.lane);
+        else
+            sign_zero<LEVEL, 1>(sig, 0, v.lane);
+        if (v.lane == 0) {
+            if (b.status) b.status[task] = ok ? DIL_OK : DIL_EITER;
+            if (b.iters) b.iters[task] = it;
+        }
+        __syncwarp();
+    }
+}
+
+// ---------------------------------------------------------------- host side
+namespace {
+
+// Mean acceptance of one repetition (Alg 2; 1 / 4.25, 1 / 5.1, 1 / 3.85).
+double accept_of(int level) { return level == 2 ? 1 / 4.25 : level == 3 ? 1 / 5.1 : 1 / 3.85; }
+
+constexpr int MAX_ROUNDS = 24;
+constexpr int CTL_WORDS = 64;   // the hashing warps' counter, then the rounds' task counts
+static_assert(MAX_ROUNDS + 3 <= CTL_WORDS, "a count per round, the counter and the round after the last");
+
+size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+template <int LEVEL>
+int min_slots() { return (Scratch<LEVEL>::ITR_POLYS + Slot<LEVEL>::POLYS - 1) / Slot<LEVEL>::POLYS; }
+
+struct Layout {
+    size_t pre, slots, mu, rhop, pending, best, done, ctl, total;
+};
+
+template <int LEVEL>
+Layout layout_of(int src, size_t n, size_t slots) {
+    Layout L;
+    size_t at = 0;
+    auto take = [&](size_t bytes) {
+        const size_t here = at;
+        at += al256(bytes);
+        return here;
+    };
+    L.pre = take(src == SIGN_KEYED ? 0 : n * Scratch<LEVEL>::PRE_POLYS * N * 4);
+    L.slots = take(slots * Slot<LEVEL>::POLYS * N * 4);
+    L.mu = take(64 * n);
+    L.rhop = take(64 * n);
+    L.pending = take(8 * n);
+    L.best = take(4 * n);
+    L.done = take(4 * n);
+    L.ctl = take(4 * CTL_WORDS);
+    L.total = at;
+    return L;
+}
+
+// Rounds after which fewer than 0.02 tasks are expected to be left.
+int rounds_of(int level, int n, int slots) {
+    double left = n;
+    int r = 0;
+    while (left > 0.02 && r < MAX_ROUNDS) {
+        const int m = round_reps(left < 1 ? 1 : (int)left, slots);
+        for (int i = 0; i < m; ++i) left *= 1 - accept_of(level);
+        ++r;
+    }
+    return r;
+}
+
+template <class Kern>
+cudaError_t dynamic_smem(Kern kern, size_t bytes) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+int blocks_for(long long items, int per) { return (int)((items + per - 1) / per); }
+
+template <int LEVEL, int SRC>
+cudaError_t launch_rounds(SignBatch b, void *ws, cudaStream_t s) {
+    using V = Lv<LEVEL>;
+    const Layout L = layout_of<LEVEL>(SRC, b.n, b.slots);
+    uint8_t *base = static_cast<uint8_t *>(ws);
+    b.pre = reinterpret_cast<int32_t *>(base + L.pre);
+    b.slot_polys = reinterpret_cast<int32_t *>(base + L.slots);
+    b.mu = reinterpret_cast<uint32_t *>(base + L.mu);
+    b.rhop = reinterpret_cast<uint32_t *>(base + L.rhop);
+    b.pending = reinterpret_cast<int *>(base + L.pending);
+    b.best = reinterpret_cast<int *>(base + L.best);
+    b.done = reinterpret_cast<int *>(base + L.done);
+    b.next = reinterpret_cast<int *>(base + L.ctl);
+    b.count = b.next + 1;
+    cudaError_t e = cudaMemsetAsync(b.next, 0, 4 * CTL_WORDS, s);
+    if (e != cudaSuccess) return e;
+
+    // prepare
+    b.hash_warps = batch_hash_warps(b.n);
+    b.hash_blocks = blocks_for(b.hash_warps, ROUND_WARPS);
+    b.expand_blocks = SRC == SIGN_PLAIN ? blocks_for((long long)b.n * V::K * V::L, K16_STATES * ROUND_WARPS) : 0;
+    const int secret_blocks = SRC == SIGN_KEYED ? 0 : blocks_for(b.n, ROUND_WARPS);
+    const size_t tables = 4 * NTT_TABLE_WORDS;
+    const size_t prep_smem = 4 * ROUND_WARPS * (SRC == SIGN_PLAIN ? EXPAND16_WORDS : HASH16_STAGE_WORDS);
+    static_assert(4 * NTT_TABLE_WORDS + 4 * 288 * ROUND_WARPS <= 4 * ROUND_WARPS * HASH16_STAGE_WORDS,
+                  "the secrets' blocks fit the hashing blocks' shared memory");
+    if ((e = dynamic_smem(k_sign_prepare<LEVEL, SRC>, prep_smem)) != cudaSuccess) return e;
+    k_sign_prepare<LEVEL, SRC>
+        <<<b.hash_blocks + b.expand_blocks + secret_blocks, 32 * ROUND_WARPS, prep_smem, s>>>(b);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+
+    const size_t mask_smem = 4 * ROUND_WARPS * MASK_WORDS;
+    const size_t front_smem = 2 * tables + 4 * ROUND_WARPS * front_warp_words<LEVEL>();
+    const size_t back_smem = 2 * tables + 4 * ROUND_WARPS * 288;
+    if ((e = dynamic_smem(k_sign_mask<LEVEL>, mask_smem)) != cudaSuccess) return e;
+    if ((e = dynamic_smem(k_sign_front<LEVEL, SRC>, front_smem)) != cudaSuccess) return e;
+    const int rounds = rounds_of(LEVEL, b.n, b.slots);
+    const int most = b.slots;   // attempts of a round; blocks beyond the actual count return at once
+    const HashGrid h = hash_grid(most);
+    for (int r = 0; r < rounds; ++r) {
+        k_sign_mask<LEVEL><<<blocks_for(most, ROUND_WARPS * (K16_STATES / V::L)), 32 * ROUND_WARPS, mask_smem, s>>>(b, r);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        k_sign_front<LEVEL, SRC><<<blocks_for(most, ROUND_WARPS), 32 * ROUND_WARPS, front_smem, s>>>(b, r);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        k_sign_hash<LEVEL><<<h.blocks, h.threads, 0, s>>>(b, r);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        k_sign_back<LEVEL, SRC><<<blocks_for(most, ROUND_WARPS), 32 * ROUND_WARPS, back_smem, s>>>(b, r);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    const size_t room = (size_t)b.slots * Slot<LEVEL>::POLYS / Scratch<LEVEL>::ITR_POLYS;
+    const int workers = (int)(room < 64 ? room : 64), ctas = blocks_for(workers, 4);
+    const size_t rest_smem = cta_bytes(4, 1);
+    if ((e = dynamic_smem(k_sign_rest<LEVEL, SRC>, rest_smem)) != cudaSuccess) return e;
+    k_sign_rest<LEVEL, SRC><<<ctas, 128, rest_smem, s>>>(b, rounds, workers);
+    return cudaGetLastError();
+}
+
+template <int LEVEL>
+cudaError_t launch_src(int src, const SignBatch &b, void *ws, cudaStream_t s) {
+    switch (src) {
+        case SIGN_PLAIN: return launch_rounds<LEVEL, SIGN_PLAIN>(b, ws, s);
+        case SIGN_AHAT: return launch_rounds<LEVEL, SIGN_AHAT>(b, ws, s);
+        case SIGN_KEYED: return launch_rounds<LEVEL, SIGN_KEYED>(b, ws, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+// Slots of a batch: one per task, and for a small batch enough for
+// ROUND_MAX_REPS repetitions of each while that does not overfill the GPU.
+int sign_batch_slots(int level, int n) {
+    const int least = level == 2 ? min_slots<2>() : level == 3 ? min_slots<3>() : min_slots<5>();
+    long long s = (long long)n * ROUND_MAX_REPS;
+    if (s > ROUND_FILL) s = n > ROUND_FILL ? n : ROUND_FILL;
+    return (int)(s < least ? least : s);
+}
+
+size_t sign_batch_bytes(int level, int src, size_t n, size_t slots) {
+    return level == 2   ? layout_of<2>(src, n, slots).total
+           : level == 3 ? layout_of<3>(src, n, slots).total
+                        : layout_of<5>(src, n, slots).total;
+}
+
+int sign_batch_min_slots(int level, int n) {
+    const int least = level == 2 ? min_slots<2>() : level == 3 ? min_slots<3>() : min_slots<5>();
+    return n > least ? n : least;
+}
+
+cudaError_t launch_sign_batch(int level, int src, const SignBatch &b, void *ws, cudaStream_t s) {
+    if (b.n <= 0) return cudaSuccess;
+    if (b.slots < sign_batch_min_slots(level, b.n)) return cudaErrorInvalidValue;
+    switch (level) {
+        case 2: return launch_src<2>(src, b, ws, s);
+        case 3: return launch_src<3>(src, b, ws, s);
+        case 5: return launch_src<5>(src, b, ws, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace dil
