@@ -191,6 +191,7 @@ void carve_verify(dil::VerifyBatch &b, void *ws, size_t m, size_t polys) {
     b.mu = reinterpret_cast<uint32_t *>(aux);
     b.tr = reinterpret_cast<uint32_t *>(aux + 64 * m);
     b.next = reinterpret_cast<int *>(aux + 96 * m);
+    b.challenge = aux + 128 * m;
 }
 
 void sizes_of(int level, size_t &pk, size_t &sk, size_t &sig) { dil_sizes(level, &pk, &sk, &sig); }
@@ -404,10 +405,8 @@ int dil_expand_a(dil_ctx *c, int level, size_t n, const uint8_t *rho, size_t rho
     if (!rho || !ahat || !aligned16(ahat) || n > (size_t)INT32_MAX) return DIL_EINVAL;
     std::lock_guard<std::mutex> lk(c->mu);
     DeviceGuard g(c->device);
-    // one warp per key, in the CTA size of Verify's tuning (the other kernel
-    // whose first step is ExpandA); the output needs no workspace
     cudaError_t e = dil::launch_expand_a(level, (int)n, rho, rho_stride, reinterpret_cast<int32_t *>(ahat),
-                                         fused_warps(c, 2, level), (cudaStream_t)stream);
+                                         (cudaStream_t)stream);
     return e != cudaSuccess ? cuda_fail(e) : DIL_OK;
 }
 

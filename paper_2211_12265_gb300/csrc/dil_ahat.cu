@@ -1,26 +1,23 @@
 // Resident-A^ forms of the plain kernels: A^ = ExpandA(rho) written to a
 // caller's buffer (Alg 4; the matrix Alg 1 samples and Alg 2 / Alg 3 use in the
 // NTT domain), and Sign reading that A^ instead of sampling it (Verify's is a
-// source of its batch form, dil_verify.cu).  A task runs on one warp; its body
-// is the plain one (dil_procs.cuh) with the A^ source switched.
+// source of its batch form, dil_verify.cu; Sign's usual form, too, is one of
+// the batch's, dil_rounds.cu).  The Sign here runs a task on one warp with the
+// plain body (dil_procs.cuh) and the A^ source switched.
 #include "dil_kern.cuh"
+#include "dil_sample16.cuh"
 
 namespace dil {
 
-// A^ of task `task` at ahat + task k l N, polynomial (i, j) at index i l + j,
+// A^ of task t at ahat + t k l N, polynomial (i, j) at index i l + j,
 // coefficients in index order, each in [0, q).
 template <int LEVEL>
-__global__ void __launch_bounds__(256, 4) k_expand_a(int n, const uint8_t *__restrict__ rho, size_t rho_stride,
-                                                     int32_t *ahat) {
-    extern __shared__ __align__(16) uint8_t smem[];
-    const CtaView v = cta_setup<1>(smem);
-    const int task = blockIdx.x * v.groups + v.group;
-    if (task >= n) return;
-    using V = Lv<LEVEL>;
-    constexpr int KL = V::K * V::L;
-    stage_bytes(v.gs->rho, rho + (size_t)task * rho_stride, 32, v.lane);
-    __syncwarp();
-    expand_a_range<LEVEL>(v.gs->rho, 0, KL, ahat + (size_t)task * KL * N, *v.ws, v.lane);
+__global__ void __launch_bounds__(32, 16) k_expand_a(int n, const uint8_t *rho, size_t rho_stride, int32_t *ahat) {
+    __shared__ __align__(16) uint32_t st[EXPAND16_WORDS];
+    constexpr int KL = Lv<LEVEL>::K * Lv<LEVEL>::L;
+    expand_a_batch<LEVEL>((long long)blockIdx.x * K16_STATES, (long long)n * KL,
+                          [&](int t) { return rho + (size_t)t * rho_stride; },
+                          [&](int t) { return ahat + (size_t)t * KL * N; }, st, threadIdx.x);
 }
 
 template <int LEVEL>
@@ -66,12 +63,19 @@ __global__ void __launch_bounds__(256, 4) k_sign_a(int n, const uint8_t *__restr
     }
 }
 
-cudaError_t launch_expand_a(int level, int n, const uint8_t *rho, size_t rho_stride, int32_t *ahat, int warps,
-                            cudaStream_t s) {
+template <int LEVEL>
+static cudaError_t launch_expand(int n, const uint8_t *rho, size_t rho_stride, int32_t *ahat, cudaStream_t s) {
+    if (n <= 0) return cudaSuccess;
+    const long long polys = (long long)n * Lv<LEVEL>::K * Lv<LEVEL>::L;
+    k_expand_a<LEVEL><<<(int)((polys + K16_STATES - 1) / K16_STATES), 32, 0, s>>>(n, rho, rho_stride, ahat);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_expand_a(int level, int n, const uint8_t *rho, size_t rho_stride, int32_t *ahat, cudaStream_t s) {
     switch (level) {
-        case 2: return launch_plain(k_expand_a<2>, n, warps, 1, s, rho, rho_stride, ahat);
-        case 3: return launch_plain(k_expand_a<3>, n, warps, 1, s, rho, rho_stride, ahat);
-        case 5: return launch_plain(k_expand_a<5>, n, warps, 1, s, rho, rho_stride, ahat);
+        case 2: return launch_expand<2>(n, rho, rho_stride, ahat, s);
+        case 3: return launch_expand<3>(n, rho, rho_stride, ahat, s);
+        case 5: return launch_expand<5>(n, rho, rho_stride, ahat, s);
     }
     return cudaErrorInvalidValue;
 }

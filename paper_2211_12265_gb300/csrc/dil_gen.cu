@@ -1,32 +1,28 @@
 // KeyGen of a batch (Alg 1).
 //
-// Batch form: one task per group of P warps up to the packed keys, then a
-// kernel that hashes tr = H(pk) sixteen tasks to a warp.  In the task's own
-// warp (k_keygen, kept for the launch shapes a caller asks for) the ten blocks
-// of a Dilithium2 key cost 4.5 k of the task's 19.4 k SM clocks (10,000 keys:
-// 616 -> 550 us).
-#include "dil_hash16.cuh"
+// Batch form, four kernels: H(zeta), sixteen tasks to a warp; ExpandA and
+// ExpandS, sixteen polynomials to a warp whatever tasks they belong to
+// (dil_sample16.cuh); t = A s1 + s2 and the packed keys, one task per group of P
+// warps; tr = H(pk), sixteen tasks to a warp.  In the task's own warp
+// (k_keygen, kept for the launch shapes a caller asks for) the eleven blocks of
+// a Dilithium2 key's hashes cost 4.9 k of the task's 19.4 k SM clocks (10,000
+// keys, fused -> batch: 616 -> 533 us).
 #include "dil_kern.cuh"
+#include "dil_sample16.cuh"
 
 namespace dil {
 
-template <int LEVEL, int P, bool SPLIT>
-__device__ __forceinline__ void keygen_body(int n, const uint8_t *__restrict__ seeds, uint8_t *pk, uint8_t *sk,
-                                            int32_t *scratch) {
+template <int LEVEL, int P>
+__global__ void __launch_bounds__(256, 4) k_keygen(int n, const uint8_t *__restrict__ seeds, uint8_t *pk,
+                                                   uint8_t *sk, int32_t *scratch) {
     extern __shared__ __align__(16) uint8_t smem[];
     const CtaView v = cta_setup<P>(smem);
     const int task = blockIdx.x * v.groups + v.group;
     if (task >= n) return;
     using V = Lv<LEVEL>;
-    gen_task<LEVEL, P, SPLIT>(seeds + (size_t)task * 32, pk + (size_t)task * V::PK, sk + (size_t)task * V::SK,
-                              scratch + (size_t)task * Scratch<LEVEL>::GEN_POLYS * N, *v.gs, *v.ws, v.zt, v.izt, v.g,
-                              v.bar, v.lane);
-}
-
-template <int LEVEL, int P>
-__global__ void __launch_bounds__(256, 4) k_keygen(int n, const uint8_t *__restrict__ seeds, uint8_t *pk,
-                                                   uint8_t *sk, int32_t *scratch) {
-    keygen_body<LEVEL, P, false>(n, seeds, pk, sk, scratch);
+    gen_task<LEVEL, P>(seeds + (size_t)task * 32, pk + (size_t)task * V::PK, sk + (size_t)task * V::SK,
+                       scratch + (size_t)task * Scratch<LEVEL>::GEN_POLYS * N, *v.gs, *v.ws, v.zt, v.izt, v.g, v.bar,
+                       v.lane);
 }
 
 cudaError_t launch_keygen(int level, int n, const uint8_t *seeds, uint8_t *pk, uint8_t *sk, int32_t *scratch,
@@ -36,10 +32,94 @@ cudaError_t launch_keygen(int level, int n, const uint8_t *seeds, uint8_t *pk, u
 
 // ---------------------------------------------------------------- batch form
 
+// Bytes this thread of a pair writes of 4-byte words a[lo .. lo + cnt) (every
+// other word of a byte string of any alignment).
+__device__ __forceinline__ void put_words(uint8_t *dst, const uint32_t (&a)[25], int lo, int cnt) {
+#pragma unroll
+    for (int i = 0; i < 25; ++i) {
+        if (i < lo || i >= lo + cnt) continue;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) dst[8 * (i - lo) + q] = (uint8_t)(a[i] >> (8 * q));
+    }
+}
+
+// (rho, rho', K) = H(zeta) of task `pair`: rho to pk, sk and the first words of
+// its scratch's s^1 (which the arithmetic writes last), rho' behind it, K to sk.
+template <int LEVEL>
+struct KeygenSeedJob {
+    const uint8_t *seed;
+    uint8_t *pk, *sk;
+    uint32_t *out;
+    bool todo;
+    int lane;
+
+    __device__ __forceinline__ bool next(HashInput &in) {
+        if (!todo) return false;
+        todo = false;
+        in = {nullptr, seed, 32, 0};
+        return true;
+    }
+
+    __device__ __forceinline__ void done(const uint32_t (&a)[25]) {
+        const int p = lane & 1;
+#pragma unroll
+        for (int i = 0; i < 12; ++i) out[2 * i + p] = a[i];   // rho (32 bytes), rho' (64)
+        put_words(pk + 4 * p, a, 0, 4);
+        put_words(sk + 4 * p, a, 0, 4);
+        put_words(sk + 32 + 4 * p, a, 12, 4);
+    }
+};
+
+template <int LEVEL>
+__device__ __forceinline__ int32_t *gen_scratch(int32_t *scratch, int t) {
+    return scratch + (size_t)t * Scratch<LEVEL>::GEN_POLYS * N;
+}
+
+template <int LEVEL>
+__global__ void __launch_bounds__(128) k_keygen_seeds(int n, const uint8_t *seeds, uint8_t *pk, uint8_t *sk,
+                                                      int32_t *scratch) {
+    __shared__ __align__(16) uint32_t stage[4][HASH16_STAGE_WORDS];
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (w * K16_STATES >= n) return;
+    const int t = w * K16_STATES + (lane >> 1);
+    const bool mine = t < n;
+    const size_t at = mine ? t : 0;
+    KeygenSeedJob<LEVEL> job{seeds + at * 32, pk + at * Lv<LEVEL>::PK, sk + at * Lv<LEVEL>::SK,
+                             reinterpret_cast<uint32_t *>(gen_scratch<LEVEL>(scratch, (int)at)), mine, lane};
+    hash16_run(job, stage[threadIdx.x >> 5], lane);
+}
+
+// Blocks [0, s_blocks) sample s1 || s2, the others A^.  One warp per CTA, as in
+// Sign's prepare kernel.
+template <int LEVEL>
+__global__ void __launch_bounds__(32, 16) k_keygen_expand(int n, int32_t *scratch, int s_blocks) {
+    __shared__ __align__(16) uint32_t st[EXPAND16_WORDS];
+    using V = Lv<LEVEL>;
+    using S = Scratch<LEVEL>;
+    const int lane = threadIdx.x;
+    const int blk = blockIdx.x;
+    if (blk < s_blocks) {
+        expand_s_batch<LEVEL>(
+            (long long)blk * K16_STATES, (long long)n * (V::K + V::L),
+            [&](int t) { return reinterpret_cast<const uint8_t *>(gen_scratch<LEVEL>(scratch, t)) + 32; },
+            [&](int t) { return gen_scratch<LEVEL>(scratch, t) + S::GEN_S * N; }, st, lane);
+    } else {
+        expand_a_batch<LEVEL>(
+            (long long)(blk - s_blocks) * K16_STATES, (long long)n * V::K * V::L,
+            [&](int t) { return reinterpret_cast<const uint8_t *>(gen_scratch<LEVEL>(scratch, t)); },
+            [&](int t) { return gen_scratch<LEVEL>(scratch, t) + V::L * N; }, st, lane);
+    }
+}
+
 template <int LEVEL, int P>
-__global__ void __launch_bounds__(256, 4) k_keygen_batch(int n, const uint8_t *__restrict__ seeds, uint8_t *pk,
-                                                         uint8_t *sk, int32_t *scratch) {
-    keygen_body<LEVEL, P, true>(n, seeds, pk, sk, scratch);
+__global__ void __launch_bounds__(256, 4) k_keygen_rows(int n, uint8_t *pk, uint8_t *sk, int32_t *scratch) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    const CtaView v = cta_setup<P>(smem);
+    const int task = blockIdx.x * v.groups + v.group;
+    if (task >= n) return;
+    using V = Lv<LEVEL>;
+    gen_rows<LEVEL, P>(pk + (size_t)task * V::PK, sk + (size_t)task * V::SK, gen_scratch<LEVEL>(scratch, task),
+                       *v.ws, v.zt, v.izt, v.g, v.bar, v.lane);
 }
 
 // tr = H(pk) of task `pair` into its secret key.
@@ -57,18 +137,12 @@ struct KeygenTrJob {
         return true;
     }
 
-    __device__ __forceinline__ void done(const uint32_t (&a)[25]) {
-        uint8_t *tr = sk + 64 + 4 * (lane & 1);
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) tr[8 * i + q] = (uint8_t)(a[i] >> (8 * q));
-    }
+    __device__ __forceinline__ void done(const uint32_t (&a)[25]) { put_words(sk + 64 + 4 * (lane & 1), a, 0, 4); }
 };
 
 template <int LEVEL>
 __global__ void __launch_bounds__(128) k_keygen_tr(int n, const uint8_t *pk, uint8_t *sk) {
-    __shared__ uint32_t stage[4][HASH16_STAGE_WORDS];
+    __shared__ __align__(16) uint32_t stage[4][HASH16_STAGE_WORDS];
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (w * K16_STATES >= n) return;
     const int t = w * K16_STATES + (lane >> 1);
@@ -81,10 +155,18 @@ namespace {
 template <int LEVEL>
 cudaError_t launch_batch(int n, const uint8_t *seeds, uint8_t *pk, uint8_t *sk, int32_t *scratch, int warps, int p,
                          cudaStream_t s) {
-    const cudaError_t e = p == 1 ? launch_plain(k_keygen_batch<LEVEL, 1>, n, warps, p, s, seeds, pk, sk, scratch)
-                                 : launch_plain(k_keygen_batch<LEVEL, 4>, n, warps, p, s, seeds, pk, sk, scratch);
-    if (e != cudaSuccess) return e;
+    using V = Lv<LEVEL>;
     const HashGrid h = hash_grid(n);
+    k_keygen_seeds<LEVEL><<<h.blocks, h.threads, 0, s>>>(n, seeds, pk, sk, scratch);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const auto blocks = [&](long long polys) { return (int)((polys * n + K16_STATES - 1) / K16_STATES); };
+    const int s_blocks = blocks(V::K + V::L);
+    k_keygen_expand<LEVEL><<<s_blocks + blocks(V::K * V::L), 32, 0, s>>>(n, scratch, s_blocks);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = p == 1 ? launch_plain(k_keygen_rows<LEVEL, 1>, n, warps, p, s, pk, sk, scratch)
+               : launch_plain(k_keygen_rows<LEVEL, 4>, n, warps, p, s, pk, sk, scratch);
+    if (e != cudaSuccess) return e;
     k_keygen_tr<LEVEL><<<h.blocks, h.threads, 0, s>>>(n, pk, sk);
     return cudaGetLastError();
 }

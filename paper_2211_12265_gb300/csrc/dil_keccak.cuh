@@ -180,6 +180,24 @@ __device__ __forceinline__ void absorb_smem(uint32_t &lo, uint32_t &hi, const ui
     keccak_f(lo, hi);
 }
 
+// 4 bytes of global memory at p (any alignment), bytes from p + have on read
+// as 0.  Only aligned words that hold a byte below p + have are loaded, and
+// such a word lies in that byte's page, so no load can fault.  CG: through L2
+// (see ld_word_cg).
+template <bool CG = false>
+__device__ __forceinline__ uint32_t ld_bytes4(const uint8_t *p, long long have) {
+    if (have <= 0) return 0;
+    const uint32_t mis = (uint32_t)reinterpret_cast<uintptr_t>(p) & 3u;
+    const uint32_t *q = reinterpret_cast<const uint32_t *>(p - mis);
+    uint32_t v = CG ? __ldcg(q) : q[0];
+    if (mis) {
+        uint32_t w = 0;
+        if (have > (long long)(4 - mis)) w = CG ? __ldcg(q + 1) : q[1];
+        v = __funnelshift_r(v, w, 8 * mis);
+    }
+    return have < 4 ? v & ((1u << (8 * (int)have)) - 1u) : v;
+}
+
 // Aligned 8-byte word of global memory, loaded through L2: coherent with
 // stores and copies made while the kernel runs (a serving kernel reuses its
 // request buffers), unlike the L1 and read-only paths.

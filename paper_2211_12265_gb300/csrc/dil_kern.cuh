@@ -31,7 +31,7 @@ __device__ __forceinline__ CtaView cta_setup(uint8_t *smem) {
     v.izt = v.zt + NTT_TABLE_WORDS;
     GroupSmem *gsa = reinterpret_cast<GroupSmem *>(smem + CTA_TABLE_BYTES);
     WarpSmem *wsa = reinterpret_cast<WarpSmem *>(smem + CTA_TABLE_BYTES + v.groups * sizeof(GroupSmem));
-    load_zetas(v.zt, v.izt);
+    load_zetas(v.zt);
     __syncthreads();
     const int warp = threadIdx.x >> 5;
     v.lane = threadIdx.x & 31;

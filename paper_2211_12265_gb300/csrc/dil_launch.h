@@ -55,12 +55,13 @@ struct VerifyBatch {
     const uint8_t *key_tr;
     int n_keys;
     uint32_t *mu, *tr;       // per task 16 and (not VERIFY_KEYED) 8 words
+    uint8_t *challenge;      // per task 256 bytes
     int *next;               // counter of the hashing warps
-    int hash_warps, hash_blocks;   // set by the launch
+    int hash_warps, hash_blocks, challenge_blocks;   // set by the launch
 };
-// Per task beside the polynomials: mu (64), tr (32) and 32 more, of which the
-// batch's counter takes the first.
-constexpr size_t VERIFY_AUX_BYTES = 128;
+// Per task beside the polynomials: mu (64), tr (32), 32 more, of which the
+// batch's counter takes the first, and the challenge (256).
+constexpr size_t VERIFY_AUX_BYTES = 384;
 cudaError_t launch_verify_batch(int level, int src, const VerifyBatch &b, int warps, int p, cudaStream_t s);
 // Sign in rounds (dil_rounds.cu).  Where a task's A^, s^1, s^2 and t^0 come from:
 // its secret key, that with the caller's A^, or a resident key.
@@ -82,7 +83,7 @@ struct SignBatch {
     int32_t *pre, *slot_polys;
     uint32_t *mu, *rhop;
     int *pending, *best, *done, *next, *count;
-    int hash_warps, hash_blocks, expand_blocks;
+    int hash_warps, expand_blocks;
 };
 int sign_batch_slots(int level, int n);       // slots worth having
 int sign_batch_min_slots(int level, int n);   // slots needed
@@ -96,8 +97,7 @@ cudaError_t warm_sign(int level, int warps, int p, cudaStream_t s);
 // from rho (task i's 32 bytes at rho + i rho_stride) into ahat (n x k l x 256
 // words, 16-byte aligned); Sign with task i's A^ at ahat + i k l 256 instead of
 // ExpandA (Verify: launch_verify_batch).
-cudaError_t launch_expand_a(int level, int n, const uint8_t *rho, size_t rho_stride, int32_t *ahat, int warps,
-                            cudaStream_t s);
+cudaError_t launch_expand_a(int level, int n, const uint8_t *rho, size_t rho_stride, int32_t *ahat, cudaStream_t s);
 cudaError_t launch_sign_a(int level, int n, const uint8_t *sk, const uint8_t *msg, const uint64_t *off,
                           const int32_t *ahat, uint8_t *sig, int32_t *status, int32_t *iters, int32_t *scratch,
                           int max_iter, int warps, cudaStream_t s);

@@ -22,7 +22,7 @@
 
 namespace dil {
 
-struct Zetas {
+struct __align__(16) Zetas {
     int32_t z[256], zs[256];     // zeta^brv8(k) mod q, centred, and its quotient
     int32_t iz[256], izs[256];   // zeta^-brv8(k)
 };
@@ -72,7 +72,8 @@ constexpr Zetas make_zetas() {
 }
 }  // namespace detail
 
-static __constant__ Zetas c_zetas = detail::make_zetas();
+static __constant__ Zetas c_zetas = detail::make_zetas();       // factors the code names one by one
+static __device__ const Zetas g_zetas = detail::make_zetas();   // the source of the shared tables
 
 // Final INTT level scale: mont(F, x) = x * 2^32 / 256 and
 // mont(G, x) = x * zeta^-brv8(1) * 2^32 / 256 (mod q).
@@ -321,20 +322,15 @@ __device__ __forceinline__ void ntt_inv(int32_t r[8], int32_t *buf, const int32_
     for (int m = 0; m < 8; ++m) r[m] = p.v[m];
 }
 
-// Loads the twiddle tables (NTT_TABLE_WORDS each) into shared memory (whole
-// block participates).
-__device__ __forceinline__ void load_zetas_fwd(int32_t *zt) {
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
-        zt[i] = c_zetas.z[i];
-        zt[256 + i] = c_zetas.zs[i];
-    }
-}
-__device__ __forceinline__ void load_zetas(int32_t *zt, int32_t *izt) {
-    load_zetas_fwd(zt);
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
-        izt[i] = c_zetas.iz[i];
-        izt[256 + i] = c_zetas.izs[i];
-    }
+// Copies the forward twiddles (NTT_TABLE_WORDS), or those and behind them the
+// inverse ones, to 16-byte aligned shared memory (whole block participates).
+// From global memory: constant memory serves lanes that ask for different words
+// one after the other, 32 reads per warp and word.
+template <int TABLES = 2>
+__device__ __forceinline__ void load_zetas(int32_t *zt) {
+    static_assert(sizeof(Zetas) == 2 * NTT_TABLE_WORDS * sizeof(int32_t), "forward, then inverse");
+    for (int i = threadIdx.x; i < TABLES * NTT_TABLE_WORDS / 4; i += blockDim.x)
+        reinterpret_cast<int4 *>(zt)[i] = __ldg(reinterpret_cast<const int4 *>(&g_zetas) + i);
 }
 
 // Transposes 8 values from L0 to 8 consecutive coefficients (8 lane + m).

@@ -174,7 +174,7 @@ template <int LEVEL> struct Scratch {
     static constexpr int Z = W + V::K;
     static constexpr int ITR_POLYS = Z + V::L;
     static constexpr int SIGN_POLYS = PRE_POLYS + ITR_POLYS;
-    static constexpr int GEN_S = V::L + V::K * V::L;         // s1 || s2, coefficient order (one-warp groups)
+    static constexpr int GEN_S = V::L + V::K * V::L;         // s1 || s2, coefficient order
     static constexpr int GEN_POLYS = GEN_S + V::L + V::K;     // s^1 | A^ | s1 || s2
     static constexpr int VERIFY_POLYS = V::L + V::K * V::L;   // z^, A^
     static constexpr int KEYED_VERIFY_POLYS = V::L;           // z^ (A^ is resident)
@@ -307,21 +307,25 @@ __device__ void mask_stream(const uint8_t *rhop, int kappa, MaskStream &ms, int3
     }
 }
 
-// acc = sum_j A^_ij o v^_j (pointwise Montgomery products) for one row i of A^
-// (ahat: the row's l polynomials, index order; read through L2 since another
-// warp or kernel may have written them); v^_j (index order) at `vhat`.
+// acc = sum_j A^_ij o v^_j 2^-32, |acc| < q, for one row i of A^ (ahat: the row's
+// l polynomials, index order; read through L2 since another warp or kernel may
+// have written them); v^_j (index order) at `vhat`.  The products are summed in
+// 64 bits (|sum| < 7 q 9.1q < 2^31 q) and reduced once.
 __device__ __forceinline__ void accumulate_row(int32_t acc[8], const int32_t *ahat, int l, const int32_t *vhat,
                                                int lane) {
-    int32_t a[8], v[8];
+    long long sum[8];
 #pragma unroll
-    for (int m = 0; m < 8; ++m) acc[m] = 0;
+    for (int m = 0; m < 8; ++m) sum[m] = 0;
 #pragma unroll 1
     for (int j = 0; j < l; ++j) {
+        int32_t a[8], v[8];
         load_l2_cg(a, ahat + j * N, lane);
         load_l2(v, vhat + j * N, lane);
 #pragma unroll
-        for (int m = 0; m < 8; ++m) acc[m] += mont_mul(a[m], v[m]);
+        for (int m = 0; m < 8; ++m) sum[m] += (long long)a[m] * v[m];
     }
+#pragma unroll
+    for (int m = 0; m < 8; ++m) acc[m] = mont_reduce(sum[m]);
 }
 
 // c^ = NTT(SampleInBall(c~)) in layout L2 (every warp of a group computes it).
@@ -335,15 +339,56 @@ __device__ __forceinline__ void challenge_hat(int32_t ch[8], const uint8_t *ctil
 }
 
 // -------------------------------------------------------------------------
-// Alg 1: Gen.  seed: 32 bytes.  pk, sk: outputs.  scratch: GEN_POLYS polys.
-// SPLIT: tr = H(pk) is left to a later kernel (dil_gen.cu).
+// Alg 1: Gen.  pk, sk: outputs.  scratch: GEN_POLYS polys.
 // -------------------------------------------------------------------------
-template <int LEVEL, int P, bool SPLIT = false>
+
+// From A^ and s1 || s2 in scratch: s1 and s2 packed into sk, t = A s1 + s2, and
+// t1, t0 packed into pk and sk.
+template <int LEVEL, int P>
+__device__ void gen_rows(uint8_t *pk, uint8_t *sk, int32_t *scratch, WarpSmem &ws, const int32_t *zt,
+                         const int32_t *izt, int g, int bar, int lane) {
+    using V = Lv<LEVEL>;
+    const int32_t *sraw = scratch + Scratch<LEVEL>::GEN_S * N;
+    int32_t r[8], a[8], acc[8];
+    // s^1 over the start of scratch, which holds nothing that is still read
+#pragma unroll 1
+    for (int j = g; j < V::L; j += P) {
+        load_l2(a, sraw + j * N, lane);
+        pack_seq<V::ETABITS>(sk + V::SK_S1 + j * V::POLYETA, a, V::ETA, -1, lane);
+        load_l0(r, sraw + j * N, lane);
+        ntt_fwd(r, ws.buf, zt, lane);
+        store_l2(scratch + j * N, r, lane);
+    }
+    group_sync<P>(bar);
+    // t = INTT(A^ o s^1) + s2; (t1, t0) = Power2Round(t), row i into pk and sk
+#pragma unroll 1
+    for (int i = g; i < V::K; i += P) {
+        accumulate_row(acc, scratch + (V::L + i * V::L) * N, V::L, scratch, lane);
+        ntt_inv(acc, ws.buf, izt, lane);
+        load_l2(a, sraw + (V::L + i) * N, lane);
+        load_l0(r, sraw + (V::L + i) * N, lane);
+        pack_seq<V::ETABITS>(sk + V::SK_S2 + i * V::POLYETA, a, V::ETA, -1, lane);
+        int32_t t1[8], t0[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            int32_t t = to_canonical(acc[m]) + r[m];      // (-eta, q + eta)
+            t += (t < 0) ? Q : 0;
+            t -= (t >= Q) ? Q : 0;
+            power2round(t, t1[m], t0[m]);
+        }
+        l0_to_seq(t1, ws.buf, lane);
+        pack_seq<10>(pk + 32 + i * V::POLYT1, t1, 0, 1, lane);
+        l0_to_seq(t0, ws.buf, lane);
+        pack_seq<D>(sk + V::SK_T0 + i * V::POLYT0, t0, 1 << (D - 1), -1, lane);
+    }
+}
+
+// A whole key from its 32-byte seed.
+template <int LEVEL, int P>
 __device__ void gen_task(const uint8_t *__restrict__ seed, uint8_t *pk, uint8_t *sk, int32_t *scratch,
                          GroupSmem &gs, WarpSmem &ws, const int32_t *zt, const int32_t *izt, int g, int bar,
                          int lane) {
     using V = Lv<LEVEL>;
-    int32_t r[8], a[8], acc[8];
     // (rho, rho', K) = H(zeta)  (Alg 1)
     if (g == 0) {
         stage_bytes(gs.hb, seed, 32, lane);
@@ -361,79 +406,29 @@ __device__ void gen_task(const uint8_t *__restrict__ seed, uint8_t *pk, uint8_t 
         gs.rhop[32 + lane] = gs.hb[64 + lane];
     }
     group_sync<P>(bar);
-    using S = Scratch<LEVEL>;
-    int32_t *sraw = scratch + S::GEN_S * N;
-    if constexpr (P == 1) {
-        // s1 || s2 = ExpandS(rho'): all l + k sponges in one sixteen-state batch,
-        // then s1: pack into sk, NTT
-        expand_s_16<V::ETA>(gs.rhop, V::L + V::K, sraw, ws.k16, lane);
+    // s1 || s2 = ExpandS(rho') and A^ = ExpandA(rho) into scratch
+    int32_t *sraw = scratch + Scratch<LEVEL>::GEN_S * N;
+    constexpr int SP = V::L + V::K, U = Units<SP, P>::SIZE;
 #pragma unroll 1
-        for (int j = 0; j < V::L; ++j) {
-            load_l2(a, sraw + j * N, lane);
-            pack_seq<V::ETABITS>(sk + V::SK_S1 + j * V::POLYETA, a, V::ETA, -1, lane);
-            load_l0(r, sraw + j * N, lane);
-            ntt_fwd(r, ws.buf, zt, lane);
-            store_l2(scratch + j * N, r, lane);
-        }
-    }
-    // s1: sample, pack into sk, NTT (task groups of several warps)
-    constexpr int U1 = Units<V::L, P>::SIZE;
-#pragma unroll 1
-    for (int j = U1 * g; j < V::L && P > 1; j += U1 * P) {
-        const bool two = U1 == 2 && j + 1 < V::L;
-        if (two)
+    for (int j = U * g; j < SP; j += U * P) {
+        const bool two = U == 2 && j + 1 < SP;
+        int32_t r[8];
+        if (two) {
             expand_s_pair<V::ETA>(gs.rhop, j, j + 1, ws.buf, ws.buf2, ws.sq, ws.sq2, lane);
-        else
-            expand_s_poly<V::ETA>(gs.rhop, j, ws.buf2, ws.sq, lane);
-        for (int h = two ? 0 : 1; h < 2; ++h) {
-            const int32_t *src = h ? ws.buf2 : ws.buf;
-            const int jj = two ? j + h : j;
-#pragma unroll
-            for (int m = 0; m < 8; ++m) a[m] = src[8 * lane + m + 4 * (lane >> 2)];
-            pack_seq<V::ETABITS>(sk + V::SK_S1 + jj * V::POLYETA, a, V::ETA, -1, lane);
-            read_buf_l0(r, src, lane);
-            __syncwarp();
-            ntt_fwd(r, ws.buf, zt, lane);
-            store_l2(scratch + jj * N, r, lane);
-        }
-    }
-    // t = INTT(A^ o s^1) + s2; (t1, t0) = Power2Round(t), row i into pk and sk
-    auto row = [&](int i) {
-        accumulate_row(acc, scratch + (V::L + i * V::L) * N, V::L, scratch, lane);
-#pragma unroll
-        for (int m = 0; m < 8; ++m) acc[m] = reduce_q(acc[m]);
-        ntt_inv(acc, ws.buf, izt, lane);
-        if constexpr (P == 1) {
-            load_l2(a, sraw + (V::L + i) * N, lane);
-            load_l0(r, sraw + (V::L + i) * N, lane);
+            read_buf_l0(r, ws.buf2, lane);
+            store_l0(sraw + (j + 1) * N, r, lane);
         } else {
-            expand_s_poly<V::ETA>(gs.rhop, V::L + i, ws.buf, ws.sq, lane);
-#pragma unroll
-            for (int m = 0; m < 8; ++m) a[m] = ws.buf[8 * lane + m + 4 * (lane >> 2)];
-            read_buf_l0(r, ws.buf, lane);
-            __syncwarp();
+            expand_s_poly<V::ETA>(gs.rhop, j, ws.buf, ws.sq, lane);
         }
-        pack_seq<V::ETABITS>(sk + V::SK_S2 + i * V::POLYETA, a, V::ETA, -1, lane);
-        int32_t t1[8], t0[8];
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            int32_t t = to_canonical(acc[m]) + r[m];      // (-eta, q + eta)
-            t += (t < 0) ? Q : 0;
-            t -= (t >= Q) ? Q : 0;
-            power2round(t, t1[m], t0[m]);
-        }
-        l0_to_seq(t1, ws.buf, lane);
-        pack_seq<10>(pk + 32 + i * V::POLYT1, t1, 0, 1, lane);
-        l0_to_seq(t0, ws.buf, lane);
-        pack_seq<D>(sk + V::SK_T0 + i * V::POLYT0, t0, 1 << (D - 1), -1, lane);
-    };
+        read_buf_l0(r, ws.buf, lane);
+        store_l0(sraw + j * N, r, lane);
+        __syncwarp();
+    }
     constexpr int KL = V::K * V::L;
-    // A^ = ExpandA(rho) into scratch after s^1, then the rows of t
     expand_a_range<LEVEL>(gs.rho, share_lo<KL, P>(g), share_lo<KL, P>(g + 1), scratch + V::L * N, ws, lane);
+    __threadfence_block();
     group_sync<P>(bar);
-#pragma unroll 1
-    for (int i = g; i < V::K; i += P) row(i);
-    if constexpr (SPLIT) return;
+    gen_rows<LEVEL, P>(pk, sk, scratch, ws, zt, izt, g, bar, lane);
     __threadfence_block();
     group_sync<P>(bar);
     // tr = H(rho || t1)
@@ -594,7 +589,7 @@ __device__ bool sign_front(int kappa, const int32_t *pre, int32_t *itr, MaskStre
     using V = Lv<LEVEL>;
     using S = Scratch<LEVEL>;
     volatile int *vflag = &gs.flag;
-    int32_t r[8], a[8], acc[8];
+    int32_t r[8], acc[8];
     // y = ExpandMask(rho', kappa); y^ = NTT(y)
     if constexpr (P == 1)
         mask_stream<LEVEL>(gs.rhop, kappa, ms, itr + S::Y * N, itr + S::YH * N, ws, zt, lane);
@@ -605,17 +600,7 @@ __device__ bool sign_front(int kappa, const int32_t *pre, int32_t *itr, MaskStre
     // w = INTT(A^ o y^); w1 = HighBits(w)
 #pragma unroll 1
     for (int i = g; i < V::K; i += P) {
-#pragma unroll
-        for (int m = 0; m < 8; ++m) acc[m] = 0;
-#pragma unroll 1
-        for (int j = 0; j < V::L; ++j) {
-            load_l2_cg(a, pre + (S::AH + i * V::L + j) * N, lane);
-            load_l2(r, itr + (S::YH + j) * N, lane);
-#pragma unroll
-            for (int m = 0; m < 8; ++m) acc[m] += mont_mul(a[m], r[m]);
-        }
-#pragma unroll
-        for (int m = 0; m < 8; ++m) acc[m] = reduce_q(acc[m]);
+        accumulate_row(acc, pre + (S::AH + i * V::L) * N, V::L, itr + S::YH * N, lane);
         ntt_inv(acc, ws.buf, izt, lane);
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
@@ -797,13 +782,14 @@ __device__ void sign_zero(uint8_t *sig, int g, int lane) {
 // beforehand.
 // SPLIT: the task's hashes run elsewhere (dil_verify.cu): nothing of msg or tr
 // is read, the packed w1' goes to the start of scratch instead of into
-// c~ = H(mu || w1'), and 1 means that only that comparison is left.
+// c~ = H(mu || w1'), and 1 means that only that comparison is left.  c_in
+// (nullable): SampleInBall(c~), 256 signed bytes.
 template <int LEVEL, int P, bool KEYED = false, bool AHAT = false, bool SPLIT = false>
 __device__ int verify_task(const uint8_t *__restrict__ pk, const uint8_t *__restrict__ msg, size_t mlen,
                            const uint8_t *__restrict__ sig, int32_t *scratch, GroupSmem &gs, WarpSmem &ws,
                            const int32_t *zt, const int32_t *izt, int g, int bar, int lane,
                            const int32_t *key = nullptr, const uint8_t *tr = nullptr,
-                           const uint8_t *mu_in = nullptr) {
+                           const uint8_t *mu_in = nullptr, const int8_t *c_in = nullptr) {
     using V = Lv<LEVEL>;
     volatile int *vflag = &gs.flag;
     int32_t r[8], acc[8], ch[8];
@@ -880,7 +866,13 @@ __device__ int verify_task(const uint8_t *__restrict__ pk, const uint8_t *__rest
     group_sync<P>(bar);
     if (*vflag) return 0;
     // c^ = NTT(SampleInBall(c~))
-    challenge_hat<LEVEL>(ch, gs.ctilde, ws, zt, lane);
+    if (SPLIT && c_in) {
+#pragma unroll
+        for (int m = 0; m < 8; ++m) ch[m] = c_in[lane + 32 * m];
+        ntt_fwd(ch, ws.buf, zt, lane);
+    } else {
+        challenge_hat<LEVEL>(ch, gs.ctilde, ws, zt, lane);
+    }
     // v = INTT(A^ o z^ - c^ o NTT(t1 2^d)); w1' = UseHint(h, v)
     using S = Scratch<LEVEL>;
     const int32_t *ahat = KEYED ? key + S::AH * N : AHAT ? key : scratch + V::L * N;

@@ -21,9 +21,9 @@
 // its output unused (masks sampled sixteen nonces ahead), each kernel's code
 // fits the instruction cache (the fused kernel's first stall is instruction
 // fetch), and no SM idles while a few tasks run 20 to 30 repetitions one after
-// the other.  Fused -> rounds: 10,000 Dilithium2 tasks 3396 -> 2021 us, 10,000
-// Dilithium3 (32 B - 4 KB) 5350 -> 3209 us, 150 Dilithium5 1580 -> 455 us, one
-// Dilithium2 task 318 -> 126 us.
+// the other.  Fused -> rounds: 10,000 Dilithium2 tasks 3396 -> 1848 us, 10,000
+// Dilithium3 (32 B - 4 KB) 5350 -> 2945 us, 150 Dilithium5 1580 -> 408 us, one
+// Dilithium2 task 176 -> 119 us.
 #include <climits>
 
 #include "dil_kern.cuh"
@@ -145,21 +145,11 @@ struct SignMuJob {
     }
 };
 
-// Copies nbytes (a multiple of 4) from global memory to shared memory.
-__device__ __forceinline__ void stage_words(uint8_t *dst, const uint8_t *src, int nbytes, int lane) {
-    if ((reinterpret_cast<uintptr_t>(src) & 3) == 0) {
-        for (int i = lane; i < nbytes / 4; i += 32)
-            reinterpret_cast<uint32_t *>(dst)[i] = reinterpret_cast<const uint32_t *>(src)[i];
-    } else {
-        for (int i = lane; i < nbytes; i += 32) dst[i] = src[i];
-    }
-}
-
 // As unpack_poly_l0, with buf (a warp's exchange buffer) as staging.
 template <int BITS>
 __device__ __forceinline__ void unpack_words_l0(int32_t v[8], const uint8_t *src, int32_t off, int32_t *buf, int lane) {
     uint8_t *sq = reinterpret_cast<uint8_t *>(buf);
-    stage_words(sq, src, N * BITS / 8, lane);
+    stage_bytes(sq, src, N * BITS / 8, lane);
     __syncwarp();
 #pragma unroll
     for (int m = 0; m < 8; ++m) v[m] = off - (int32_t)get_field(sq, BITS * (lane + 32 * m), BITS);
@@ -184,41 +174,38 @@ __device__ __forceinline__ void sign_secrets(const uint8_t *sk, int32_t *pre, in
     }
 }
 
-constexpr int ROUND_WARPS = 4;   // warps per CTA of every kernel here
+constexpr int ROUND_WARPS = 4;   // warps per CTA of the kernels with a warp per attempt
 
-// Blocks [0, hash_blocks) hash, [.., + expand_blocks) sample A^ (SIGN_AHAT:
-// none), the rest transform the secrets (SIGN_KEYED: none), one task per warp;
-// with SIGN_AHAT they also copy the caller's A^.
+// One warp per CTA: a sampling warp's 11 to 13 KB of shared memory let sixteen
+// be resident on an SM, and single warps spread over the SMs to within one (in
+// fours, 2,500 mask warps made 625 CTAs for 608 places, a second wave of 17).
+// Blocks [0, hash_warps) hash, [.., + expand_blocks) sample A^ (SIGN_AHAT:
+// none), the rest transform the secrets (SIGN_KEYED: none), one task each; with
+// SIGN_AHAT they also copy the caller's A^.
 template <int LEVEL, int SRC>
-__global__ void __launch_bounds__(32 * ROUND_WARPS, 4) k_sign_prepare(const SignBatch b) {
+__global__ void __launch_bounds__(32, 16) k_sign_prepare(const SignBatch b) {
     extern __shared__ __align__(16) uint32_t sm[];
     using V = Lv<LEVEL>;
     constexpr int KL = V::K * V::L;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int lane = threadIdx.x;
     int blk = blockIdx.x;
-    if (blk < b.hash_blocks) {
-        const int w = blk * ROUND_WARPS + warp;
-        if (w >= b.hash_warps) return;
-        SignMuJob<LEVEL, SRC> job(b, w * K16_STATES + (lane >> 1), lane);
-        hash16_run(job, sm + warp * HASH16_STAGE_WORDS, lane);
+    if (blk < b.hash_warps) {
+        SignMuJob<LEVEL, SRC> job(b, blk * K16_STATES + (lane >> 1), lane);
+        hash16_run(job, sm, lane);
         return;
     }
     if constexpr (SRC != SIGN_KEYED) {
-        blk -= b.hash_blocks;
+        blk -= b.hash_warps;
         if (blk < b.expand_blocks) {
-            const long long first = (long long)(blk * ROUND_WARPS + warp) * K16_STATES;
             expand_a_batch<LEVEL>(
-                first, (long long)b.n * KL, [&](int t) { return b.sk + (size_t)t * V::SK; },
-                [&](int t) { return b.pre + (size_t)t * Scratch<LEVEL>::PRE_POLYS * N; }, sm + warp * EXPAND16_WORDS,
-                lane);
+                (long long)blk * K16_STATES, (long long)b.n * KL, [&](int t) { return b.sk + (size_t)t * V::SK; },
+                [&](int t) { return b.pre + (size_t)t * Scratch<LEVEL>::PRE_POLYS * N; }, sm, lane);
             return;
         }
-        blk -= b.expand_blocks;
-        int32_t *zt = reinterpret_cast<int32_t *>(sm), *buf = zt + NTT_TABLE_WORDS + warp * 288;
-        load_zetas_fwd(zt);
-        __syncthreads();
-        const int t = blk * ROUND_WARPS + warp;
-        if (t >= b.n) return;
+        const int t = blk - b.expand_blocks;
+        int32_t *zt = reinterpret_cast<int32_t *>(sm), *buf = zt + NTT_TABLE_WORDS;
+        load_zetas<1>(zt);
+        __syncwarp();
         int32_t *pre = b.pre + (size_t)t * Scratch<LEVEL>::PRE_POLYS * N;
         if (SRC == SIGN_AHAT) copy_polys(b.ahat + (size_t)t * KL * N, 0, KL, pre, lane);
         sign_secrets<LEVEL>(b.sk + (size_t)t * V::SK, pre, buf, zt, lane);
@@ -232,15 +219,14 @@ constexpr int MASK_STRIDE = 178;
 constexpr int MASK_WORDS = K16_STATES * MASK_STRIDE;
 
 template <int LEVEL>
-__global__ void __launch_bounds__(32 * ROUND_WARPS, 4) k_sign_mask(const SignBatch b, int r) {
-    extern __shared__ __align__(16) uint32_t sm[];
+__global__ void __launch_bounds__(32, 16) k_sign_mask(const SignBatch b, int r) {
+    __shared__ __align__(16) uint32_t st[MASK_WORDS];
     using V = Lv<LEVEL>;
     constexpr int G = K16_STATES / V::L;   // attempts per warp
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int lane = threadIdx.x;
     const Round q = round_of(b, r);
-    const int attempts = q.p * q.m, first = (blockIdx.x * ROUND_WARPS + warp) * G;
+    const int attempts = q.p * q.m, first = blockIdx.x * G;
     if (first >= attempts) return;
-    uint32_t *st = sm + warp * MASK_WORDS;
     const int s = lane >> 1, p = lane & 1;
     const int slot = min(first + s / V::L, attempts - 1), i = slot / q.m;
     const int rep = q.base + slot - i * q.m;
@@ -305,7 +291,7 @@ template <int LEVEL>
 constexpr int front_warp_words() { return 288 + Lv<LEVEL>::L * N; }
 
 template <int LEVEL, int SRC>
-__global__ void __launch_bounds__(32 * ROUND_WARPS, LEVEL == 5 ? 6 : 8) k_sign_front(const SignBatch b, int r) {
+__global__ void __launch_bounds__(32 * ROUND_WARPS, LEVEL == 2 ? 7 : 5) k_sign_front(const SignBatch b, int r) {
     extern __shared__ __align__(16) uint32_t sm[];
     using V = Lv<LEVEL>;
     using S = Scratch<LEVEL>;
@@ -313,7 +299,7 @@ __global__ void __launch_bounds__(32 * ROUND_WARPS, LEVEL == 5 ? 6 : 8) k_sign_f
     const int attempts = q.p * q.m;
     if ((int)blockIdx.x * ROUND_WARPS >= attempts) return;
     int32_t *zt = reinterpret_cast<int32_t *>(sm), *izt = zt + NTT_TABLE_WORDS;
-    load_zetas(zt, izt);
+    load_zetas(zt);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int s = blockIdx.x * ROUND_WARPS + warp;
@@ -334,13 +320,16 @@ __global__ void __launch_bounds__(32 * ROUND_WARPS, LEVEL == 5 ? 6 : 8) k_sign_f
         long long acc[8];
 #pragma unroll
         for (int m = 0; m < 8; ++m) acc[m] = 0;
-#pragma unroll 1
+        // every load of the row is in flight before the first product: A^ comes from L2 or DRAM
+        int32_t a[V::L][8];
+#pragma unroll
+        for (int j = 0; j < V::L; ++j) load_l2(a[j], pre + (S::AH + i * V::L + j) * N, lane);
+#pragma unroll
         for (int j = 0; j < V::L; ++j) {
-            int32_t a[8], y[8];
-            load_l2(a, pre + (S::AH + i * V::L + j) * N, lane);
+            int32_t y[8];
             load_l2(y, yh + j * N, lane);
 #pragma unroll
-            for (int m = 0; m < 8; ++m) acc[m] += (long long)a[m] * y[m];
+            for (int m = 0; m < 8; ++m) acc[m] += (long long)a[j][m] * y[m];
         }
 #pragma unroll
         for (int m = 0; m < 8; ++m) v[m] = mont_reduce(acc[m]);
@@ -378,14 +367,9 @@ struct SignCtJob {
     }
 };
 
-// Shared words of a hashing warp: the stage, then sixteen challenges of 256
-// bytes.
-constexpr int CHALLENGE_STRIDE = 65;   // words from one pair's challenge to the next
-constexpr int HASH_WARP_WORDS = HASH16_STAGE_WORDS + K16_STATES * CHALLENGE_STRIDE;
-
 template <int LEVEL>
 __global__ void __launch_bounds__(32 * ROUND_WARPS, 4) k_sign_hash(const SignBatch b, int r) {
-    __shared__ uint32_t sm[ROUND_WARPS][HASH_WARP_WORDS];
+    __shared__ __align__(16) uint32_t sm[ROUND_WARPS][CHALLENGE_WORDS];
     using V = Lv<LEVEL>;
     using SL = Slot<LEVEL>;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, pair = lane >> 1, p = lane & 1;
@@ -393,7 +377,6 @@ __global__ void __launch_bounds__(32 * ROUND_WARPS, 4) k_sign_hash(const SignBat
     const int attempts = q.p * q.m, first = (blockIdx.x * (blockDim.x >> 5) + warp) * K16_STATES;
     if (first >= attempts) return;
     uint32_t *stage = sm[warp];
-    uint8_t *c = reinterpret_cast<uint8_t *>(stage + HASH16_STAGE_WORDS + pair * CHALLENGE_STRIDE);
     const int s = first + pair;
     const bool mine = s < attempts;
     const int task = mine ? pending_list(b, r)[s / q.m] : 0;
@@ -404,50 +387,10 @@ __global__ void __launch_bounds__(32 * ROUND_WARPS, 4) k_sign_hash(const SignBat
 #pragma unroll
         for (int i = 0; i < 4; ++i) reinterpret_cast<uint32_t *>(x + SL::XCT)[2 * i + p] = job.ct[i];
     }
-    // c = SampleInBall(c~): the blocks go through the stage, the even thread of
-    // each pair draws and swaps (the order Alg 2 gives)
-    uint32_t a[25];
-#pragma unroll
-    for (int i = 0; i < 25; ++i) a[i] = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) a[i] = job.ct[i];
-    if (!p) a[4] = 0x1Fu;
-    if (p) a[16] = 0x80000000u;
-    for (int i = p; i < 64; i += 2) reinterpret_cast<uint32_t *>(c)[i] = 0;
-    bool more = mine;
-    int i = N - V::TAU, pos = 8;
-    uint64_t signs = 0;
-    for (int blk = 0; blk < MAX_SQUEEZE_BLOCKS && __any_sync(FULL, more); ++blk) {
-        hash16_permute(a, p);
-        __syncwarp();
-#pragma unroll
-        for (int w = 0; w < 17; ++w) stage[k16_word(pair, 2 * w + p)] = a[w];
-        __syncwarp();
-        if (more && !p) {
-            if (blk == 0)
-                signs = ((uint64_t)stage[k16_word(pair, 1)] << 32) | stage[k16_word(pair, 0)];
-            while (i < N && pos < 136) {
-                const int at = (stage[k16_word(pair, pos >> 2)] >> (8 * (pos & 3))) & 0xFF;
-                ++pos;
-                if (at > i) continue;
-                c[i] = c[at];
-                c[at] = (signs & 1) ? 0xFF : 1;
-                signs >>= 1;
-                ++i;
-            }
-            pos = 0;
-        }
-        more = more && pair_bcast(i, lane) < N;
-    }
-    __syncwarp();
-    // 256 bytes of each challenge over its slot's w1, which every pair of the
-    // warp has absorbed
-    for (int u = 0; u < K16_STATES && first + u < attempts; ++u) {
-        const uint32_t *src = stage + HASH16_STAGE_WORDS + u * CHALLENGE_STRIDE;
-        uint32_t *dst = reinterpret_cast<uint32_t *>(slot_of<LEVEL>(b, first + u) + SL::X * N);
-        dst[lane] = src[lane];
-        dst[lane + 32] = src[lane + 32];
-    }
+    challenge16<V::TAU>(job.ct, mine, stage, lane);
+    // over the slot's w1, which every pair of the warp has absorbed
+    for (int u = 0; u < K16_STATES && first + u < attempts; ++u)
+        put_challenge(reinterpret_cast<uint8_t *>(slot_of<LEVEL>(b, first + u) + SL::X * N), stage, u, lane);
 }
 
 // ---------------------------------------------------------------- back
@@ -573,7 +516,7 @@ __global__ void __launch_bounds__(32 * ROUND_WARPS, 8) k_sign_back(const SignBat
     const int attempts = q.p * q.m;
     if ((int)blockIdx.x * ROUND_WARPS >= attempts) return;
     int32_t *zt = reinterpret_cast<int32_t *>(sm), *izt = zt + NTT_TABLE_WORDS;
-    load_zetas(zt, izt);
+    load_zetas(zt);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int s = blockIdx.x * ROUND_WARPS + warp;
@@ -743,28 +686,23 @@ cudaError_t launch_rounds(SignBatch b, void *ws, cudaStream_t s) {
 
     // prepare
     b.hash_warps = batch_hash_warps(b.n);
-    b.hash_blocks = blocks_for(b.hash_warps, ROUND_WARPS);
-    b.expand_blocks = SRC == SIGN_PLAIN ? blocks_for((long long)b.n * V::K * V::L, K16_STATES * ROUND_WARPS) : 0;
-    const int secret_blocks = SRC == SIGN_KEYED ? 0 : blocks_for(b.n, ROUND_WARPS);
+    b.expand_blocks = SRC == SIGN_PLAIN ? blocks_for((long long)b.n * V::K * V::L, K16_STATES) : 0;
+    const int secret_blocks = SRC == SIGN_KEYED ? 0 : b.n;
     const size_t tables = 4 * NTT_TABLE_WORDS;
-    const size_t prep_smem = 4 * ROUND_WARPS * (SRC == SIGN_PLAIN ? EXPAND16_WORDS : HASH16_STAGE_WORDS);
-    static_assert(4 * NTT_TABLE_WORDS + 4 * 288 * ROUND_WARPS <= 4 * ROUND_WARPS * HASH16_STAGE_WORDS,
-                  "the secrets' blocks fit the hashing blocks' shared memory");
+    const size_t prep_smem = 4 * (SRC == SIGN_PLAIN ? EXPAND16_WORDS : HASH16_STAGE_WORDS + NTT_TABLE_WORDS);
+    static_assert(NTT_TABLE_WORDS + 288 <= EXPAND16_WORDS && 288 <= HASH16_STAGE_WORDS, "the secrets' blocks");
     if ((e = dynamic_smem(k_sign_prepare<LEVEL, SRC>, prep_smem)) != cudaSuccess) return e;
-    k_sign_prepare<LEVEL, SRC>
-        <<<b.hash_blocks + b.expand_blocks + secret_blocks, 32 * ROUND_WARPS, prep_smem, s>>>(b);
+    k_sign_prepare<LEVEL, SRC><<<b.hash_warps + b.expand_blocks + secret_blocks, 32, prep_smem, s>>>(b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
-    const size_t mask_smem = 4 * ROUND_WARPS * MASK_WORDS;
     const size_t front_smem = 2 * tables + 4 * ROUND_WARPS * front_warp_words<LEVEL>();
     const size_t back_smem = 2 * tables + 4 * ROUND_WARPS * 288;
-    if ((e = dynamic_smem(k_sign_mask<LEVEL>, mask_smem)) != cudaSuccess) return e;
     if ((e = dynamic_smem(k_sign_front<LEVEL, SRC>, front_smem)) != cudaSuccess) return e;
     const int rounds = rounds_of(LEVEL, b.n, b.slots);
     const int most = b.slots;   // attempts of a round; blocks beyond the actual count return at once
     const HashGrid h = hash_grid(most);
     for (int r = 0; r < rounds; ++r) {
-        k_sign_mask<LEVEL><<<blocks_for(most, ROUND_WARPS * (K16_STATES / V::L)), 32 * ROUND_WARPS, mask_smem, s>>>(b, r);
+        k_sign_mask<LEVEL><<<blocks_for(most, K16_STATES / V::L), 32, 0, s>>>(b, r);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         k_sign_front<LEVEL, SRC><<<blocks_for(most, ROUND_WARPS), 32 * ROUND_WARPS, front_smem, s>>>(b, r);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;

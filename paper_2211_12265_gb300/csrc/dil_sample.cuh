@@ -561,10 +561,12 @@ __device__ __forceinline__ void pack8(uint8_t *out, const uint32_t v[8]) {
     }
 }
 
-// Copies nbytes from global to shared memory, one byte per lane per step,
-// through L2 (coherent with copies into the source made while the kernel runs).
-__device__ __forceinline__ void stage_bytes(uint8_t *dst, const uint8_t *__restrict__ src, int nbytes, int lane) {
-    for (int i = lane; i < nbytes; i += 32) dst[i] = __ldcg(src + i);
+// Copies nbytes from global memory (any alignment) to 4-byte aligned shared
+// memory, a word per lane and step, through L2 (coherent with copies into the
+// source made while the kernel runs).  Up to 3 bytes beyond nbytes are zeroed.
+__device__ __forceinline__ void stage_bytes(uint8_t *dst, const uint8_t *src, int nbytes, int lane) {
+    for (int i = lane; 4 * i < nbytes; i += 32)
+        reinterpret_cast<uint32_t *>(dst)[i] = ld_bytes4<true>(src + 4 * i, nbytes - 4 * i);
 }
 
 }  // namespace dil

@@ -1,5 +1,5 @@
-// ExpandA over the polynomials of a batch, sixteen to a warp whatever tasks they
-// belong to, with the states in registers (dil_hash16.cuh).
+// ExpandA and ExpandS over the polynomials of a batch, sixteen to a warp
+// whatever tasks they belong to, with the states in registers (dil_hash16.cuh).
 #pragma once
 #include "dil_hash16.cuh"
 #include "dil_sample.cuh"
@@ -78,6 +78,88 @@ __device__ __forceinline__ void expand_a_batch(long long first, long long total,
         __syncwarp();
         expand_a_poly(seed, q / V::L, q % V::L, buf, sq, lane);
         for (int m = 0; m < 8; ++m) out_of(t)[q * N + 8 * lane + m] = buf[9 * lane + m];
+        __syncwarp();
+    }
+}
+
+// As expand_a_batch for ExpandS: polynomials [first, first + 16) of the `total` =
+// tasks (l + k), s1 then s2 of each task, coefficients in order.  seed_of(t):
+// the 64 bytes of rho' (4-byte aligned); out_of(t): l + k polynomials.  Two
+// blocks hold 544 candidates: always enough for eta = 2 (15 in 16 accepted),
+// and for eta = 4 (9 in 16) in all but one polynomial of 10^5.
+template <int LEVEL, class Seed, class Out>
+__device__ __forceinline__ void expand_s_batch(long long first, long long total, Seed seed_of, Out out_of,
+                                               uint32_t *st, int lane) {
+    using V = Lv<LEVEL>;
+    constexpr int KL = V::K + V::L;
+    if (first >= total) return;
+    const int s = lane >> 1, p = lane & 1;
+    const long long at = first + s < total ? first + s : total - 1;
+    const int task = (int)(at / KL), nonce = (int)(at - (long long)task * KL);
+    const uint32_t *rhop = reinterpret_cast<const uint32_t *>(seed_of(task));
+    uint32_t a[25];
+#pragma unroll
+    for (int i = 0; i < 25; ++i) a[i] = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) a[i] = rhop[2 * i + p];
+    if (!p) a[8] = (uint32_t)nonce | (0x1Fu << 16);
+    if (p) a[16] = 0x80000000u;
+#pragma unroll 1
+    for (int blk = 0; blk < 2; ++blk) {
+        hash16_permute(a, p);
+#pragma unroll
+        for (int i = 0; i < 17; ++i) st[s * EXPAND16_STRIDE + 34 * blk + 2 * i + p] = a[i];
+    }
+    __syncwarp();
+    uint32_t few = 0;
+#pragma unroll 1
+    for (int u = 0; u < K16_STATES && first + u < total; ++u) {
+        const int t = (int)((first + u) / KL);
+        int32_t *dst = out_of(t) + (int)(first + u - (long long)t * KL) * N;
+        int c = 0;
+        // a lane takes the four bytes of word lane + 32 m (68 words), in stream order
+        for (int m = 0; m < 3 && c < N; ++m) {
+            const int w = lane + 32 * m;
+            const uint32_t x = w < 68 ? st[u * EXPAND16_STRIDE + w] : 0xFFFFFFFFu;
+            uint32_t take = 0;
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                const uint32_t v = (x >> (4 * b)) & 15u;
+                take |= (uint32_t)(V::ETA == 2 ? v < 15u : v < 9u) << b;
+            }
+            // candidates taken by the lanes before this one
+            int before = __popc(take);
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int y = __shfl_up_sync(FULL, before, d);
+                if (lane >= d) before += y;
+            }
+            const int all = __shfl_sync(FULL, before, 31);
+            int to = c + before - __popc(take);
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                if (!((take >> b) & 1u)) continue;
+                const uint32_t v = (x >> (4 * b)) & 15u;
+                if (to < N) dst[to] = V::ETA == 2 ? 2 - (int32_t)(v % 5u) : 4 - (int32_t)v;
+                ++to;
+            }
+            c += all;
+        }
+        few |= (uint32_t)(c < N) << u;
+    }
+    if (!few) return;
+    __syncwarp();
+    uint8_t *seed = reinterpret_cast<uint8_t *>(st), *sq = seed + 64;
+    int32_t *buf = reinterpret_cast<int32_t *>(st) + 64;
+#pragma unroll 1
+    for (int u = 0; u < K16_STATES; ++u) {
+        if (!((few >> u) & 1u)) continue;
+        const int t = (int)((first + u) / KL), q = (int)(first + u - (long long)t * KL);
+        seed[lane] = seed_of(t)[lane];
+        seed[lane + 32] = seed_of(t)[lane + 32];
+        __syncwarp();
+        expand_s_poly<V::ETA>(seed, q, buf, sq, lane);
+        for (int m = 0; m < 8; ++m) out_of(t)[q * N + lane + 32 * m] = buf[lane + 36 * m];
         __syncwarp();
     }
 }

@@ -1,16 +1,19 @@
 // Verify of a batch (Alg 3).
 //
-// Batch form: two kernels.  The first gives its leading blocks to the hashes
-// tr = H(pk) and mu = H(tr || M), sixteen tasks to a warp, and the others to
-// the arithmetic, one task per group of P warps up to the packed w1'; the two
-// halves of a task never wait on each other.  The second recomputes
-// c~ = H(mu || w1'), sixteen tasks to a warp, and compares.  Hashing inside
+// Batch form.  The first kernel gives its leading blocks to the hashes
+// tr = H(pk) and mu = H(tr || M) and to SampleInBall(c~), sixteen tasks to a
+// warp, and the others to sampling A^, sixteen polynomials to a warp whatever tasks they belong to
+// (dil_sample16.cuh).  The second does the arithmetic, one task per group of P
+// warps up to the packed w1'; with a resident key's or the caller's A^ it is
+// the other blocks of the first.  The last recomputes c~ = H(mu || w1'),
+// sixteen tasks to a warp, and compares.  Hashing inside
 // the task's own warp (k_verify, kept for the launch shapes a caller asks for)
 // runs the 18 blocks of a Dilithium2 task at 18.7 SM clocks per round, 8.1 k
-// of the task's 20.7 k clocks; sixteen to a warp they take 1.4 k.  10,000 tasks:
-// Dilithium2 656 -> 491 us, Dilithium5 (32 B - 4 KB) 1815 -> 1564 us.
-#include "dil_hash16.cuh"
+// of the task's 20.7 k clocks; sixteen to a warp they take 1.4 k.  10,000 tasks,
+// fused -> batch: Dilithium2 655 -> 462 us, Dilithium5 (32 B - 4 KB)
+// 1813 -> 1351 us; 13 Dilithium3 tasks 162 -> 138 us.
 #include "dil_kern.cuh"
+#include "dil_sample16.cuh"
 
 namespace dil {
 
@@ -118,35 +121,94 @@ struct VerifyMuJob {
     }
 };
 
+// One hashing warp of the batch (w < hash_warps).
+template <int LEVEL, int SRC>
+__device__ __forceinline__ void verify_hashes(const VerifyBatch &b, int w, uint32_t *stage, int lane) {
+    VerifyMuJob<LEVEL, SRC> job(b, w * K16_STATES + (lane >> 1), lane);
+    hash16_run(job, stage, lane);
+}
+
+// The arithmetic of the tasks of CTA `blk`.
 template <int LEVEL, int P, int SRC>
-__global__ void __launch_bounds__(256, 4) k_verify_batch(int, const VerifyBatch b) {
-    extern __shared__ __align__(16) uint8_t smem[];
+__device__ __forceinline__ void verify_tasks(const VerifyBatch &b, int blk, uint8_t *smem) {
     using V = Lv<LEVEL>;
-    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if ((int)blockIdx.x < b.hash_blocks) {
-        const int w = blockIdx.x * warps + warp;
-        if (w >= b.hash_warps) return;
-        VerifyMuJob<LEVEL, SRC> job(b, w * K16_STATES + (lane >> 1), lane);
-        hash16_run(job, reinterpret_cast<uint32_t *>(smem) + warp * HASH16_STAGE_WORDS, lane);
-        return;
-    }
     const CtaView v = cta_setup<P>(smem);
-    const int task = (blockIdx.x - b.hash_blocks) * v.groups + v.group;
+    const int task = blk * v.groups + v.group;
     if (task >= b.n) return;
     int key;
     uint64_t m0;
     size_t mlen;
     int r = 0;
     if (verify_input<SRC>(b, task, key, m0, mlen)) {
+        int32_t *scr = b.scratch + (size_t)task * verify_polys<LEVEL, SRC>() * N;
         const int32_t *a = SRC == VERIFY_AHAT    ? b.ahat + (size_t)task * V::K * V::L * N
                            : SRC == VERIFY_KEYED ? b.keys + (size_t)key * Scratch<LEVEL>::KEY_POLYS * N
-                                                 : nullptr;
-        r = verify_task<LEVEL, P, SRC == VERIFY_KEYED, SRC == VERIFY_AHAT, true>(
-            b.pk + (size_t)key * V::PK, nullptr, 0, b.sig + (size_t)task * V::SIG,
-            b.scratch + (size_t)task * verify_polys<LEVEL, SRC>() * N, *v.gs, *v.ws, v.zt, v.izt, v.g, v.bar, v.lane,
-            a);
+                                                 : scr + V::L * N;
+        r = verify_task<LEVEL, P, SRC == VERIFY_KEYED, SRC != VERIFY_KEYED, true>(
+            b.pk + (size_t)key * V::PK, nullptr, 0, b.sig + (size_t)task * V::SIG, scr, *v.gs, *v.ws, v.zt, v.izt,
+            v.g, v.bar, v.lane, a, nullptr, nullptr,
+            b.challenge_blocks ? reinterpret_cast<const int8_t *>(b.challenge) + (size_t)task * 256 : nullptr);
     }
     if (v.g == 0 && v.lane == 0) b.ok[task] = (uint8_t)r;   // 1: c~ decides (k_verify_compare)
+}
+
+// VERIFY_AHAT, VERIFY_KEYED: hashes and arithmetic.
+template <int LEVEL, int P, int SRC>
+__global__ void __launch_bounds__(256, 4) k_verify_batch(const VerifyBatch b) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if ((int)blockIdx.x < b.hash_blocks) {
+        const int w = blockIdx.x * warps + warp;
+        if (w < b.hash_warps)
+            verify_hashes<LEVEL, SRC>(b, w, reinterpret_cast<uint32_t *>(smem) + warp * HASH16_STAGE_WORDS, lane);
+        return;
+    }
+    verify_tasks<LEVEL, P, SRC>(b, blockIdx.x - b.hash_blocks, smem);
+}
+
+// c = SampleInBall(c~) of the signatures of tasks [first, first + 16), one warp.
+template <int LEVEL>
+__device__ __forceinline__ void verify_challenges(const VerifyBatch &b, int first, uint32_t *stage, int lane) {
+    using V = Lv<LEVEL>;
+    if (first >= b.n) return;
+    const int t = first + (lane >> 1);
+    const uint8_t *ct = b.sig + (size_t)(t < b.n ? t : first) * V::SIG + 4 * (lane & 1);
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = ld_bytes4(ct + 8 * i, 4);
+    challenge16<V::TAU>(w, t < b.n, stage, lane);
+    for (int u = 0; u < K16_STATES && first + u < b.n; ++u)
+        put_challenge(b.challenge + (size_t)(first + u) * 256, stage, u, lane);
+}
+
+// VERIFY_PLAIN: blocks [0, hash_warps) hash tr and mu, [.., + challenge_blocks)
+// draw challenges, the others sample A^; the arithmetic follows.  One warp per
+// CTA, as in Sign's prepare kernel.
+template <int LEVEL>
+__global__ void __launch_bounds__(32, 16) k_verify_prepare(const VerifyBatch b) {
+    extern __shared__ __align__(16) uint32_t sm[];
+    using V = Lv<LEVEL>;
+    const int lane = threadIdx.x;
+    int blk = blockIdx.x;
+    if (blk < b.hash_warps) {
+        verify_hashes<LEVEL, VERIFY_PLAIN>(b, blk, sm, lane);
+        return;
+    }
+    blk -= b.hash_warps;
+    if (blk < b.challenge_blocks) {
+        verify_challenges<LEVEL>(b, blk * K16_STATES, sm, lane);
+        return;
+    }
+    blk -= b.challenge_blocks;
+    expand_a_batch<LEVEL>(
+        (long long)blk * K16_STATES, (long long)b.n * V::K * V::L, [&](int t) { return b.pk + (size_t)t * V::PK; },
+        [&](int t) { return b.scratch + ((size_t)t * verify_polys<LEVEL, VERIFY_PLAIN>() + V::L) * N; }, sm, lane);
+}
+
+template <int LEVEL, int P>
+__global__ void __launch_bounds__(256, 4) k_verify_rows(const VerifyBatch b) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    verify_tasks<LEVEL, P, VERIFY_PLAIN>(b, blockIdx.x, smem);
 }
 
 // c~ = H(mu || w1') of task `pair` against the signature's.
@@ -181,7 +243,7 @@ struct VerifyCompareJob {
 
 template <int LEVEL, int SRC>
 __global__ void __launch_bounds__(128) k_verify_compare(const VerifyBatch b) {
-    __shared__ uint32_t stage[4][HASH16_STAGE_WORDS];
+    __shared__ __align__(16) uint32_t stage[4][HASH16_STAGE_WORDS];
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (w * K16_STATES >= b.n) return;
     VerifyCompareJob<LEVEL, SRC> job(b, w * K16_STATES + (lane >> 1), lane);
@@ -193,17 +255,32 @@ namespace {
 template <int LEVEL, int P, int SRC>
 cudaError_t launch_batch(VerifyBatch b, int warps, cudaStream_t s) {
     b.hash_warps = batch_hash_warps(b.n);
-    b.hash_blocks = (b.hash_warps + warps - 1) / warps;
     cudaError_t e = cudaSuccess;
     if (b.n > b.hash_warps * K16_STATES) e = cudaMemsetAsync(b.next, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
-    const int groups = warps / P;
+    const int blocks = (b.n + warps / P - 1) / (warps / P);
     const size_t smem = cta_bytes(warps, P);
-    e = cudaFuncSetAttribute(k_verify_batch<LEVEL, P, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_verify_batch<LEVEL, P, SRC><<<b.hash_blocks + (b.n + groups - 1) / groups, warps * 32, smem, s>>>(b.n, b);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if constexpr (SRC == VERIFY_PLAIN) {
+        b.challenge_blocks = (b.n + K16_STATES - 1) / K16_STATES;
+        const long long polys = (long long)b.n * Lv<LEVEL>::K * Lv<LEVEL>::L;
+        const int expand_blocks = (int)((polys + K16_STATES - 1) / K16_STATES);
+        const int bytes = EXPAND16_WORDS * (int)sizeof(uint32_t);
+        static_assert(CHALLENGE_WORDS <= EXPAND16_WORDS, "the hashing blocks' shared memory");
+        e = cudaFuncSetAttribute(k_verify_prepare<LEVEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+        k_verify_prepare<LEVEL><<<b.hash_warps + b.challenge_blocks + expand_blocks, 32, bytes, s>>>(b);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(k_verify_rows<LEVEL, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        k_verify_rows<LEVEL, P><<<blocks, warps * 32, smem, s>>>(b);
+    } else {
+        b.hash_blocks = (b.hash_warps + warps - 1) / warps;
+        b.challenge_blocks = 0;
+        e = cudaFuncSetAttribute(k_verify_batch<LEVEL, P, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        k_verify_batch<LEVEL, P, SRC><<<b.hash_blocks + blocks, warps * 32, smem, s>>>(b);
+    }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const HashGrid h = hash_grid(b.n);
     k_verify_compare<LEVEL, SRC><<<h.blocks, h.threads, 0, s>>>(b);
     return cudaGetLastError();
