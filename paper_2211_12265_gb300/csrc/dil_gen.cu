@@ -2,8 +2,8 @@
 //
 // Batch form, four kernels: H(zeta), sixteen tasks to a warp; ExpandA and
 // ExpandS, sixteen polynomials to a warp whatever tasks they belong to
-// (dil_sample16.cuh); t = A s1 + s2 and the packed keys, one task per group of P
-// warps; tr = H(pk), sixteen tasks to a warp.  In the task's own warp
+// (dil_sample16.cuh); t = A s1 + s2 and the packed keys, one task per warp;
+// tr = H(pk), sixteen tasks to a warp.  In the task's own warp
 // (k_keygen, kept for the launch shapes a caller asks for) the eleven blocks of
 // a Dilithium2 key's hashes cost 4.9 k of the task's 19.4 k SM clocks (10,000
 // keys, fused -> batch: 616 -> 533 us).
@@ -43,8 +43,8 @@ __device__ __forceinline__ void put_words(uint8_t *dst, const uint32_t (&a)[25],
     }
 }
 
-// (rho, rho', K) = H(zeta) of task `pair`: rho to pk, sk and the first words of
-// its scratch's s^1 (which the arithmetic writes last), rho' behind it, K to sk.
+// (rho, rho', K) = H(zeta) of task `pair`: rho to pk, sk and the start of its
+// scratch, rho' behind it, K to sk.
 template <int LEVEL>
 struct KeygenSeedJob {
     const uint8_t *seed;
@@ -111,15 +111,49 @@ __global__ void __launch_bounds__(32, 16) k_keygen_expand(int n, int32_t *scratc
     }
 }
 
-template <int LEVEL, int P>
-__global__ void __launch_bounds__(256, 4) k_keygen_rows(int n, uint8_t *pk, uint8_t *sk, int32_t *scratch) {
-    extern __shared__ __align__(16) uint8_t smem[];
-    const CtaView v = cta_setup<P>(smem);
-    const int task = blockIdx.x * v.groups + v.group;
-    if (task >= n) return;
+// s1, s2, t1 and t0 of one task, one warp: gen_rows with s^1 in shared memory and
+// every load of a row of A^ in flight at once.
+template <int LEVEL>
+__global__ void __launch_bounds__(32, LEVEL == 2 ? 28 : 20) k_keygen_rows(uint8_t *pk, uint8_t *sk,
+                                                                       const int32_t *scratch) {
+    __shared__ __align__(16) int32_t buf[288], sh[Lv<LEVEL>::L * N];
     using V = Lv<LEVEL>;
-    gen_rows<LEVEL, P>(pk + (size_t)task * V::PK, sk + (size_t)task * V::SK, gen_scratch<LEVEL>(scratch, task),
-                       *v.ws, v.zt, v.izt, v.g, v.bar, v.lane);
+    const int task = blockIdx.x, lane = threadIdx.x;
+    pk += (size_t)task * V::PK;
+    sk += (size_t)task * V::SK;
+    const int32_t *ah = scratch + ((size_t)task * Scratch<LEVEL>::GEN_POLYS + V::L) * N;
+    const int32_t *sraw = scratch + ((size_t)task * Scratch<LEVEL>::GEN_POLYS + Scratch<LEVEL>::GEN_S) * N;
+    int32_t v[8], s[8];
+#pragma unroll 1
+    for (int j = 0; j < V::L; ++j) {
+        load_l2(s, sraw + j * N, lane);
+        load_l0(v, sraw + j * N, lane);
+        pack_poly<V::ETABITS>(sk + V::SK_S1 + j * V::POLYETA, s, V::ETA, -1, buf, lane);
+        ntt_fwd_global(v, buf);
+        store_l2(sh + j * N, v, lane);   // read back by the same lane
+    }
+#pragma unroll 1
+    for (int i = 0; i < V::K; ++i) {
+        int32_t a[V::L][8];
+#pragma unroll
+        for (int j = 0; j < V::L; ++j) load_l2(a[j], ah + (i * V::L + j) * N, lane);
+        load_l2(s, sraw + (V::L + i) * N, lane);
+        pack_poly<V::ETABITS>(sk + V::SK_S2 + i * V::POLYETA, s, V::ETA, -1, buf, lane);
+        long long acc[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) acc[m] = 0;
+#pragma unroll
+        for (int j = 0; j < V::L; ++j) {
+            load_l2(v, sh + j * N, lane);
+#pragma unroll
+            for (int m = 0; m < 8; ++m) acc[m] += (long long)a[j][m] * v[m];
+        }
+        load_l0(s, sraw + (V::L + i) * N, lane);
+#pragma unroll
+        for (int m = 0; m < 8; ++m) v[m] = mont_reduce(acc[m]);
+        ntt_inv_global(v, buf);
+        gen_split<LEVEL>(pk + 32 + i * V::POLYT1, sk + V::SK_T0 + i * V::POLYT0, v, s, buf, lane);
+    }
 }
 
 // tr = H(pk) of task `pair` into its secret key.
@@ -153,8 +187,7 @@ __global__ void __launch_bounds__(128) k_keygen_tr(int n, const uint8_t *pk, uin
 namespace {
 
 template <int LEVEL>
-cudaError_t launch_batch(int n, const uint8_t *seeds, uint8_t *pk, uint8_t *sk, int32_t *scratch, int warps, int p,
-                         cudaStream_t s) {
+cudaError_t launch_batch(int n, const uint8_t *seeds, uint8_t *pk, uint8_t *sk, int32_t *scratch, cudaStream_t s) {
     using V = Lv<LEVEL>;
     const HashGrid h = hash_grid(n);
     k_keygen_seeds<LEVEL><<<h.blocks, h.threads, 0, s>>>(n, seeds, pk, sk, scratch);
@@ -164,9 +197,8 @@ cudaError_t launch_batch(int n, const uint8_t *seeds, uint8_t *pk, uint8_t *sk, 
     const int s_blocks = blocks(V::K + V::L);
     k_keygen_expand<LEVEL><<<s_blocks + blocks(V::K * V::L), 32, 0, s>>>(n, scratch, s_blocks);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    e = p == 1 ? launch_plain(k_keygen_rows<LEVEL, 1>, n, warps, p, s, pk, sk, scratch)
-               : launch_plain(k_keygen_rows<LEVEL, 4>, n, warps, p, s, pk, sk, scratch);
-    if (e != cudaSuccess) return e;
+    k_keygen_rows<LEVEL><<<n, 32, 0, s>>>(pk, sk, scratch);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_keygen_tr<LEVEL><<<h.blocks, h.threads, 0, s>>>(n, pk, sk);
     return cudaGetLastError();
 }
@@ -174,13 +206,12 @@ cudaError_t launch_batch(int n, const uint8_t *seeds, uint8_t *pk, uint8_t *sk, 
 }  // namespace
 
 cudaError_t launch_keygen_batch(int level, int n, const uint8_t *seeds, uint8_t *pk, uint8_t *sk, int32_t *scratch,
-                                int warps, int p, cudaStream_t s) {
+                                cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    if (p != 1 && p != 4) return cudaErrorInvalidValue;
     switch (level) {
-        case 2: return launch_batch<2>(n, seeds, pk, sk, scratch, warps, p, s);
-        case 3: return launch_batch<3>(n, seeds, pk, sk, scratch, warps, p, s);
-        case 5: return launch_batch<5>(n, seeds, pk, sk, scratch, warps, p, s);
+        case 2: return launch_batch<2>(n, seeds, pk, sk, scratch, s);
+        case 3: return launch_batch<3>(n, seeds, pk, sk, scratch, s);
+        case 5: return launch_batch<5>(n, seeds, pk, sk, scratch, s);
     }
     return cudaErrorInvalidValue;
 }

@@ -36,9 +36,10 @@ cudaError_t launch_verify(int level, int n, const uint8_t *pk, const uint8_t *ms
                           const uint8_t *sig, uint8_t *ok, int32_t *scratch, int warps, int p, cudaStream_t s);
 
 // Batch forms: the hashes of independent tasks run sixteen to a warp (dil_gen.cu,
-// dil_verify.cu); p: warps per task of the arithmetic (1 or 4; divides warps).
+// dil_verify.cu).  warps and p (1 or 4) shape the arithmetic of VERIFY_AHAT and
+// VERIFY_KEYED; otherwise it runs on single warps.
 cudaError_t launch_keygen_batch(int level, int n, const uint8_t *seeds, uint8_t *pk, uint8_t *sk, int32_t *scratch,
-                                int warps, int p, cudaStream_t s);
+                                cudaStream_t s);
 // Where a Verify's A^ comes from: sampled, the caller's, or a resident key's.
 enum VerifySource { VERIFY_PLAIN = 0, VERIFY_AHAT = 1, VERIFY_KEYED = 2 };
 struct VerifyBatch {
@@ -85,7 +86,7 @@ struct SignBatch {
     int *pending, *best, *done, *next, *count;
     int hash_warps, expand_blocks;
 };
-int sign_batch_slots(int level, int n);       // slots worth having
+int sign_batch_slots(int level, int n, int parts);   // slots worth having beside parts - 1 other batches
 int sign_batch_min_slots(int level, int n);   // slots needed
 size_t sign_batch_bytes(int level, int src, size_t n, size_t slots);   // workspace
 cudaError_t launch_sign_batch(int level, int src, const SignBatch &b, void *ws, cudaStream_t s);

@@ -132,6 +132,30 @@ __device__ __forceinline__ int4 ldz128(uint32_t a) {
     return v;
 }
 
+// Twiddles z and zs [i, i + 1 / 2 / 4) of one direction, from a CTA's shared
+// table or (kernels whose CTAs are too short-lived to fill one) from the global
+// one through L1.
+struct SharedTwiddles {
+    uint32_t at;   // shared-memory address
+    __device__ __forceinline__ int32_t z32(int i) const { return ldz32(at + 4 * i); }
+    __device__ __forceinline__ int32_t zs32(int i) const { return ldz32(at + 1024 + 4 * i); }
+    __device__ __forceinline__ int2 z64(int i) const { return ldz64(at + 4 * i); }
+    __device__ __forceinline__ int2 zs64(int i) const { return ldz64(at + 1024 + 4 * i); }
+    __device__ __forceinline__ int4 z128(int i) const { return ldz128(at + 4 * i); }
+    __device__ __forceinline__ int4 zs128(int i) const { return ldz128(at + 1024 + 4 * i); }
+};
+template <bool INV>
+struct GlobalTwiddles {
+    __device__ __forceinline__ const int32_t *z(int i) const { return (INV ? g_zetas.iz : g_zetas.z) + i; }
+    __device__ __forceinline__ const int32_t *zs(int i) const { return (INV ? g_zetas.izs : g_zetas.zs) + i; }
+    __device__ __forceinline__ int32_t z32(int i) const { return __ldg(z(i)); }
+    __device__ __forceinline__ int32_t zs32(int i) const { return __ldg(zs(i)); }
+    __device__ __forceinline__ int2 z64(int i) const { return __ldg(reinterpret_cast<const int2 *>(z(i))); }
+    __device__ __forceinline__ int2 zs64(int i) const { return __ldg(reinterpret_cast<const int2 *>(zs(i))); }
+    __device__ __forceinline__ int4 z128(int i) const { return __ldg(reinterpret_cast<const int4 *>(z(i))); }
+    __device__ __forceinline__ int4 zs128(int i) const { return __ldg(reinterpret_cast<const int4 *>(zs(i))); }
+};
+
 // Eight coefficients of one lane, passed by value to the out-of-line transforms.
 struct Poly8 {
     int32_t v[8];
@@ -140,11 +164,9 @@ struct Poly8 {
 // Forward NTT.  In: L0, |r| < q.  Out: L2, |r| < 9.1q, unscaled (a level adds
 // at most 1.01q).  buf: the warp's exchange buffer (288 words), zt: the
 // forward twiddles (shared).
-// Out of line: one copy of the code serves every call site, which keeps the
-// fused kernels' instruction footprint small.
-static __device__ __noinline__ Poly8 ntt_fwd_impl(Poly8 p, uint32_t buf, uint32_t zt) {
+template <class Table>
+__device__ __forceinline__ void ntt_fwd_body(int32_t (&r)[8], uint32_t buf, Table zt) {
     const int lane = threadIdx.x & 31;
-    int32_t *r = p.v;
     // level 1 (len 128): pairs (m, m+4)
     {
         const int32_t z = c_zetas.z[1], zs = c_zetas.zs[1];
@@ -172,13 +194,13 @@ static __device__ __noinline__ Poly8 ntt_fwd_impl(Poly8 p, uint32_t buf, uint32_
     __syncwarp();
     // level 4 (len 16): pairs (m, m+4), twiddle 8 + b
     {
-        const int32_t z = ldz32(zt + 4 * (8 + b)), zs = ldz32(zt + 1024 + 4 * (8 + b));
+        const int32_t z = zt.z32(8 + b), zs = zt.zs32(8 + b);
 #pragma unroll
         for (int m = 0; m < 4; ++m) ct_bfly(r[m], r[m + 4], z, zs);
     }
     // level 5 (len 8): pairs (m, m+2), twiddles 16 + 2b + {0, 1}
     {
-        const int2 z = ldz64(zt + 4 * (16 + 2 * b)), zs = ldz64(zt + 1024 + 4 * (16 + 2 * b));
+        const int2 z = zt.z64(16 + 2 * b), zs = zt.zs64(16 + 2 * b);
         ct_bfly(r[0], r[2], z.x, zs.x);
         ct_bfly(r[1], r[3], z.x, zs.x);
         ct_bfly(r[4], r[6], z.y, zs.y);
@@ -186,7 +208,7 @@ static __device__ __noinline__ Poly8 ntt_fwd_impl(Poly8 p, uint32_t buf, uint32_
     }
     // level 6 (len 4): pairs (m, m+1), twiddles 32 + 4b + {0..3}
     {
-        const int4 z = ldz128(zt + 4 * (32 + 4 * b)), zs = ldz128(zt + 1024 + 4 * (32 + 4 * b));
+        const int4 z = zt.z128(32 + 4 * b), zs = zt.zs128(32 + 4 * b);
         ct_bfly(r[0], r[1], z.x, zs.x);
         ct_bfly(r[2], r[3], z.y, zs.y);
         ct_bfly(r[4], r[5], z.z, zs.z);
@@ -202,7 +224,7 @@ static __device__ __noinline__ Poly8 ntt_fwd_impl(Poly8 p, uint32_t buf, uint32_
     // level 7 (len 2): pairs (m, m+2), twiddles 64 + 2t + {0, 1} (one 8-byte
     // load per lane: a half-warp reads 128 contiguous bytes, conflict-free)
     {
-        const int2 z = ldz64(zt + 4 * (64 + 2 * lane)), zs = ldz64(zt + 1024 + 4 * (64 + 2 * lane));
+        const int2 z = zt.z64(64 + 2 * lane), zs = zt.zs64(64 + 2 * lane);
         ct_bfly(r[0], r[2], z.x, zs.x);
         ct_bfly(r[1], r[3], z.x, zs.x);
         ct_bfly(r[4], r[6], z.y, zs.y);
@@ -210,13 +232,12 @@ static __device__ __noinline__ Poly8 ntt_fwd_impl(Poly8 p, uint32_t buf, uint32_
     }
     // level 8 (len 1): pairs (m, m+1), twiddles 128 + 4t + {0..3} (16-byte load)
     {
-        const int4 z = ldz128(zt + 4 * (128 + 4 * lane)), zs = ldz128(zt + 1024 + 4 * (128 + 4 * lane));
+        const int4 z = zt.z128(128 + 4 * lane), zs = zt.zs128(128 + 4 * lane);
         ct_bfly(r[0], r[1], z.x, zs.x);
         ct_bfly(r[2], r[3], z.y, zs.y);
         ct_bfly(r[4], r[5], z.z, zs.z);
         ct_bfly(r[6], r[7], z.w, zs.w);
     }
-    return p;
 }
 
 // Inverse NTT.  In: L2, |r| < q.  Out: L0, |r| < q, equal to INTT(in) * 2^32,
@@ -225,12 +246,12 @@ static __device__ __noinline__ Poly8 ntt_fwd_impl(Poly8 p, uint32_t buf, uint32_
 // lies in [-q/4, 5q/4), so it never exceeds the sums of its level.  The last
 // level keeps the Montgomery product, whose result is below q.
 // izt: the inverse twiddles in shared memory.
-static __device__ __noinline__ Poly8 ntt_inv_impl(Poly8 p, uint32_t buf, uint32_t izt) {
+template <class Table>
+__device__ __forceinline__ void ntt_inv_body(int32_t (&r)[8], uint32_t buf, Table izt) {
     const int lane = threadIdx.x & 31;
-    int32_t *r = p.v;
     // len 1: pairs (m, m+1), twiddles 128 + 4t + {0..3}
     {
-        const int4 z = ldz128(izt + 4 * (128 + 4 * lane)), zs = ldz128(izt + 1024 + 4 * (128 + 4 * lane));
+        const int4 z = izt.z128(128 + 4 * lane), zs = izt.zs128(128 + 4 * lane);
         gs_bfly(r[0], r[1], z.x, zs.x);
         gs_bfly(r[2], r[3], z.y, zs.y);
         gs_bfly(r[4], r[5], z.z, zs.z);
@@ -238,7 +259,7 @@ static __device__ __noinline__ Poly8 ntt_inv_impl(Poly8 p, uint32_t buf, uint32_
     }
     // len 2: pairs (m, m+2), twiddles 64 + 2t + {0, 1}
     {
-        const int2 z = ldz64(izt + 4 * (64 + 2 * lane)), zs = ldz64(izt + 1024 + 4 * (64 + 2 * lane));
+        const int2 z = izt.z64(64 + 2 * lane), zs = izt.zs64(64 + 2 * lane);
         gs_bfly(r[0], r[2], z.x, zs.x);
         gs_bfly(r[1], r[3], z.x, zs.x);
         gs_bfly(r[4], r[6], z.y, zs.y);
@@ -255,7 +276,7 @@ static __device__ __noinline__ Poly8 ntt_inv_impl(Poly8 p, uint32_t buf, uint32_
     __syncwarp();
     // len 4: pairs (m, m+1), twiddles 32 + 4b + {0..3}
     {
-        const int4 z = ldz128(izt + 4 * (32 + 4 * b)), zs = ldz128(izt + 1024 + 4 * (32 + 4 * b));
+        const int4 z = izt.z128(32 + 4 * b), zs = izt.zs128(32 + 4 * b);
         gs_bfly(r[0], r[1], z.x, zs.x);
         gs_bfly(r[2], r[3], z.y, zs.y);
         gs_bfly(r[4], r[5], z.z, zs.z);
@@ -263,7 +284,7 @@ static __device__ __noinline__ Poly8 ntt_inv_impl(Poly8 p, uint32_t buf, uint32_
     }
     // len 8: pairs (m, m+2), twiddles 16 + 2b + {0, 1}
     {
-        const int2 z = ldz64(izt + 4 * (16 + 2 * b)), zs = ldz64(izt + 1024 + 4 * (16 + 2 * b));
+        const int2 z = izt.z64(16 + 2 * b), zs = izt.zs64(16 + 2 * b);
         gs_bfly(r[0], r[2], z.x, zs.x);
         gs_bfly(r[1], r[3], z.x, zs.x);
         gs_bfly(r[4], r[6], z.y, zs.y);
@@ -271,7 +292,7 @@ static __device__ __noinline__ Poly8 ntt_inv_impl(Poly8 p, uint32_t buf, uint32_
     }
     // len 16: pairs (m, m+4), twiddle 8 + b
     {
-        const int32_t z = ldz32(izt + 4 * (8 + b)), zs = ldz32(izt + 1024 + 4 * (8 + b));
+        const int32_t z = izt.z32(8 + b), zs = izt.zs32(8 + b);
 #pragma unroll
         for (int m = 0; m < 4; ++m) gs_bfly(r[m], r[m + 4], z, zs);
     }
@@ -299,6 +320,24 @@ static __device__ __noinline__ Poly8 ntt_inv_impl(Poly8 p, uint32_t buf, uint32_
         r[m] = mont_mul(NTT_F, a + c);
         r[m + 4] = mont_mul(NTT_G, a - c);
     }
+}
+
+// Out of line: one copy of the code serves every call site, which keeps the
+// fused kernels' instruction footprint small.
+static __device__ __noinline__ Poly8 ntt_fwd_impl(Poly8 p, uint32_t buf, uint32_t zt) {
+    ntt_fwd_body(p.v, buf, SharedTwiddles{zt});
+    return p;
+}
+static __device__ __noinline__ Poly8 ntt_inv_impl(Poly8 p, uint32_t buf, uint32_t izt) {
+    ntt_inv_body(p.v, buf, SharedTwiddles{izt});
+    return p;
+}
+static __device__ __noinline__ Poly8 ntt_fwd_global_impl(Poly8 p, uint32_t buf) {
+    ntt_fwd_body(p.v, buf, GlobalTwiddles<false>{});
+    return p;
+}
+static __device__ __noinline__ Poly8 ntt_inv_global_impl(Poly8 p, uint32_t buf) {
+    ntt_inv_body(p.v, buf, GlobalTwiddles<true>{});
     return p;
 }
 
@@ -318,6 +357,24 @@ __device__ __forceinline__ void ntt_inv(int32_t r[8], int32_t *buf, const int32_
 #pragma unroll
     for (int m = 0; m < 8; ++m) p.v[m] = r[m];
     p = ntt_inv_impl(p, smem_addr(buf), smem_addr(izt));
+#pragma unroll
+    for (int m = 0; m < 8; ++m) r[m] = p.v[m];
+}
+
+// The same with the twiddles of the global table.
+__device__ __forceinline__ void ntt_fwd_global(int32_t r[8], int32_t *buf) {
+    Poly8 p;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) p.v[m] = r[m];
+    p = ntt_fwd_global_impl(p, smem_addr(buf));
+#pragma unroll
+    for (int m = 0; m < 8; ++m) r[m] = p.v[m];
+}
+__device__ __forceinline__ void ntt_inv_global(int32_t r[8], int32_t *buf) {
+    Poly8 p;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) p.v[m] = r[m];
+    p = ntt_inv_global_impl(p, smem_addr(buf));
 #pragma unroll
     for (int m = 0; m < 8; ++m) r[m] = p.v[m];
 }

@@ -133,6 +133,40 @@ __device__ __forceinline__ void unpack_poly_l0(int32_t v[8], const uint8_t *__re
     __syncwarp();
 }
 
+// As unpack_poly_l0, with the exchange buffer (288 words) as staging.
+template <int BITS>
+__device__ __forceinline__ void unpack_buf_l0(int32_t v[8], const uint8_t *src, int32_t off, int32_t *buf, int lane) {
+    uint8_t *sq = reinterpret_cast<uint8_t *>(buf);
+    stage_bytes(sq, src, N * BITS / 8, lane);
+    __syncwarp();
+#pragma unroll
+    for (int m = 0; m < 8; ++m) v[m] = off - (int32_t)get_field(sq, BITS * (lane + 32 * m), BITS);
+    __syncwarp();
+}
+
+// Packs 8 consecutive w1 values of this lane at dst (4-byte aligned).
+template <int LEVEL>
+__device__ __forceinline__ void pack_w1(uint8_t *dst, const int32_t v[8], int lane) {
+    using V = Lv<LEVEL>;
+    if constexpr (V::W1BITS == 4) {
+        uint32_t x = 0;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) x |= (uint32_t)v[m] << (4 * m);
+        reinterpret_cast<uint32_t *>(dst)[lane] = x;
+    } else {
+        uint32_t lo = 0, hi = 0;   // 24 bits each
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            lo |= (uint32_t)v[m] << (6 * m);
+            hi |= (uint32_t)v[m + 4] << (6 * m);
+        }
+        uint16_t *d = reinterpret_cast<uint16_t *>(dst) + 3 * lane;
+        d[0] = (uint16_t)lo;
+        d[1] = (uint16_t)((lo >> 16) | (hi << 8));
+        d[2] = (uint16_t)(hi >> 8);
+    }
+}
+
 // Writes 8 consecutive coefficients (lane t: 8t..8t+7) as `off + sign v` in BITS bits.
 template <int BITS>
 __device__ __forceinline__ void pack_seq(uint8_t *dst_poly, const int32_t v[8], int32_t off, int sign, int lane) {
@@ -342,6 +376,24 @@ __device__ __forceinline__ void challenge_hat(int32_t ch[8], const uint8_t *ctil
 // Alg 1: Gen.  pk, sk: outputs.  scratch: GEN_POLYS polys.
 // -------------------------------------------------------------------------
 
+// (t1, t0) = Power2Round(INTT(A^ s^1) + s2) of one row, packed (both in L0).
+template <int LEVEL>
+__device__ __forceinline__ void gen_split(uint8_t *t1_out, uint8_t *t0_out, const int32_t as1[8], const int32_t s2[8],
+                                          int32_t *buf, int lane) {
+    int32_t t1[8], t0[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        int32_t t = to_canonical(as1[m]) + s2[m];      // (-eta, q + eta)
+        t += (t < 0) ? Q : 0;
+        t -= (t >= Q) ? Q : 0;
+        power2round(t, t1[m], t0[m]);
+    }
+    l0_to_seq(t1, buf, lane);
+    pack_poly<10>(t1_out, t1, 0, 1, buf, lane);
+    l0_to_seq(t0, buf, lane);
+    pack_poly<D>(t0_out, t0, 1 << (D - 1), -1, buf, lane);
+}
+
 // From A^ and s1 || s2 in scratch: s1 and s2 packed into sk, t = A s1 + s2, and
 // t1, t0 packed into pk and sk.
 template <int LEVEL, int P>
@@ -354,7 +406,7 @@ __device__ void gen_rows(uint8_t *pk, uint8_t *sk, int32_t *scratch, WarpSmem &w
 #pragma unroll 1
     for (int j = g; j < V::L; j += P) {
         load_l2(a, sraw + j * N, lane);
-        pack_seq<V::ETABITS>(sk + V::SK_S1 + j * V::POLYETA, a, V::ETA, -1, lane);
+        pack_poly<V::ETABITS>(sk + V::SK_S1 + j * V::POLYETA, a, V::ETA, -1, ws.buf, lane);
         load_l0(r, sraw + j * N, lane);
         ntt_fwd(r, ws.buf, zt, lane);
         store_l2(scratch + j * N, r, lane);
@@ -367,19 +419,8 @@ __device__ void gen_rows(uint8_t *pk, uint8_t *sk, int32_t *scratch, WarpSmem &w
         ntt_inv(acc, ws.buf, izt, lane);
         load_l2(a, sraw + (V::L + i) * N, lane);
         load_l0(r, sraw + (V::L + i) * N, lane);
-        pack_seq<V::ETABITS>(sk + V::SK_S2 + i * V::POLYETA, a, V::ETA, -1, lane);
-        int32_t t1[8], t0[8];
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            int32_t t = to_canonical(acc[m]) + r[m];      // (-eta, q + eta)
-            t += (t < 0) ? Q : 0;
-            t -= (t >= Q) ? Q : 0;
-            power2round(t, t1[m], t0[m]);
-        }
-        l0_to_seq(t1, ws.buf, lane);
-        pack_seq<10>(pk + 32 + i * V::POLYT1, t1, 0, 1, lane);
-        l0_to_seq(t0, ws.buf, lane);
-        pack_seq<D>(sk + V::SK_T0 + i * V::POLYT0, t0, 1 << (D - 1), -1, lane);
+        pack_poly<V::ETABITS>(sk + V::SK_S2 + i * V::POLYETA, a, V::ETA, -1, ws.buf, lane);
+        gen_split<LEVEL>(pk + 32 + i * V::POLYT1, sk + V::SK_T0 + i * V::POLYT0, acc, r, ws.buf, lane);
     }
 }
 
@@ -782,14 +823,13 @@ __device__ void sign_zero(uint8_t *sig, int g, int lane) {
 // beforehand.
 // SPLIT: the task's hashes run elsewhere (dil_verify.cu): nothing of msg or tr
 // is read, the packed w1' goes to the start of scratch instead of into
-// c~ = H(mu || w1'), and 1 means that only that comparison is left.  c_in
-// (nullable): SampleInBall(c~), 256 signed bytes.
+// c~ = H(mu || w1'), and 1 means that only that comparison is left.
 template <int LEVEL, int P, bool KEYED = false, bool AHAT = false, bool SPLIT = false>
 __device__ int verify_task(const uint8_t *__restrict__ pk, const uint8_t *__restrict__ msg, size_t mlen,
                            const uint8_t *__restrict__ sig, int32_t *scratch, GroupSmem &gs, WarpSmem &ws,
                            const int32_t *zt, const int32_t *izt, int g, int bar, int lane,
                            const int32_t *key = nullptr, const uint8_t *tr = nullptr,
-                           const uint8_t *mu_in = nullptr, const int8_t *c_in = nullptr) {
+                           const uint8_t *mu_in = nullptr) {
     using V = Lv<LEVEL>;
     volatile int *vflag = &gs.flag;
     int32_t r[8], acc[8], ch[8];
@@ -866,13 +906,7 @@ __device__ int verify_task(const uint8_t *__restrict__ pk, const uint8_t *__rest
     group_sync<P>(bar);
     if (*vflag) return 0;
     // c^ = NTT(SampleInBall(c~))
-    if (SPLIT && c_in) {
-#pragma unroll
-        for (int m = 0; m < 8; ++m) ch[m] = c_in[lane + 32 * m];
-        ntt_fwd(ch, ws.buf, zt, lane);
-    } else {
-        challenge_hat<LEVEL>(ch, gs.ctilde, ws, zt, lane);
-    }
+    challenge_hat<LEVEL>(ch, gs.ctilde, ws, zt, lane);
     // v = INTT(A^ o z^ - c^ o NTT(t1 2^d)); w1' = UseHint(h, v)
     using S = Scratch<LEVEL>;
     const int32_t *ahat = KEYED ? key + S::AH * N : AHAT ? key : scratch + V::L * N;

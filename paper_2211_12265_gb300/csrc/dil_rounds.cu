@@ -42,7 +42,13 @@ template <int LEVEL> struct Slot {
 };
 
 constexpr int ROUND_MAX_REPS = 32;     // repetitions of one task in one round
-constexpr int ROUND_FILL = 152 * 32;   // attempts that fill the GPU with a warp each
+// Attempts of a round that are worth having in flight, speculative ones included:
+// a round of fewer takes almost as long (its hashes alone are a chain of eight
+// permutations), more are only wasted repetitions.  10,000 Dilithium2 tasks with
+// 10, 15, 20, 30 k slots: 1770, 1662, 1579, 1812 us; 150 Dilithium5 tasks with
+// 1.2, 2.4, 3.6, 4.8 k: 422, 460, 409, 430 us; 1,000 of them: 954, 687, 725, 776.
+template <int LEVEL> constexpr int round_fill() { return 152 * (LEVEL == 2 ? 32 : LEVEL == 3 ? 28 : 24); }
+constexpr int ROUND_MOST = 152 * 128;
 
 __host__ __device__ __forceinline__ int round_reps(int pending, int slots) {
     if (pending <= 0) return 0;
@@ -145,36 +151,24 @@ struct SignMuJob {
     }
 };
 
-// As unpack_poly_l0, with buf (a warp's exchange buffer) as staging.
-template <int BITS>
-__device__ __forceinline__ void unpack_words_l0(int32_t v[8], const uint8_t *src, int32_t off, int32_t *buf, int lane) {
-    uint8_t *sq = reinterpret_cast<uint8_t *>(buf);
-    stage_bytes(sq, src, N * BITS / 8, lane);
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < 8; ++m) v[m] = off - (int32_t)get_field(sq, BITS * (lane + 32 * m), BITS);
-    __syncwarp();
-}
-
 // s^1, s^2, t^0 of one task (one warp).
 template <int LEVEL>
-__device__ __forceinline__ void sign_secrets(const uint8_t *sk, int32_t *pre, int32_t *buf, const int32_t *zt,
-                                             int lane) {
+__device__ __forceinline__ void sign_secrets(const uint8_t *sk, int32_t *pre, int32_t *buf, int lane) {
     using V = Lv<LEVEL>;
     using S = Scratch<LEVEL>;
     int32_t r[8];
 #pragma unroll 1
     for (int u = 0; u < V::L + 2 * V::K; ++u) {
         if (u < V::L + V::K)
-            unpack_words_l0<V::ETABITS>(r, sk + V::SK_S1 + u * V::POLYETA, V::ETA, buf, lane);   // s1, then s2
+            unpack_buf_l0<V::ETABITS>(r, sk + V::SK_S1 + u * V::POLYETA, V::ETA, buf, lane);   // s1, then s2
         else
-            unpack_words_l0<D>(r, sk + V::SK_T0 + (u - V::L - V::K) * V::POLYT0, 1 << (D - 1), buf, lane);
-        ntt_fwd(r, buf, zt, lane);
+            unpack_buf_l0<D>(r, sk + V::SK_T0 + (u - V::L - V::K) * V::POLYT0, 1 << (D - 1), buf, lane);
+        ntt_fwd_global(r, buf);
         store_l2(pre + (S::S1H + u) * N, r, lane);
     }
 }
 
-constexpr int ROUND_WARPS = 4;   // warps per CTA of the kernels with a warp per attempt
+constexpr int ROUND_WARPS = 4;   // warps per CTA of the hashing and checking kernels
 
 // One warp per CTA: a sampling warp's 11 to 13 KB of shared memory let sixteen
 // be resident on an SM, and single warps spread over the SMs to within one (in
@@ -203,12 +197,9 @@ __global__ void __launch_bounds__(32, 16) k_sign_prepare(const SignBatch b) {
             return;
         }
         const int t = blk - b.expand_blocks;
-        int32_t *zt = reinterpret_cast<int32_t *>(sm), *buf = zt + NTT_TABLE_WORDS;
-        load_zetas<1>(zt);
-        __syncwarp();
         int32_t *pre = b.pre + (size_t)t * Scratch<LEVEL>::PRE_POLYS * N;
         if (SRC == SIGN_AHAT) copy_polys(b.ahat + (size_t)t * KL * N, 0, KL, pre, lane);
-        sign_secrets<LEVEL>(b.sk + (size_t)t * V::SK, pre, buf, zt, lane);
+        sign_secrets<LEVEL>(b.sk + (size_t)t * V::SK, pre, reinterpret_cast<int32_t *>(sm), lane);
     }
 }
 
@@ -263,60 +254,26 @@ __global__ void __launch_bounds__(32, 16) k_sign_mask(const SignBatch b, int r) 
 }
 
 // ---------------------------------------------------------------- front
-// Packs 8 consecutive w1 values of this lane at dst (2-byte aligned).
-template <int LEVEL>
-__device__ __forceinline__ void pack_w1(uint8_t *dst, const int32_t v[8], int lane) {
-    using V = Lv<LEVEL>;
-    if constexpr (V::W1BITS == 4) {
-        uint32_t x = 0;
-#pragma unroll
-        for (int m = 0; m < 8; ++m) x |= (uint32_t)v[m] << (4 * m);
-        reinterpret_cast<uint32_t *>(dst)[lane] = x;
-    } else {
-        uint32_t lo = 0, hi = 0;   // 24 bits each
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            lo |= (uint32_t)v[m] << (6 * m);
-            hi |= (uint32_t)v[m + 4] << (6 * m);
-        }
-        uint16_t *d = reinterpret_cast<uint16_t *>(dst) + 3 * lane;
-        d[0] = (uint16_t)lo;
-        d[1] = (uint16_t)((lo >> 16) | (hi << 8));
-        d[2] = (uint16_t)(hi >> 8);
-    }
-}
-
-// Shared words of a front warp: the exchange buffer and y^ (l polynomials).
-template <int LEVEL>
-constexpr int front_warp_words() { return 288 + Lv<LEVEL>::L * N; }
-
 template <int LEVEL, int SRC>
-__global__ void __launch_bounds__(32 * ROUND_WARPS, LEVEL == 2 ? 7 : 5) k_sign_front(const SignBatch b, int r) {
-    extern __shared__ __align__(16) uint32_t sm[];
+__global__ void __launch_bounds__(32, LEVEL == 2 ? 28 : 20) k_sign_front(const SignBatch b, int r) {
+    __shared__ __align__(16) int32_t buf[288], yh[Lv<LEVEL>::L * N];
     using V = Lv<LEVEL>;
     using S = Scratch<LEVEL>;
     const Round q = round_of(b, r);
-    const int attempts = q.p * q.m;
-    if ((int)blockIdx.x * ROUND_WARPS >= attempts) return;
-    int32_t *zt = reinterpret_cast<int32_t *>(sm), *izt = zt + NTT_TABLE_WORDS;
-    load_zetas(zt);
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int s = blockIdx.x * ROUND_WARPS + warp;
+    const int attempts = q.p * q.m, s = blockIdx.x, lane = threadIdx.x;
     if (s >= attempts) return;
-    int32_t *buf = izt + NTT_TABLE_WORDS + warp * front_warp_words<LEVEL>(), *yh = buf + 288;
     const int32_t *pre = pre_of<LEVEL, SRC>(b, pending_list(b, r)[s / q.m]);
     int32_t *slot = slot_of<LEVEL>(b, s);
     int32_t v[8];
 #pragma unroll 1
     for (int j = 0; j < V::L; ++j) {
         load_l0(v, slot + (Slot<LEVEL>::Y + j) * N, lane);
-        ntt_fwd(v, buf, zt, lane);
+        ntt_fwd_global(v, buf);
         store_l2(yh + j * N, v, lane);   // read back by the same lane
     }
 #pragma unroll 1
     for (int i = 0; i < V::K; ++i) {
-        // the l products of a row are summed in 64 bits (|sum| < 7 q 9q < 2^31 q) and reduced once
+        // the l products of a row are summed in 64 bits (|sum| < 7 q 9.1q < 2^31 q) and reduced once
         long long acc[8];
 #pragma unroll
         for (int m = 0; m < 8; ++m) acc[m] = 0;
@@ -333,7 +290,7 @@ __global__ void __launch_bounds__(32 * ROUND_WARPS, LEVEL == 2 ? 7 : 5) k_sign_f
         }
 #pragma unroll
         for (int m = 0; m < 8; ++m) v[m] = mont_reduce(acc[m]);
-        ntt_inv(v, buf, izt, lane);
+        ntt_inv_global(v, buf);
         int32_t h[8];
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
@@ -396,84 +353,75 @@ __global__ void __launch_bounds__(32 * ROUND_WARPS, 4) k_sign_hash(const SignBat
 // ---------------------------------------------------------------- back
 // The checks of the attempt in `slot` with challenge ch (L2 layout); z
 // replaces y, the hint masks go behind the challenge.  True when accepted.
+// One loop over the r0 polynomials (LowBits(w - c s2)), then z = y + c s1, then
+// the hints (c t0), so that the transform exists once: r0 first, since its
+// polynomials reject more often (Dilithium3: 0.17 against 0.09 each; 5.3
+// transforms an attempt instead of 6.6).
 template <int LEVEL>
-__device__ __forceinline__ bool sign_checks(const int32_t *pre, int32_t *slot, const int32_t ch[8], int32_t *buf,
+__device__ __forceinline__ bool sign_checks(const int32_t *pre, int32_t *slot, const int32_t (&ch)[8], int32_t *buf,
                                             const int32_t *izt, int lane) {
     using V = Lv<LEVEL>;
     using S = Scratch<LEVEL>;
     using SL = Slot<LEVEL>;
-    int32_t v[8], a[8];
-    // z = y + INTT(c^ o s^1); reject if ||z|| >= gamma1 - beta
-#pragma unroll 1
-    for (int j = 0; j < V::L; ++j) {
-        int32_t *y = slot + (SL::Y + j) * N;
-        load_l2(a, pre + (S::S1H + j) * N, lane);
-#pragma unroll
-        for (int m = 0; m < 8; ++m) v[m] = mont_mul(ch[m], a[m]);
-        load_l0(a, y, lane);
-        ntt_inv(v, buf, izt, lane);
-        bool bad = false;
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            v[m] = centre_small(to_canonical(v[m]) + a[m]);
-            bad |= iabs(v[m]) >= V::GAMMA1 - V::BETA;
-        }
-        if (__any_sync(FULL, bad)) return false;
-        store_l0(y, v, lane);
-    }
-    // v_s = INTT(c^ o s^2); r0 = LowBits(w - v_s)
-#pragma unroll 1
-    for (int i = 0; i < V::K; ++i) {
-        int32_t *w = slot + (SL::W + i) * N;
-        load_l2(a, pre + (S::S2H + i) * N, lane);
-#pragma unroll
-        for (int m = 0; m < 8; ++m) v[m] = mont_mul(ch[m], a[m]);
-        load_l0(a, w, lane);
-        ntt_inv(v, buf, izt, lane);
-        bool bad = false;
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            int32_t d = a[m] - v[m];                 // (-q, 2q)
-            d += (d < 0) ? Q : 0;
-            d -= (d >= Q) ? Q : 0;
-            int32_t h1, l0;
-            decompose<LEVEL>(d, h1, l0);
-            bad |= iabs(l0) >= V::GAMMA2 - V::BETA;
-            a[m] = d;
-        }
-        if (__any_sync(FULL, bad)) return false;
-        store_l0(w, a, lane);   // w - c s2, for the hint
-    }
-    // v_t = INTT(c^ o t^0); h = MakeHint(-v_t, w - v_s + v_t)
+    constexpr int R0 = V::K, ZS = V::K + V::L, ALL = 2 * V::K + V::L;   // ends of the three parts
+    static_assert(SL::W == SL::Y + V::L, "w behind y");
     uint32_t *hint = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(slot + SL::X * N) + SL::XHINT);
+    int32_t v[8], a[8], d[8];
     int count = 0;
 #pragma unroll 1
-    for (int i = 0; i < V::K; ++i) {
-        load_l2(a, pre + (S::T0H + i) * N, lane);
+    for (int u = 0; u < ALL; ++u) {
+        int32_t *data = slot + (u < R0 ? SL::W + u : SL::Y + u - R0) * N;   // w, y, w again
+        load_l2(a, pre + (u < R0 ? S::S2H + u : u < ZS ? S::S1H + u - R0 : S::T0H + u - ZS) * N, lane);
+        load_l0(d, data, lane);
 #pragma unroll
         for (int m = 0; m < 8; ++m) v[m] = mont_mul(ch[m], a[m]);
-        load_l0(a, slot + (SL::W + i) * N, lane);
         ntt_inv(v, buf, izt, lane);
         bool bad = false;
-        uint32_t hbits = 0;
+        if (u < R0) {
+            // v_s = INTT(c^ o s^2); r0 = LowBits(w - v_s); w - v_s is kept for the hint
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            int32_t vt = to_canonical(v[m]);
-            bad |= iabs(to_centred(vt)) >= V::GAMMA2;
-            int32_t rr = a[m] + vt;
-            rr -= (rr >= Q) ? Q : 0;
-            int32_t z = vt ? Q - vt : 0;
-            hbits |= (uint32_t)make_hint<LEVEL>(z, rr) << m;
-        }
-        if (__any_sync(FULL, bad)) return false;
-        uint32_t mine = 0;
+            for (int m = 0; m < 8; ++m) {
+                int32_t e = d[m] - v[m];                 // (-q, 2q)
+                e += (e < 0) ? Q : 0;
+                e -= (e >= Q) ? Q : 0;
+                int32_t h1, l0;
+                decompose<LEVEL>(e, h1, l0);
+                bad |= iabs(l0) >= V::GAMMA2 - V::BETA;
+                d[m] = e;
+            }
+            if (__any_sync(FULL, bad)) return false;
+            store_l0(data, d, lane);
+        } else if (u < ZS) {
+            // z = y + INTT(c^ o s^1); reject if ||z|| >= gamma1 - beta
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            const uint32_t w = __ballot_sync(FULL, (hbits >> m) & 1u);
-            if (lane == m) mine = w;
-            count += __popc(w);
+            for (int m = 0; m < 8; ++m) {
+                v[m] = centre_small(to_canonical(v[m]) + d[m]);
+                bad |= iabs(v[m]) >= V::GAMMA1 - V::BETA;
+            }
+            if (__any_sync(FULL, bad)) return false;
+            store_l0(data, v, lane);
+        } else {
+            // v_t = INTT(c^ o t^0); h = MakeHint(-v_t, w - v_s + v_t)
+            uint32_t hbits = 0;
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+                int32_t vt = to_canonical(v[m]);
+                bad |= iabs(to_centred(vt)) >= V::GAMMA2;
+                int32_t rr = d[m] + vt;
+                rr -= (rr >= Q) ? Q : 0;
+                int32_t z = vt ? Q - vt : 0;
+                hbits |= (uint32_t)make_hint<LEVEL>(z, rr) << m;
+            }
+            if (__any_sync(FULL, bad)) return false;
+            uint32_t mine = 0;
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+                const uint32_t x = __ballot_sync(FULL, (hbits >> m) & 1u);
+                if (lane == m) mine = x;
+                count += __popc(x);
+            }
+            if (lane < 8) hint[(u - ZS) * 8 + lane] = mine;
         }
-        if (lane < 8) hint[i * 8 + lane] = mine;
     }
     return count <= V::OMEGA;
 }
@@ -481,14 +429,14 @@ __device__ __forceinline__ bool sign_checks(const int32_t *pre, int32_t *slot, c
 // sig = c~ || z || h of the accepted attempt in `slot` (read through L2:
 // another warp may have written it).
 template <int LEVEL>
-__device__ __forceinline__ void sign_emit(uint8_t *sig, const int32_t *slot, int lane) {
+__device__ __forceinline__ void sign_emit(uint8_t *sig, const int32_t *slot, int32_t *buf, int lane) {
     using V = Lv<LEVEL>;
     using SL = Slot<LEVEL>;
 #pragma unroll 1
     for (int j = 0; j < V::L; ++j) {
         int32_t v[8];
         load_l2_cg(v, slot + (SL::Y + j) * N, lane);   // 8 consecutive coefficients
-        pack_seq<V::ZBITS>(sig + V::SIG_Z + j * V::POLYZ, v, V::GAMMA1, -1, lane);
+        pack_poly<V::ZBITS>(sig + V::SIG_Z + j * V::POLYZ, v, V::GAMMA1, -1, buf, lane);
     }
     const uint8_t *x = reinterpret_cast<const uint8_t *>(slot + SL::X * N);
     sig[lane] = __ldcg(x + SL::XCT + lane);
@@ -508,47 +456,15 @@ __device__ __forceinline__ void sign_emit(uint8_t *sig, const int32_t *slot, int
     for (int p = base + lane; p < V::OMEGA; p += 32) h[p] = 0;
 }
 
-template <int LEVEL, int SRC>
-__global__ void __launch_bounds__(32 * ROUND_WARPS, 8) k_sign_back(const SignBatch b, int r) {
-    extern __shared__ __align__(16) uint32_t sm[];
+// Task `task` (i-th of round r) after the last of its attempts: its signature,
+// the cap, or the next round.
+template <int LEVEL>
+__device__ __forceinline__ void settle(const SignBatch &b, const Round &q, int r, int i, int task, int best, int32_t *buf,
+                                       int lane) {
     using V = Lv<LEVEL>;
-    const Round q = round_of(b, r);
-    const int attempts = q.p * q.m;
-    if ((int)blockIdx.x * ROUND_WARPS >= attempts) return;
-    int32_t *zt = reinterpret_cast<int32_t *>(sm), *izt = zt + NTT_TABLE_WORDS;
-    load_zetas(zt);
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int s = blockIdx.x * ROUND_WARPS + warp;
-    if (s >= attempts) return;
-    int32_t *buf = izt + NTT_TABLE_WORDS + warp * 288;
-    const int i = s / q.m, task = pending_list(b, r)[i], rep = q.base + s - i * q.m;
-    int32_t *slot = slot_of<LEVEL>(b, s);
-    // a repetition past the cap, or past one that has been accepted, is not looked at
-    int skip = 0;
-    if (lane == 0) skip = rep >= b.max_iter || atomicOr(&b.best[task], 0) < rep;
-    if (!__shfl_sync(FULL, skip, 0)) {
-        int32_t ch[8];
-        const int8_t *c = reinterpret_cast<const int8_t *>(slot + Slot<LEVEL>::X * N);
-#pragma unroll
-        for (int m = 0; m < 8; ++m) ch[m] = c[lane + 32 * m];
-        ntt_fwd(ch, buf, zt, lane);
-        if (sign_checks<LEVEL>(pre_of<LEVEL, SRC>(b, task), slot, ch, buf, izt, lane) && lane == 0)
-            atomicMin(&b.best[task], rep);
-    }
-    // the last of the task's attempts settles the round
-    __threadfence();
-    int arrived = 0;
-    __syncwarp();
-    if (lane == 0) arrived = atomicAdd(&b.done[task], 1);
-    if (__shfl_sync(FULL, arrived, 0) != q.m - 1) return;
-    __threadfence();
-    int best = 0;
-    if (lane == 0) best = atomicOr(&b.best[task], 0);
-    best = __shfl_sync(FULL, best, 0);
     uint8_t *sig = b.sig + (size_t)task * V::SIG;
     if (best != INT_MAX) {
-        sign_emit<LEVEL>(sig, slot_of<LEVEL>(b, i * q.m + best - q.base), lane);
+        sign_emit<LEVEL>(sig, slot_of<LEVEL>(b, i * q.m + best - q.base), buf, lane);
         if (lane == 0) {
             if (b.status) b.status[task] = DIL_OK;
             if (b.iters) b.iters[task] = best + 1;
@@ -564,6 +480,53 @@ __global__ void __launch_bounds__(32 * ROUND_WARPS, 8) k_sign_back(const SignBat
         int *list = b.pending + (size_t)((r + 1) & 1) * b.n;
         list[atomicAdd(b.count + r + 1, 1)] = task;
     }
+}
+
+template <int LEVEL, int SRC>
+__global__ void __launch_bounds__(32 * ROUND_WARPS, 8) k_sign_back(const SignBatch b, int r) {
+    __shared__ __align__(16) int32_t tables[2 * NTT_TABLE_WORDS], bufs[ROUND_WARPS][288];
+    const Round q = round_of(b, r);
+    const int attempts = q.p * q.m;
+    if ((int)blockIdx.x * ROUND_WARPS >= attempts) return;
+    load_zetas(tables);
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, s = blockIdx.x * ROUND_WARPS + warp;
+    if (s >= attempts) return;
+    int32_t *buf = bufs[warp], *zt = tables, *izt = tables + NTT_TABLE_WORDS;
+    const int i = s / q.m, task = pending_list(b, r)[i], rep = q.base + s - i * q.m;
+    int32_t *slot = slot_of<LEVEL>(b, s);
+    // a repetition past the cap, or past one that has been accepted, is not looked at
+    int skip = 0;
+    if (lane == 0) skip = rep >= b.max_iter || (q.m > 1 && atomicOr(&b.best[task], 0) < rep);
+    bool accepted = false;
+    if (!__shfl_sync(FULL, skip, 0)) {
+        int32_t ch[8];
+        const int8_t *c = reinterpret_cast<const int8_t *>(slot + Slot<LEVEL>::X * N);
+#pragma unroll
+        for (int m = 0; m < 8; ++m) ch[m] = c[lane + 32 * m];
+        ntt_fwd(ch, buf, zt, lane);
+        accepted = sign_checks<LEVEL>(pre_of<LEVEL, SRC>(b, task), slot, ch, buf, izt, lane);
+    }
+    if (accepted) __threadfence();   // settle reads what other lanes (or, with m > 1, other warps) wrote, through L2
+    __syncwarp();
+    int best = accepted ? rep : INT_MAX;
+    if (q.m > 1) {
+        // the last of the task's attempts settles the round; what an accepted one
+        // wrote is visible before its repetition, and that before its arrival
+        int arrived = 0;
+        if (lane == 0) {
+            if (accepted) {
+                atomicMin(&b.best[task], rep);
+                __threadfence();
+            }
+            arrived = atomicAdd(&b.done[task], 1);
+        }
+        if (__shfl_sync(FULL, arrived, 0) != q.m - 1) return;
+        __threadfence();
+        if (lane == 0) best = atomicOr(&b.best[task], 0);
+        best = __shfl_sync(FULL, best, 0);
+    }
+    settle<LEVEL>(b, q, r, i, task, best, buf, lane);
 }
 
 // ---------------------------------------------------------------- what is left
@@ -688,27 +651,23 @@ cudaError_t launch_rounds(SignBatch b, void *ws, cudaStream_t s) {
     b.hash_warps = batch_hash_warps(b.n);
     b.expand_blocks = SRC == SIGN_PLAIN ? blocks_for((long long)b.n * V::K * V::L, K16_STATES) : 0;
     const int secret_blocks = SRC == SIGN_KEYED ? 0 : b.n;
-    const size_t tables = 4 * NTT_TABLE_WORDS;
-    const size_t prep_smem = 4 * (SRC == SIGN_PLAIN ? EXPAND16_WORDS : HASH16_STAGE_WORDS + NTT_TABLE_WORDS);
-    static_assert(NTT_TABLE_WORDS + 288 <= EXPAND16_WORDS && 288 <= HASH16_STAGE_WORDS, "the secrets' blocks");
+    const size_t prep_smem = 4 * (SRC == SIGN_PLAIN ? EXPAND16_WORDS : HASH16_STAGE_WORDS);
+    static_assert(288 <= HASH16_STAGE_WORDS && HASH16_STAGE_WORDS <= EXPAND16_WORDS, "every block's shared memory");
     if ((e = dynamic_smem(k_sign_prepare<LEVEL, SRC>, prep_smem)) != cudaSuccess) return e;
     k_sign_prepare<LEVEL, SRC><<<b.hash_warps + b.expand_blocks + secret_blocks, 32, prep_smem, s>>>(b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
-    const size_t front_smem = 2 * tables + 4 * ROUND_WARPS * front_warp_words<LEVEL>();
-    const size_t back_smem = 2 * tables + 4 * ROUND_WARPS * 288;
-    if ((e = dynamic_smem(k_sign_front<LEVEL, SRC>, front_smem)) != cudaSuccess) return e;
     const int rounds = rounds_of(LEVEL, b.n, b.slots);
     const int most = b.slots;   // attempts of a round; blocks beyond the actual count return at once
     const HashGrid h = hash_grid(most);
     for (int r = 0; r < rounds; ++r) {
         k_sign_mask<LEVEL><<<blocks_for(most, K16_STATES / V::L), 32, 0, s>>>(b, r);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_sign_front<LEVEL, SRC><<<blocks_for(most, ROUND_WARPS), 32 * ROUND_WARPS, front_smem, s>>>(b, r);
+        k_sign_front<LEVEL, SRC><<<most, 32, 0, s>>>(b, r);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         k_sign_hash<LEVEL><<<h.blocks, h.threads, 0, s>>>(b, r);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_sign_back<LEVEL, SRC><<<blocks_for(most, ROUND_WARPS), 32 * ROUND_WARPS, back_smem, s>>>(b, r);
+        k_sign_back<LEVEL, SRC><<<blocks_for(most, ROUND_WARPS), 32 * ROUND_WARPS, 0, s>>>(b, r);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     const size_t room = (size_t)b.slots * Slot<LEVEL>::POLYS / Scratch<LEVEL>::ITR_POLYS;
@@ -731,13 +690,20 @@ cudaError_t launch_src(int src, const SignBatch &b, void *ws, cudaStream_t s) {
 
 }  // namespace
 
-// Slots of a batch: one per task, and for a small batch enough for
-// ROUND_MAX_REPS repetitions of each while that does not overfill the GPU.
-int sign_batch_slots(int level, int n) {
-    const int least = level == 2 ? min_slots<2>() : level == 3 ? min_slots<3>() : min_slots<5>();
+// Slots of a batch that has 1 / parts of the GPU: one per task at least, and for
+// further repetitions up to ROUND_MAX_REPS per task within the fill, two per
+// task within ROUND_MOST.
+template <int LEVEL>
+static int slots_of(int n, int parts) {
+    const long long fill = round_fill<LEVEL>() / parts, most = ROUND_MOST / parts;
     long long s = (long long)n * ROUND_MAX_REPS;
-    if (s > ROUND_FILL) s = n > ROUND_FILL ? n : ROUND_FILL;
-    return (int)(s < least ? least : s);
+    if (s > fill) s = 2LL * n > fill ? 2LL * n : fill;
+    if (s > most) s = n > most ? n : most;
+    return (int)(s < min_slots<LEVEL>() ? min_slots<LEVEL>() : s);
+}
+
+int sign_batch_slots(int level, int n, int parts) {
+    return level == 2 ? slots_of<2>(n, parts) : level == 3 ? slots_of<3>(n, parts) : slots_of<5>(n, parts);
 }
 
 size_t sign_batch_bytes(int level, int src, size_t n, size_t slots) {

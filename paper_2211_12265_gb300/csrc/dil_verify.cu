@@ -3,9 +3,9 @@
 // Batch form.  The first kernel gives its leading blocks to the hashes
 // tr = H(pk) and mu = H(tr || M) and to SampleInBall(c~), sixteen tasks to a
 // warp, and the others to sampling A^, sixteen polynomials to a warp whatever tasks they belong to
-// (dil_sample16.cuh).  The second does the arithmetic, one task per group of P
-// warps up to the packed w1'; with a resident key's or the caller's A^ it is
-// the other blocks of the first.  The last recomputes c~ = H(mu || w1'),
+// (dil_sample16.cuh).  The second does the arithmetic up to the packed w1', one
+// task per warp; with a resident key's or the caller's A^ it is the other blocks
+// of the first, one task per group of P warps.  The last recomputes c~ = H(mu || w1'),
 // sixteen tasks to a warp, and compares.  Hashing inside
 // the task's own warp (k_verify, kept for the launch shapes a caller asks for)
 // runs the 18 blocks of a Dilithium2 task at 18.7 SM clocks per round, 8.1 k
@@ -141,13 +141,11 @@ __device__ __forceinline__ void verify_tasks(const VerifyBatch &b, int blk, uint
     int r = 0;
     if (verify_input<SRC>(b, task, key, m0, mlen)) {
         int32_t *scr = b.scratch + (size_t)task * verify_polys<LEVEL, SRC>() * N;
-        const int32_t *a = SRC == VERIFY_AHAT    ? b.ahat + (size_t)task * V::K * V::L * N
-                           : SRC == VERIFY_KEYED ? b.keys + (size_t)key * Scratch<LEVEL>::KEY_POLYS * N
-                                                 : scr + V::L * N;
-        r = verify_task<LEVEL, P, SRC == VERIFY_KEYED, SRC != VERIFY_KEYED, true>(
+        const int32_t *a = SRC == VERIFY_AHAT ? b.ahat + (size_t)task * V::K * V::L * N
+                                              : b.keys + (size_t)key * Scratch<LEVEL>::KEY_POLYS * N;
+        r = verify_task<LEVEL, P, SRC == VERIFY_KEYED, SRC == VERIFY_AHAT, true>(
             b.pk + (size_t)key * V::PK, nullptr, 0, b.sig + (size_t)task * V::SIG, scr, *v.gs, *v.ws, v.zt, v.izt,
-            v.g, v.bar, v.lane, a, nullptr, nullptr,
-            b.challenge_blocks ? reinterpret_cast<const int8_t *>(b.challenge) + (size_t)task * 256 : nullptr);
+            v.g, v.bar, v.lane, a);
     }
     if (v.g == 0 && v.lane == 0) b.ok[task] = (uint8_t)r;   // 1: c~ decides (k_verify_compare)
 }
@@ -205,10 +203,100 @@ __global__ void __launch_bounds__(32, 16) k_verify_prepare(const VerifyBatch b) 
         [&](int t) { return b.scratch + ((size_t)t * verify_polys<LEVEL, VERIFY_PLAIN>() + V::L) * N; }, sm, lane);
 }
 
-template <int LEVEL, int P>
-__global__ void __launch_bounds__(256, 4) k_verify_rows(const VerifyBatch b) {
-    extern __shared__ __align__(16) uint8_t smem[];
-    verify_tasks<LEVEL, P, VERIFY_PLAIN>(b, blockIdx.x, smem);
+// The arithmetic of one task, one warp: hint decoding, z^, and per row
+// w1' = UseHint(h, INTT(A^ z^ - c^ NTT(t1 2^d))), packed to the start of its
+// scratch.  False when the signature is malformed or z too large.
+template <int LEVEL>
+__device__ __forceinline__ bool verify_rows(const VerifyBatch &b, int task, int32_t *buf, int32_t *zh, uint32_t *hmask,
+                                            int lane) {
+    using V = Lv<LEVEL>;
+    const uint8_t *sig = b.sig + (size_t)task * V::SIG, *pk = b.pk + (size_t)task * V::PK;
+    uint8_t *sq = reinterpret_cast<uint8_t *>(buf);
+    int32_t v[8], ch[8];
+    // strict hint decoding into bit masks
+    stage_bytes(sq, sig + V::SIG_H, V::OMEGA + V::K, lane);
+    hmask[lane] = 0;
+    hmask[32 + lane] = 0;
+    __syncwarp();
+    bool bad = false;
+    int prev = 0;
+#pragma unroll 1
+    for (int i = 0; i < V::K; ++i) {
+        const int end = sq[V::OMEGA + i];
+        if (end < prev || end > V::OMEGA) {
+            bad = true;
+            break;
+        }
+        for (int j = prev + lane; j < end; j += 32) {
+            const int idx = sq[j];
+            if (j > prev && idx <= sq[j - 1]) bad = true;
+            atomicOr(&hmask[i * 8 + (idx >> 5)], 1u << (idx & 31));
+        }
+        prev = end;
+    }
+    if (!bad)
+        for (int j = prev + lane; j < V::OMEGA; j += 32)
+            if (sq[j]) bad = true;
+    if (__any_sync(FULL, bad)) return false;
+    // z^ = NTT(z), ||z|| < gamma1 - beta
+#pragma unroll 1
+    for (int j = 0; j < V::L; ++j) {
+        unpack_buf_l0<V::ZBITS>(v, sig + V::SIG_Z + j * V::POLYZ, V::GAMMA1, buf, lane);
+#pragma unroll
+        for (int m = 0; m < 8; ++m) bad |= iabs(v[m]) >= V::GAMMA1 - V::BETA;
+        if (__any_sync(FULL, bad)) return false;
+        ntt_fwd_global(v, buf);
+        store_l2(zh + j * N, v, lane);   // read back by the same lane
+    }
+    const int8_t *c = reinterpret_cast<const int8_t *>(b.challenge) + (size_t)task * 256;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) ch[m] = c[lane + 32 * m];
+    ntt_fwd_global(ch, buf);
+    int32_t *scr = b.scratch + (size_t)task * verify_polys<LEVEL, VERIFY_PLAIN>() * N;
+#pragma unroll 1
+    for (int i = 0; i < V::K; ++i) {
+        int32_t a[V::L][8];   // every load of the row in flight during t1's transform
+#pragma unroll
+        for (int j = 0; j < V::L; ++j) load_l2(a[j], scr + (V::L + i * V::L + j) * N, lane);
+        unpack_buf_l0<10>(v, pk + 32 + i * V::POLYT1, 0, buf, lane);
+#pragma unroll
+        for (int m = 0; m < 8; ++m) v[m] = (-v[m]) << D;   // t1 2^d, t1 unpacked as 0 - field
+        ntt_fwd_global(v, buf);
+        // summed in 64 bits, |sum| < 7 q 9.1q + 9.1q 9.1q < 2^31 q
+        long long acc[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) acc[m] = -(long long)ch[m] * v[m];
+#pragma unroll
+        for (int j = 0; j < V::L; ++j) {
+            load_l2(v, zh + j * N, lane);
+#pragma unroll
+            for (int m = 0; m < 8; ++m) acc[m] += (long long)a[j][m] * v[m];
+        }
+#pragma unroll
+        for (int m = 0; m < 8; ++m) v[m] = mont_reduce(acc[m]);
+        ntt_inv_global(v, buf);
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            const int hbit = (hmask[i * 8 + m] >> lane) & 1u;
+            v[m] = use_hint<LEVEL>(hbit, to_canonical(v[m]));
+        }
+        l0_to_seq(v, buf, lane);
+        pack_w1<LEVEL>(reinterpret_cast<uint8_t *>(scr) + i * V::POLYW1, v, lane);
+    }
+    return true;
+}
+
+template <int LEVEL>
+__global__ void __launch_bounds__(32, LEVEL == 2 ? 24 : 20) k_verify_rows(const VerifyBatch b) {
+    __shared__ __align__(16) int32_t buf[288], zh[Lv<LEVEL>::L * N];
+    __shared__ uint32_t hmask[64];
+    const int task = blockIdx.x, lane = threadIdx.x;
+    int key;
+    uint64_t m0;
+    size_t mlen;
+    const bool r = verify_input<VERIFY_PLAIN>(b, task, key, m0, mlen) &&
+                   verify_rows<LEVEL>(b, task, buf, zh, hmask, lane);
+    if (lane == 0) b.ok[task] = r;   // 1: c~ decides (k_verify_compare)
 }
 
 // c~ = H(mu || w1') of task `pair` against the signature's.
@@ -258,8 +346,6 @@ cudaError_t launch_batch(VerifyBatch b, int warps, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     if (b.n > b.hash_warps * K16_STATES) e = cudaMemsetAsync(b.next, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
-    const int blocks = (b.n + warps / P - 1) / (warps / P);
-    const size_t smem = cta_bytes(warps, P);
     if constexpr (SRC == VERIFY_PLAIN) {
         b.challenge_blocks = (b.n + K16_STATES - 1) / K16_STATES;
         const long long polys = (long long)b.n * Lv<LEVEL>::K * Lv<LEVEL>::L;
@@ -270,12 +356,11 @@ cudaError_t launch_batch(VerifyBatch b, int warps, cudaStream_t s) {
         if (e != cudaSuccess) return e;
         k_verify_prepare<LEVEL><<<b.hash_warps + b.challenge_blocks + expand_blocks, 32, bytes, s>>>(b);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(k_verify_rows<LEVEL, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_verify_rows<LEVEL, P><<<blocks, warps * 32, smem, s>>>(b);
+        k_verify_rows<LEVEL><<<b.n, 32, 0, s>>>(b);
     } else {
+        const int blocks = (b.n + warps / P - 1) / (warps / P);
+        const size_t smem = cta_bytes(warps, P);
         b.hash_blocks = (b.hash_warps + warps - 1) / warps;
-        b.challenge_blocks = 0;
         e = cudaFuncSetAttribute(k_verify_batch<LEVEL, P, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         k_verify_batch<LEVEL, P, SRC><<<b.hash_blocks + blocks, warps * 32, smem, s>>>(b);
@@ -288,6 +373,7 @@ cudaError_t launch_batch(VerifyBatch b, int warps, cudaStream_t s) {
 
 template <int LEVEL, int SRC>
 cudaError_t launch_batch_p(const VerifyBatch &b, int warps, int p, cudaStream_t s) {
+    if constexpr (SRC == VERIFY_PLAIN) return launch_batch<LEVEL, 1, SRC>(b, warps, s);
     switch (p) {
         case 1: return launch_batch<LEVEL, 1, SRC>(b, warps, s);
         case 4: return launch_batch<LEVEL, 4, SRC>(b, warps, s);
