@@ -48,10 +48,6 @@ namespace {
 
 constexpr size_t POLY_BYTES = 256 * sizeof(int32_t);
 
-// Up to this many tasks the batch forms' arithmetic runs four warps per task:
-// a task's latency is what counts while the SMs are not full.
-constexpr size_t BATCH_WIDE_TASKS = 600;
-
 // NVTX range over one API call (a no-op unless a profiler is attached), so
 // traces show which entry point issued which launches.
 struct TraceRange {
@@ -114,12 +110,11 @@ struct Shape {
     int warps, p;
 };
 
-Shape shape_of(const dil_ctx *c, int op, int level, size_t n, size_t per) {
+Shape shape_of(const dil_ctx *c, int op, int level, size_t per) {
     const int w = c->warps[op][lidx(level)], p = c->wpt[op][lidx(level)];
     if (p > 1) return {true, w, p};
     if (c->budget < per) return {true, 8, 2};
-    if (n <= BATCH_WIDE_TASKS) return {false, 4, 4};
-    return {false, w ? w : 4, 1};
+    return {false, 0, 0};
 }
 
 // The fused kernels' launch shape where a caller set none.
@@ -155,7 +150,9 @@ cudaError_t keygen_chunk(const Shape &sh, int level, int m, const uint8_t *seeds
                     : dil::launch_keygen_batch(level, m, seeds, pk, sk, scratch, s);
 }
 
-size_t verify_task_bytes(size_t polys) { return polys * POLY_BYTES + dil::VERIFY_AUX_BYTES; }
+size_t verify_task_bytes(int level, int src) {
+    return dil::verify_batch_polys(level, src) * POLY_BYTES + dil::VERIFY_AUX_BYTES;
+}
 
 constexpr size_t PIPE_MIN_TASKS = 2048;   // smaller batches run as one chunk
 constexpr size_t PIPE_STREAMS = 4;
@@ -241,6 +238,8 @@ int sign_cap(const dil_ctx *c, int level) {
     return (c->max_iter > 0 && c->max_iter < cap) ? c->max_iter : cap;
 }
 
+void sizes_of(int level, size_t &pk, size_t &sk, size_t &sig) { dil_sizes(level, &pk, &sk, &sig); }
+
 // Carves m tasks of a Verify batch out of a workspace of m verify_task_bytes.
 void carve_verify(dil::VerifyBatch &b, void *ws, size_t m, size_t polys) {
     uint8_t *aux = static_cast<uint8_t *>(ws) + m * polys * POLY_BYTES;
@@ -252,7 +251,33 @@ void carve_verify(dil::VerifyBatch &b, void *ws, size_t m, size_t polys) {
     b.challenge = aux + 128 * m;
 }
 
-void sizes_of(int level, size_t &pk, size_t &sk, size_t &sig) { dil_sizes(level, &pk, &sk, &sig); }
+// Runs Verify's batch form over the n tasks of `all` (whose per-task pointers are
+// those of task 0), in as many launches as the budget asks for.
+int run_verify_batch(dil_ctx *c, int level, int src, size_t n, const dil::VerifyBatch &all, cudaStream_t s) {
+    const size_t polys = dil::verify_batch_polys(level, src), per = verify_task_bytes(level, src);
+    const size_t chunk = chunk_tasks(c, per, n);
+    if (chunk == 0) return DIL_ENOMEM;
+    int rc = ensure_ws(c, chunk * per);
+    if (!rc) rc = ensure_aux(c);
+    if (rc) return rc;
+    size_t pkb, skb, sigb;
+    sizes_of(level, pkb, skb, sigb);
+    const size_t k = level == 2 ? 4 : level == 3 ? 6 : 8, l = level == 2 ? 4 : level == 3 ? 5 : 7;
+    for (size_t s0 = 0; s0 < n; s0 += chunk) {
+        const size_t m = std::min(chunk, n - s0);
+        dil::VerifyBatch b = all;
+        carve_verify(b, c->ws, m, polys);
+        if (src != dil::VERIFY_KEYED) b.pk += pkb * s0;
+        if (b.ahat) b.ahat += k * l * 256 * s0;
+        if (b.key_idx) b.key_idx += s0;
+        b.off += s0;
+        b.sig += sigb * s0;
+        b.ok += s0;
+        const cudaError_t e = dil::launch_verify_batch(level, src, b, {c->aux[0], c->ev_fork, c->ev_join}, s);
+        if (e != cudaSuccess) return cuda_fail(e);
+    }
+    return DIL_OK;
+}
 
 }  // namespace
 
@@ -357,7 +382,7 @@ int dil_keygen(dil_ctx *c, int level, size_t n, const uint8_t *seeds, uint8_t *p
     if (rc) return rc;
     for (size_t s0 = 0; s0 < n; s0 += chunk) {
         int m = (int)std::min(chunk, n - s0);
-        const Shape sh = shape_of(c, 0, level, m, per);
+        const Shape sh = shape_of(c, 0, level, per);
         cudaError_t e = keygen_chunk(sh, level, m, seeds + 32 * s0, pk + pkb * s0, sk + skb * s0, (int32_t *)c->ws,
                                      (cudaStream_t)stream);
         if (e != cudaSuccess) return cuda_fail(e);
@@ -417,29 +442,26 @@ int dil_verify(dil_ctx *c, int level, size_t n, const uint8_t *pk, const uint8_t
     DeviceGuard g(c->device);
     size_t pkb, skb, sigb;
     sizes_of(level, pkb, skb, sigb);
-    const size_t polys = dil::scratch_polys(dil::OP_VERIFY, level);
-    const Shape sh = shape_of(c, 2, level, n, verify_task_bytes(polys));
-    const size_t per = sh.fused ? polys * POLY_BYTES : verify_task_bytes(polys);
+    const size_t batch = verify_task_bytes(level, dil::VERIFY_PLAIN);
+    const Shape sh = shape_of(c, 2, level, batch);
+    if (!sh.fused) {
+        dil::VerifyBatch b{};
+        b.pk = pk;
+        b.msg = msg;
+        b.off = msg_off;
+        b.sig = sig;
+        b.ok = ok;
+        return run_verify_batch(c, level, dil::VERIFY_PLAIN, n, b, (cudaStream_t)stream);
+    }
+    const size_t per = dil::scratch_polys(dil::OP_VERIFY, level) * POLY_BYTES;
     size_t chunk = chunk_tasks(c, per, n);
     if (chunk == 0) return DIL_ENOMEM;
     int rc = ensure_ws(c, chunk * per);
     if (rc) return rc;
     for (size_t s0 = 0; s0 < n; s0 += chunk) {
         int m = (int)std::min(chunk, n - s0);
-        cudaError_t e;
-        if (sh.fused) {
-            e = dil::launch_verify(level, m, pk + pkb * s0, msg, msg_off + s0, sig + sigb * s0, ok + s0,
-                                   (int32_t *)c->ws, sh.warps, sh.p, (cudaStream_t)stream);
-        } else {
-            dil::VerifyBatch b{};
-            carve_verify(b, c->ws, m, polys);
-            b.pk = pk + pkb * s0;
-            b.msg = msg;
-            b.off = msg_off + s0;
-            b.sig = sig + sigb * s0;
-            b.ok = ok + s0;
-            e = dil::launch_verify_batch(level, dil::VERIFY_PLAIN, b, sh.warps, sh.p, (cudaStream_t)stream);
-        }
+        cudaError_t e = dil::launch_verify(level, m, pk + pkb * s0, msg, msg_off + s0, sig + sigb * s0, ok + s0,
+                                           (int32_t *)c->ws, sh.warps, sh.p, (cudaStream_t)stream);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     return DIL_OK;
@@ -517,32 +539,14 @@ int dil_verify_a(dil_ctx *c, int level, size_t n, const uint8_t *pk, const uint8
     if (!pk || !msg_off || !sig || !ok || !aligned16(ahat) || n > (size_t)INT32_MAX) return DIL_EINVAL;
     std::lock_guard<std::mutex> lk(c->mu);
     DeviceGuard g(c->device);
-    size_t pkb, skb, sigb;
-    sizes_of(level, pkb, skb, sigb);
-    // z^ and what a task's hashes leave, less than dil_verify's scratch
-    const size_t polys = dil::keyed_verify_polys(level), per = verify_task_bytes(polys);
-    const size_t chunk = chunk_tasks(c, per, n);
-    if (chunk == 0) return DIL_ENOMEM;
-    int rc = ensure_ws(c, chunk * per);
-    if (rc) return rc;
-    const int32_t *a = reinterpret_cast<const int32_t *>(ahat);
-    for (size_t s0 = 0; s0 < n; s0 += chunk) {
-        const int m = (int)std::min(chunk, n - s0);
-        dil::VerifyBatch b{};
-        carve_verify(b, c->ws, m, polys);
-        b.pk = pk + pkb * s0;
-        b.msg = msg;
-        b.off = msg_off + s0;
-        b.sig = sig + sigb * s0;
-        b.ok = ok + s0;
-        b.ahat = a + ahat_words(level) * s0;
-        const int w = c->warps[2][lidx(level)];
-        const bool wide = (size_t)m <= BATCH_WIDE_TASKS;
-        cudaError_t e = dil::launch_verify_batch(level, dil::VERIFY_AHAT, b, wide ? 4 : w ? w : 4, wide ? 4 : 1,
-                                                 (cudaStream_t)stream);
-        if (e != cudaSuccess) return cuda_fail(e);
-    }
-    return DIL_OK;
+    dil::VerifyBatch b{};
+    b.pk = pk;
+    b.msg = msg;
+    b.off = msg_off;
+    b.sig = sig;
+    b.ok = ok;
+    b.ahat = reinterpret_cast<const int32_t *>(ahat);
+    return run_verify_batch(c, level, dil::VERIFY_AHAT, n, b, (cudaStream_t)stream);
 }
 
 // ---------------------------------------------------------------- persistent
@@ -788,34 +792,30 @@ int dil_verify_keyed(dil_ctx *c, const dil_keystore *ks, size_t n, const int32_t
     DeviceGuard g(c->device);
     size_t pkb, skb, sigb;
     sizes_of(ks->level, pkb, skb, sigb);
-    const size_t polys = dil::keyed_verify_polys(ks->level);
-    const Shape sh = shape_of(c, 2, ks->level, n, verify_task_bytes(polys));
-    const size_t per = sh.fused ? polys * POLY_BYTES : verify_task_bytes(polys);
+    const Shape sh = shape_of(c, 2, ks->level, verify_task_bytes(ks->level, dil::VERIFY_KEYED));
+    if (!sh.fused) {
+        dil::VerifyBatch b{};
+        b.pk = ks->pk;
+        b.msg = msg;
+        b.off = msg_off;
+        b.sig = sig;
+        b.ok = ok;
+        b.keys = ks->keys;
+        b.key_idx = key_idx;
+        b.key_tr = ks->tr;
+        b.n_keys = (int)ks->n;
+        return run_verify_batch(c, ks->level, dil::VERIFY_KEYED, n, b, (cudaStream_t)stream);
+    }
+    const size_t per = dil::keyed_verify_polys(ks->level) * POLY_BYTES;
     size_t chunk = chunk_tasks(c, per, n);
     if (chunk == 0) return DIL_ENOMEM;
     int rc = ensure_ws(c, chunk * per);
     if (rc) return rc;
     for (size_t s0 = 0; s0 < n; s0 += chunk) {
         int m = (int)std::min(chunk, n - s0);
-        cudaError_t e;
-        if (sh.fused) {
-            e = dil::launch_verify_keyed(ks->level, m, (int)ks->n, key_idx + s0, ks->pk, ks->keys, ks->tr, msg,
-                                         msg_off + s0, sig + sigb * s0, ok + s0, (int32_t *)c->ws, sh.warps, sh.p,
-                                         (cudaStream_t)stream);
-        } else {
-            dil::VerifyBatch b{};
-            carve_verify(b, c->ws, m, polys);
-            b.pk = ks->pk;
-            b.msg = msg;
-            b.off = msg_off + s0;
-            b.sig = sig + sigb * s0;
-            b.ok = ok + s0;
-            b.keys = ks->keys;
-            b.key_idx = key_idx + s0;
-            b.key_tr = ks->tr;
-            b.n_keys = (int)ks->n;
-            e = dil::launch_verify_batch(ks->level, dil::VERIFY_KEYED, b, sh.warps, sh.p, (cudaStream_t)stream);
-        }
+        cudaError_t e = dil::launch_verify_keyed(ks->level, m, (int)ks->n, key_idx + s0, ks->pk, ks->keys, ks->tr, msg,
+                                                 msg_off + s0, sig + sigb * s0, ok + s0, (int32_t *)c->ws, sh.warps,
+                                                 sh.p, (cudaStream_t)stream);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     return DIL_OK;
@@ -904,7 +904,7 @@ int dil_keygen_host(dil_ctx *c, int level, size_t n, const uint8_t *seeds, uint8
     if (rc) return rc;
     uint8_t *d_seed = (uint8_t *)c->stage, *d_pk = d_seed + al(32 * n), *d_sk = d_pk + al(pkb * n);
     const size_t per = dil::scratch_polys(dil::OP_KEYGEN, level) * POLY_BYTES;
-    const Shape sh = shape_of(c, 0, level, n, per);
+    const Shape sh = shape_of(c, 0, level, per);
     const size_t tasks = pipe_tasks(c, n, per);
     return run_pipeline(c, n, tasks, tasks * per, (cudaStream_t)stream,
                         [&](size_t c0, size_t c1, cudaStream_t s, int32_t *scratch) -> int {
@@ -997,9 +997,10 @@ int dil_verify_host(dil_ctx *c, int level, size_t n, const uint8_t *pk, const ui
     uint64_t *d_off = (uint64_t *)(d_msg + al(mlen + 1));
     uint8_t *d_sig = (uint8_t *)d_off + al(8 * (n + 1));
     uint8_t *d_ok = d_sig + al(sigb * n);
-    const size_t polys = dil::scratch_polys(dil::OP_VERIFY, level);
-    const Shape sh = shape_of(c, 2, level, n, pipe_streams(n) * verify_task_bytes(polys));
-    const size_t per = sh.fused ? polys * POLY_BYTES : verify_task_bytes(polys), tasks = pipe_tasks(c, n, per);
+    const size_t batch = verify_task_bytes(level, dil::VERIFY_PLAIN);
+    const Shape sh = shape_of(c, 2, level, pipe_streams(n) * batch);
+    const size_t per = sh.fused ? dil::scratch_polys(dil::OP_VERIFY, level) * POLY_BYTES : batch;
+    const size_t tasks = pipe_tasks(c, n, per);
     return run_pipeline(c, n, tasks, tasks * per, (cudaStream_t)stream,
                         [&](size_t c0, size_t c1, cudaStream_t s, int32_t *scratch) -> int {
                             const size_t m = c1 - c0;
@@ -1015,13 +1016,13 @@ int dil_verify_host(dil_ctx *c, int level, size_t n, const uint8_t *pk, const ui
                                                        d_sig + sigb * c0, d_ok + c0, scratch, sh.warps, sh.p, s);
                             } else {
                                 dil::VerifyBatch b{};
-                                carve_verify(b, scratch, m, polys);
+                                carve_verify(b, scratch, m, dil::verify_batch_polys(level, dil::VERIFY_PLAIN));
                                 b.pk = d_pk + pkb * c0;
                                 b.msg = d_msg;
                                 b.off = d_off + c0;
                                 b.sig = d_sig + sigb * c0;
                                 b.ok = d_ok + c0;
-                                e = dil::launch_verify_batch(level, dil::VERIFY_PLAIN, b, sh.warps, sh.p, s);
+                                e = dil::launch_verify_batch(level, dil::VERIFY_PLAIN, b, dil::VerifyFork{}, s);
                             }
                             if (e != cudaSuccess) return cuda_fail(e);
                             if (!d2h(ok + c0, d_ok + c0, m, s)) return DIL_ECUDA;

@@ -15,9 +15,9 @@ template <int LEVEL>
 __global__ void __launch_bounds__(32, 16) k_expand_a(int n, const uint8_t *rho, size_t rho_stride, int32_t *ahat) {
     __shared__ __align__(16) uint32_t st[EXPAND16_WORDS];
     constexpr int KL = Lv<LEVEL>::K * Lv<LEVEL>::L;
-    expand_a_batch<LEVEL>((long long)blockIdx.x * K16_STATES, (long long)n * KL,
-                          [&](int t) { return rho + (size_t)t * rho_stride; },
-                          [&](int t) { return ahat + (size_t)t * KL * N; }, st, threadIdx.x);
+    expand_a_batch<LEVEL, true>((long long)blockIdx.x * K16_STATES, (long long)n * KL,
+                                [&](int t) { return rho + (size_t)t * rho_stride; },
+                                [&](int t) { return ahat + (size_t)t * KL * N; }, st, threadIdx.x);
 }
 
 template <int LEVEL>

@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(32, 16) k_keygen_expand(int n, int32_t *scratc
             [&](int t) { return reinterpret_cast<const uint8_t *>(gen_scratch<LEVEL>(scratch, t)) + 32; },
             [&](int t) { return gen_scratch<LEVEL>(scratch, t) + S::GEN_S * N; }, st, lane);
     } else {
-        expand_a_batch<LEVEL>(
+        expand_a_batch<LEVEL, false>(
             (long long)(blk - s_blocks) * K16_STATES, (long long)n * V::K * V::L,
             [&](int t) { return reinterpret_cast<const uint8_t *>(gen_scratch<LEVEL>(scratch, t)); },
             [&](int t) { return gen_scratch<LEVEL>(scratch, t) + V::L * N; }, st, lane);
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(32, LEVEL == 2 ? 28 : 20) k_keygen_rows(uint8_
     int32_t v[8], s[8];
 #pragma unroll 1
     for (int j = 0; j < V::L; ++j) {
-        load_l2(s, sraw + j * N, lane);
+        load_seq(s, sraw + j * N, lane);
         load_l0(v, sraw + j * N, lane);
         pack_poly<V::ETABITS>(sk + V::SK_S1 + j * V::POLYETA, s, V::ETA, -1, buf, lane);
         ntt_fwd_global(v, buf);
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(32, LEVEL == 2 ? 28 : 20) k_keygen_rows(uint8_
         int32_t a[V::L][8];
 #pragma unroll
         for (int j = 0; j < V::L; ++j) load_l2(a[j], ah + (i * V::L + j) * N, lane);
-        load_l2(s, sraw + (V::L + i) * N, lane);
+        load_seq(s, sraw + (V::L + i) * N, lane);
         pack_poly<V::ETABITS>(sk + V::SK_S2 + i * V::POLYETA, s, V::ETA, -1, buf, lane);
         long long acc[8];
 #pragma unroll

@@ -36,8 +36,7 @@ cudaError_t launch_verify(int level, int n, const uint8_t *pk, const uint8_t *ms
                           const uint8_t *sig, uint8_t *ok, int32_t *scratch, int warps, int p, cudaStream_t s);
 
 // Batch forms: the hashes of independent tasks run sixteen to a warp (dil_gen.cu,
-// dil_verify.cu).  warps and p (1 or 4) shape the arithmetic of VERIFY_AHAT and
-// VERIFY_KEYED; otherwise it runs on single warps.
+// dil_verify.cu).
 cudaError_t launch_keygen_batch(int level, int n, const uint8_t *seeds, uint8_t *pk, uint8_t *sk, int32_t *scratch,
                                 cudaStream_t s);
 // Where a Verify's A^ comes from: sampled, the caller's, or a resident key's.
@@ -49,7 +48,7 @@ struct VerifyBatch {
     const uint64_t *off;
     const uint8_t *sig;
     uint8_t *ok;
-    int32_t *scratch;        // VERIFY_PLAIN: scratch_polys(OP_VERIFY) per task, else keyed_verify_polys
+    int32_t *scratch;        // verify_batch_polys polynomials per task
     const int32_t *ahat;     // VERIFY_AHAT
     const int32_t *keys;     // VERIFY_KEYED: KEY_POLYS polynomials, index and tr of each key
     const int32_t *key_idx;
@@ -58,12 +57,19 @@ struct VerifyBatch {
     uint32_t *mu, *tr;       // per task 16 and (not VERIFY_KEYED) 8 words
     uint8_t *challenge;      // per task 256 bytes
     int *next;               // counter of the hashing warps
-    int hash_warps, hash_blocks, challenge_blocks;   // set by the launch
+    int hash_warps, challenge_blocks;   // set by the launch
 };
 // Per task beside the polynomials: mu (64), tr (32), 32 more, of which the
 // batch's counter takes the first, and the challenge (256).
 constexpr size_t VERIFY_AUX_BYTES = 384;
-cudaError_t launch_verify_batch(int level, int src, const VerifyBatch &b, int warps, int p, cudaStream_t s);
+// A stream for the hashes of tr and mu beside the rest (null: none), which starts
+// after what is on the launch's stream and which that waits for.
+struct VerifyFork {
+    cudaStream_t stream;
+    cudaEvent_t fork, join;
+};
+size_t verify_batch_polys(int level, int src);   // scratch polynomials of one task
+cudaError_t launch_verify_batch(int level, int src, const VerifyBatch &b, const VerifyFork &f, cudaStream_t s);
 // Sign in rounds (dil_rounds.cu).  Where a task's A^, s^1, s^2 and t^0 come from:
 // its secret key, that with the caller's A^, or a resident key.
 enum SignSource { SIGN_PLAIN = 0, SIGN_AHAT = 1, SIGN_KEYED = 2 };

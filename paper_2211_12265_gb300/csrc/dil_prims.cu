@@ -94,10 +94,10 @@ __global__ void k_test_ntt(int n, const int32_t *in, int32_t *out, int inverse) 
         ntt_fwd(r, ws.buf, zt, lane);
 #pragma unroll
         for (int m = 0; m < 8; ++m) r[m] = to_canonical(reduce_q(r[m]));
-        store_l2(dst, r, lane);
+        store_seq(dst, r, lane);
     } else {
         // ntt_inv returns INTT(x) * 2^32; feed x * 2^-32 = mont_mul(x, 1)
-        load_l2(r, src, lane);
+        load_seq(r, src, lane);
 #pragma unroll
         for (int m = 0; m < 8; ++m) r[m] = mont_mul(reduce_q(r[m]), 1);
         ntt_inv(r, ws.buf, izt, lane);
@@ -169,10 +169,10 @@ __global__ void k_test_expand_a(int n, const uint8_t *rho, int32_t *out) {
     stage_bytes(gs.rho, rho + (size_t)item * 32, 32, lane);
     __syncwarp();
     int32_t *o = out + (size_t)item * V::K * V::L * N;
-    expand_a_range<LEVEL>(gs.rho, 0, 1, o, ws, lane);
-    expand_a_range<LEVEL>(gs.rho, 1, 3, o, ws, lane);
-    expand_a_range<LEVEL>(gs.rho, 3, 9, o, ws, lane);
-    expand_a_range<LEVEL>(gs.rho, 9, V::K * V::L, o, ws, lane);
+    expand_a_range<LEVEL, true>(gs.rho, 0, 1, o, ws, lane);
+    expand_a_range<LEVEL, true>(gs.rho, 1, 3, o, ws, lane);
+    expand_a_range<LEVEL, true>(gs.rho, 3, 9, o, ws, lane);
+    expand_a_range<LEVEL, true>(gs.rho, 9, V::K * V::L, o, ws, lane);
 }
 
 // ---------------------------------------------------------------- t^0 = NTT(t0)
@@ -264,7 +264,7 @@ __device__ __forceinline__ void t0_unpack(int32_t r[8], const uint8_t *sk, int i
 __device__ __forceinline__ void t0_store(int32_t *dst, int32_t r[8], int lane) {
 #pragma unroll
     for (int m = 0; m < 8; ++m) r[m] = to_canonical(reduce_q(r[m]));
-    store_l2(dst, r, lane);
+    store_seq(dst, r, lane);
 }
 
 // (0a) unpack kernel: t0 of task `item` to tmp (natural order)

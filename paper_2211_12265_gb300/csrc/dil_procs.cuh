@@ -10,9 +10,9 @@
 // NTT exchange buffers and squeezed blocks; per-group shared memory holds the
 // task's seeds, the packed w1 hash input, c~ and the hint masks.  Per-task
 // vectors that do not fit on chip (A^, s^1, s^2, t^0, y, y^, w, z) live in a
-// global scratch area: NTT-domain polynomials in index order (lane t reads
-// 8t..8t+7 with two 16-byte loads), plain ones in coefficient order (lane t
-// reads t + 32m, coalesced).
+// global scratch area: NTT-domain polynomials in lane order (lane t reads indexes
+// 8t..8t+7 with two coalesced 16-byte loads), plain ones in coefficient order
+// (lane t reads t + 32m, coalesced).
 #pragma once
 #include "dil_sample.cuh"
 
@@ -80,25 +80,55 @@ struct Units {
     static constexpr int SIZE = (M >= 2 * P) ? 2 : 1;
 };
 
-__device__ __forceinline__ void load_l2(int32_t v[8], const int32_t *p, int lane) {
+// Eight consecutive coefficients of lane t (8t..8t+7) of a polynomial in
+// coefficient order, or an NTT-domain one in index order (the order A^ has
+// outside this library).
+__device__ __forceinline__ void load_seq(int32_t v[8], const int32_t *p, int lane) {
     const int4 *q = reinterpret_cast<const int4 *>(p + 8 * lane);
     int4 a = q[0], b = q[1];
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
     v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
 
-// As load_l2, through L2 only (data written by warps on other SMs).
-__device__ __forceinline__ void load_l2_cg(int32_t v[8], const int32_t *p, int lane) {
+// As load_seq, through L2 only (data written by warps on other SMs).
+__device__ __forceinline__ void load_seq_cg(int32_t v[8], const int32_t *p, int lane) {
     const int4 *q = reinterpret_cast<const int4 *>(p + 8 * lane);
     int4 a = __ldcg(q), b = __ldcg(q + 1);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
     v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
 
-__device__ __forceinline__ void store_l2(int32_t *p, const int32_t v[8], int lane) {
+__device__ __forceinline__ void store_seq(int32_t *p, const int32_t v[8], int lane) {
     int4 *q = reinterpret_cast<int4 *>(p + 8 * lane);
     q[0] = make_int4(v[0], v[1], v[2], v[3]);
     q[1] = make_int4(v[4], v[5], v[6], v[7]);
+}
+
+// The same eight coefficients of an NTT-domain polynomial in lane order, the
+// order of every scratch and resident key: indexes 8t..8t+3 at 4t, 8t+4..8t+7 at
+// 128 + 4t.  Each 16-byte access of a warp then covers 512 consecutive bytes;
+// in index order it used half of every 32-byte sector and met two-way bank
+// conflicts in shared memory (l1tex was the busiest unit of Sign's front kernel,
+// 83%).
+__device__ __forceinline__ void load_l2(int32_t v[8], const int32_t *p, int lane) {
+    const int4 *q = reinterpret_cast<const int4 *>(p) + lane;
+    int4 a = q[0], b = q[32];
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+
+// As load_l2, through L2 only (data written by warps on other SMs).
+__device__ __forceinline__ void load_l2_cg(int32_t v[8], const int32_t *p, int lane) {
+    const int4 *q = reinterpret_cast<const int4 *>(p) + lane;
+    int4 a = __ldcg(q), b = __ldcg(q + 32);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+
+__device__ __forceinline__ void store_l2(int32_t *p, const int32_t v[8], int lane) {
+    int4 *q = reinterpret_cast<int4 *>(p) + lane;
+    q[0] = make_int4(v[0], v[1], v[2], v[3]);
+    q[32] = make_int4(v[4], v[5], v[6], v[7]);
 }
 
 __device__ __forceinline__ void load_l0(int32_t v[8], const int32_t *p, int lane) {
@@ -222,34 +252,36 @@ template <int LEVEL> struct Scratch {
 template <int M, int P>
 __device__ __forceinline__ int share_lo(int g) { return g * M / P; }
 
-// A^_p (p = i l + j) for p in [lo, hi) into out + p N in index order: up to
-// sixteen sponges at a time while at least seven remain, six at a time while
+// A^_p (p = i l + j) for p in [lo, hi) into out + p N in lane order (INDEX: in
+// index order): up to sixteen sponges at a time while at least seven remain, six at a time while
 // at least three remain, then a pair or a single.
-template <int LEVEL>
+template <int LEVEL, bool INDEX = false>
 __device__ void expand_a_range(const uint8_t *rho, int lo, int hi, int32_t *out, WarpSmem &ws, int lane) {
     constexpr int L = Lv<LEVEL>::L;
     int p = lo;
     while (hi - p >= 7) {
         const int c = min(K16_STATES, hi - p);
-        expand_a_16<L>(rho, p, c, out + p * N, ws.k16, lane);
+        expand_a_16<L, INDEX>(rho, p, c, out + p * N, ws.k16, lane);
         p += c;
     }
     while (hi - p >= 3) {
         const int c = min(K6_STATES, hi - p);
-        expand_a_six<L>(rho, p, c, out + p * N, ws.kst, ws.kpi(), lane);
+        expand_a_six<L, INDEX>(rho, p, c, out + p * N, ws.kst, ws.kpi(), lane);
         p += c;
     }
     int32_t a[8];
     if (hi - p == 2) {
         expand_a_pair(rho, p / L, p % L, (p + 1) / L, (p + 1) % L, ws.buf, ws.buf2, ws.sq, ws.sq2, lane);
         read_buf_l2(a, ws.buf2, lane);
-        store_l2(out + (p + 1) * N, a, lane);
+        if (INDEX) store_seq(out + (p + 1) * N, a, lane);
+        else store_l2(out + (p + 1) * N, a, lane);
     } else if (hi - p == 1) {
         expand_a_poly(rho, p / L, p % L, ws.buf, ws.sq, lane);
     }
     if (hi - p >= 1) {
         read_buf_l2(a, ws.buf, lane);
-        store_l2(out + p * N, a, lane);
+        if (INDEX) store_seq(out + p * N, a, lane);
+        else store_l2(out + p * N, a, lane);
     }
     __syncwarp();
 }
@@ -261,7 +293,7 @@ __device__ __forceinline__ int32_t *y_slot(int32_t *ring, int u) {
 }
 
 // y_j = ExpandMask(rho', kappa + j) into its ring slot and y^_j = NTT(y_j) in
-// index order to yh + j N, for j in [lo, hi) (one warp's share of a
+// lane order to yh + j N, for j in [lo, hi) (one warp's share of a
 // repetition when a task group has several warps).
 template <int LEVEL>
 __device__ void expand_mask_range(const uint8_t *rhop, int kappa, int lo, int hi, int32_t *ring, int32_t *yh,
@@ -342,8 +374,8 @@ __device__ void mask_stream(const uint8_t *rhop, int kappa, MaskStream &ms, int3
 }
 
 // acc = sum_j A^_ij o v^_j 2^-32, |acc| < q, for one row i of A^ (ahat: the row's
-// l polynomials, index order; read through L2 since another warp or kernel may
-// have written them); v^_j (index order) at `vhat`.  The products are summed in
+// l polynomials; read through L2 since another warp or kernel may have written
+// them); v^_j at `vhat`.  The products are summed in
 // 64 bits (|sum| < 7 q 9.1q < 2^31 q) and reduced once.
 __device__ __forceinline__ void accumulate_row(int32_t acc[8], const int32_t *ahat, int l, const int32_t *vhat,
                                                int lane) {
@@ -405,7 +437,7 @@ __device__ void gen_rows(uint8_t *pk, uint8_t *sk, int32_t *scratch, WarpSmem &w
     // s^1 over the start of scratch, which holds nothing that is still read
 #pragma unroll 1
     for (int j = g; j < V::L; j += P) {
-        load_l2(a, sraw + j * N, lane);
+        load_seq(a, sraw + j * N, lane);
         pack_poly<V::ETABITS>(sk + V::SK_S1 + j * V::POLYETA, a, V::ETA, -1, ws.buf, lane);
         load_l0(r, sraw + j * N, lane);
         ntt_fwd(r, ws.buf, zt, lane);
@@ -417,7 +449,7 @@ __device__ void gen_rows(uint8_t *pk, uint8_t *sk, int32_t *scratch, WarpSmem &w
     for (int i = g; i < V::K; i += P) {
         accumulate_row(acc, scratch + (V::L + i * V::L) * N, V::L, scratch, lane);
         ntt_inv(acc, ws.buf, izt, lane);
-        load_l2(a, sraw + (V::L + i) * N, lane);
+        load_seq(a, sraw + (V::L + i) * N, lane);
         load_l0(r, sraw + (V::L + i) * N, lane);
         pack_poly<V::ETABITS>(sk + V::SK_S2 + i * V::POLYETA, a, V::ETA, -1, ws.buf, lane);
         gen_split<LEVEL>(pk + 32 + i * V::POLYT1, sk + V::SK_T0 + i * V::POLYT0, acc, r, ws.buf, lane);
@@ -487,13 +519,14 @@ __device__ void gen_task(const uint8_t *__restrict__ seed, uint8_t *pk, uint8_t 
 // Alg 2: Sign
 // -------------------------------------------------------------------------
 
-// Copies polynomials [lo, hi) of src (a caller's A^, 256 words each) to dst
-// with 16-byte loads and stores.
+// Copies polynomials [lo, hi) of src (a caller's A^ in index order, 256 words
+// each) to dst in lane order, 16 bytes at a time.
 __device__ __forceinline__ void copy_polys(const int32_t *__restrict__ src, int lo, int hi, int32_t *dst, int lane) {
     const int4 *q = reinterpret_cast<const int4 *>(src + lo * N);
     int4 *d = reinterpret_cast<int4 *>(dst + lo * N);
 #pragma unroll 2
-    for (int i = lane; i < (hi - lo) * (N / 4); i += 32) d[i] = __ldg(q + i);
+    for (int i = lane; i < (hi - lo) * (N / 4); i += 32)   // unit u of a polynomial: lane u / 2, half u mod 2
+        d[(i & ~63) + ((i & 1) << 5) + ((i & 63) >> 1)] = __ldg(q + i);
 }
 
 // Precomputation shared by every repetition: mu, rho', A^, s^1, s^2, t^0.
@@ -786,7 +819,7 @@ __device__ void sign_pack(uint8_t *sig, const int32_t *itr, const GroupSmem &gs,
 #pragma unroll 1
     for (int j = g; j < V::L; j += P) {
         int32_t v[8];
-        load_l2(v, itr + (S::Z + j) * N, lane);   // 8 consecutive coefficients
+        load_seq(v, itr + (S::Z + j) * N, lane);   // 8 consecutive coefficients
         pack_seq<V::ZBITS>(sig + V::SIG_Z + j * V::POLYZ, v, V::GAMMA1, -1, lane);
     }
     if (g != P - 1) return;
@@ -817,14 +850,9 @@ __device__ void sign_zero(uint8_t *sig, int g, int lane) {
 // -------------------------------------------------------------------------
 // KEYED: the public key is resident; `key` holds its A^ and NTT(t1 2^d)
 // (KEY_POLYS layout) and `tr` its H(pk), so neither is recomputed.
-// AHAT: `key` is the caller's A^ of this key (k l polynomials, ExpandA(rho));
-// t1 and H(pk) come from pk as in the plain form.
 // mu_in (nullable, KEYED only, global memory, 8-byte aligned): mu computed
 // beforehand.
-// SPLIT: the task's hashes run elsewhere (dil_verify.cu): nothing of msg or tr
-// is read, the packed w1' goes to the start of scratch instead of into
-// c~ = H(mu || w1'), and 1 means that only that comparison is left.
-template <int LEVEL, int P, bool KEYED = false, bool AHAT = false, bool SPLIT = false>
+template <int LEVEL, int P, bool KEYED = false>
 __device__ int verify_task(const uint8_t *__restrict__ pk, const uint8_t *__restrict__ msg, size_t mlen,
                            const uint8_t *__restrict__ sig, int32_t *scratch, GroupSmem &gs, WarpSmem &ws,
                            const int32_t *zt, const int32_t *izt, int g, int bar, int lane,
@@ -881,10 +909,10 @@ __device__ int verify_task(const uint8_t *__restrict__ pk, const uint8_t *__rest
     }
     // A^ = ExpandA(rho) into scratch after z^ (unless resident)
     constexpr int KL = V::K * V::L;
-    if constexpr (!KEYED && !AHAT)
+    if constexpr (!KEYED)
         expand_a_range<LEVEL>(gs.rho, share_lo<KL, P>(g), share_lo<KL, P>(g + 1), scratch + V::L * N, ws, lane);
     // mu = H(H(rho || t1) || M), on the last warp
-    if (!SPLIT && g == P - 1) {
+    if (g == P - 1) {
         uint32_t lo = 0, hi = 0;
         if (KEYED) {
             gs.tr[lane] = __ldcg(tr + lane);
@@ -909,7 +937,7 @@ __device__ int verify_task(const uint8_t *__restrict__ pk, const uint8_t *__rest
     challenge_hat<LEVEL>(ch, gs.ctilde, ws, zt, lane);
     // v = INTT(A^ o z^ - c^ o NTT(t1 2^d)); w1' = UseHint(h, v)
     using S = Scratch<LEVEL>;
-    const int32_t *ahat = KEYED ? key + S::AH * N : AHAT ? key : scratch + V::L * N;
+    const int32_t *ahat = KEYED ? key + S::AH * N : scratch + V::L * N;
 #pragma unroll 1
     for (int i = g; i < V::K; i += P) {
         accumulate_row(acc, ahat + i * V::L * N, V::L, scratch, lane);
@@ -933,11 +961,6 @@ __device__ int verify_task(const uint8_t *__restrict__ pk, const uint8_t *__rest
         pack_seq<V::W1BITS>(gs.hb + HB_W1 + i * V::POLYW1, r, 0, 1, lane);
     }
     group_sync<P>(bar);
-    if constexpr (SPLIT) {   // every row has read z^ by now
-        const uint32_t *w1 = reinterpret_cast<const uint32_t *>(gs.hb + HB_W1);
-        for (int i = 32 * g + lane; i < V::K * V::POLYW1 / 4; i += 32 * P) scratch[i] = (int32_t)w1[i];
-        return 1;
-    }
     // c~ == H(mu || w1')
     if (g == 0) {
         uint32_t lo = 0, hi = 0;

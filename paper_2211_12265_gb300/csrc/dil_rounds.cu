@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(32, 16) k_sign_prepare(const SignBatch b) {
     if constexpr (SRC != SIGN_KEYED) {
         blk -= b.hash_warps;
         if (blk < b.expand_blocks) {
-            expand_a_batch<LEVEL>(
+            expand_a_batch<LEVEL, false>(
                 (long long)blk * K16_STATES, (long long)b.n * KL, [&](int t) { return b.sk + (size_t)t * V::SK; },
                 [&](int t) { return b.pre + (size_t)t * Scratch<LEVEL>::PRE_POLYS * N; }, sm, lane);
             return;
@@ -435,7 +435,7 @@ __device__ __forceinline__ void sign_emit(uint8_t *sig, const int32_t *slot, int
 #pragma unroll 1
     for (int j = 0; j < V::L; ++j) {
         int32_t v[8];
-        load_l2_cg(v, slot + (SL::Y + j) * N, lane);   // 8 consecutive coefficients
+        load_seq_cg(v, slot + (SL::Y + j) * N, lane);   // 8 consecutive coefficients
         pack_poly<V::ZBITS>(sig + V::SIG_Z + j * V::POLYZ, v, V::GAMMA1, -1, buf, lane);
     }
     const uint8_t *x = reinterpret_cast<const uint8_t *>(slot + SL::X * N);

@@ -28,6 +28,10 @@ __device__ __forceinline__ uint32_t get_field(const uint8_t *buf, int pos, int b
     return v & ((1u << bits) - 1u);
 }
 
+// Word of index c of an NTT-domain polynomial in lane order (load_l2 of
+// dil_procs.cuh): lane c / 8's first or second half.
+__device__ __forceinline__ int lane_order(int c) { return ((c & 4) << 5) + ((c >> 3) << 2) + (c & 3); }
+
 // ---------------------------------------------------------------- ExpandA
 // A^_ij from SHAKE128(rho || j || i).  Candidates are 3-byte little-endian
 // words with the top bit cleared, kept when < q, in stream order; coefficient
@@ -90,8 +94,9 @@ __device__ __forceinline__ void expand_a_pair(const uint8_t *rho, int i0, int j0
 // Six-instance ExpandA: polynomials p0 .. p0 + count - 1 (count <= 6) of A^
 // (p = i l + j), rejection-sampled with the same warp vote straight from the
 // states' squeezed blocks into global memory, coefficient c of polynomial p at
-// out[(p - p0) 256 + c] (index order).  rho: 32 bytes of shared memory.
-template <int L>
+// out[(p - p0) 256 + c] (INDEX: index order) or where lane order puts it.  rho:
+// 32 bytes of shared memory.
+template <int L, bool INDEX>
 __device__ __forceinline__ void expand_a_six(const uint8_t *rho, int p0, int count, int32_t *out, uint32_t *kst,
                                              uint32_t *kpi, int lane) {
     keccak6_seed(
@@ -116,7 +121,7 @@ __device__ __forceinline__ void expand_a_six(const uint8_t *rho, int p0, int cou
                 const bool acc = valid && v < (uint32_t)Q;
                 const uint32_t mask = __ballot_sync(FULL, acc);
                 const int pos = c + __popc(mask & lanemask_lt(lane));
-                if (acc && pos < N) dst[pos] = (int32_t)v;
+                if (acc && pos < N) dst[INDEX ? pos : lane_order(pos)] = (int32_t)v;
                 c += __popc(mask);
             }
             if (lane == g) mine = c;
@@ -130,7 +135,7 @@ __device__ __forceinline__ void expand_a_six(const uint8_t *rho, int p0, int cou
 // written like expand_a_six.  The candidates of two instances
 // are voted on at once, one per half-warp (4 x 16 candidate slots for a
 // block's 56).
-template <int L>
+template <int L, bool INDEX>
 __device__ __forceinline__ void expand_a_16(const uint8_t *rho, int p0, int count, int32_t *out, uint32_t *kst,
                                             int lane) {
     keccak16_seed(
@@ -159,7 +164,7 @@ __device__ __forceinline__ void expand_a_16(const uint8_t *rho, int p0, int coun
                 const bool acc = live && k < 56 && v < (uint32_t)Q;
                 const uint32_t m = __ballot_sync(FULL, acc) >> (16 * half) & 0xFFFFu;
                 const int at = c + __popc(m & below);
-                if (acc && at < N) dst[at] = (int32_t)v;
+                if (acc && at < N) dst[INDEX ? at : lane_order(at)] = (int32_t)v;
                 c += __popc(m);
             }
             const int c_new = __shfl_sync(FULL, c, (lane & 1) << 4);

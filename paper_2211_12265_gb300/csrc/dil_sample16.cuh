@@ -15,7 +15,8 @@ constexpr int EXPAND16_WORDS = K16_STATES * EXPAND16_STRIDE + 8;
 
 // ExpandA over a batch: polynomials [first, first + 16) of the `total` = tasks
 // k l polynomials, numbered task by task, one warp.  seed_of(t): the 32 bytes
-// of task t's rho (global memory, any alignment); out_of(t): task t's A^.
+// of task t's rho (global memory, any alignment); out_of(t): task t's A^, in
+// index order with INDEX, else in lane order.
 // The states stay in registers over the five permutations; the blocks of all
 // go to shared memory, and a lane then takes candidates lane + 32 m of one
 // stream: 24 bits times 32 are whole words, so its shift is fixed and its
@@ -23,7 +24,7 @@ constexpr int EXPAND16_WORDS = K16_STATES * EXPAND16_STRIDE + 8;
 // time, took a quarter of ExpandA's time.)  A stream of 280 candidates leaves
 // fewer than 256 with probability below 1e-30; such a polynomial is sampled
 // again by the form that squeezes until it has enough.
-template <int LEVEL, class Seed, class Out>
+template <int LEVEL, bool INDEX, class Seed, class Out>
 __device__ __forceinline__ void expand_a_batch(long long first, long long total, Seed seed_of, Out out_of,
                                                uint32_t *st, int lane) {
     using V = Lv<LEVEL>;
@@ -61,7 +62,7 @@ __device__ __forceinline__ void expand_a_batch(long long first, long long total,
             const bool acc = v < (uint32_t)Q && (m < 8 || lane < 24);   // 280 candidates
             const uint32_t mask = __ballot_sync(FULL, acc);
             const int to = c + __popc(mask & lanemask_lt(lane));
-            if (acc && to < N) dst[to] = (int32_t)v;
+            if (acc && to < N) dst[INDEX ? to : lane_order(to)] = (int32_t)v;
             c += __popc(mask);
         }
         few |= (uint32_t)(c < N) << u;
@@ -77,7 +78,8 @@ __device__ __forceinline__ void expand_a_batch(long long first, long long total,
         seed[lane] = seed_of(t)[lane];
         __syncwarp();
         expand_a_poly(seed, q / V::L, q % V::L, buf, sq, lane);
-        for (int m = 0; m < 8; ++m) out_of(t)[q * N + 8 * lane + m] = buf[9 * lane + m];
+        for (int m = 0; m < 8; ++m)
+            out_of(t)[q * N + (INDEX ? 8 * lane + m : lane_order(8 * lane + m))] = buf[9 * lane + m];
         __syncwarp();
     }
 }

@@ -1,17 +1,15 @@
 // Verify of a batch (Alg 3).
 //
-// Batch form.  The first kernel gives its leading blocks to the hashes
-// tr = H(pk) and mu = H(tr || M) and to SampleInBall(c~), sixteen tasks to a
-// warp, and the others to sampling A^, sixteen polynomials to a warp whatever tasks they belong to
-// (dil_sample16.cuh).  The second does the arithmetic up to the packed w1', one
-// task per warp; with a resident key's or the caller's A^ it is the other blocks
-// of the first, one task per group of P warps.  The last recomputes c~ = H(mu || w1'),
-// sixteen tasks to a warp, and compares.  Hashing inside
-// the task's own warp (k_verify, kept for the launch shapes a caller asks for)
-// runs the 18 blocks of a Dilithium2 task at 18.7 SM clocks per round, 8.1 k
-// of the task's 20.7 k clocks; sixteen to a warp they take 1.4 k.  10,000 tasks,
-// fused -> batch: Dilithium2 655 -> 462 us, Dilithium5 (32 B - 4 KB)
-// 1813 -> 1351 us; 13 Dilithium3 tasks 162 -> 138 us.
+// Batch form.  One kernel hashes tr = H(pk) and mu = H(tr || M), sixteen tasks
+// to a warp.  Beside it, on a stream of their own where the caller has one to
+// spare, run SampleInBall(c~), sixteen tasks to a warp, with ExpandA, sixteen
+// polynomials to a warp whatever tasks they belong to (dil_sample16.cuh; not
+// with a resident key's or the caller's A^), and then the arithmetic up to the
+// packed w1', one task per warp.  The last kernel recomputes c~ = H(mu || w1'),
+// sixteen tasks to a warp, and compares.  Hashing inside the task's own warp
+// (k_verify, kept for the launch shapes a caller asks for) runs the 18 blocks of
+// a Dilithium2 task at 18.7 SM clocks per round, 8.1 k of the task's 20.7 k
+// clocks; sixteen to a warp they take 1.4 k.
 #include "dil_kern.cuh"
 #include "dil_sample16.cuh"
 
@@ -47,10 +45,10 @@ cudaError_t launch_verify(int level, int n, const uint8_t *pk, const uint8_t *ms
 
 // ---------------------------------------------------------------- batch form
 
-// Scratch polynomials of one task of the batch form.
+// Scratch polynomials of one task of the batch form: the packed w1', then A^.
 template <int LEVEL, int SRC>
 __host__ __device__ constexpr int verify_polys() {
-    return SRC == VERIFY_PLAIN ? Scratch<LEVEL>::VERIFY_POLYS : Scratch<LEVEL>::KEYED_VERIFY_POLYS;
+    return SRC == VERIFY_PLAIN ? 1 + Lv<LEVEL>::K * Lv<LEVEL>::L : 1;
 }
 
 // Task t's message (and resident key); false when the task is to be rejected.
@@ -63,8 +61,6 @@ __device__ __forceinline__ bool verify_input(const VerifyBatch &b, int t, int &k
     }
     return message_of(b.off, t, m0, mlen);
 }
-
-static_assert(HASH16_STAGE_WORDS * sizeof(uint32_t) <= sizeof(WarpSmem), "the hashing warps' shared memory");
 
 // tr = H(pk) (not for resident keys) and mu = H(tr || M) of a pair's tasks:
 // the first by the pair's index, the next ones from the batch's counter.
@@ -121,47 +117,14 @@ struct VerifyMuJob {
     }
 };
 
-// One hashing warp of the batch (w < hash_warps).
+// The hashing warps, each a CTA of its own: they are chains (a 16 KB message is
+// 121 blocks, 3.4 us each on a warp of its own), so they get the registers to
+// keep a state and its input (at 64, a block took 4.5 us) and start first.
 template <int LEVEL, int SRC>
-__device__ __forceinline__ void verify_hashes(const VerifyBatch &b, int w, uint32_t *stage, int lane) {
-    VerifyMuJob<LEVEL, SRC> job(b, w * K16_STATES + (lane >> 1), lane);
-    hash16_run(job, stage, lane);
-}
-
-// The arithmetic of the tasks of CTA `blk`.
-template <int LEVEL, int P, int SRC>
-__device__ __forceinline__ void verify_tasks(const VerifyBatch &b, int blk, uint8_t *smem) {
-    using V = Lv<LEVEL>;
-    const CtaView v = cta_setup<P>(smem);
-    const int task = blk * v.groups + v.group;
-    if (task >= b.n) return;
-    int key;
-    uint64_t m0;
-    size_t mlen;
-    int r = 0;
-    if (verify_input<SRC>(b, task, key, m0, mlen)) {
-        int32_t *scr = b.scratch + (size_t)task * verify_polys<LEVEL, SRC>() * N;
-        const int32_t *a = SRC == VERIFY_AHAT ? b.ahat + (size_t)task * V::K * V::L * N
-                                              : b.keys + (size_t)key * Scratch<LEVEL>::KEY_POLYS * N;
-        r = verify_task<LEVEL, P, SRC == VERIFY_KEYED, SRC == VERIFY_AHAT, true>(
-            b.pk + (size_t)key * V::PK, nullptr, 0, b.sig + (size_t)task * V::SIG, scr, *v.gs, *v.ws, v.zt, v.izt,
-            v.g, v.bar, v.lane, a);
-    }
-    if (v.g == 0 && v.lane == 0) b.ok[task] = (uint8_t)r;   // 1: c~ decides (k_verify_compare)
-}
-
-// VERIFY_AHAT, VERIFY_KEYED: hashes and arithmetic.
-template <int LEVEL, int P, int SRC>
-__global__ void __launch_bounds__(256, 4) k_verify_batch(const VerifyBatch b) {
-    extern __shared__ __align__(16) uint8_t smem[];
-    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if ((int)blockIdx.x < b.hash_blocks) {
-        const int w = blockIdx.x * warps + warp;
-        if (w < b.hash_warps)
-            verify_hashes<LEVEL, SRC>(b, w, reinterpret_cast<uint32_t *>(smem) + warp * HASH16_STAGE_WORDS, lane);
-        return;
-    }
-    verify_tasks<LEVEL, P, SRC>(b, blockIdx.x - b.hash_blocks, smem);
+__global__ void __launch_bounds__(32, 16) k_verify_hash(const VerifyBatch b) {
+    __shared__ __align__(16) uint32_t stage[HASH16_STAGE_WORDS];
+    VerifyMuJob<LEVEL, SRC> job(b, blockIdx.x * K16_STATES + (threadIdx.x >> 1), threadIdx.x);
+    hash16_run(job, stage, threadIdx.x);
 }
 
 // c = SampleInBall(c~) of the signatures of tasks [first, first + 16), one warp.
@@ -179,38 +142,32 @@ __device__ __forceinline__ void verify_challenges(const VerifyBatch &b, int firs
         put_challenge(b.challenge + (size_t)(first + u) * 256, stage, u, lane);
 }
 
-// VERIFY_PLAIN: blocks [0, hash_warps) hash tr and mu, [.., + challenge_blocks)
-// draw challenges, the others sample A^; the arithmetic follows.  One warp per
-// CTA, as in Sign's prepare kernel.
+// Blocks [0, challenge_blocks) draw challenges, the others (VERIFY_PLAIN only)
+// sample A^.  One warp per CTA, as in Sign's prepare kernel.
 template <int LEVEL>
-__global__ void __launch_bounds__(32, 16) k_verify_prepare(const VerifyBatch b) {
-    extern __shared__ __align__(16) uint32_t sm[];
+__global__ void __launch_bounds__(32, 16) k_verify_sample(const VerifyBatch b) {
+    __shared__ __align__(16) uint32_t sm[EXPAND16_WORDS];
+    static_assert(CHALLENGE_WORDS <= EXPAND16_WORDS, "the challenge blocks' shared memory");
     using V = Lv<LEVEL>;
-    const int lane = threadIdx.x;
-    int blk = blockIdx.x;
-    if (blk < b.hash_warps) {
-        verify_hashes<LEVEL, VERIFY_PLAIN>(b, blk, sm, lane);
-        return;
-    }
-    blk -= b.hash_warps;
+    const int lane = threadIdx.x, blk = blockIdx.x;
     if (blk < b.challenge_blocks) {
         verify_challenges<LEVEL>(b, blk * K16_STATES, sm, lane);
         return;
     }
-    blk -= b.challenge_blocks;
-    expand_a_batch<LEVEL>(
-        (long long)blk * K16_STATES, (long long)b.n * V::K * V::L, [&](int t) { return b.pk + (size_t)t * V::PK; },
-        [&](int t) { return b.scratch + ((size_t)t * verify_polys<LEVEL, VERIFY_PLAIN>() + V::L) * N; }, sm, lane);
+    expand_a_batch<LEVEL, false>(
+        (long long)(blk - b.challenge_blocks) * K16_STATES, (long long)b.n * V::K * V::L,
+        [&](int t) { return b.pk + (size_t)t * V::PK; },
+        [&](int t) { return b.scratch + ((size_t)t * verify_polys<LEVEL, VERIFY_PLAIN>() + 1) * N; }, sm, lane);
 }
 
 // The arithmetic of one task, one warp: hint decoding, z^, and per row
 // w1' = UseHint(h, INTT(A^ z^ - c^ NTT(t1 2^d))), packed to the start of its
 // scratch.  False when the signature is malformed or z too large.
-template <int LEVEL>
-__device__ __forceinline__ bool verify_rows(const VerifyBatch &b, int task, int32_t *buf, int32_t *zh, uint32_t *hmask,
-                                            int lane) {
+template <int LEVEL, int SRC>
+__device__ __forceinline__ bool verify_rows(const VerifyBatch &b, int task, int key, int32_t *buf, int32_t *zh,
+                                            uint32_t *hmask, int lane) {
     using V = Lv<LEVEL>;
-    const uint8_t *sig = b.sig + (size_t)task * V::SIG, *pk = b.pk + (size_t)task * V::PK;
+    const uint8_t *sig = b.sig + (size_t)task * V::SIG, *pk = b.pk + (size_t)key * V::PK;
     uint8_t *sq = reinterpret_cast<uint8_t *>(buf);
     int32_t v[8], ch[8];
     // strict hint decoding into bit masks
@@ -252,16 +209,27 @@ __device__ __forceinline__ bool verify_rows(const VerifyBatch &b, int task, int3
 #pragma unroll
     for (int m = 0; m < 8; ++m) ch[m] = c[lane + 32 * m];
     ntt_fwd_global(ch, buf);
-    int32_t *scr = b.scratch + (size_t)task * verify_polys<LEVEL, VERIFY_PLAIN>() * N;
+    int32_t *scr = b.scratch + (size_t)task * verify_polys<LEVEL, SRC>() * N;
+    const int32_t *keyp = SRC == VERIFY_KEYED ? b.keys + (size_t)key * Scratch<LEVEL>::KEY_POLYS * N : nullptr;
+    const int32_t *ah = SRC == VERIFY_KEYED  ? keyp + Scratch<LEVEL>::AH * N
+                        : SRC == VERIFY_AHAT ? b.ahat + (size_t)task * V::K * V::L * N
+                                             : scr + N;
 #pragma unroll 1
     for (int i = 0; i < V::K; ++i) {
         int32_t a[V::L][8];   // every load of the row in flight during t1's transform
 #pragma unroll
-        for (int j = 0; j < V::L; ++j) load_l2(a[j], scr + (V::L + i * V::L + j) * N, lane);
-        unpack_buf_l0<10>(v, pk + 32 + i * V::POLYT1, 0, buf, lane);
+        for (int j = 0; j < V::L; ++j) {
+            if (SRC == VERIFY_AHAT) load_seq(a[j], ah + (i * V::L + j) * N, lane);
+            else load_l2(a[j], ah + (i * V::L + j) * N, lane);
+        }
+        if (SRC == VERIFY_KEYED) {
+            load_l2(v, keyp + (Scratch<LEVEL>::T1H + i) * N, lane);
+        } else {
+            unpack_buf_l0<10>(v, pk + 32 + i * V::POLYT1, 0, buf, lane);
 #pragma unroll
-        for (int m = 0; m < 8; ++m) v[m] = (-v[m]) << D;   // t1 2^d, t1 unpacked as 0 - field
-        ntt_fwd_global(v, buf);
+            for (int m = 0; m < 8; ++m) v[m] = (-v[m]) << D;   // t1 2^d, t1 unpacked as 0 - field
+            ntt_fwd_global(v, buf);
+        }
         // summed in 64 bits, |sum| < 7 q 9.1q + 9.1q 9.1q < 2^31 q
         long long acc[8];
 #pragma unroll
@@ -286,7 +254,7 @@ __device__ __forceinline__ bool verify_rows(const VerifyBatch &b, int task, int3
     return true;
 }
 
-template <int LEVEL>
+template <int LEVEL, int SRC>
 __global__ void __launch_bounds__(32, LEVEL == 2 ? 24 : 20) k_verify_rows(const VerifyBatch b) {
     __shared__ __align__(16) int32_t buf[288], zh[Lv<LEVEL>::L * N];
     __shared__ uint32_t hmask[64];
@@ -294,8 +262,8 @@ __global__ void __launch_bounds__(32, LEVEL == 2 ? 24 : 20) k_verify_rows(const 
     int key;
     uint64_t m0;
     size_t mlen;
-    const bool r = verify_input<VERIFY_PLAIN>(b, task, key, m0, mlen) &&
-                   verify_rows<LEVEL>(b, task, buf, zh, hmask, lane);
+    const bool r = verify_input<SRC>(b, task, key, m0, mlen) &&
+                   verify_rows<LEVEL, SRC>(b, task, key, buf, zh, hmask, lane);
     if (lane == 0) b.ok[task] = r;   // 1: c~ decides (k_verify_compare)
 }
 
@@ -340,67 +308,62 @@ __global__ void __launch_bounds__(128) k_verify_compare(const VerifyBatch b) {
 
 namespace {
 
-template <int LEVEL, int P, int SRC>
-cudaError_t launch_batch(VerifyBatch b, int warps, cudaStream_t s) {
+template <int LEVEL, int SRC>
+cudaError_t launch_batch(VerifyBatch b, const VerifyFork &f, cudaStream_t s) {
     b.hash_warps = batch_hash_warps(b.n);
+    b.challenge_blocks = (b.n + K16_STATES - 1) / K16_STATES;
+    const cudaStream_t hs = f.stream ? f.stream : s;
     cudaError_t e = cudaSuccess;
-    if (b.n > b.hash_warps * K16_STATES) e = cudaMemsetAsync(b.next, 0, sizeof(int), s);
-    if (e != cudaSuccess) return e;
-    if constexpr (SRC == VERIFY_PLAIN) {
-        b.challenge_blocks = (b.n + K16_STATES - 1) / K16_STATES;
-        const long long polys = (long long)b.n * Lv<LEVEL>::K * Lv<LEVEL>::L;
-        const int expand_blocks = (int)((polys + K16_STATES - 1) / K16_STATES);
-        const int bytes = EXPAND16_WORDS * (int)sizeof(uint32_t);
-        static_assert(CHALLENGE_WORDS <= EXPAND16_WORDS, "the hashing blocks' shared memory");
-        e = cudaFuncSetAttribute(k_verify_prepare<LEVEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e != cudaSuccess) return e;
-        k_verify_prepare<LEVEL><<<b.hash_warps + b.challenge_blocks + expand_blocks, 32, bytes, s>>>(b);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_verify_rows<LEVEL><<<b.n, 32, 0, s>>>(b);
-    } else {
-        const int blocks = (b.n + warps / P - 1) / (warps / P);
-        const size_t smem = cta_bytes(warps, P);
-        b.hash_blocks = (b.hash_warps + warps - 1) / warps;
-        e = cudaFuncSetAttribute(k_verify_batch<LEVEL, P, SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_verify_batch<LEVEL, P, SRC><<<b.hash_blocks + blocks, warps * 32, smem, s>>>(b);
-    }
+    if (f.stream && ((e = cudaEventRecord(f.fork, s)) != cudaSuccess ||
+                     (e = cudaStreamWaitEvent(hs, f.fork, 0)) != cudaSuccess))
+        return e;
+    if (b.n > b.hash_warps * K16_STATES && (e = cudaMemsetAsync(b.next, 0, sizeof(int), hs)) != cudaSuccess) return e;
+    k_verify_hash<LEVEL, SRC><<<b.hash_warps, 32, 0, hs>>>(b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const long long polys = SRC == VERIFY_PLAIN ? (long long)b.n * Lv<LEVEL>::K * Lv<LEVEL>::L : 0;
+    k_verify_sample<LEVEL><<<b.challenge_blocks + (int)((polys + K16_STATES - 1) / K16_STATES), 32, 0, s>>>(b);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) {
+        k_verify_rows<LEVEL, SRC><<<b.n, 32, 0, s>>>(b);
+        e = cudaGetLastError();
+    }
+    // the caller's stream waits for the hashes whatever went wrong on it
+    if (f.stream) {
+        const cudaError_t r = cudaEventRecord(f.join, hs), w = cudaStreamWaitEvent(s, f.join, 0);
+        if (e == cudaSuccess) e = r != cudaSuccess ? r : w;
+    }
+    if (e != cudaSuccess) return e;
     const HashGrid h = hash_grid(b.n);
     k_verify_compare<LEVEL, SRC><<<h.blocks, h.threads, 0, s>>>(b);
     return cudaGetLastError();
 }
 
-template <int LEVEL, int SRC>
-cudaError_t launch_batch_p(const VerifyBatch &b, int warps, int p, cudaStream_t s) {
-    if constexpr (SRC == VERIFY_PLAIN) return launch_batch<LEVEL, 1, SRC>(b, warps, s);
-    switch (p) {
-        case 1: return launch_batch<LEVEL, 1, SRC>(b, warps, s);
-        case 4: return launch_batch<LEVEL, 4, SRC>(b, warps, s);
-    }
-    return cudaErrorInvalidValue;
-}
-
 template <int LEVEL>
-cudaError_t launch_batch_src(int src, const VerifyBatch &b, int warps, int p, cudaStream_t s) {
+cudaError_t launch_batch_src(int src, const VerifyBatch &b, const VerifyFork &f, cudaStream_t s) {
     switch (src) {
-        case VERIFY_PLAIN: return launch_batch_p<LEVEL, VERIFY_PLAIN>(b, warps, p, s);
-        case VERIFY_AHAT: return launch_batch_p<LEVEL, VERIFY_AHAT>(b, warps, p, s);
-        case VERIFY_KEYED: return launch_batch_p<LEVEL, VERIFY_KEYED>(b, warps, p, s);
+        case VERIFY_PLAIN: return launch_batch<LEVEL, VERIFY_PLAIN>(b, f, s);
+        case VERIFY_AHAT: return launch_batch<LEVEL, VERIFY_AHAT>(b, f, s);
+        case VERIFY_KEYED: return launch_batch<LEVEL, VERIFY_KEYED>(b, f, s);
     }
     return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
-cudaError_t launch_verify_batch(int level, int src, const VerifyBatch &b, int warps, int p, cudaStream_t s) {
+cudaError_t launch_verify_batch(int level, int src, const VerifyBatch &b, const VerifyFork &f, cudaStream_t s) {
     if (b.n <= 0) return cudaSuccess;
     switch (level) {
-        case 2: return launch_batch_src<2>(src, b, warps, p, s);
-        case 3: return launch_batch_src<3>(src, b, warps, p, s);
-        case 5: return launch_batch_src<5>(src, b, warps, p, s);
+        case 2: return launch_batch_src<2>(src, b, f, s);
+        case 3: return launch_batch_src<3>(src, b, f, s);
+        case 5: return launch_batch_src<5>(src, b, f, s);
     }
     return cudaErrorInvalidValue;
+}
+
+size_t verify_batch_polys(int level, int src) {
+    const int all = level == 2 ? verify_polys<2, VERIFY_PLAIN>() : level == 3 ? verify_polys<3, VERIFY_PLAIN>()
+                                                                           : verify_polys<5, VERIFY_PLAIN>();
+    return src == VERIFY_PLAIN ? all : 1;
 }
 
 size_t cta_smem_bytes(int warps, int p) { return cta_bytes(warps, p); }
