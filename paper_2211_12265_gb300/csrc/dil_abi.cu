@@ -29,11 +29,13 @@ struct dil_ctx {
     void *pws = nullptr;
     size_t pws_bytes = 0;
     dil::PersistTuning ptune;
+    bool ptune_set = false;   // by dil_set_persistent_tuning
     cudaStream_t cap_stream = nullptr;
     cudaStream_t cancel_stream = nullptr;   // carries the cancel word's copy
     cudaGraphExec_t gexec = nullptr;
     dil::PersistJobs gjobs{};
     dil::PersistTuning gtune;
+    bool grounds = false;     // the captured launch runs in rounds
     int gmax_iter = -1;
     int spin_limit = 0;       // polls per bounded device wait (0 = PERSIST_SPIN_LIMIT); tests lower it
     int gspin_limit = -1;
@@ -100,6 +102,13 @@ size_t chunk_tasks(const dil_ctx *c, size_t per, size_t n) {
 }
 size_t chunk_tasks(const dil_ctx *c, int op, int level, size_t n) {
     return chunk_tasks(c, dil::scratch_polys(op, level) * POLY_BYTES, n);
+}
+
+// Tasks of a part when a batch runs in parts on ns streams, each with a part's
+// scratch; one stream when the budget does not hold ns tasks' scratch.
+size_t part_tasks(const dil_ctx *c, size_t n, size_t per, size_t &ns) {
+    if (c->budget < ns * per) ns = 1;
+    return std::min((n + ns - 1) / ns, chunk_tasks(c, ns * per, n));
 }
 
 // Launch shape of one call.  The fused forms run when the caller asked for two
@@ -233,13 +242,6 @@ int run_sign_batch(dil_ctx *c, int level, int src, size_t n, const dil::SignBatc
                        });
 }
 
-int sign_cap(const dil_ctx *c, int level) {
-    const int l = level == 2 ? 4 : level == 3 ? 5 : 7, cap = (65536 - l) / l + 1;
-    return (c->max_iter > 0 && c->max_iter < cap) ? c->max_iter : cap;
-}
-
-void sizes_of(int level, size_t &pk, size_t &sk, size_t &sig) { dil_sizes(level, &pk, &sk, &sig); }
-
 // Carves m tasks of a Verify batch out of a workspace of m verify_task_bytes.
 void carve_verify(dil::VerifyBatch &b, void *ws, size_t m, size_t polys) {
     uint8_t *aux = static_cast<uint8_t *>(ws) + m * polys * POLY_BYTES;
@@ -252,32 +254,37 @@ void carve_verify(dil::VerifyBatch &b, void *ws, size_t m, size_t polys) {
 }
 
 // Runs Verify's batch form over the n tasks of `all` (whose per-task pointers are
-// those of task 0), in as many launches as the budget asks for.
+// those of task 0), in as many launches as the budget asks for, with the hashes
+// on a stream of their own.  (Parts of a large batch on several streams gain
+// nothing: 10,000 Dilithium2 tasks take 442 us in one, 450 to 461 in two to four.)
 int run_verify_batch(dil_ctx *c, int level, int src, size_t n, const dil::VerifyBatch &all, cudaStream_t s) {
     const size_t polys = dil::verify_batch_polys(level, src), per = verify_task_bytes(level, src);
-    const size_t chunk = chunk_tasks(c, per, n);
-    if (chunk == 0) return DIL_ENOMEM;
-    int rc = ensure_ws(c, chunk * per);
-    if (!rc) rc = ensure_aux(c);
+    const size_t tasks = chunk_tasks(c, per, n);
+    const int rc = ensure_aux(c);
     if (rc) return rc;
     size_t pkb, skb, sigb;
-    sizes_of(level, pkb, skb, sigb);
+    dil_sizes(level, &pkb, &skb, &sigb);
     const size_t k = level == 2 ? 4 : level == 3 ? 6 : 8, l = level == 2 ? 4 : level == 3 ? 5 : 7;
-    for (size_t s0 = 0; s0 < n; s0 += chunk) {
-        const size_t m = std::min(chunk, n - s0);
+    return run_streams(c, n, tasks, tasks * per, 1, s, [&](size_t c0, size_t c1, cudaStream_t st, int32_t *scratch) -> int {
         dil::VerifyBatch b = all;
-        carve_verify(b, c->ws, m, polys);
-        if (src != dil::VERIFY_KEYED) b.pk += pkb * s0;
-        if (b.ahat) b.ahat += k * l * 256 * s0;
-        if (b.key_idx) b.key_idx += s0;
-        b.off += s0;
-        b.sig += sigb * s0;
-        b.ok += s0;
-        const cudaError_t e = dil::launch_verify_batch(level, src, b, {c->aux[0], c->ev_fork, c->ev_join}, s);
-        if (e != cudaSuccess) return cuda_fail(e);
-    }
-    return DIL_OK;
+        carve_verify(b, scratch, c1 - c0, polys);
+        if (src != dil::VERIFY_KEYED) b.pk += pkb * c0;
+        if (b.ahat) b.ahat += k * l * 256 * c0;
+        if (b.key_idx) b.key_idx += c0;
+        b.off += c0;
+        b.sig += sigb * c0;
+        b.ok += c0;
+        const cudaError_t e = dil::launch_verify_batch(level, src, b, {c->aux[0], c->ev_fork, c->ev_join}, st);
+        return e == cudaSuccess ? DIL_OK : cuda_fail(e);
+    });
 }
+
+int sign_cap(const dil_ctx *c, int level) {
+    const int l = level == 2 ? 4 : level == 3 ? 5 : 7, cap = (65536 - l) / l + 1;
+    return (c->max_iter > 0 && c->max_iter < cap) ? c->max_iter : cap;
+}
+
+void sizes_of(int level, size_t &pk, size_t &sk, size_t &sig) { dil_sizes(level, &pk, &sk, &sig); }
 
 }  // namespace
 
@@ -376,18 +383,15 @@ int dil_keygen(dil_ctx *c, int level, size_t n, const uint8_t *seeds, uint8_t *p
     size_t pkb, skb, sigb;
     sizes_of(level, pkb, skb, sigb);
     const size_t per = dil::scratch_polys(dil::OP_KEYGEN, level) * POLY_BYTES;
-    size_t chunk = chunk_tasks(c, per, n);
-    if (chunk == 0) return DIL_ENOMEM;
-    int rc = ensure_ws(c, chunk * per);
-    if (rc) return rc;
-    for (size_t s0 = 0; s0 < n; s0 += chunk) {
-        int m = (int)std::min(chunk, n - s0);
-        const Shape sh = shape_of(c, 0, level, per);
-        cudaError_t e = keygen_chunk(sh, level, m, seeds + 32 * s0, pk + pkb * s0, sk + skb * s0, (int32_t *)c->ws,
-                                     (cudaStream_t)stream);
-        if (e != cudaSuccess) return cuda_fail(e);
-    }
-    return DIL_OK;
+    const Shape sh = shape_of(c, 0, level, per);
+    size_t ns = sh.fused || n < PIPE_MIN_TASKS ? 1 : 2;   // 10,000 Dilithium2 keys: 476 us on one stream, 458 on two
+    const size_t tasks = part_tasks(c, n, per, ns);
+    return run_streams(c, n, tasks, tasks * per, ns, (cudaStream_t)stream,
+                       [&](size_t c0, size_t c1, cudaStream_t s, int32_t *scratch) -> int {
+                           const cudaError_t e = keygen_chunk(sh, level, (int)(c1 - c0), seeds + 32 * c0, pk + pkb * c0,
+                                                              sk + skb * c0, scratch, s);
+                           return e == cudaSuccess ? DIL_OK : cuda_fail(e);
+                       });
 }
 
 int dil_sign_ex(dil_ctx *c, int level, size_t n, const uint8_t *sk, const uint8_t *msg, const uint64_t *msg_off,
@@ -562,6 +566,7 @@ int dil_set_persistent_tuning(dil_ctx *c, int warps_per_cta, int warps_per_task,
     c->ptune.ctas_per_sm = ctas_per_sm;
     c->ptune.chunk = chunk;
     c->ptune.spec = speculation;
+    c->ptune_set = true;
     return DIL_OK;
 }
 
@@ -570,6 +575,68 @@ bool same_jobs(const dil::PersistJobs &a, const dil::PersistJobs &b) { return me
 bool same_tune(const dil::PersistTuning &a, const dil::PersistTuning &b) {
     return a.warps == b.warps && a.p == b.p && a.ctas_per_sm == b.ctas_per_sm && a.chunk == b.chunk &&
            a.spec == b.spec;
+}
+}  // namespace
+
+namespace {
+// A persistent launch in rounds: each job in parts, the parts dealt over the four
+// streams; a part's workspace serves one after the other.  At most PART_MOST
+// tasks a part: a cancel ends the parts that have not started at once.
+constexpr size_t PART_MOST = 16384;
+struct RoundPlan {
+    RoundSize size[dil::PERSIST_MAX_JOBS];
+    size_t region = 0, bytes = 0;   // a stream's workspace, the launch's (0: does not fit the budget)
+};
+
+RoundPlan round_plan(const dil_ctx *c, const dil::PersistJobs &J) {
+    RoundPlan p;
+    const size_t budget = c->budget > dil::PERSIST_HEADER_BYTES ? (c->budget - dil::PERSIST_HEADER_BYTES) / PIPE_STREAMS : 0;
+    for (int j = 0; j < J.njobs; ++j) {
+        const size_t n = J.job[j].n;
+        if (n == 0) continue;
+        const size_t part = n < PIPE_MIN_TASKS ? n : std::min((n + PIPE_STREAMS - 1) / PIPE_STREAMS, PART_MOST);
+        p.size[j] = round_size(J.job[j].level, dil::SIGN_PLAIN, part, budget, PIPE_STREAMS);
+        if (p.size[j].tasks == 0) return RoundPlan{};
+        p.region = std::max(p.region, dil::sign_batch_bytes(J.job[j].level, dil::SIGN_PLAIN, p.size[j].tasks,
+                                                            p.size[j].slots));
+    }
+    p.bytes = dil::PERSIST_HEADER_BYTES + PIPE_STREAMS * p.region;
+    return p;
+}
+
+// Enqueues the launch on s and the context's other streams.
+cudaError_t launch_rounds(dil_ctx *c, const dil::PersistJobs &J, const RoundPlan &p, cudaStream_t s) {
+    cudaStream_t st[PIPE_STREAMS] = {s, c->aux[0], c->aux[1], c->aux[2]};
+    cudaError_t e = cudaMemsetAsync(c->pws, 0, dil::PERSIST_HEADER_BYTES, s);
+    if (e == cudaSuccess) e = cudaEventRecord(c->ev_fork, s);
+    for (size_t k = 1; k < PIPE_STREAMS && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(st[k], c->ev_fork, 0);
+    size_t turn = 0;
+    for (int j = 0; j < J.njobs && e == cudaSuccess; ++j) {
+        const dil::PersistJob &x = J.job[j];
+        size_t pkb, skb, sigb;
+        dil_sizes(x.level, &pkb, &skb, &sigb);
+        for (size_t c0 = 0; c0 < (size_t)x.n && e == cudaSuccess; c0 += p.size[j].tasks, ++turn) {
+            dil::SignBatch b{};
+            b.n = (int)std::min(p.size[j].tasks, x.n - c0);
+            b.slots = (int)p.size[j].slots;
+            b.sk = x.sk + skb * c0;
+            b.msg = x.msg;
+            b.off = x.off + c0;
+            b.sig = x.sig + sigb * c0;
+            b.status = x.status ? x.status + c0 : nullptr;
+            b.iters = x.iters ? x.iters + c0 : nullptr;
+            b.max_iter = sign_cap(c, x.level);
+            b.cancel = dil::persist_cancel_word(c->pws);
+            const size_t k = turn % PIPE_STREAMS;
+            e = dil::launch_sign_batch(x.level, dil::SIGN_PLAIN, b,
+                                       static_cast<uint8_t *>(c->pws) + dil::PERSIST_HEADER_BYTES + k * p.region, st[k]);
+        }
+    }
+    for (size_t k = 1; k < PIPE_STREAMS; ++k) {
+        const cudaError_t r = cudaEventRecord(c->ev_join, st[k]), w = cudaStreamWaitEvent(s, c->ev_join, 0);
+        if (e == cudaSuccess) e = r != cudaSuccess ? r : w;
+    }
+    return e;
 }
 }  // namespace
 
@@ -600,8 +667,14 @@ int dil_sign_persistent(dil_ctx *c, int njobs, const dil_sign_job *jobs, void *s
     if (total == 0) return DIL_OK;
     std::lock_guard<std::mutex> lk(c->mu);
     DeviceGuard g(c->device);
-    {   // SMs per job in proportion to its work (a task's relative cost by level:
-        // persistent Sign rates 3.65 / 2.42 / 1.98 M/s at 10,000 tasks)
+    // One-warp launches run in rounds; shapes of two or four warps per task, a
+    // budget too small for a round, and the hook that makes bounded waits run out
+    // keep the device queue.
+    RoundPlan plan;
+    if (!(c->ptune_set && c->ptune.p > 1) && c->spin_limit == 0) plan = round_plan(c, J);
+    const bool rounds = plan.bytes != 0;
+    if (!rounds) {   // SMs per job in proportion to its work (a task's relative cost by level:
+                     // persistent Sign rates 3.65 / 2.42 / 1.98 M/s at 10,000 tasks)
         int sms = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) return DIL_ECUDA;
         double w[dil::PERSIST_MAX_JOBS], sum = 0;
@@ -616,9 +689,13 @@ int dil_sign_persistent(dil_ctx *c, int njobs, const dil_sign_job *jobs, void *s
             J.sm_end[j] = j + 1 == njobs ? (1 << 30) : (int)(sms * acc / sum + 0.5);
         }
     }
-    const size_t need = dil::persist_workspace_bytes(J, c->ptune, c->device);
+    const size_t need = rounds ? plan.bytes : dil::persist_workspace_bytes(J, c->ptune, c->device);
     if (need == 0) return DIL_ECUDA;
     if (need > c->budget) return DIL_ENOMEM;
+    if (rounds) {
+        const int rc = ensure_aux(c);
+        if (rc) return rc;
+    }
     if (need > c->pws_bytes) {
         if (c->pws) {
             cudaDeviceSynchronize();
@@ -634,7 +711,7 @@ int dil_sign_persistent(dil_ctx *c, int njobs, const dil_sign_job *jobs, void *s
     }
     const int max_iter = c->max_iter;
     if (!c->gexec || !same_jobs(J, c->gjobs) || !same_tune(c->ptune, c->gtune) || max_iter != c->gmax_iter ||
-        c->spin_limit != c->gspin_limit || c->gws != c->pws) {
+        c->spin_limit != c->gspin_limit || rounds != c->grounds || c->gws != c->pws) {
         if (c->gexec) {
             cudaGraphExecDestroy(c->gexec);
             c->gexec = nullptr;
@@ -642,11 +719,12 @@ int dil_sign_persistent(dil_ctx *c, int njobs, const dil_sign_job *jobs, void *s
         if (!c->cap_stream && cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
             return DIL_ECUDA;
         // warm the attribute / occupancy queries outside the capture
-        if (dil::persist_workspace_bytes(J, c->ptune, c->device) == 0) return DIL_ECUDA;
+        if (!rounds && dil::persist_workspace_bytes(J, c->ptune, c->device) == 0) return DIL_ECUDA;
         cudaGraph_t graph = nullptr;
         if (cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) return DIL_ECUDA;
-        cudaError_t e = dil::launch_sign_persist(J, c->pws, c->ptune, max_iter, c->spin_limit, c->device,
-                                                 c->cap_stream);
+        cudaError_t e = rounds ? launch_rounds(c, J, plan, c->cap_stream)
+                               : dil::launch_sign_persist(J, c->pws, c->ptune, max_iter, c->spin_limit, c->device,
+                                                          c->cap_stream);
         cudaError_t e2 = cudaStreamEndCapture(c->cap_stream, &graph);
         if (e != cudaSuccess || e2 != cudaSuccess) {
             if (graph) cudaGraphDestroy(graph);
@@ -663,6 +741,7 @@ int dil_sign_persistent(dil_ctx *c, int njobs, const dil_sign_job *jobs, void *s
         c->gtune = c->ptune;
         c->gmax_iter = max_iter;
         c->gspin_limit = c->spin_limit;
+        c->grounds = rounds;
         c->gws = c->pws;
     }
     return cudaGraphLaunch(c->gexec, (cudaStream_t)stream) == cudaSuccess ? DIL_OK : DIL_ECUDA;

@@ -184,6 +184,19 @@ __global__ void __launch_bounds__(128) k_keygen_tr(int n, const uint8_t *pk, uin
     hash16_run(job, stage[threadIdx.x >> 5], lane);
 }
 
+// The same for a small batch, a warp per key on the 25-lane form.
+template <int LEVEL>
+__global__ void __launch_bounds__(32) k_keygen_tr_wide(const uint8_t *pk, uint8_t *sk) {
+    __shared__ __align__(16) uint8_t none[8];
+    const int t = blockIdx.x, lane = threadIdx.x;
+    uint32_t lo = 0, hi = 0;
+    absorb_concat(lo, hi, none, 0, pk + (size_t)t * Lv<LEVEL>::PK, Lv<LEVEL>::PK, 136, lane);
+    if (lane >= 4) return;
+    uint8_t *tr = sk + (size_t)t * Lv<LEVEL>::SK + 64 + 8 * lane;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) tr[q] = (uint8_t)((q < 4 ? lo : hi) >> (8 * (q & 3)));
+}
+
 namespace {
 
 template <int LEVEL>
@@ -199,7 +212,10 @@ cudaError_t launch_batch(int n, const uint8_t *seeds, uint8_t *pk, uint8_t *sk, 
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_keygen_rows<LEVEL><<<n, 32, 0, s>>>(pk, sk, scratch);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_keygen_tr<LEVEL><<<h.blocks, h.threads, 0, s>>>(n, pk, sk);
+    if (n <= HASH_WIDE_MOST)
+        k_keygen_tr_wide<LEVEL><<<n, 32, 0, s>>>(pk, sk);
+    else
+        k_keygen_tr<LEVEL><<<h.blocks, h.threads, 0, s>>>(n, pk, sk);
     return cudaGetLastError();
 }
 

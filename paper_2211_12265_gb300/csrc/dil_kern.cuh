@@ -64,6 +64,12 @@ inline int batch_hash_warps(int n) {
     return all <= 608 ? all : (n + 31) / 32 > 608 ? (n + 31) / 32 : 608;
 }
 
+// Up to this many hashes a warp each, on the 25-lane form: while every warp has a
+// sub-partition to itself a block takes 2.7 us that way and 3.4 two threads to a
+// state (224 and 250 clocks a round; absorbing costs 150 and 1,000), and the
+// chain of a hash's blocks is what a small batch waits for.
+constexpr int HASH_WIDE_MOST = 608;
+
 // Launch shape of a kernel that only hashes, one task per pair of threads:
 // single-warp CTAs spread a small batch over the SMs, four-warp ones put one
 // warp on each of an SM's sub-partitions.

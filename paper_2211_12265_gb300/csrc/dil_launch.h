@@ -85,6 +85,7 @@ struct SignBatch {
     const int32_t *key_idx;
     int n_keys;
     int max_iter;
+    const int *cancel;       // nullable: tasks without an accepted repetition end once it is set
     int slots;               // attempts of a round, at least sign_batch_min_slots
     // set by the launch: the workspace and the prepare kernel's blocks
     int32_t *pre, *slot_polys;
@@ -195,6 +196,11 @@ struct PersistTuning {
     int chunk = 1;        // fresh tasks claimed per queue access
     int spec = 4;         // helper groups per unfinished task (0 = no speculation)
 };
+// Header bytes of a persistent launch's workspace (the queue, which a launch in
+// rounds shares for its error and cancel words), and the latter's address.
+constexpr size_t PERSIST_HEADER_BYTES = 256;
+static_assert(sizeof(PersistQueue) <= PERSIST_HEADER_BYTES, "queue header");
+inline const int *persist_cancel_word(const void *ws) { return &static_cast<const PersistQueue *>(ws)->cancel; }
 // Device bytes a persistent launch needs for `total` tasks of the given levels.
 size_t persist_workspace_bytes(const PersistJobs &J, const PersistTuning &t, int device);
 // Polls of a bounded device wait before it gives up (the default of a launch).

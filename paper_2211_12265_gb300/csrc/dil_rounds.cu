@@ -83,11 +83,20 @@ __device__ __forceinline__ const int32_t *pre_of(const SignBatch &b, int t) {
     return b.pre + (size_t)t * Scratch<LEVEL>::PRE_POLYS * N;
 }
 
+// A host cancel of the batch (seen through L2; any lane).
+__device__ __forceinline__ bool canceled(const SignBatch &b) { return b.cancel && __ldcg(b.cancel) != 0; }
+
+// Status and repetitions of a task without a signature.
+__device__ __forceinline__ void report(const SignBatch &b, int task, int status, int iters) {
+    if (b.status) b.status[task] = status;
+    if (b.iters) b.iters[task] = iters;
+}
+
 // ---------------------------------------------------------------- prepare
 // mu = H(tr || M) and rho' = H(K || mu) of a pair's tasks: the first by the
 // pair's index, the next ones from the batch's counter.  A task with an
-// unknown key or decreasing offsets is rejected here, every other one enters
-// round 0.
+// unknown key or decreasing offsets is rejected here (and one met after a cancel
+// ends), every other one enters round 0.
 template <int LEVEL, int SRC>
 struct SignMuJob {
     const SignBatch &b;
@@ -126,13 +135,11 @@ struct SignMuJob {
             }
             first = false;
             if (task >= b.n) return false;
-            if (input(key, m0, mlen)) break;
+            const bool valid = input(key, m0, mlen), stop = pair_bcast(canceled(b), lane);
+            if (valid && !stop) break;
             uint8_t *sig = b.sig + (size_t)task * V::SIG;
             for (int i = lane & 1; i < V::SIG; i += 2) sig[i] = 0;
-            if (!(lane & 1)) {
-                if (b.status) b.status[task] = DIL_EINVAL;
-                if (b.iters) b.iters[task] = 0;
-            }
+            if (!(lane & 1)) report(b, task, valid ? DIL_ECANCELED : DIL_EINVAL, 0);
         }
         in = {b.sk + (size_t)key * V::SK + 64, b.msg + m0, 32 + mlen, 32};
         return true;
@@ -350,7 +357,105 @@ __global__ void __launch_bounds__(32 * ROUND_WARPS, 4) k_sign_hash(const SignBat
         put_challenge(reinterpret_cast<uint8_t *>(slot_of<LEVEL>(b, first + u) + SL::X * N), stage, u, lane);
 }
 
+// The same for a small round, a warp per attempt on the 25-lane form.
+template <int LEVEL>
+__global__ void __launch_bounds__(32) k_sign_hash_wide(const SignBatch b, int r) {
+    using V = Lv<LEVEL>;
+    using SL = Slot<LEVEL>;
+    constexpr int W1 = V::K * V::POLYW1;
+    __shared__ __align__(16) uint32_t in[(64 + W1) / 4 + 2];
+    __shared__ __align__(16) int32_t buf[288];
+    __shared__ __align__(16) uint8_t sq[688], ct[32];
+    const Round q = round_of(b, r);
+    const int s = blockIdx.x, lane = threadIdx.x;
+    if (s >= q.p * q.m) return;
+    const int task = pending_list(b, r)[s / q.m];
+    uint32_t *x = reinterpret_cast<uint32_t *>(slot_of<LEVEL>(b, s) + SL::X * N);
+    if (lane < 16) in[lane] = b.mu[(size_t)task * 16 + lane];
+#pragma unroll
+    for (int i = 0; i < W1 / 128; ++i) in[16 + lane + 32 * i] = x[lane + 32 * i];
+    __syncwarp();
+    uint32_t lo = 0, hi = 0;
+    absorb_smem(lo, hi, reinterpret_cast<const uint8_t *>(in), 64 + W1, 136, lane);
+    squeeze_words(lo, hi, ct, 4, lane);
+    __syncwarp();
+    sample_in_ball<V::TAU>(ct, buf, sq, lane);
+    int32_t c[8];
+    read_buf_l0(c, buf, lane);
+    int8_t *out = reinterpret_cast<int8_t *>(x);
+#pragma unroll
+    for (int m = 0; m < 8; ++m) out[SL::XC + lane + 32 * m] = (int8_t)c[m];
+    if (lane < 8) x[SL::XCT / 4 + lane] = reinterpret_cast<const uint32_t *>(ct)[lane];
+}
+
 // ---------------------------------------------------------------- back
+// v_s = INTT(c^ o s^2) in v, w in d: d = w - v_s (kept for the hint); true when
+// r0 = LowBits(w - v_s) is too large.
+template <int LEVEL>
+__device__ __forceinline__ bool check_r0(const int32_t (&v)[8], int32_t (&d)[8]) {
+    using V = Lv<LEVEL>;
+    bool bad = false;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        int32_t e = d[m] - v[m];                 // (-q, 2q)
+        e += (e < 0) ? Q : 0;
+        e -= (e >= Q) ? Q : 0;
+        int32_t h1, l0;
+        decompose<LEVEL>(e, h1, l0);
+        bad |= iabs(l0) >= V::GAMMA2 - V::BETA;
+        d[m] = e;
+    }
+    return __any_sync(FULL, bad);
+}
+
+// INTT(c^ o s^1) in v, y in d: v = z; true when ||z|| >= gamma1 - beta.
+template <int LEVEL>
+__device__ __forceinline__ bool check_z(int32_t (&v)[8], const int32_t (&d)[8]) {
+    using V = Lv<LEVEL>;
+    bool bad = false;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        v[m] = centre_small(to_canonical(v[m]) + d[m]);
+        bad |= iabs(v[m]) >= V::GAMMA1 - V::BETA;
+    }
+    return __any_sync(FULL, bad);
+}
+
+// v_t = INTT(c^ o t^0) in v, w - v_s in d: h = MakeHint(-v_t, w - v_s + v_t) into
+// eight masks, its ones added to count; true when ||v_t|| >= gamma2.
+template <int LEVEL>
+__device__ __forceinline__ bool check_hint(const int32_t (&v)[8], const int32_t (&d)[8], uint32_t *hint, int &count,
+                                           int lane) {
+    using V = Lv<LEVEL>;
+    bool bad = false;
+    uint32_t hbits = 0;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        int32_t vt = to_canonical(v[m]);
+        bad |= iabs(to_centred(vt)) >= V::GAMMA2;
+        int32_t rr = d[m] + vt;
+        rr -= (rr >= Q) ? Q : 0;
+        int32_t z = vt ? Q - vt : 0;
+        hbits |= (uint32_t)make_hint<LEVEL>(z, rr) << m;
+    }
+    if (__any_sync(FULL, bad)) return true;
+    uint32_t mine = 0;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        const uint32_t x = __ballot_sync(FULL, (hbits >> m) & 1u);
+        if (lane == m) mine = x;
+        count += __popc(x);
+    }
+    if (lane < 8) hint[lane] = mine;
+    return false;
+}
+
+// The hint masks of a slot, eight words per polynomial.
+template <int LEVEL>
+__device__ __forceinline__ uint32_t *hint_of(int32_t *slot) {
+    return reinterpret_cast<uint32_t *>(slot + Slot<LEVEL>::X * N) + Slot<LEVEL>::XHINT / 4;
+}
+
 // The checks of the attempt in `slot` with challenge ch (L2 layout); z
 // replaces y, the hint masks go behind the challenge.  True when accepted.
 // One loop over the r0 polynomials (LowBits(w - c s2)), then z = y + c s1, then
@@ -365,7 +470,7 @@ __device__ __forceinline__ bool sign_checks(const int32_t *pre, int32_t *slot, c
     using SL = Slot<LEVEL>;
     constexpr int R0 = V::K, ZS = V::K + V::L, ALL = 2 * V::K + V::L;   // ends of the three parts
     static_assert(SL::W == SL::Y + V::L, "w behind y");
-    uint32_t *hint = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(slot + SL::X * N) + SL::XHINT);
+    uint32_t *hint = hint_of<LEVEL>(slot);
     int32_t v[8], a[8], d[8];
     int count = 0;
 #pragma unroll 1
@@ -376,51 +481,14 @@ __device__ __forceinline__ bool sign_checks(const int32_t *pre, int32_t *slot, c
 #pragma unroll
         for (int m = 0; m < 8; ++m) v[m] = mont_mul(ch[m], a[m]);
         ntt_inv(v, buf, izt, lane);
-        bool bad = false;
         if (u < R0) {
-            // v_s = INTT(c^ o s^2); r0 = LowBits(w - v_s); w - v_s is kept for the hint
-#pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                int32_t e = d[m] - v[m];                 // (-q, 2q)
-                e += (e < 0) ? Q : 0;
-                e -= (e >= Q) ? Q : 0;
-                int32_t h1, l0;
-                decompose<LEVEL>(e, h1, l0);
-                bad |= iabs(l0) >= V::GAMMA2 - V::BETA;
-                d[m] = e;
-            }
-            if (__any_sync(FULL, bad)) return false;
+            if (check_r0<LEVEL>(v, d)) return false;
             store_l0(data, d, lane);
         } else if (u < ZS) {
-            // z = y + INTT(c^ o s^1); reject if ||z|| >= gamma1 - beta
-#pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                v[m] = centre_small(to_canonical(v[m]) + d[m]);
-                bad |= iabs(v[m]) >= V::GAMMA1 - V::BETA;
-            }
-            if (__any_sync(FULL, bad)) return false;
+            if (check_z<LEVEL>(v, d)) return false;
             store_l0(data, v, lane);
-        } else {
-            // v_t = INTT(c^ o t^0); h = MakeHint(-v_t, w - v_s + v_t)
-            uint32_t hbits = 0;
-#pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                int32_t vt = to_canonical(v[m]);
-                bad |= iabs(to_centred(vt)) >= V::GAMMA2;
-                int32_t rr = d[m] + vt;
-                rr -= (rr >= Q) ? Q : 0;
-                int32_t z = vt ? Q - vt : 0;
-                hbits |= (uint32_t)make_hint<LEVEL>(z, rr) << m;
-            }
-            if (__any_sync(FULL, bad)) return false;
-            uint32_t mine = 0;
-#pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                const uint32_t x = __ballot_sync(FULL, (hbits >> m) & 1u);
-                if (lane == m) mine = x;
-                count += __popc(x);
-            }
-            if (lane < 8) hint[(u - ZS) * 8 + lane] = mine;
+        } else if (check_hint<LEVEL>(v, d, hint + (u - ZS) * 8, count, lane)) {
+            return false;
         }
     }
     return count <= V::OMEGA;
@@ -457,7 +525,7 @@ __device__ __forceinline__ void sign_emit(uint8_t *sig, const int32_t *slot, int
 }
 
 // Task `task` (i-th of round r) after the last of its attempts: its signature,
-// the cap, or the next round.
+// the cap, a cancel, or the next round.
 template <int LEVEL>
 __device__ __forceinline__ void settle(const SignBatch &b, const Round &q, int r, int i, int task, int best, int32_t *buf,
                                        int lane) {
@@ -465,21 +533,43 @@ __device__ __forceinline__ void settle(const SignBatch &b, const Round &q, int r
     uint8_t *sig = b.sig + (size_t)task * V::SIG;
     if (best != INT_MAX) {
         sign_emit<LEVEL>(sig, slot_of<LEVEL>(b, i * q.m + best - q.base), buf, lane);
-        if (lane == 0) {
-            if (b.status) b.status[task] = DIL_OK;
-            if (b.iters) b.iters[task] = best + 1;
-        }
-    } else if (q.base + q.m >= b.max_iter) {
+        if (lane == 0) report(b, task, DIL_OK, best + 1);
+        return;
+    }
+    const bool capped = q.base + q.m >= b.max_iter;
+    if (__shfl_sync(FULL, capped || canceled(b), 0)) {
         sign_zero<LEVEL, 1>(sig, 0, lane);
-        if (lane == 0) {
-            if (b.status) b.status[task] = DIL_EITER;
-            if (b.iters) b.iters[task] = b.max_iter;
-        }
+        if (lane == 0) report(b, task, capped ? DIL_EITER : DIL_ECANCELED, capped ? b.max_iter : 0);
     } else if (lane == 0) {
         b.done[task] = 0;
         int *list = b.pending + (size_t)((r + 1) & 1) * b.n;
         list[atomicAdd(b.count + r + 1, 1)] = task;
     }
+}
+
+// One warp per attempt, after its checks (what they wrote has been fenced: it is
+// read through L2): the last of the task's attempts settles the round.  What an
+// accepted one wrote is visible before its repetition, and that before its
+// arrival.
+template <int LEVEL>
+__device__ __forceinline__ void arrive(const SignBatch &b, const Round &q, int r, int i, int task, int rep,
+                                       bool accepted, int32_t *buf, int lane) {
+    int best = accepted ? rep : INT_MAX;
+    if (q.m > 1) {
+        int arrived = 0;
+        if (lane == 0) {
+            if (accepted) {
+                atomicMin(&b.best[task], rep);
+                __threadfence();
+            }
+            arrived = atomicAdd(&b.done[task], 1);
+        }
+        if (__shfl_sync(FULL, arrived, 0) != q.m - 1) return;
+        __threadfence();
+        if (lane == 0) best = atomicOr(&b.best[task], 0);
+        best = __shfl_sync(FULL, best, 0);
+    }
+    settle<LEVEL>(b, q, r, i, task, best, buf, lane);
 }
 
 template <int LEVEL, int SRC>
@@ -507,26 +597,73 @@ __global__ void __launch_bounds__(32 * ROUND_WARPS, 8) k_sign_back(const SignBat
         ntt_fwd(ch, buf, zt, lane);
         accepted = sign_checks<LEVEL>(pre_of<LEVEL, SRC>(b, task), slot, ch, buf, izt, lane);
     }
-    if (accepted) __threadfence();   // settle reads what other lanes (or, with m > 1, other warps) wrote, through L2
+    if (accepted) __threadfence();
     __syncwarp();
-    int best = accepted ? rep : INT_MAX;
-    if (q.m > 1) {
-        // the last of the task's attempts settles the round; what an accepted one
-        // wrote is visible before its repetition, and that before its arrival
-        int arrived = 0;
-        if (lane == 0) {
-            if (accepted) {
-                atomicMin(&b.best[task], rep);
-                __threadfence();
+    arrive<LEVEL>(b, q, r, i, task, rep, accepted, buf, lane);
+}
+
+// The same for a small round, four warps per attempt: its checks are 2 k + l
+// transforms in a row on a warp of its own (20 us for Dilithium2), a quarter of
+// that here, and the SMs have the room.
+template <int LEVEL, int SRC>
+__global__ void __launch_bounds__(128) k_sign_back_wide(const SignBatch b, int r) {
+    __shared__ __align__(16) int32_t tables[2 * NTT_TABLE_WORDS], bufs[4][288];
+    __shared__ int hints;
+    using V = Lv<LEVEL>;
+    using S = Scratch<LEVEL>;
+    using SL = Slot<LEVEL>;
+    const Round q = round_of(b, r);
+    const int s = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (s >= q.p * q.m) return;
+    load_zetas(tables);
+    if (threadIdx.x == 0) hints = 0;
+    __syncthreads();
+    int32_t *buf = bufs[warp], *zt = tables, *izt = tables + NTT_TABLE_WORDS;
+    const int i = s / q.m, task = pending_list(b, r)[i], rep = q.base + s - i * q.m;
+    int32_t *slot = slot_of<LEVEL>(b, s);
+    const int32_t *pre = pre_of<LEVEL, SRC>(b, task);
+    bool bad = threadIdx.x == 0 && (rep >= b.max_iter || (q.m > 1 && atomicOr(&b.best[task], 0) < rep));
+    bool accepted = !__syncthreads_or(bad);
+    if (accepted) {
+        int32_t ch[8];
+        const int8_t *c = reinterpret_cast<const int8_t *>(slot + SL::X * N);
+#pragma unroll
+        for (int m = 0; m < 8; ++m) ch[m] = c[lane + 32 * m];
+        ntt_fwd(ch, buf, zt, lane);
+        // r0, z and hint polynomials in turn, a quarter of each to a warp
+#pragma unroll 1
+        for (int part = 0; part < 3 && accepted; ++part) {
+            const int polys = part == 1 ? V::L : V::K;
+            bad = false;
+#pragma unroll 1
+            for (int u = warp; u < polys && !bad; u += 4) {
+                int32_t v[8], a[8], d[8];
+                load_l2(a, pre + ((part == 0 ? S::S2H : part == 1 ? S::S1H : S::T0H) + u) * N, lane);
+                int32_t *data = slot + ((part == 1 ? SL::Y : SL::W) + u) * N;
+                load_l0(d, data, lane);
+#pragma unroll
+                for (int m = 0; m < 8; ++m) v[m] = mont_mul(ch[m], a[m]);
+                ntt_inv(v, buf, izt, lane);
+                if (part == 0) {
+                    bad = check_r0<LEVEL>(v, d);
+                    if (!bad) store_l0(data, d, lane);
+                } else if (part == 1) {
+                    bad = check_z<LEVEL>(v, d);
+                    if (!bad) store_l0(data, v, lane);
+                } else {
+                    int count = 0;
+                    bad = check_hint<LEVEL>(v, d, hint_of<LEVEL>(slot) + 8 * u, count, lane);
+                    if (!bad && lane == 0) atomicAdd(&hints, count);
+                }
             }
-            arrived = atomicAdd(&b.done[task], 1);
+            accepted = !__syncthreads_or(bad);
         }
-        if (__shfl_sync(FULL, arrived, 0) != q.m - 1) return;
-        __threadfence();
-        if (lane == 0) best = atomicOr(&b.best[task], 0);
-        best = __shfl_sync(FULL, best, 0);
+        accepted = accepted && *(volatile int *)&hints <= V::OMEGA;
     }
-    settle<LEVEL>(b, q, r, i, task, best, buf, lane);
+    // every warp of the CTA has written its part by the last barrier; warp 0 settles
+    if (accepted) __threadfence();
+    __syncthreads();
+    if (warp == 0) arrive<LEVEL>(b, q, r, i, task, rep, accepted, buf, lane);
 }
 
 // ---------------------------------------------------------------- what is left
@@ -551,9 +688,9 @@ __global__ void __launch_bounds__(256, 4) k_sign_rest(const SignBatch b, int r, 
         }
         __syncwarp();
         int it = q.base;
-        bool ok = false;
+        bool ok = false, stop = false;
         MaskStream ms{0, 0};
-        while (it < b.max_iter) {
+        while (it < b.max_iter && !(stop = __shfl_sync(FULL, canceled(b), 0))) {
             ok = sign_attempt<LEVEL, 1>(it * V::L, pre, itr, ms, *v.gs, *v.ws, v.zt, v.izt, 0, v.bar, v.lane);
             ++it;
             if (ok) break;
@@ -563,10 +700,7 @@ __global__ void __launch_bounds__(256, 4) k_sign_rest(const SignBatch b, int r, 
             sign_pack<LEVEL, 1>(sig, itr, *v.gs, 0, v.lane);
         else
             sign_zero<LEVEL, 1>(sig, 0, v.lane);
-        if (v.lane == 0) {
-            if (b.status) b.status[task] = ok ? DIL_OK : DIL_EITER;
-            if (b.iters) b.iters[task] = it;
-        }
+        if (v.lane == 0) report(b, task, ok ? DIL_OK : stop ? DIL_ECANCELED : DIL_EITER, !ok && stop ? 0 : it);
         __syncwarp();
     }
 }
@@ -665,9 +799,15 @@ cudaError_t launch_rounds(SignBatch b, void *ws, cudaStream_t s) {
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         k_sign_front<LEVEL, SRC><<<most, 32, 0, s>>>(b, r);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_sign_hash<LEVEL><<<h.blocks, h.threads, 0, s>>>(b, r);
+        if (most <= HASH_WIDE_MOST)
+            k_sign_hash_wide<LEVEL><<<most, 32, 0, s>>>(b, r);
+        else
+            k_sign_hash<LEVEL><<<h.blocks, h.threads, 0, s>>>(b, r);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_sign_back<LEVEL, SRC><<<blocks_for(most, ROUND_WARPS), 32 * ROUND_WARPS, 0, s>>>(b, r);
+        if (most <= HASH_WIDE_MOST)
+            k_sign_back_wide<LEVEL, SRC><<<most, 128, 0, s>>>(b, r);
+        else
+            k_sign_back<LEVEL, SRC><<<blocks_for(most, ROUND_WARPS), 32 * ROUND_WARPS, 0, s>>>(b, r);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     const size_t room = (size_t)b.slots * Slot<LEVEL>::POLYS / Scratch<LEVEL>::ITR_POLYS;

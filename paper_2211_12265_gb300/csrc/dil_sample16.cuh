@@ -118,34 +118,17 @@ __device__ __forceinline__ void expand_s_batch(long long first, long long total,
     for (int u = 0; u < K16_STATES && first + u < total; ++u) {
         const int t = (int)((first + u) / KL);
         int32_t *dst = out_of(t) + (int)(first + u - (long long)t * KL) * N;
+        // candidate lane + 32 m: nibble lane mod 8 of word lane / 8 + 4 m
+        const uint32_t *src = st + u * EXPAND16_STRIDE + (lane >> 3);
         int c = 0;
-        // a lane takes the four bytes of word lane + 32 m (68 words), in stream order
-        for (int m = 0; m < 3 && c < N; ++m) {
-            const int w = lane + 32 * m;
-            const uint32_t x = w < 68 ? st[u * EXPAND16_STRIDE + w] : 0xFFFFFFFFu;
-            uint32_t take = 0;
-#pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                const uint32_t v = (x >> (4 * b)) & 15u;
-                take |= (uint32_t)(V::ETA == 2 ? v < 15u : v < 9u) << b;
-            }
-            // candidates taken by the lanes before this one
-            int before = __popc(take);
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const int y = __shfl_up_sync(FULL, before, d);
-                if (lane >= d) before += y;
-            }
-            const int all = __shfl_sync(FULL, before, 31);
-            int to = c + before - __popc(take);
-#pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                if (!((take >> b) & 1u)) continue;
-                const uint32_t v = (x >> (4 * b)) & 15u;
-                if (to < N) dst[to] = V::ETA == 2 ? 2 - (int32_t)(v % 5u) : 4 - (int32_t)v;
-                ++to;
-            }
-            c += all;
+#pragma unroll 1
+        for (int m = 0; m < 17 && c < N; ++m) {
+            const uint32_t v = (src[4 * m] >> (4 * (lane & 7))) & 15u;
+            const bool acc = V::ETA == 2 ? v < 15u : v < 9u;
+            const uint32_t mask = __ballot_sync(FULL, acc);
+            const int to = c + __popc(mask & lanemask_lt(lane));
+            if (acc && to < N) dst[to] = V::ETA == 2 ? 2 - (int32_t)(v % 5u) : 4 - (int32_t)v;
+            c += __popc(mask);
         }
         few |= (uint32_t)(c < N) << u;
     }

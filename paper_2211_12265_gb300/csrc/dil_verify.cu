@@ -127,6 +127,30 @@ __global__ void __launch_bounds__(32, 16) k_verify_hash(const VerifyBatch b) {
     hash16_run(job, stage, threadIdx.x);
 }
 
+// The same for a small batch, a warp per task on the 25-lane form.
+template <int LEVEL, int SRC>
+__global__ void __launch_bounds__(32) k_verify_hash_wide(const VerifyBatch b) {
+    __shared__ __align__(16) uint8_t tr[32];
+    using V = Lv<LEVEL>;
+    const int task = blockIdx.x, lane = threadIdx.x;
+    int key;
+    uint64_t m0;
+    size_t mlen;
+    if (!verify_input<SRC>(b, task, key, m0, mlen)) return;
+    uint32_t lo = 0, hi = 0;
+    if (SRC == VERIFY_KEYED) {
+        tr[lane] = b.key_tr[(size_t)key * 32 + lane];
+    } else {
+        absorb_concat(lo, hi, tr, 0, b.pk + (size_t)task * V::PK, V::PK, 136, lane);
+        squeeze_words(lo, hi, tr, 4, lane);
+    }
+    __syncwarp();
+    lo = 0;
+    hi = 0;
+    absorb_concat(lo, hi, tr, 32, b.msg + m0, mlen, 136, lane);
+    squeeze_words(lo, hi, reinterpret_cast<uint8_t *>(b.mu + (size_t)task * 16), 8, lane);
+}
+
 // c = SampleInBall(c~) of the signatures of tasks [first, first + 16), one warp.
 template <int LEVEL>
 __device__ __forceinline__ void verify_challenges(const VerifyBatch &b, int first, uint32_t *stage, int lane) {
@@ -306,6 +330,29 @@ __global__ void __launch_bounds__(128) k_verify_compare(const VerifyBatch b) {
     hash16_run(job, stage[threadIdx.x >> 5], lane);
 }
 
+// The same for a small batch, a warp per task on the 25-lane form.
+template <int LEVEL, int SRC>
+__global__ void __launch_bounds__(32) k_verify_compare_wide(const VerifyBatch b) {
+    using V = Lv<LEVEL>;
+    constexpr int W1 = V::K * V::POLYW1;
+    __shared__ __align__(16) uint32_t in[(64 + W1) / 4 + 2];
+    const int task = blockIdx.x, lane = threadIdx.x;
+    if (!b.ok[task]) return;
+    const uint32_t *w1 = reinterpret_cast<const uint32_t *>(b.scratch + (size_t)task * verify_polys<LEVEL, SRC>() * N);
+    if (lane < 16) in[lane] = b.mu[(size_t)task * 16 + lane];
+#pragma unroll
+    for (int i = 0; i < W1 / 128; ++i) in[16 + lane + 32 * i] = w1[lane + 32 * i];
+    __syncwarp();
+    uint32_t lo = 0, hi = 0;
+    absorb_smem(lo, hi, reinterpret_cast<const uint8_t *>(in), 64 + W1, 136, lane);
+    bool eq = true;
+    if (lane < 4) {
+        const uint8_t *ct = b.sig + (size_t)task * V::SIG + 8 * lane;
+        eq = ld_bytes4(ct, 4) == lo && ld_bytes4(ct + 4, 4) == hi;
+    }
+    if (!__all_sync(FULL, eq) && lane == 0) b.ok[task] = 0;
+}
+
 namespace {
 
 template <int LEVEL, int SRC>
@@ -317,8 +364,12 @@ cudaError_t launch_batch(VerifyBatch b, const VerifyFork &f, cudaStream_t s) {
     if (f.stream && ((e = cudaEventRecord(f.fork, s)) != cudaSuccess ||
                      (e = cudaStreamWaitEvent(hs, f.fork, 0)) != cudaSuccess))
         return e;
+    const bool wide = b.n <= HASH_WIDE_MOST;
     if (b.n > b.hash_warps * K16_STATES && (e = cudaMemsetAsync(b.next, 0, sizeof(int), hs)) != cudaSuccess) return e;
-    k_verify_hash<LEVEL, SRC><<<b.hash_warps, 32, 0, hs>>>(b);
+    if (wide)
+        k_verify_hash_wide<LEVEL, SRC><<<b.n, 32, 0, hs>>>(b);
+    else
+        k_verify_hash<LEVEL, SRC><<<b.hash_warps, 32, 0, hs>>>(b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const long long polys = SRC == VERIFY_PLAIN ? (long long)b.n * Lv<LEVEL>::K * Lv<LEVEL>::L : 0;
     k_verify_sample<LEVEL><<<b.challenge_blocks + (int)((polys + K16_STATES - 1) / K16_STATES), 32, 0, s>>>(b);
@@ -334,7 +385,10 @@ cudaError_t launch_batch(VerifyBatch b, const VerifyFork &f, cudaStream_t s) {
     }
     if (e != cudaSuccess) return e;
     const HashGrid h = hash_grid(b.n);
-    k_verify_compare<LEVEL, SRC><<<h.blocks, h.threads, 0, s>>>(b);
+    if (wide)
+        k_verify_compare_wide<LEVEL, SRC><<<b.n, 32, 0, s>>>(b);
+    else
+        k_verify_compare<LEVEL, SRC><<<h.blocks, h.threads, 0, s>>>(b);
     return cudaGetLastError();
 }
 
