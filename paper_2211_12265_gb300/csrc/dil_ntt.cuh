@@ -101,6 +101,18 @@ __device__ __forceinline__ void gs_bfly(int32_t &a, int32_t &b, int32_t z, int32
     b = mul_add_z(0, d, z, zs);
 }
 
+// The same on coefficients a and b of C polynomials.
+template <int C>
+__device__ __forceinline__ void ct_bflies(int32_t (&r)[C][8], int a, int b, int32_t z, int32_t zs) {
+#pragma unroll
+    for (int c = 0; c < C; ++c) ct_bfly(r[c][a], r[c][b], z, zs);
+}
+template <int C>
+__device__ __forceinline__ void gs_bflies(int32_t (&r)[C][8], int a, int b, int32_t z, int32_t zs) {
+#pragma unroll
+    for (int c = 0; c < C; ++c) gs_bfly(r[c][a], r[c][b], z, zs);
+}
+
 // Shared-memory accesses by 32-bit shared-window address (the out-of-line
 // transforms receive addresses, not generic pointers).  Exchange-buffer
 // accesses are ordered (volatile, memory clobber); twiddle loads read
@@ -160,83 +172,96 @@ struct GlobalTwiddles {
 struct Poly8 {
     int32_t v[8];
 };
+// The same for C polynomials that are transformed together.
+template <int C>
+struct Polys8 {
+    int32_t v[C][8];
+};
 
 // Forward NTT.  In: L0, |r| < q.  Out: L2, |r| < 9.1q, unscaled (a level adds
 // at most 1.01q).  buf: the warp's exchange buffer (288 words), zt: the
 // forward twiddles (shared).
-template <class Table>
-__device__ __forceinline__ void ntt_fwd_body(int32_t (&r)[8], uint32_t buf, Table zt) {
+template <int C, class Table>
+__device__ __forceinline__ void ntt_fwd_body(int32_t (&r)[C][8], uint32_t buf, Table zt) {
     const int lane = threadIdx.x & 31;
     // level 1 (len 128): pairs (m, m+4)
     {
         const int32_t z = c_zetas.z[1], zs = c_zetas.zs[1];
 #pragma unroll
-        for (int m = 0; m < 4; ++m) ct_bfly(r[m], r[m + 4], z, zs);
+        for (int m = 0; m < 4; ++m) ct_bflies(r, m, m + 4, z, zs);
     }
     // level 2 (len 64): pairs (m, m+2), twiddle 2 + m/4
-    ct_bfly(r[0], r[2], c_zetas.z[2], c_zetas.zs[2]);
-    ct_bfly(r[1], r[3], c_zetas.z[2], c_zetas.zs[2]);
-    ct_bfly(r[4], r[6], c_zetas.z[3], c_zetas.zs[3]);
-    ct_bfly(r[5], r[7], c_zetas.z[3], c_zetas.zs[3]);
+    ct_bflies(r, 0, 2, c_zetas.z[2], c_zetas.zs[2]);
+    ct_bflies(r, 1, 3, c_zetas.z[2], c_zetas.zs[2]);
+    ct_bflies(r, 4, 6, c_zetas.z[3], c_zetas.zs[3]);
+    ct_bflies(r, 5, 7, c_zetas.z[3], c_zetas.zs[3]);
     // level 3 (len 32): pairs (m, m+1), twiddle 4 + m/2
-    ct_bfly(r[0], r[1], c_zetas.z[4], c_zetas.zs[4]);
-    ct_bfly(r[2], r[3], c_zetas.z[5], c_zetas.zs[5]);
-    ct_bfly(r[4], r[5], c_zetas.z[6], c_zetas.zs[6]);
-    ct_bfly(r[6], r[7], c_zetas.z[7], c_zetas.zs[7]);
+    ct_bflies(r, 0, 1, c_zetas.z[4], c_zetas.zs[4]);
+    ct_bflies(r, 2, 3, c_zetas.z[5], c_zetas.zs[5]);
+    ct_bflies(r, 4, 5, c_zetas.z[6], c_zetas.zs[6]);
+    ct_bflies(r, 6, 7, c_zetas.z[7], c_zetas.zs[7]);
     // exchange L0 -> L1
 #pragma unroll
-    for (int m = 0; m < 8; ++m) sts32(buf + 4 * (lane + 36 * m), r[m]);
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+        for (int m = 0; m < 8; ++m) sts32(4 * 288 * c + buf + 4 * (lane + 36 * m), r[c][m]);
     __syncwarp();
     const int b = lane >> 2;
     const uint32_t base1 = buf + 4 * (36 * b + (lane & 3));
 #pragma unroll
-    for (int m = 0; m < 8; ++m) r[m] = lds32(base1 + 16 * m);
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+        for (int m = 0; m < 8; ++m) r[c][m] = lds32(4 * 288 * c + base1 + 16 * m);
     __syncwarp();
     // level 4 (len 16): pairs (m, m+4), twiddle 8 + b
     {
         const int32_t z = zt.z32(8 + b), zs = zt.zs32(8 + b);
 #pragma unroll
-        for (int m = 0; m < 4; ++m) ct_bfly(r[m], r[m + 4], z, zs);
+        for (int m = 0; m < 4; ++m) ct_bflies(r, m, m + 4, z, zs);
     }
     // level 5 (len 8): pairs (m, m+2), twiddles 16 + 2b + {0, 1}
     {
         const int2 z = zt.z64(16 + 2 * b), zs = zt.zs64(16 + 2 * b);
-        ct_bfly(r[0], r[2], z.x, zs.x);
-        ct_bfly(r[1], r[3], z.x, zs.x);
-        ct_bfly(r[4], r[6], z.y, zs.y);
-        ct_bfly(r[5], r[7], z.y, zs.y);
+        ct_bflies(r, 0, 2, z.x, zs.x);
+        ct_bflies(r, 1, 3, z.x, zs.x);
+        ct_bflies(r, 4, 6, z.y, zs.y);
+        ct_bflies(r, 5, 7, z.y, zs.y);
     }
     // level 6 (len 4): pairs (m, m+1), twiddles 32 + 4b + {0..3}
     {
         const int4 z = zt.z128(32 + 4 * b), zs = zt.zs128(32 + 4 * b);
-        ct_bfly(r[0], r[1], z.x, zs.x);
-        ct_bfly(r[2], r[3], z.y, zs.y);
-        ct_bfly(r[4], r[5], z.z, zs.z);
-        ct_bfly(r[6], r[7], z.w, zs.w);
+        ct_bflies(r, 0, 1, z.x, zs.x);
+        ct_bflies(r, 2, 3, z.y, zs.y);
+        ct_bflies(r, 4, 5, z.z, zs.z);
+        ct_bflies(r, 6, 7, z.w, zs.w);
     }
     // exchange L1 -> L2
 #pragma unroll
-    for (int m = 0; m < 8; ++m) sts32(base1 + 4 * (4 * m + (m >> 1)), r[m]);
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+        for (int m = 0; m < 8; ++m) sts32(4 * 288 * c + base1 + 4 * (4 * m + (m >> 1)), r[c][m]);
     __syncwarp();
 #pragma unroll
-    for (int m = 0; m < 8; ++m) r[m] = lds32(buf + 4 * (9 * lane + m));
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+        for (int m = 0; m < 8; ++m) r[c][m] = lds32(4 * 288 * c + buf + 4 * (9 * lane + m));
     __syncwarp();
     // level 7 (len 2): pairs (m, m+2), twiddles 64 + 2t + {0, 1} (one 8-byte
     // load per lane: a half-warp reads 128 contiguous bytes, conflict-free)
     {
         const int2 z = zt.z64(64 + 2 * lane), zs = zt.zs64(64 + 2 * lane);
-        ct_bfly(r[0], r[2], z.x, zs.x);
-        ct_bfly(r[1], r[3], z.x, zs.x);
-        ct_bfly(r[4], r[6], z.y, zs.y);
-        ct_bfly(r[5], r[7], z.y, zs.y);
+        ct_bflies(r, 0, 2, z.x, zs.x);
+        ct_bflies(r, 1, 3, z.x, zs.x);
+        ct_bflies(r, 4, 6, z.y, zs.y);
+        ct_bflies(r, 5, 7, z.y, zs.y);
     }
     // level 8 (len 1): pairs (m, m+1), twiddles 128 + 4t + {0..3} (16-byte load)
     {
         const int4 z = zt.z128(128 + 4 * lane), zs = zt.zs128(128 + 4 * lane);
-        ct_bfly(r[0], r[1], z.x, zs.x);
-        ct_bfly(r[2], r[3], z.y, zs.y);
-        ct_bfly(r[4], r[5], z.z, zs.z);
-        ct_bfly(r[6], r[7], z.w, zs.w);
+        ct_bflies(r, 0, 1, z.x, zs.x);
+        ct_bflies(r, 2, 3, z.y, zs.y);
+        ct_bflies(r, 4, 5, z.z, zs.z);
+        ct_bflies(r, 6, 7, z.w, zs.w);
     }
 }
 
@@ -246,137 +271,160 @@ __device__ __forceinline__ void ntt_fwd_body(int32_t (&r)[8], uint32_t buf, Tabl
 // lies in [-q/4, 5q/4), so it never exceeds the sums of its level.  The last
 // level keeps the Montgomery product, whose result is below q.
 // izt: the inverse twiddles in shared memory.
-template <class Table>
-__device__ __forceinline__ void ntt_inv_body(int32_t (&r)[8], uint32_t buf, Table izt) {
+template <int C, class Table>
+__device__ __forceinline__ void ntt_inv_body(int32_t (&r)[C][8], uint32_t buf, Table izt) {
     const int lane = threadIdx.x & 31;
     // len 1: pairs (m, m+1), twiddles 128 + 4t + {0..3}
     {
         const int4 z = izt.z128(128 + 4 * lane), zs = izt.zs128(128 + 4 * lane);
-        gs_bfly(r[0], r[1], z.x, zs.x);
-        gs_bfly(r[2], r[3], z.y, zs.y);
-        gs_bfly(r[4], r[5], z.z, zs.z);
-        gs_bfly(r[6], r[7], z.w, zs.w);
+        gs_bflies(r, 0, 1, z.x, zs.x);
+        gs_bflies(r, 2, 3, z.y, zs.y);
+        gs_bflies(r, 4, 5, z.z, zs.z);
+        gs_bflies(r, 6, 7, z.w, zs.w);
     }
     // len 2: pairs (m, m+2), twiddles 64 + 2t + {0, 1}
     {
         const int2 z = izt.z64(64 + 2 * lane), zs = izt.zs64(64 + 2 * lane);
-        gs_bfly(r[0], r[2], z.x, zs.x);
-        gs_bfly(r[1], r[3], z.x, zs.x);
-        gs_bfly(r[4], r[6], z.y, zs.y);
-        gs_bfly(r[5], r[7], z.y, zs.y);
+        gs_bflies(r, 0, 2, z.x, zs.x);
+        gs_bflies(r, 1, 3, z.x, zs.x);
+        gs_bflies(r, 4, 6, z.y, zs.y);
+        gs_bflies(r, 5, 7, z.y, zs.y);
     }
     // exchange L2 -> L1
 #pragma unroll
-    for (int m = 0; m < 8; ++m) sts32(buf + 4 * (9 * lane + m), r[m]);
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+        for (int m = 0; m < 8; ++m) sts32(4 * 288 * c + buf + 4 * (9 * lane + m), r[c][m]);
     __syncwarp();
     const int b = lane >> 2;
     const uint32_t base1 = buf + 4 * (36 * b + (lane & 3));
 #pragma unroll
-    for (int m = 0; m < 8; ++m) r[m] = lds32(base1 + 4 * (4 * m + (m >> 1)));
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+        for (int m = 0; m < 8; ++m) r[c][m] = lds32(4 * 288 * c + base1 + 4 * (4 * m + (m >> 1)));
     __syncwarp();
     // len 4: pairs (m, m+1), twiddles 32 + 4b + {0..3}
     {
         const int4 z = izt.z128(32 + 4 * b), zs = izt.zs128(32 + 4 * b);
-        gs_bfly(r[0], r[1], z.x, zs.x);
-        gs_bfly(r[2], r[3], z.y, zs.y);
-        gs_bfly(r[4], r[5], z.z, zs.z);
-        gs_bfly(r[6], r[7], z.w, zs.w);
+        gs_bflies(r, 0, 1, z.x, zs.x);
+        gs_bflies(r, 2, 3, z.y, zs.y);
+        gs_bflies(r, 4, 5, z.z, zs.z);
+        gs_bflies(r, 6, 7, z.w, zs.w);
     }
     // len 8: pairs (m, m+2), twiddles 16 + 2b + {0, 1}
     {
         const int2 z = izt.z64(16 + 2 * b), zs = izt.zs64(16 + 2 * b);
-        gs_bfly(r[0], r[2], z.x, zs.x);
-        gs_bfly(r[1], r[3], z.x, zs.x);
-        gs_bfly(r[4], r[6], z.y, zs.y);
-        gs_bfly(r[5], r[7], z.y, zs.y);
+        gs_bflies(r, 0, 2, z.x, zs.x);
+        gs_bflies(r, 1, 3, z.x, zs.x);
+        gs_bflies(r, 4, 6, z.y, zs.y);
+        gs_bflies(r, 5, 7, z.y, zs.y);
     }
     // len 16: pairs (m, m+4), twiddle 8 + b
     {
         const int32_t z = izt.z32(8 + b), zs = izt.zs32(8 + b);
 #pragma unroll
-        for (int m = 0; m < 4; ++m) gs_bfly(r[m], r[m + 4], z, zs);
+        for (int m = 0; m < 4; ++m) gs_bflies(r, m, m + 4, z, zs);
     }
     // exchange L1 -> L0
 #pragma unroll
-    for (int m = 0; m < 8; ++m) sts32(base1 + 16 * m, r[m]);
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+        for (int m = 0; m < 8; ++m) sts32(4 * 288 * c + base1 + 16 * m, r[c][m]);
     __syncwarp();
 #pragma unroll
-    for (int m = 0; m < 8; ++m) r[m] = lds32(buf + 4 * (lane + 36 * m));
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+        for (int m = 0; m < 8; ++m) r[c][m] = lds32(4 * 288 * c + buf + 4 * (lane + 36 * m));
     __syncwarp();
     // len 32: pairs (m, m+1), twiddle 4 + m/2
-    gs_bfly(r[0], r[1], c_zetas.iz[4], c_zetas.izs[4]);
-    gs_bfly(r[2], r[3], c_zetas.iz[5], c_zetas.izs[5]);
-    gs_bfly(r[4], r[5], c_zetas.iz[6], c_zetas.izs[6]);
-    gs_bfly(r[6], r[7], c_zetas.iz[7], c_zetas.izs[7]);
+    gs_bflies(r, 0, 1, c_zetas.iz[4], c_zetas.izs[4]);
+    gs_bflies(r, 2, 3, c_zetas.iz[5], c_zetas.izs[5]);
+    gs_bflies(r, 4, 5, c_zetas.iz[6], c_zetas.izs[6]);
+    gs_bflies(r, 6, 7, c_zetas.iz[7], c_zetas.izs[7]);
     // len 64: pairs (m, m+2), twiddle 2 + m/4
-    gs_bfly(r[0], r[2], c_zetas.iz[2], c_zetas.izs[2]);
-    gs_bfly(r[1], r[3], c_zetas.iz[2], c_zetas.izs[2]);
-    gs_bfly(r[4], r[6], c_zetas.iz[3], c_zetas.izs[3]);
-    gs_bfly(r[5], r[7], c_zetas.iz[3], c_zetas.izs[3]);
+    gs_bflies(r, 0, 2, c_zetas.iz[2], c_zetas.izs[2]);
+    gs_bflies(r, 1, 3, c_zetas.iz[2], c_zetas.izs[2]);
+    gs_bflies(r, 4, 6, c_zetas.iz[3], c_zetas.izs[3]);
+    gs_bflies(r, 5, 7, c_zetas.iz[3], c_zetas.izs[3]);
     // len 128 with the factor 2^32/n folded in (twiddle 1)
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        int32_t a = r[m], c = r[m + 4];
-        r[m] = mont_mul(NTT_F, a + c);
-        r[m + 4] = mont_mul(NTT_G, a - c);
-    }
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int32_t a = r[c][m], b2 = r[c][m + 4];
+            r[c][m] = mont_mul(NTT_F, a + b2);
+            r[c][m + 4] = mont_mul(NTT_G, a - b2);
+        }
 }
 
 // Out of line: one copy of the code serves every call site, which keeps the
 // fused kernels' instruction footprint small.
-static __device__ __noinline__ Poly8 ntt_fwd_impl(Poly8 p, uint32_t buf, uint32_t zt) {
+static __device__ __noinline__ Polys8<1> ntt_fwd_impl(Polys8<1> p, uint32_t buf, uint32_t zt) {
     ntt_fwd_body(p.v, buf, SharedTwiddles{zt});
     return p;
 }
-static __device__ __noinline__ Poly8 ntt_inv_impl(Poly8 p, uint32_t buf, uint32_t izt) {
+static __device__ __noinline__ Polys8<1> ntt_inv_impl(Polys8<1> p, uint32_t buf, uint32_t izt) {
     ntt_inv_body(p.v, buf, SharedTwiddles{izt});
     return p;
 }
-static __device__ __noinline__ Poly8 ntt_fwd_global_impl(Poly8 p, uint32_t buf) {
+// With the twiddles of the global table, on one polynomial or on two whose
+// chains fill each other's latencies and share the twiddles (exchange buffer:
+// 288 words each).
+template <int C>
+__device__ __noinline__ Polys8<C> ntt_fwd_global_impl(Polys8<C> p, uint32_t buf) {
     ntt_fwd_body(p.v, buf, GlobalTwiddles<false>{});
     return p;
 }
-static __device__ __noinline__ Poly8 ntt_inv_global_impl(Poly8 p, uint32_t buf) {
+template <int C>
+__device__ __noinline__ Polys8<C> ntt_inv_global_impl(Polys8<C> p, uint32_t buf) {
     ntt_inv_body(p.v, buf, GlobalTwiddles<true>{});
     return p;
 }
 
 __device__ __forceinline__ void ntt_fwd(int32_t r[8], int32_t *buf, const int32_t *zt, int lane) {
     (void)lane;
-    Poly8 p;
+    Polys8<1> p;
 #pragma unroll
-    for (int m = 0; m < 8; ++m) p.v[m] = r[m];
+    for (int m = 0; m < 8; ++m) p.v[0][m] = r[m];
     p = ntt_fwd_impl(p, smem_addr(buf), smem_addr(zt));
 #pragma unroll
-    for (int m = 0; m < 8; ++m) r[m] = p.v[m];
+    for (int m = 0; m < 8; ++m) r[m] = p.v[0][m];
 }
 
 __device__ __forceinline__ void ntt_inv(int32_t r[8], int32_t *buf, const int32_t *izt, int lane) {
     (void)lane;
-    Poly8 p;
+    Polys8<1> p;
 #pragma unroll
-    for (int m = 0; m < 8; ++m) p.v[m] = r[m];
+    for (int m = 0; m < 8; ++m) p.v[0][m] = r[m];
     p = ntt_inv_impl(p, smem_addr(buf), smem_addr(izt));
 #pragma unroll
-    for (int m = 0; m < 8; ++m) r[m] = p.v[m];
+    for (int m = 0; m < 8; ++m) r[m] = p.v[0][m];
 }
 
-// The same with the twiddles of the global table.
-__device__ __forceinline__ void ntt_fwd_global(int32_t r[8], int32_t *buf) {
-    Poly8 p;
+// The same with the twiddles of the global table, on C polynomials.
+template <int C>
+__device__ __forceinline__ void ntt_fwd_global(int32_t (&r)[C][8], int32_t *buf) {
+    Polys8<C> p;
 #pragma unroll
-    for (int m = 0; m < 8; ++m) p.v[m] = r[m];
-    p = ntt_fwd_global_impl(p, smem_addr(buf));
+    for (int i = 0; i < 8 * C; ++i) p.v[i / 8][i % 8] = r[i / 8][i % 8];
+    p = ntt_fwd_global_impl<C>(p, smem_addr(buf));
 #pragma unroll
-    for (int m = 0; m < 8; ++m) r[m] = p.v[m];
+    for (int i = 0; i < 8 * C; ++i) r[i / 8][i % 8] = p.v[i / 8][i % 8];
 }
-__device__ __forceinline__ void ntt_inv_global(int32_t r[8], int32_t *buf) {
-    Poly8 p;
+template <int C>
+__device__ __forceinline__ void ntt_inv_global(int32_t (&r)[C][8], int32_t *buf) {
+    Polys8<C> p;
 #pragma unroll
-    for (int m = 0; m < 8; ++m) p.v[m] = r[m];
-    p = ntt_inv_global_impl(p, smem_addr(buf));
+    for (int i = 0; i < 8 * C; ++i) p.v[i / 8][i % 8] = r[i / 8][i % 8];
+    p = ntt_inv_global_impl<C>(p, smem_addr(buf));
 #pragma unroll
-    for (int m = 0; m < 8; ++m) r[m] = p.v[m];
+    for (int i = 0; i < 8 * C; ++i) r[i / 8][i % 8] = p.v[i / 8][i % 8];
+}
+__device__ __forceinline__ void ntt_fwd_global(int32_t (&r)[8], int32_t *buf) {
+    ntt_fwd_global(reinterpret_cast<int32_t (&)[1][8]>(r), buf);
+}
+__device__ __forceinline__ void ntt_inv_global(int32_t (&r)[8], int32_t *buf) {
+    ntt_inv_global(reinterpret_cast<int32_t (&)[1][8]>(r), buf);
 }
 
 // Copies the forward twiddles (NTT_TABLE_WORDS), or those and behind them the

@@ -42,6 +42,7 @@ template <int LEVEL> struct Slot {
 };
 
 constexpr int ROUND_MAX_REPS = 32;     // repetitions of one task in one round
+constexpr int MAX_ROUNDS = 24;
 // Attempts of a round that are worth having in flight, speculative ones included:
 // a round of fewer takes almost as long (its hashes alone are a chain of eight
 // permutations), more are only wasted repetitions.  10,000 Dilithium2 tasks with
@@ -261,9 +262,12 @@ __global__ void __launch_bounds__(32, 16) k_sign_mask(const SignBatch b, int r) 
 }
 
 // ---------------------------------------------------------------- front
+// Two polynomials at a time share their twiddles and y^ (10,000 Dilithium3 tasks
+// 2586 -> 2556 us, Dilithium5 3353 -> 3309, Dilithium2 unchanged: the kernel waits
+// for DRAM more than for its transforms, 69% of the copy rate).
 template <int LEVEL, int SRC>
-__global__ void __launch_bounds__(32, LEVEL == 2 ? 28 : 20) k_sign_front(const SignBatch b, int r) {
-    __shared__ __align__(16) int32_t buf[288], yh[Lv<LEVEL>::L * N];
+__global__ void __launch_bounds__(32, 20) k_sign_front(const SignBatch b, int r) {
+    __shared__ __align__(16) int32_t buf[2 * 288], yh[Lv<LEVEL>::L * N];
     using V = Lv<LEVEL>;
     using S = Scratch<LEVEL>;
     const Round q = round_of(b, r);
@@ -271,42 +275,58 @@ __global__ void __launch_bounds__(32, LEVEL == 2 ? 28 : 20) k_sign_front(const S
     if (s >= attempts) return;
     const int32_t *pre = pre_of<LEVEL, SRC>(b, pending_list(b, r)[s / q.m]);
     int32_t *slot = slot_of<LEVEL>(b, s);
-    int32_t v[8];
+    int32_t v[2][8];
 #pragma unroll 1
-    for (int j = 0; j < V::L; ++j) {
-        load_l0(v, slot + (Slot<LEVEL>::Y + j) * N, lane);
+    for (int j = 0; j + 1 < V::L; j += 2) {
+        load_l0(v[0], slot + (Slot<LEVEL>::Y + j) * N, lane);
+        load_l0(v[1], slot + (Slot<LEVEL>::Y + j + 1) * N, lane);
         ntt_fwd_global(v, buf);
-        store_l2(yh + j * N, v, lane);   // read back by the same lane
+        store_l2(yh + j * N, v[0], lane);   // read back by the same lane
+        store_l2(yh + (j + 1) * N, v[1], lane);
     }
+    if (V::L % 2) {
+        load_l0(v[0], slot + (Slot<LEVEL>::Y + V::L - 1) * N, lane);
+        ntt_fwd_global(v[0], buf);
+        store_l2(yh + (V::L - 1) * N, v[0], lane);
+    }
+    static_assert(V::K % 2 == 0, "rows in pairs");
 #pragma unroll 1
-    for (int i = 0; i < V::K; ++i) {
+    for (int i = 0; i < V::K; i += 2) {
         // the l products of a row are summed in 64 bits (|sum| < 7 q 9.1q < 2^31 q) and reduced once
-        long long acc[8];
+        long long acc[2][8];
 #pragma unroll
-        for (int m = 0; m < 8; ++m) acc[m] = 0;
-        // every load of the row is in flight before the first product: A^ comes from L2 or DRAM
-        int32_t a[V::L][8];
-#pragma unroll
-        for (int j = 0; j < V::L; ++j) load_l2(a[j], pre + (S::AH + i * V::L + j) * N, lane);
+        for (int m = 0; m < 8; ++m) acc[0][m] = acc[1][m] = 0;
+        const int32_t *row = pre + (S::AH + i * V::L) * N;
 #pragma unroll
         for (int j = 0; j < V::L; ++j) {
-            int32_t y[8];
+            int32_t a0[8], a1[8], y[8];
+            load_l2(a0, row + j * N, lane);
+            load_l2(a1, row + (V::L + j) * N, lane);
             load_l2(y, yh + j * N, lane);
 #pragma unroll
-            for (int m = 0; m < 8; ++m) acc[m] += (long long)a[j][m] * y[m];
+            for (int m = 0; m < 8; ++m) {
+                acc[0][m] += (long long)a0[m] * y[m];
+                acc[1][m] += (long long)a1[m] * y[m];
+            }
         }
-#pragma unroll
-        for (int m = 0; m < 8; ++m) v[m] = mont_reduce(acc[m]);
-        ntt_inv_global(v, buf);
-        int32_t h[8];
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
-            v[m] = to_canonical(v[m]);
-            h[m] = highbits<LEVEL>(v[m]);
+            v[0][m] = mont_reduce(acc[0][m]);
+            v[1][m] = mont_reduce(acc[1][m]);
         }
-        store_l0(slot + (Slot<LEVEL>::W + i) * N, v, lane);
-        l0_to_seq(h, buf, lane);
-        pack_w1<LEVEL>(reinterpret_cast<uint8_t *>(slot + Slot<LEVEL>::X * N) + i * V::POLYW1, h, lane);
+        ntt_inv_global(v, buf);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            int32_t h[8];
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+                v[c][m] = to_canonical(v[c][m]);
+                h[m] = highbits<LEVEL>(v[c][m]);
+            }
+            store_l0(slot + (Slot<LEVEL>::W + i + c) * N, v[c], lane);
+            l0_to_seq(h, buf, lane);
+            pack_w1<LEVEL>(reinterpret_cast<uint8_t *>(slot + Slot<LEVEL>::X * N) + (i + c) * V::POLYW1, h, lane);
+        }
     }
 }
 
@@ -711,7 +731,6 @@ namespace {
 // Mean acceptance of one repetition (Alg 2; 1 / 4.25, 1 / 5.1, 1 / 3.85).
 double accept_of(int level) { return level == 2 ? 1 / 4.25 : level == 3 ? 1 / 5.1 : 1 / 3.85; }
 
-constexpr int MAX_ROUNDS = 24;
 constexpr int CTL_WORDS = 64;   // the hashing warps' counter, then the rounds' task counts
 static_assert(MAX_ROUNDS + 3 <= CTL_WORDS, "a count per round, the counter and the round after the last");
 

@@ -55,14 +55,28 @@ __device__ __forceinline__ void expand_a_batch(long long first, long long total,
         const int t = (int)((first + u) / KL);
         int32_t *dst = out_of(t) + (int)(first + u - (long long)t * KL) * N;
         const uint32_t *src = st + u * EXPAND16_STRIDE + w0;
+        // the first 256 candidates all below q (0.78 of the polynomials): in place
+        uint32_t v[9];
+        bool all = true;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            v[m] = __funnelshift_r(src[24 * m], src[24 * m + 1], sh) & 0x7FFFFFu;
+            all = all && v[m] < (uint32_t)Q;
+        }
+        if (__all_sync(FULL, all)) {
+            const int to = INDEX ? lane : lane_order(lane);   // candidate + 32: 32 or 16 words on
+#pragma unroll
+            for (int m = 0; m < 8; ++m) dst[to + (INDEX ? 32 : 16) * m] = (int32_t)v[m];
+            continue;
+        }
+        v[8] = __funnelshift_r(src[192], src[193], sh) & 0x7FFFFFu;
         int c = 0;
 #pragma unroll
         for (int m = 0; m < 9; ++m) {
-            const uint32_t v = __funnelshift_r(src[24 * m], src[24 * m + 1], sh) & 0x7FFFFFu;
-            const bool acc = v < (uint32_t)Q && (m < 8 || lane < 24);   // 280 candidates
+            const bool acc = v[m] < (uint32_t)Q && (m < 8 || lane < 24);   // 280 candidates
             const uint32_t mask = __ballot_sync(FULL, acc);
             const int to = c + __popc(mask & lanemask_lt(lane));
-            if (acc && to < N) dst[INDEX ? to : lane_order(to)] = (int32_t)v;
+            if (acc && to < N) dst[INDEX ? to : lane_order(to)] = (int32_t)v[m];
             c += __popc(mask);
         }
         few |= (uint32_t)(c < N) << u;
