@@ -212,8 +212,9 @@ int run_streams(dil_ctx *c, size_t n, size_t per, size_t region, size_t ns, cuda
 
 // Streams a Sign batch of n tasks is spread over: the rounds of one part fill
 // the gaps of the others' (the hashes' chains, the ends of kernels).
-// 10,000 Dilithium2 tasks on 1, 2, 3, 4 streams: 1925, 1678, 1611, 1579 us; 5,000:
-// 1130, 1073, 1009, 1004; 2,048: 652, 645, 628, 619.
+// 10,000 Dilithium2 tasks on 2, 3, 4 streams: 1593, 1546, 1524 us; 10,000
+// Dilithium3 2295, 2253, 2233; 3,000 Dilithium2 707, 680, 672.  (Streams of
+// falling priority: 1700 and 2460 us for the first two.)
 size_t sign_parts(size_t n) { return n >= PIPE_MIN_TASKS ? PIPE_STREAMS : 1; }
 
 // Runs Sign in rounds over the n tasks of `all` (whose per-task pointers are
@@ -230,6 +231,7 @@ int run_sign_batch(dil_ctx *c, int level, int src, size_t n, const dil::SignBatc
                            dil::SignBatch b = all;
                            b.n = (int)(c1 - c0);
                            b.slots = (int)z.slots;
+                           b.parts = (int)ns;
                            if (src != dil::SIGN_KEYED) b.sk += skb * c0;
                            if (b.ahat) b.ahat += k * l * 256 * c0;
                            if (b.key_idx) b.key_idx += c0;
@@ -256,7 +258,9 @@ void carve_verify(dil::VerifyBatch &b, void *ws, size_t m, size_t polys) {
 // Runs Verify's batch form over the n tasks of `all` (whose per-task pointers are
 // those of task 0), in as many launches as the budget asks for, with the hashes
 // on a stream of their own.  (Parts of a large batch on several streams gain
-// nothing: 10,000 Dilithium2 tasks take 442 us in one, 450 to 461 in two to four.)
+// nothing that holds: with the hashes between two halves' sampling 10,000
+// Dilithium2 tasks take 408 us instead of 416, 10,000 Dilithium5 1264 instead of
+// 1202; the hashes before the sampling cost both 5 to 12%.)
 int run_verify_batch(dil_ctx *c, int level, int src, size_t n, const dil::VerifyBatch &all, cudaStream_t s) {
     const size_t polys = dil::verify_batch_polys(level, src), per = verify_task_bytes(level, src);
     const size_t tasks = chunk_tasks(c, per, n);
@@ -619,6 +623,7 @@ cudaError_t launch_rounds(dil_ctx *c, const dil::PersistJobs &J, const RoundPlan
             dil::SignBatch b{};
             b.n = (int)std::min(p.size[j].tasks, x.n - c0);
             b.slots = (int)p.size[j].slots;
+            b.parts = PIPE_STREAMS;
             b.sk = x.sk + skb * c0;
             b.msg = x.msg;
             b.off = x.off + c0;
@@ -1038,6 +1043,7 @@ int dil_sign_host(dil_ctx *c, int level, size_t n, const uint8_t *sk, const uint
                                 dil::SignBatch b{};
                                 b.n = (int)m;
                                 b.slots = (int)z.slots;
+                                b.parts = (int)ns;
                                 b.sk = d_sk + skb * c0;
                                 b.msg = d_msg;
                                 b.off = d_off + c0;

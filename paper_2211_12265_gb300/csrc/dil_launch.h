@@ -87,11 +87,12 @@ struct SignBatch {
     int max_iter;
     const int *cancel;       // nullable: tasks without an accepted repetition end once it is set
     int slots;               // attempts of a round, at least sign_batch_min_slots
+    int parts;               // batches that share the GPU
     // set by the launch: the workspace and the prepare kernel's blocks
     int32_t *pre, *slot_polys;
     uint32_t *mu, *rhop;
     int *pending, *best, *done, *next, *count;
-    int hash_warps, expand_blocks;
+    int hash_warps, expand_blocks, fill;
 };
 int sign_batch_slots(int level, int n, int parts);   // slots worth having beside parts - 1 other batches
 int sign_batch_min_slots(int level, int n);   // slots needed

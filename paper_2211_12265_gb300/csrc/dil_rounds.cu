@@ -4,14 +4,14 @@
 // while its other blocks sample A^ and transform s1, s2 and t0.  Then every
 // round evaluates the next m repetitions of each unfinished task (an
 // "attempt" each, in a slot of its own), phase by phase over the whole batch:
-//   mask   y = ExpandMask: sixteen polynomials to a warp, those of whole attempts
+//   mask   y = ExpandMask: sixteen polynomials to a warp
 //   front  y^, w = INTT(A^ y^), w1: a warp per attempt
 //   hash   c~ = H(mu || w1) and SampleInBall: sixteen attempts to a warp
 //   back   z, r0 and hint checks: a warp per attempt; the warp that finishes a
 //          task's last attempt of the round writes the signature of the
 //          smallest accepting repetition, or keeps the task for the next round
-// m grows as tasks finish (slots / unfinished tasks), so the long tail of the
-// rejection loop is evaluated in parallel and a round keeps filling the GPU.
+// m grows as tasks finish (round_reps), so the long tail of the rejection loop
+// is evaluated in parallel and a round keeps filling the GPU.
 // The host launches as many rounds as leave no task over in all but a
 // vanishing share of batches, and then a kernel that runs the plain loop on
 // whatever is left.
@@ -21,9 +21,13 @@
 // its output unused (masks sampled sixteen nonces ahead), each kernel's code
 // fits the instruction cache (the fused kernel's first stall is instruction
 // fetch), and no SM idles while a few tasks run 20 to 30 repetitions one after
-// the other.  Fused -> rounds: 10,000 Dilithium2 tasks 3396 -> 1848 us, 10,000
-// Dilithium3 (32 B - 4 KB) 5350 -> 2945 us, 150 Dilithium5 1580 -> 408 us, one
-// Dilithium2 task 176 -> 119 us.
+// the other.  Fused -> rounds: 10,000 Dilithium2 tasks 3396 -> 1521 us, 10,000
+// Dilithium3 (32 B - 4 KB) 5350 -> 2345 us, 150 Dilithium5 1580 -> 387 us, one
+// Dilithium2 task 176 -> 101 us.
+//
+// What bounds the phases at 20,000 Dilithium2 attempts: mask the ALU pipe (87%),
+// prepare and hash the same (75%), front DRAM (69% of the copy rate), back its
+// issue slots (51%, the multiplier 51% of its rate; 20 of 32 warps).
 #include <climits>
 
 #include "dil_kern.cuh"
@@ -49,11 +53,26 @@ constexpr int MAX_ROUNDS = 24;
 // 10, 15, 20, 30 k slots: 1770, 1662, 1579, 1812 us; 150 Dilithium5 tasks with
 // 1.2, 2.4, 3.6, 4.8 k: 422, 460, 409, 430 us; 1,000 of them: 954, 687, 725, 776.
 template <int LEVEL> constexpr int round_fill() { return 152 * (LEVEL == 2 ? 32 : LEVEL == 3 ? 28 : 24); }
-constexpr int ROUND_MOST = 152 * 128;
+// The same for all of several batches that share the GPU: the rounds of one fill
+// the gaps of the others', and their last rounds, of a few tasks each, come at
+// the same time.  10,000 Dilithium2 tasks in four batches with 4.8, 9.7, 14.6 k:
+// 1517, 1524, 1566 us; Dilithium3: 2270, 2233, 2233; 3,000 Dilithium2: 784, 672
+// (9.7 k slots; 723 with 6 k), 666.
+constexpr int ROUND_SHARED = 152 * 64;
+constexpr int ROUND_MOST = 152 * 192;
+// Repetitions of a task in one round that are worth their time on a full GPU:
+// all of a task's are run though the first accepted one ends it.  100,000
+// Dilithium2 tasks with 1, 2, 3, 4, 6, 32: 12.5, 12.5, 12.1, 12.0, 12.3, 12.8 ms;
+// 10,000 with 3, 5, 32: 1535, 1524, 1591 us; 10,000 Dilithium3: 2271, 2233, 2326.
+constexpr int ROUND_CAP = 5;
 
-__host__ __device__ __forceinline__ int round_reps(int pending, int slots) {
+// Repetitions of each of `pending` tasks in a round: as many as there are slots
+// for, but more than ROUND_CAP only up to `fill` attempts in all.
+__host__ __device__ __forceinline__ int round_reps(int pending, int slots, int fill) {
     if (pending <= 0) return 0;
-    const int m = slots / pending;
+    const int worth = fill / pending > ROUND_CAP ? fill / pending : ROUND_CAP;
+    int m = slots / pending;
+    if (m > worth) m = worth;
     return m < 1 ? 1 : m > ROUND_MAX_REPS ? ROUND_MAX_REPS : m;
 }
 
@@ -63,8 +82,8 @@ struct Round {
 };
 __device__ __forceinline__ Round round_of(const SignBatch &b, int r) {
     Round q{b.count[r], 0, 0};
-    for (int i = 0; i < r; ++i) q.base += round_reps(b.count[i], b.slots);
-    q.m = round_reps(q.p, b.slots);
+    for (int i = 0; i < r; ++i) q.base += round_reps(b.count[i], b.slots, b.fill);
+    q.m = round_reps(q.p, b.slots, b.fill);
     return q;
 }
 
@@ -221,13 +240,13 @@ template <int LEVEL>
 __global__ void __launch_bounds__(32, 16) k_sign_mask(const SignBatch b, int r) {
     __shared__ __align__(16) uint32_t st[MASK_WORDS];
     using V = Lv<LEVEL>;
-    constexpr int G = K16_STATES / V::L;   // attempts per warp
     const int lane = threadIdx.x;
     const Round q = round_of(b, r);
-    const int attempts = q.p * q.m, first = blockIdx.x * G;
-    if (first >= attempts) return;
+    // a state per polynomial: polynomial j of the attempt in slot i is the round's i l + j-th
+    const int polys = q.p * q.m * V::L, first = blockIdx.x * K16_STATES;
+    if (first >= polys) return;
     const int s = lane >> 1, p = lane & 1;
-    const int slot = min(first + s / V::L, attempts - 1), i = slot / q.m;
+    const int mine = min(first + s, polys - 1), slot = mine / V::L, i = slot / q.m;
     const int rep = q.base + slot - i * q.m;
     const uint32_t *seed = b.rhop + (size_t)pending_list(b, r)[i] * 16;
     uint32_t a[25];
@@ -235,7 +254,7 @@ __global__ void __launch_bounds__(32, 16) k_sign_mask(const SignBatch b, int r) 
     for (int w = 0; w < 25; ++w) a[w] = 0;
 #pragma unroll
     for (int w = 0; w < 8; ++w) a[w] = seed[2 * w + p];
-    if (!p) a[8] = ((uint32_t)(V::L * rep + s % V::L) & 0xFFFFu) | (0x1Fu << 16);
+    if (!p) a[8] = ((uint32_t)(V::L * rep + mine - slot * V::L) & 0xFFFFu) | (0x1Fu << 16);
     if (p) a[16] = 0x80000000u;
 #pragma unroll 1
     for (int blk = 0; blk < 5; ++blk) {
@@ -248,10 +267,10 @@ __global__ void __launch_bounds__(32, 16) k_sign_mask(const SignBatch b, int r) 
     // the shift is the lane's own and the word advances by ZBITS
     const int w0 = (V::ZBITS * lane) >> 5, sh = (V::ZBITS * lane) & 31;
 #pragma unroll 1
-    for (int u = 0; u < G * V::L; ++u) {
-        const int at = first + u / V::L;
-        if (at >= attempts) break;
-        int32_t *dst = slot_of<LEVEL>(b, at) + (Slot<LEVEL>::Y + u % V::L) * N;
+    for (int u = 0; u < K16_STATES; ++u) {
+        const int at = (first + u) / V::L;
+        if (first + u >= polys) break;
+        int32_t *dst = slot_of<LEVEL>(b, at) + (Slot<LEVEL>::Y + first + u - at * V::L) * N;
         const uint32_t *src = st + u * MASK_STRIDE + w0;
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
@@ -764,12 +783,15 @@ Layout layout_of(int src, size_t n, size_t slots) {
     return L;
 }
 
+// Attempts worth having in flight in a batch that has 1 / parts of the GPU.
+template <int LEVEL> int fill_of(int parts) { return parts > 1 ? ROUND_SHARED / parts : round_fill<LEVEL>(); }
+
 // Rounds after which fewer than 0.02 tasks are expected to be left.
-int rounds_of(int level, int n, int slots) {
+int rounds_of(int level, int n, const SignBatch &b) {
     double left = n;
     int r = 0;
     while (left > 0.02 && r < MAX_ROUNDS) {
-        const int m = round_reps(left < 1 ? 1 : (int)left, slots);
+        const int m = round_reps(left < 1 ? 1 : (int)left, b.slots, b.fill);
         for (int i = 0; i < m; ++i) left *= 1 - accept_of(level);
         ++r;
     }
@@ -797,6 +819,7 @@ cudaError_t launch_rounds(SignBatch b, void *ws, cudaStream_t s) {
     b.done = reinterpret_cast<int *>(base + L.done);
     b.next = reinterpret_cast<int *>(base + L.ctl);
     b.count = b.next + 1;
+    b.fill = fill_of<LEVEL>(b.parts);
     cudaError_t e = cudaMemsetAsync(b.next, 0, 4 * CTL_WORDS, s);
     if (e != cudaSuccess) return e;
 
@@ -810,11 +833,11 @@ cudaError_t launch_rounds(SignBatch b, void *ws, cudaStream_t s) {
     k_sign_prepare<LEVEL, SRC><<<b.hash_warps + b.expand_blocks + secret_blocks, 32, prep_smem, s>>>(b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
-    const int rounds = rounds_of(LEVEL, b.n, b.slots);
+    const int rounds = rounds_of(LEVEL, b.n, b);
     const int most = b.slots;   // attempts of a round; blocks beyond the actual count return at once
     const HashGrid h = hash_grid(most);
     for (int r = 0; r < rounds; ++r) {
-        k_sign_mask<LEVEL><<<blocks_for(most, K16_STATES / V::L), 32, 0, s>>>(b, r);
+        k_sign_mask<LEVEL><<<blocks_for((long long)most * V::L, K16_STATES), 32, 0, s>>>(b, r);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         k_sign_front<LEVEL, SRC><<<most, 32, 0, s>>>(b, r);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -854,7 +877,7 @@ cudaError_t launch_src(int src, const SignBatch &b, void *ws, cudaStream_t s) {
 // task within ROUND_MOST.
 template <int LEVEL>
 static int slots_of(int n, int parts) {
-    const long long fill = round_fill<LEVEL>() / parts, most = ROUND_MOST / parts;
+    const long long fill = fill_of<LEVEL>(parts), most = ROUND_MOST / parts;
     long long s = (long long)n * ROUND_MAX_REPS;
     if (s > fill) s = 2LL * n > fill ? 2LL * n : fill;
     if (s > most) s = n > most ? n : most;
