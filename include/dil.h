@@ -77,8 +77,14 @@ int dil_set_max_iter(dil_ctx *ctx, int max_iter);
  * 2 = verify at `level` (0 = every level): warps per CTA (1..8) and warps per
  * task (1, 2 or 4, dividing warps_per_cta; 32 x warps_per_task threads
  * cooperate on one task, the paper's single-warp (1) and four-warp (4) forms).
- * Defaults: 8 warps per CTA, 2 warps per task.  The CTA shares the NTT
- * twiddle tables in shared memory. */
+ * With two or four warps per task a batch runs as one fused kernel of that
+ * shape.  With one, and where no shape was set, it runs in the batch forms,
+ * whose kernels choose their own shapes: the hashes of independent tasks
+ * sixteen to a warp, Sign's rejection loop in rounds over the whole batch.
+ * These use streams of the context beside the caller's (which waits for them)
+ * for a large batch and for Verify's hashes.  A workspace budget that holds a
+ * fused kernel's task but not a batch form's runs the fused kernel with 8
+ * warps per CTA and 2 per task.  Outputs do not depend on the shape. */
 int dil_set_tuning(dil_ctx *ctx, int op, int level, int warps_per_cta, int warps_per_task);
 
 /* Alg 1 (Gen): n 32-byte seeds -> n public keys and n secret keys. */
@@ -123,7 +129,8 @@ int dil_expand_a(dil_ctx *ctx, int level, size_t n, const uint8_t *rho, size_t r
 /* dil_sign_ex with task i's A^ read from ahat instead of expanded from the rho
  * in its secret key; ahat NULL is dil_sign_ex.  The library does not check
  * that ahat matches the keys: an A^ of another rho gives signatures that do
- * not verify.  Runs one warp per task (warps per CTA from the Sign tuning). */
+ * not verify.  Runs in rounds as dil_sign does (whatever the Sign
+ * tuning). */
 int dil_sign_a(dil_ctx *ctx, int level, size_t n, const uint8_t *sk, const uint8_t *msg,
                const uint64_t *msg_off, const uint32_t *ahat, uint8_t *sig, int32_t *task_status,
                int32_t *iterations, void *stream);
@@ -157,12 +164,16 @@ int dil_sign_noalloc(int level, size_t n, const uint8_t *sk, const uint8_t *msg,
 
 /* ----------------------------------------------------------------------------
  * Persistent Sign (section 4.3 dynamic task scheduling, on the device): one
- * launch runs every task of up to three jobs (levels may differ).  Resident
- * warp groups pull tasks from a device queue; once it is empty they evaluate
- * further nonces of unfinished tasks, and the signature of the smallest
- * accepting nonce is committed, so outputs equal dil_sign's byte for byte.
- * The launch (queue reset + kernel) is captured once into a CUDA graph per
- * distinct argument set and replayed on later identical calls.
+ * launch runs every task of up to three jobs (levels may differ).  One-warp
+ * launches (and those of a context without a persistent tuning) run in rounds:
+ * the jobs in parts over four branches of one graph, each round evaluating the
+ * next nonces of every unfinished task, more of them per task as tasks finish.
+ * Launches of two or four warps per task run on a device queue: resident warp
+ * groups pull tasks from it and, once it is empty, evaluate further nonces of
+ * unfinished tasks.  Either way the signature of the smallest accepting nonce
+ * is the output, so outputs equal dil_sign's byte for byte.  The launch is
+ * captured once into a CUDA graph per distinct argument set and replayed on
+ * later identical calls.
  * ------------------------------------------------------------------------- */
 typedef struct {
     int level;               /* 2, 3 or 5 */
@@ -190,7 +201,9 @@ int dil_sign_persistent(dil_ctx *ctx, int njobs, const dil_sign_job *jobs, void 
 /* Persistent launch shape: warps per CTA (1..8), warps per task group (1, 2
  * or 4), CTAs per SM (0 = as many as fit), fresh tasks claimed per queue
  * access (>= 1), helper groups per unfinished task (0 disables speculation).
- * Defaults 8, 2, 0, 1, 4. */
+ * The device queue's shape: with one warp per task group, or without this call,
+ * the launch runs in rounds (on the queue, in the shape 8, 2, 0, 1, 4 or the one
+ * set, where the workspace budget does not hold a round). */
 int dil_set_persistent_tuning(dil_ctx *ctx, int warps_per_cta, int warps_per_task, int ctas_per_sm, int chunk,
                               int speculation);
 
@@ -201,9 +214,10 @@ int dil_set_persistent_tuning(dil_ctx *ctx, int warps_per_cta, int warps_per_tas
 int dil_persistent_status(dil_ctx *ctx, void *stream);
 
 /* Cancels the persistent launch of this context that is running: sets its
- * queue's cancel word through a copy on a stream of its own (the launch keeps
+ * cancel word through a copy on a stream of its own (the launch keeps
  * the SMs, so no kernel is involved) and returns once the word is written.
- * The launch then claims no more repetitions: tasks that already hold an
+ * The launch then claims no more repetitions (in rounds: starts no further
+ * round): tasks that already hold an
  * accepting repetition finish as DIL_OK with their normal signature, every
  * other task ends with status DIL_ECANCELED, 0 iterations and an all-zero
  * signature, and the grid exits.  A launch that has not started yet resets
