@@ -437,7 +437,8 @@ int dil_test_rounding(dil_ctx *ctx, int level, size_t n, const int32_t *r, const
 /* Failure-detection hook: the number of polls after which each bounded wait
  * of later persistent launches on this context (the commit lock, an owner
  * waiting for its helpers) gives up, 1..4194304; 0 restores the default
- * (4194304, about half a second).  A low limit makes the real waits run out
+ * (4194304, about half a second).  While it is lowered, persistent launches run
+ * on the device queue, which has these waits.  A low limit makes them run out
  * under ordinary contention, so tests can check the per-task DIL_ETIMEOUT
  * path.  DIL_EINVAL outside that range. */
 int dil_test_set_spin_limit(dil_ctx *ctx, int limit);

@@ -1,7 +1,9 @@
 // Resident-key kernels: preparing a key store (A^, s^1, s^2, t^0, NTT(t1 2^d),
 // tr per key) and Sign / Verify of tasks that name a resident key.  With the
 // key's precomputation resident, Sign only hashes mu and rho' per message
-// before its rejection loop, and Verify skips ExpandA and H(pk).
+// before its rejection loop, and Verify skips ExpandA and H(pk).  The fused
+// Sign and Verify serve static batching and the shapes that a caller asks for;
+// otherwise batches run in the forms of dil_rounds.cu and dil_verify.cu.
 #include "dil_kern.cuh"
 
 namespace dil {

@@ -1,5 +1,8 @@
 // Plain Sign kernel (Alg 2): one task per group of P warps, whole rejection
 // loop in one launch (section 4.2 single-kernel fusion with early evaluation).
+// Serves the shapes of two or four warps per task that a caller asks for, Sign
+// without allocation, and budgets that hold no round (dil_rounds.cu otherwise:
+// 10,000 Dilithium2 tasks 3396 -> 1521 us).
 #include "dil_kern.cuh"
 
 namespace dil {
