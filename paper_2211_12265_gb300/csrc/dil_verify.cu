@@ -10,9 +10,9 @@
 // (k_verify, kept for the launch shapes a caller asks for) runs the 18 blocks of
 // a Dilithium2 task at 18.7 SM clocks per round, 8.1 k of the task's 20.7 k
 // clocks; sixteen to a warp they take 1.4 k.  Fused -> batch: 10,000 Dilithium2
-// tasks 655 -> 416 us, 10,000 Dilithium5 with messages up to 4 KB 1810 -> 1202,
-// thirteen Dilithium3 162 -> 87.  Sampling A^ takes 228 of the 416 us (ALU pipe),
-// the arithmetic 115 (latency of its loads and exchanges), the comparison 45.
+// tasks 655 -> 399 us, 10,000 Dilithium5 with messages up to 4 KB 1810 -> 1202,
+// thirteen Dilithium3 162 -> 87.  Sampling A^ takes 228 of the 399 us (ALU pipe),
+// the arithmetic about 100 (latency of its loads and exchanges), the comparison 45.
 #include "dil_kern.cuh"
 #include "dil_sample16.cuh"
 
@@ -187,6 +187,12 @@ __global__ void __launch_bounds__(32, 16) k_verify_sample(const VerifyBatch b) {
         [&](int t) { return b.scratch + ((size_t)t * verify_polys<LEVEL, VERIFY_PLAIN>() + 1) * N; }, sm, lane);
 }
 
+// Starts the lines of a byte range on their way into L2.
+__device__ __forceinline__ void prefetch_l2(const void *p, int nbytes, int lane) {
+    for (int at = 128 * lane; at < nbytes; at += 128 * 32)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const uint8_t *>(p) + at));
+}
+
 // The arithmetic of one task, one warp: hint decoding, z^, and per row
 // w1' = UseHint(h, INTT(A^ z^ - c^ NTT(t1 2^d))), packed to the start of its
 // scratch.  False when the signature is malformed or z too large.
@@ -197,6 +203,11 @@ __device__ __forceinline__ bool verify_rows(const VerifyBatch &b, int task, int 
     const uint8_t *sig = b.sig + (size_t)task * V::SIG, *pk = b.pk + (size_t)key * V::PK;
     uint8_t *sq = reinterpret_cast<uint8_t *>(buf);
     int32_t v[8], ch[8];
+    // unpacked polynomial by polynomial between transforms: without this each waits
+    // for DRAM in turn (10,000 Dilithium2 tasks 418 -> 406 us, 50,000 1837 -> 1786;
+    // A^ as well: no better, Dilithium5 0.4% worse)
+    prefetch_l2(sig, V::SIG, lane);
+    if (SRC != VERIFY_KEYED) prefetch_l2(pk, V::PK, lane);
     // strict hint decoding into bit masks
     stage_bytes(sq, sig + V::SIG_H, V::OMEGA + V::K, lane);
     hmask[lane] = 0;
@@ -281,8 +292,12 @@ __device__ __forceinline__ bool verify_rows(const VerifyBatch &b, int task, int 
     return true;
 }
 
+// Resident warps: it waits for loads more than it issues.  10,000 and 50,000
+// Dilithium2 tasks with 20, 24, 28, 32 of them: 407, 406, 401, 400 and 1808, 1786,
+// 1760, 1748 us, 5,000 (28, 32) 230, 233; 10,000 Dilithium5 with 16, 20, 24: 1201,
+// 1202, 1212.
 template <int LEVEL, int SRC>
-__global__ void __launch_bounds__(32, LEVEL == 2 ? 24 : 20) k_verify_rows(const VerifyBatch b) {
+__global__ void __launch_bounds__(32, LEVEL == 2 ? 28 : 20) k_verify_rows(const VerifyBatch b) {
     __shared__ __align__(16) int32_t buf[288], zh[Lv<LEVEL>::L * N];
     __shared__ uint32_t hmask[64];
     const int task = blockIdx.x, lane = threadIdx.x;
