@@ -131,7 +131,10 @@ __device__ __forceinline__ void hash16_run(Job &job, uint32_t *stage_words, int 
 #pragma unroll
             for (int i = 0; i < 25; ++i) a[i] = 0;
             off = 0;
+            // the next input may be what done() wrote: a thread fetches 8-byte
+            // units, of which its partner wrote half
             __threadfence_block();
+            __syncwarp(3u << (lane & 30));
             live = job.next(in);
             if (live) hash16_fetch(in, 0, stage, pair, p);
         }

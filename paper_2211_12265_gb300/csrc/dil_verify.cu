@@ -108,7 +108,7 @@ struct VerifyMuJob {
 
     __device__ __forceinline__ void done(const uint32_t (&a)[25]) {
         const int p = lane & 1;
-        if (SRC != VERIFY_KEYED && !have_tr) {   // the words this thread reads back as the prefix of mu's input
+        if (SRC != VERIFY_KEYED && !have_tr) {   // the pair reads them back as the prefix of mu's input
 #pragma unroll
             for (int i = 0; i < 4; ++i) b.tr[(size_t)task * 8 + 2 * i + p] = a[i];
             have_tr = true;
