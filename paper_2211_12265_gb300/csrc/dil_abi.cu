@@ -232,6 +232,7 @@ int run_sign_batch(dil_ctx *c, int level, int src, size_t n, const dil::SignBatc
                            b.n = (int)(c1 - c0);
                            b.slots = (int)z.slots;
                            b.parts = (int)ns;
+                           b.on_gpu = (int)std::min(n, ns * z.tasks);
                            if (src != dil::SIGN_KEYED) b.sk += skb * c0;
                            if (b.ahat) b.ahat += k * l * 256 * c0;
                            if (b.key_idx) b.key_idx += c0;
@@ -624,6 +625,7 @@ cudaError_t launch_rounds(dil_ctx *c, const dil::PersistJobs &J, const RoundPlan
             b.n = (int)std::min(p.size[j].tasks, x.n - c0);
             b.slots = (int)p.size[j].slots;
             b.parts = PIPE_STREAMS;
+            b.on_gpu = J.total;
             b.sk = x.sk + skb * c0;
             b.msg = x.msg;
             b.off = x.off + c0;
@@ -1044,6 +1046,7 @@ int dil_sign_host(dil_ctx *c, int level, size_t n, const uint8_t *sk, const uint
                                 b.n = (int)m;
                                 b.slots = (int)z.slots;
                                 b.parts = (int)ns;
+                                b.on_gpu = (int)std::min(n, ns * z.tasks);
                                 b.sk = d_sk + skb * c0;
                                 b.msg = d_msg;
                                 b.off = d_off + c0;

@@ -70,6 +70,30 @@ inline int batch_hash_warps(int n) {
 // chain of a hash's blocks is what a small batch waits for.
 constexpr int HASH_WIDE_MOST = 608;
 
+// How a batch's messages are hashed: `warps` warps of two threads to a state,
+// and `wide` warps, one per task, that take the messages of at least
+// `long_bytes` on the 25-lane form.  Beyond HASH_WIDE_MOST tasks on the GPU that
+// form still ends a long message's chain sooner, while its chains are bound by
+// latency (up to ten or twelve on an SM; more, and two threads to a state finish
+// the same work in a sixth of the issue slots).  1,000 Dilithium2 tasks of 16 KB,
+// Sign 914 us without and 818 with it, Verify 549 and 477; of 256 KB 8200 and
+// 6719, 7460 and 6401.  Messages of 4 KB as well: Verify of 609 Dilithium2 tasks
+// 203 -> 187 us, but Sign of 1,824 Dilithium3 1001 -> 1043.  Verify that samples A^
+// has the higher line, since that slows two threads to a state more: 1,824
+// Dilithium3 of 16 KB 823 -> 634 us, with resident keys 1,800 505 -> 537; Sign of
+// 1,500 Dilithium2 973 -> 936, of 1,800 of 64 KB 2536 -> 2597.
+constexpr size_t HASH_LONG_BYTES = 8192;
+constexpr int HASH_LONG_MOST = 1520, HASH_LONG_MOST_SAMPLING = 1824;
+struct HashSplit {
+    int warps, wide;
+    size_t long_bytes;
+};
+inline HashSplit hash_split(int n, int on_gpu, int most) {   // n of the on_gpu tasks that run at a time
+    if (on_gpu <= HASH_WIDE_MOST) return {0, n, 0};
+    if (on_gpu <= most) return {batch_hash_warps(n), n, HASH_LONG_BYTES};
+    return {batch_hash_warps(n), 0, (size_t)-1};
+}
+
 // Launch shape of a kernel that only hashes, one task per pair of threads:
 // single-warp CTAs spread a small batch over the SMs, four-warp ones put one
 // warp on each of an SM's sub-partitions.

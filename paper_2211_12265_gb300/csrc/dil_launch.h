@@ -58,6 +58,7 @@ struct VerifyBatch {
     uint8_t *challenge;      // per task 256 bytes
     int *next;               // counter of the hashing warps
     int hash_warps, challenge_blocks;   // set by the launch
+    size_t long_bytes;                  // messages from here on have a warp each
 };
 // Per task beside the polynomials: mu (64), tr (32), 32 more, of which the
 // batch's counter takes the first, and the challenge (256).
@@ -88,11 +89,13 @@ struct SignBatch {
     const int *cancel;       // nullable: tasks without an accepted repetition end once it is set
     int slots;               // attempts of a round, at least sign_batch_min_slots
     int parts;               // batches that share the GPU
+    int on_gpu;              // tasks of them all that run at a time
     // set by the launch: the workspace and the prepare kernel's blocks
     int32_t *pre, *slot_polys;
     uint32_t *mu, *rhop;
     int *pending, *best, *done, *next, *count;
-    int hash_warps, expand_blocks, fill;
+    int hash_warps, wide_blocks, expand_blocks, fill;
+    size_t long_bytes;       // messages from here on have one of the wide blocks
 };
 int sign_batch_slots(int level, int n, int parts);   // slots worth having beside parts - 1 other batches
 int sign_batch_min_slots(int level, int n);   // slots needed

@@ -1,7 +1,7 @@
 // Sign of a batch in rounds (Alg 2).
 //
-// A prepare kernel hashes mu and rho' of every task, sixteen tasks to a warp,
-// while its other blocks sample A^ and transform s1, s2 and t0.  Then every
+// A prepare kernel hashes mu and rho' of every task, sixteen tasks to a warp (in
+// small batches, and for their long messages, a warp each), while its other blocks sample A^ and transform s1, s2 and t0.  Then every
 // round evaluates the next m repetitions of each unfinished task (an
 // "attempt" each, in a slot of its own), phase by phase over the whole batch:
 //   mask   y = ExpandMask: sixteen polynomials to a warp
@@ -22,8 +22,9 @@
 // fits the instruction cache (the fused kernel's first stall is instruction
 // fetch), and no SM idles while a few tasks run 20 to 30 repetitions one after
 // the other.  Fused -> rounds: 10,000 Dilithium2 tasks 3396 -> 1521 us, 10,000
-// Dilithium3 (32 B - 4 KB) 5350 -> 2345 us, 150 Dilithium5 1580 -> 387 us, one
-// Dilithium2 task 176 -> 101 us.
+// Dilithium3 (32 B - 4 KB) 5350 -> 2345 us, 150 Dilithium5 1580 -> 347 us, one
+// Dilithium2 task 176 -> 101 us (of 256 KB 5568 -> 5431; 7862 with two threads to
+// its hash's state).
 //
 // What bounds the phases at 20,000 Dilithium2 attempts: mask the ALU pipe (87%),
 // prepare and hash the same (75%), front DRAM (69% of the copy rate), back its
@@ -113,6 +114,24 @@ __device__ __forceinline__ void report(const SignBatch &b, int task, int status,
 }
 
 // ---------------------------------------------------------------- prepare
+// Task t's message (and resident key); false when the task is to be rejected.
+template <int SRC>
+__device__ __forceinline__ bool sign_input(const SignBatch &b, int t, int &key, uint64_t &m0, size_t &mlen) {
+    key = t;
+    if (SRC == SIGN_KEYED) {
+        key = b.key_idx[t];
+        if (key < 0 || key >= b.n_keys) return false;
+    }
+    return message_of(b.off, t, m0, mlen);
+}
+
+// A hashed task enters round 0 (one thread).
+__device__ __forceinline__ void enter(const SignBatch &b, int task) {
+    b.best[task] = INT_MAX;
+    b.done[task] = 0;
+    b.pending[atomicAdd(b.count, 1)] = task;
+}
+
 // mu = H(tr || M) and rho' = H(K || mu) of a pair's tasks: the first by the
 // pair's index, the next ones from the batch's counter.  A task with an
 // unknown key or decreasing offsets is rejected here (and one met after a cancel
@@ -126,22 +145,13 @@ struct SignMuJob {
     __device__ SignMuJob(const SignBatch &b_, int pair, int lane_)
         : b(b_), task(pair), lane(lane_), first(true), have_mu(false) {}
 
-    __device__ __forceinline__ bool input(int &key, uint64_t &m0, size_t &mlen) const {
-        key = task;
-        if (SRC == SIGN_KEYED) {
-            key = b.key_idx[task];
-            if (key < 0 || key >= b.n_keys) return false;
-        }
-        return message_of(b.off, task, m0, mlen);
-    }
-
     __device__ __forceinline__ bool next(HashInput &in) {
         using V = Lv<LEVEL>;
         uint64_t m0 = 0;
         size_t mlen = 0;
         int key;
         if (have_mu) {   // rho' = H(K || mu)
-            input(key, m0, mlen);
+            sign_input<SRC>(b, task, key, m0, mlen);
             in = {b.sk + (size_t)key * V::SK + 32, reinterpret_cast<const uint8_t *>(b.mu + (size_t)task * 16), 96, 32};
             return true;
         }
@@ -155,7 +165,9 @@ struct SignMuJob {
             }
             first = false;
             if (task >= b.n) return false;
-            const bool valid = input(key, m0, mlen), stop = pair_bcast(canceled(b), lane);
+            const bool valid = sign_input<SRC>(b, task, key, m0, mlen);
+            if (valid && mlen >= b.long_bytes) continue;   // a wide block's
+            const bool stop = pair_bcast(canceled(b), lane);
             if (valid && !stop) break;
             uint8_t *sig = b.sig + (size_t)task * V::SIG;
             for (int i = lane & 1; i < V::SIG; i += 2) sig[i] = 0;
@@ -169,14 +181,44 @@ struct SignMuJob {
         uint32_t *dst = (have_mu ? b.rhop : b.mu) + (size_t)task * 16 + (lane & 1);
 #pragma unroll
         for (int i = 0; i < 8; ++i) dst[2 * i] = a[i];
-        if (have_mu && !(lane & 1)) {
-            b.best[task] = INT_MAX;
-            b.done[task] = 0;
-            b.pending[atomicAdd(b.count, 1)] = task;
-        }
+        if (have_mu && !(lane & 1)) enter(b, task);
         have_mu = !have_mu;
     }
 };
+
+// The same for the task of a wide block, a warp on the 25-lane form.  A task is
+// this one's if its message is long; without hashing pairs in the batch, the
+// rejected ones are too.
+template <int LEVEL, int SRC>
+__device__ __forceinline__ void sign_mu_wide(const SignBatch &b, int task, uint32_t *sm, int lane) {
+    using V = Lv<LEVEL>;
+    uint8_t *in = reinterpret_cast<uint8_t *>(sm);   // tr, then K || mu
+    uint64_t m0 = 0;
+    size_t mlen = 0;
+    int key;
+    const bool valid = sign_input<SRC>(b, task, key, m0, mlen);
+    if (valid ? mlen < b.long_bytes : b.hash_warps > 0) return;
+    if (!valid || __shfl_sync(FULL, canceled(b), 0)) {
+        sign_zero<LEVEL, 1>(b.sig + (size_t)task * V::SIG, 0, lane);
+        if (lane == 0) report(b, task, valid ? DIL_ECANCELED : DIL_EINVAL, 0);
+        return;
+    }
+    const uint8_t *sk = b.sk + (size_t)key * V::SK;
+    uint32_t lo = 0, hi = 0;
+    stage_bytes(in, sk + 64, 32, lane);
+    __syncwarp();
+    absorb_concat(lo, hi, in, 32, b.msg + m0, mlen, 136, lane);
+    squeeze_words(lo, hi, reinterpret_cast<uint8_t *>(b.mu + (size_t)task * 16), 8, lane);
+    __syncwarp();
+    stage_bytes(in, sk + 32, 32, lane);
+    squeeze_words(lo, hi, in + 32, 8, lane);
+    __syncwarp();
+    lo = 0;
+    hi = 0;
+    absorb_smem(lo, hi, in, 96, 136, lane);
+    squeeze_words(lo, hi, reinterpret_cast<uint8_t *>(b.rhop + (size_t)task * 16), 8, lane);
+    if (lane == 0) enter(b, task);
+}
 
 // s^1, s^2, t^0 of one task (one warp).
 template <int LEVEL>
@@ -200,10 +242,11 @@ constexpr int ROUND_WARPS = 4;   // warps per CTA of the hashing and checking ke
 // One warp per CTA: a sampling warp's 11 to 13 KB of shared memory let sixteen
 // be resident on an SM, and single warps spread over the SMs to within one (in
 // fours, 2,500 mask warps made 625 CTAs for 608 places, a second wave of 17).
-// Blocks [0, hash_warps) hash, [.., + expand_blocks) sample A^ (SIGN_AHAT:
+// Blocks [0, hash_warps) hash, [.., + wide_blocks) hash a long message each
+// (WIDE, hash_split), [.., + expand_blocks) sample A^ (SIGN_AHAT:
 // none), the rest transform the secrets (SIGN_KEYED: none), one task each; with
 // SIGN_AHAT they also copy the caller's A^.
-template <int LEVEL, int SRC>
+template <int LEVEL, int SRC, bool WIDE>
 __global__ void __launch_bounds__(32, 16) k_sign_prepare(const SignBatch b) {
     extern __shared__ __align__(16) uint32_t sm[];
     using V = Lv<LEVEL>;
@@ -215,8 +258,15 @@ __global__ void __launch_bounds__(32, 16) k_sign_prepare(const SignBatch b) {
         hash16_run(job, sm, lane);
         return;
     }
+    blk -= b.hash_warps;
+    if (WIDE) {
+        if (blk < b.wide_blocks) {
+            sign_mu_wide<LEVEL, SRC>(b, blk, sm, lane);
+            return;
+        }
+        blk -= b.wide_blocks;
+    }
     if constexpr (SRC != SIGN_KEYED) {
-        blk -= b.hash_warps;
         if (blk < b.expand_blocks) {
             expand_a_batch<LEVEL, false>(
                 (long long)blk * K16_STATES, (long long)b.n * KL, [&](int t) { return b.sk + (size_t)t * V::SK; },
@@ -824,13 +874,17 @@ cudaError_t launch_rounds(SignBatch b, void *ws, cudaStream_t s) {
     if (e != cudaSuccess) return e;
 
     // prepare
-    b.hash_warps = batch_hash_warps(b.n);
+    const HashSplit split = hash_split(b.n, b.on_gpu, HASH_LONG_MOST);
+    b.hash_warps = split.warps;
+    b.wide_blocks = split.wide;
+    b.long_bytes = split.long_bytes;
     b.expand_blocks = SRC == SIGN_PLAIN ? blocks_for((long long)b.n * V::K * V::L, K16_STATES) : 0;
     const int secret_blocks = SRC == SIGN_KEYED ? 0 : b.n;
     const size_t prep_smem = 4 * (SRC == SIGN_PLAIN ? EXPAND16_WORDS : HASH16_STAGE_WORDS);
     static_assert(288 <= HASH16_STAGE_WORDS && HASH16_STAGE_WORDS <= EXPAND16_WORDS, "every block's shared memory");
-    if ((e = dynamic_smem(k_sign_prepare<LEVEL, SRC>, prep_smem)) != cudaSuccess) return e;
-    k_sign_prepare<LEVEL, SRC><<<b.hash_warps + b.expand_blocks + secret_blocks, 32, prep_smem, s>>>(b);
+    const auto prepare = split.wide ? k_sign_prepare<LEVEL, SRC, true> : k_sign_prepare<LEVEL, SRC, false>;
+    if ((e = dynamic_smem(prepare, prep_smem)) != cudaSuccess) return e;
+    prepare<<<b.hash_warps + b.wide_blocks + b.expand_blocks + secret_blocks, 32, prep_smem, s>>>(b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
     const int rounds = rounds_of(LEVEL, b.n, b);

@@ -1,7 +1,7 @@
 // Verify of a batch (Alg 3).
 //
 // Batch form.  One kernel hashes tr = H(pk) and mu = H(tr || M), sixteen tasks
-// to a warp.  Beside it, on a stream of their own where the caller has one to
+// to a warp (in small batches, and for their long messages, a warp each).  Beside it, on a stream of their own where the caller has one to
 // spare, run SampleInBall(c~), sixteen tasks to a warp, with ExpandA, sixteen
 // polynomials to a warp whatever tasks they belong to (dil_sample16.cuh; not
 // with a resident key's or the caller's A^), and then the arithmetic up to the
@@ -92,7 +92,7 @@ struct VerifyMuJob {
                 }
                 first = false;
                 if (task >= b.n) return false;
-                if (verify_input<SRC>(b, task, key, m0, mlen)) break;
+                if (verify_input<SRC>(b, task, key, m0, mlen) && mlen < b.long_bytes) break;
             }
             if (SRC != VERIFY_KEYED) {
                 in = {nullptr, b.pk + (size_t)task * V::PK, (size_t)V::PK, 0};
@@ -120,26 +120,15 @@ struct VerifyMuJob {
     }
 };
 
-// The hashing warps, each a CTA of its own: they are chains (a 16 KB message is
-// 121 blocks, 3.4 us each on a warp of its own), so they get the registers to
-// keep a state and its input (at 64, a block took 4.5 us) and start first.
+// tr and mu of one task with a long message, a warp on the 25-lane form.
 template <int LEVEL, int SRC>
-__global__ void __launch_bounds__(32, 16) k_verify_hash(const VerifyBatch b) {
-    __shared__ __align__(16) uint32_t stage[HASH16_STAGE_WORDS];
-    VerifyMuJob<LEVEL, SRC> job(b, blockIdx.x * K16_STATES + (threadIdx.x >> 1), threadIdx.x);
-    hash16_run(job, stage, threadIdx.x);
-}
-
-// The same for a small batch, a warp per task on the 25-lane form.
-template <int LEVEL, int SRC>
-__global__ void __launch_bounds__(32) k_verify_hash_wide(const VerifyBatch b) {
+__device__ __forceinline__ void verify_hash_wide(const VerifyBatch &b, int task, int lane) {
     __shared__ __align__(16) uint8_t tr[32];
     using V = Lv<LEVEL>;
-    const int task = blockIdx.x, lane = threadIdx.x;
     int key;
     uint64_t m0;
     size_t mlen;
-    if (!verify_input<SRC>(b, task, key, m0, mlen)) return;
+    if (!verify_input<SRC>(b, task, key, m0, mlen) || mlen < b.long_bytes) return;
     uint32_t lo = 0, hi = 0;
     if (SRC == VERIFY_KEYED) {
         tr[lane] = b.key_tr[(size_t)key * 32 + lane];
@@ -152,6 +141,29 @@ __global__ void __launch_bounds__(32) k_verify_hash_wide(const VerifyBatch b) {
     hi = 0;
     absorb_concat(lo, hi, tr, 32, b.msg + m0, mlen, 136, lane);
     squeeze_words(lo, hi, reinterpret_cast<uint8_t *>(b.mu + (size_t)task * 16), 8, lane);
+}
+
+// The hashing warps, each a CTA of its own: they are chains (a 16 KB message is
+// 121 blocks, 3.4 us each on a warp of its own), so they get the registers to
+// keep a state and its input (at 64, a block took 4.5 us) and start first.
+// WIDE (hash_split): behind them a block per task, which hashes a long message on
+// the 25-lane form.
+template <int LEVEL, int SRC, bool WIDE>
+__global__ void __launch_bounds__(32, 16) k_verify_hash(const VerifyBatch b) {
+    __shared__ __align__(16) uint32_t stage[HASH16_STAGE_WORDS];
+    if (!WIDE || blockIdx.x < b.hash_warps) {
+        VerifyMuJob<LEVEL, SRC> job(b, blockIdx.x * K16_STATES + (threadIdx.x >> 1), threadIdx.x);
+        hash16_run(job, stage, threadIdx.x);
+    } else {
+        verify_hash_wide<LEVEL, SRC>(b, blockIdx.x - b.hash_warps, threadIdx.x);
+    }
+}
+
+// For a small batch, a block per task only.  A kernel of its own: with the code
+// above beside it thirteen Dilithium3 tasks take 92 us instead of 87.
+template <int LEVEL, int SRC>
+__global__ void __launch_bounds__(32) k_verify_hash_wide(const VerifyBatch b) {
+    verify_hash_wide<LEVEL, SRC>(b, blockIdx.x, threadIdx.x);
 }
 
 // c = SampleInBall(c~) of the signatures of tasks [first, first + 16), one warp.
@@ -375,19 +387,24 @@ namespace {
 
 template <int LEVEL, int SRC>
 cudaError_t launch_batch(VerifyBatch b, const VerifyFork &f, cudaStream_t s) {
-    b.hash_warps = batch_hash_warps(b.n);
+    const HashSplit split = hash_split(b.n, b.n, SRC == VERIFY_PLAIN ? HASH_LONG_MOST_SAMPLING : HASH_LONG_MOST);
+    b.hash_warps = split.warps;
+    b.long_bytes = split.long_bytes;
     b.challenge_blocks = (b.n + K16_STATES - 1) / K16_STATES;
     const cudaStream_t hs = f.stream ? f.stream : s;
     cudaError_t e = cudaSuccess;
     if (f.stream && ((e = cudaEventRecord(f.fork, s)) != cudaSuccess ||
                      (e = cudaStreamWaitEvent(hs, f.fork, 0)) != cudaSuccess))
         return e;
-    const bool wide = b.n <= HASH_WIDE_MOST;
-    if (b.n > b.hash_warps * K16_STATES && (e = cudaMemsetAsync(b.next, 0, sizeof(int), hs)) != cudaSuccess) return e;
-    if (wide)
-        k_verify_hash_wide<LEVEL, SRC><<<b.n, 32, 0, hs>>>(b);
+    if (split.warps && b.n > split.warps * K16_STATES &&
+        (e = cudaMemsetAsync(b.next, 0, sizeof(int), hs)) != cudaSuccess)
+        return e;
+    if (!split.warps)
+        k_verify_hash_wide<LEVEL, SRC><<<split.wide, 32, 0, hs>>>(b);
+    else if (split.wide)
+        k_verify_hash<LEVEL, SRC, true><<<split.warps + split.wide, 32, 0, hs>>>(b);
     else
-        k_verify_hash<LEVEL, SRC><<<b.hash_warps, 32, 0, hs>>>(b);
+        k_verify_hash<LEVEL, SRC, false><<<split.warps, 32, 0, hs>>>(b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const long long polys = SRC == VERIFY_PLAIN ? (long long)b.n * Lv<LEVEL>::K * Lv<LEVEL>::L : 0;
     k_verify_sample<LEVEL><<<b.challenge_blocks + (int)((polys + K16_STATES - 1) / K16_STATES), 32, 0, s>>>(b);
@@ -403,7 +420,7 @@ cudaError_t launch_batch(VerifyBatch b, const VerifyFork &f, cudaStream_t s) {
     }
     if (e != cudaSuccess) return e;
     const HashGrid h = hash_grid(b.n);
-    if (wide)
+    if (b.n <= HASH_WIDE_MOST)
         k_verify_compare_wide<LEVEL, SRC><<<b.n, 32, 0, s>>>(b);
     else
         k_verify_compare<LEVEL, SRC><<<h.blocks, h.threads, 0, s>>>(b);

@@ -42,3 +42,82 @@ def test_hash_whose_input_is_the_hash_before(torch_cuda, orc, level):
         ok = gpu_verify(ctx, level, pk, msg, off, osig)
     assert np.array_equal(sig, osig) and np.array_equal(st, ost) and np.array_equal(it, oit)
     assert ok.all()
+
+
+# (tasks, lengths): the 25-lane hashes alone (up to 608 tasks), both forms (the line
+# at 8,192 bytes and around it), and the two-thread form alone
+SPLITS = [(3, [8191, 70000, 0]), (608, [40, 8192, 300]), (609, [8191, 8192, 8193, 32]), (1520, [0, 9000, 40, 16384]),
+          (1521, [8192, 31]), (1824, [32, 12345]), (1825, [8192, 1])]
+
+
+@pytest.mark.parametrize("level", LEVELS)
+@pytest.mark.parametrize("n,lengths", SPLITS)
+def test_long_messages_beside_short_ones(torch_cuda, orc, level, n, lengths):
+    """Every task is hashed once, by the form that its length and the batch's size
+    give it, resident keys and rejected tasks among them."""
+    from gpu_util import dev, host
+    from paper_2211_12265_gb300 import dil
+    torch = torch_cuda
+    keys, m = 4, min(n, 24)   # m distinct tasks, repeated
+    pk, sk = orc.keygen_batch(level, W.seeds(keys, 1010))
+    lens = np.array([lengths[i % len(lengths)] for i in range(m)], dtype=np.int64)
+    msg, off = W.messages(lens, 1010 + n)
+    key = (np.arange(m) % keys).astype(np.int32)
+    osig, ost, oit = orc.sign_batch(level, sk[key], msg, off.astype(np.uint64))
+    pick = np.arange(n) % m
+    big = np.concatenate([msg[off[i]:off[i + 1]] for i in pick] + [np.zeros(1, np.uint8)])
+    big_off = np.concatenate([[0], np.cumsum(lens[pick])]).astype(np.uint64)
+    key = key[pick]
+    unknown = np.arange(n) % 11 == 10   # of resident keys
+    bad = osig[pick]
+    bad[::5, 40] ^= np.uint8(2)
+    with dil.Context(0) as ctx:
+        d_msg, d_off = dev(big), dev(big_off)
+        sig, st, it = (host(x) for x in ctx.sign(level, dev(sk[key]), d_msg, d_off, iterations=True))
+        ok = host(ctx.verify(level, dev(pk[key]), d_msg, d_off, dev(bad)))
+        ks = dil.dil_keystore_create(ctx.handle, level, keys, dev(pk), dev(sk))
+        d_key = dev(np.where(unknown, keys, key).astype(np.int32))
+        ksig = torch.full((n, osig.shape[1]), 0x5A, dtype=torch.uint8, device="cuda")
+        kst = torch.full((n,), 9, dtype=torch.int32, device="cuda")
+        kok = torch.full((n,), 7, dtype=torch.uint8, device="cuda")
+        dil.dil_sign_keyed(ctx.handle, ks, n, d_key, d_msg, d_off, ksig, kst)
+        dil.dil_verify_keyed(ctx.handle, ks, n, d_key, d_msg, d_off, dev(bad), kok)
+        ksig, kst, kok = host(ksig), host(kst), host(kok)
+        dil.dil_keystore_destroy(ks)
+    want_ok = np.arange(n) % 5 != 0
+    assert np.array_equal(sig, osig[pick]) and np.array_equal(st, ost[pick]) and np.array_equal(it, oit[pick])
+    assert np.array_equal(ok, want_ok.astype(np.uint8))
+    assert np.array_equal(ksig, np.where(unknown[:, None], 0, osig[pick]))
+    assert np.array_equal(kst, np.where(unknown, dil.EINVAL, ost[pick]))
+    assert np.array_equal(kok, (want_ok & ~unknown).astype(np.uint8))
+
+
+@pytest.mark.parametrize("n", [1, 400])
+def test_long_messages_end_with_the_25_lane_chain(torch_cuda, n):
+    """The hash of one long message is what such a call waits for: 24 rounds a
+    block at about 224 clocks each for a warp on the 25-lane form, 250 and the
+    absorbing for two threads to a state (1.43 times as long, measured).  The
+    bound is the fused kernel's time, which hashes that way, and a fifth."""
+    import time
+    from gpu_util import dev
+    from paper_2211_12265_gb300 import dil
+    torch = torch_cuda
+    size = 1 << 18
+    msg = torch.randint(0, 256, (size + 32 * n,), dtype=torch.uint8, device="cuda")
+    off = np.concatenate([[0], size + 32 * np.arange(n, dtype=np.uint64)]).astype(np.uint64)
+    took = {}
+    for shape in (None, (8, 2)):
+        with dil.Context(0) as ctx:
+            if shape:
+                ctx.set_tuning(1, shape[0], shape[1], 2)
+            _, sk = ctx.keygen(2, dev(W.seeds(n, 1030)))
+            d_off = dev(off)
+            ts = []
+            for _ in range(4):
+                torch.cuda.synchronize()
+                t = time.perf_counter()
+                ctx.sign(2, sk, msg, d_off)
+                torch.cuda.synchronize()
+                ts.append(time.perf_counter() - t)
+            took[shape] = min(ts)
+    assert took[None] < 1.2 * took[(8, 2)], took
