@@ -153,6 +153,14 @@ bool sign_fused(const dil_ctx *c, int level, int src) {
     return c->wpt[1][lidx(level)] > 1 || round_size(level, src, 1, c->budget).tasks == 0;
 }
 
+// Streams a KeyGen batch is spread over: one half's arithmetic and tr beside the
+// other's sampling.  On one and two streams 5,000 and 10,000 Dilithium2 keys take
+// 271, 454 and 265, 437 us, 10,000 and 16,000 Dilithium3 756, 1114 and 728, 1111;
+// but 3,000 and 4,000 Dilithium2 192, 225 and 220, 253, 2,048 and 6,000 Dilithium3
+// 234, 484 and 411, 530, 6,000, 10,000 and 20,000 Dilithium5 759, 1209, 2269 and 827,
+// 1196, 2311.
+size_t keygen_parts(int level, size_t n) { return n >= (level == 2 ? 5000u : 9000u) && level != 5 ? 2 : 1; }
+
 cudaError_t keygen_chunk(const Shape &sh, int level, int m, const uint8_t *seeds, uint8_t *pk, uint8_t *sk,
                          int32_t *scratch, cudaStream_t s) {
     return sh.fused ? dil::launch_keygen(level, m, seeds, pk, sk, scratch, sh.warps, sh.p, s)
@@ -389,7 +397,7 @@ int dil_keygen(dil_ctx *c, int level, size_t n, const uint8_t *seeds, uint8_t *p
     sizes_of(level, pkb, skb, sigb);
     const size_t per = dil::scratch_polys(dil::OP_KEYGEN, level) * POLY_BYTES;
     const Shape sh = shape_of(c, 0, level, per);
-    size_t ns = sh.fused || n < PIPE_MIN_TASKS ? 1 : 2;   // 10,000 Dilithium2 keys: 476 us on one stream, 458 on two
+    size_t ns = sh.fused ? 1 : keygen_parts(level, n);
     const size_t tasks = part_tasks(c, n, per, ns);
     return run_streams(c, n, tasks, tasks * per, ns, (cudaStream_t)stream,
                        [&](size_t c0, size_t c1, cudaStream_t s, int32_t *scratch) -> int {

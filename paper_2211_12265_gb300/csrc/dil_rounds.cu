@@ -1,9 +1,10 @@
 // Sign of a batch in rounds (Alg 2).
 //
 // A prepare kernel hashes mu and rho' of every task, sixteen tasks to a warp (in
-// small batches, and for their long messages, a warp each), while its other blocks sample A^ and transform s1, s2 and t0.  Then every
-// round evaluates the next m repetitions of each unfinished task (an
-// "attempt" each, in a slot of its own), phase by phase over the whole batch:
+// small batches, and for their long messages, a warp each), while its other
+// blocks sample A^ and transform s1, s2 and t0.  Then every round evaluates the
+// next m repetitions of each unfinished task (an "attempt" each, in a slot of its
+// own), phase by phase over the whole batch:
 //   mask   y = ExpandMask: sixteen polynomials to a warp
 //   front  y^, w = INTT(A^ y^), w1: a warp per attempt
 //   hash   c~ = H(mu || w1) and SampleInBall: sixteen attempts to a warp

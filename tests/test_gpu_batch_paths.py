@@ -121,3 +121,43 @@ def test_long_messages_end_with_the_25_lane_chain(torch_cuda, n):
                 ts.append(time.perf_counter() - t)
             took[shape] = min(ts)
     assert took[None] < 1.2 * took[(8, 2)], took
+
+
+@pytest.mark.parametrize("n", [2048, 2500])
+def test_keygen_does_not_slow_down_in_parts(torch_cuda, n):
+    """2,047 Dilithium3 keys take 236 us; in two halves beside each other 2,048 and
+    2,500 took 411 and 436.  The bound is the ratio of the counts and a quarter."""
+    from gpu_util import dev
+    from paper_2211_12265_gb300 import dil
+    torch = torch_cuda
+
+    def took(m):
+        seeds = dev(W.seeds(m, 1040))
+        pk, sk = ctx.keygen(3, seeds)
+        ts = []
+        for _ in range(9):
+            e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            e0.record()
+            for _ in range(4):
+                dil.dil_keygen(ctx.handle, 3, m, seeds, pk, sk)
+            e1.record()
+            torch.cuda.synchronize()
+            ts.append(e0.elapsed_time(e1) / 4)
+        return sorted(ts)[4]
+
+    with dil.Context(0) as ctx:
+        fewer, more = took(2047), took(n)
+    assert more < 1.25 * n / 2047 * fewer, (fewer, more)
+
+
+@pytest.mark.parametrize("level,n", [(2, 5001), (3, 9001)])
+def test_keygen_in_parts(torch_cuda, level, n):
+    """An odd batch on two streams equals its two halves, made one by one."""
+    from gpu_util import dev, host
+    from paper_2211_12265_gb300 import dil
+    seeds = W.seeds(n, 1050)
+    with dil.Context(0) as ctx:
+        pk, sk = (host(x) for x in ctx.keygen(level, dev(seeds)))
+        for part in (slice(0, 2000), slice(2000, 4500), slice(4500, n)):
+            for got, want in zip((pk, sk), ctx.keygen(level, dev(seeds[part]))):
+                assert np.array_equal(got[part], host(want))
