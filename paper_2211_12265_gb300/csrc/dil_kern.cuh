@@ -88,9 +88,11 @@ struct HashSplit {
     int warps, wide;
     size_t long_bytes;
 };
-inline HashSplit hash_split(int n, int on_gpu, int most) {   // n of the on_gpu tasks that run at a time
-    if (on_gpu <= HASH_WIDE_MOST) return {0, n, 0};
-    if (on_gpu <= most) return {batch_hash_warps(n), n, HASH_LONG_BYTES};
+// Of n of the on_gpu tasks that run at a time: a warp each up to all_most of
+// these, those with a long message up to long_most.
+inline HashSplit hash_split(int n, int on_gpu, int all_most, int long_most) {
+    if (on_gpu <= all_most) return {0, n, 0};
+    if (on_gpu <= long_most) return {batch_hash_warps(n), n, HASH_LONG_BYTES};
     return {batch_hash_warps(n), 0, (size_t)-1};
 }
 

@@ -875,7 +875,7 @@ cudaError_t launch_rounds(SignBatch b, void *ws, cudaStream_t s) {
     if (e != cudaSuccess) return e;
 
     // prepare
-    const HashSplit split = hash_split(b.n, b.on_gpu, HASH_LONG_MOST);
+    const HashSplit split = hash_split(b.n, b.on_gpu, HASH_WIDE_MOST, HASH_LONG_MOST);
     b.hash_warps = split.warps;
     b.wide_blocks = split.wide;
     b.long_bytes = split.long_bytes;

@@ -205,12 +205,13 @@ __device__ __forceinline__ void prefetch_l2(const void *p, int nbytes, int lane)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const uint8_t *>(p) + at));
 }
 
-// The arithmetic of one task, one warp: hint decoding, z^, and per row
+// The arithmetic of one task, a CTA of P warps (g: this one, with an exchange
+// buffer of its own): hint decoding, z^, and per row
 // w1' = UseHint(h, INTT(A^ z^ - c^ NTT(t1 2^d))), packed to the start of its
 // scratch.  False when the signature is malformed or z too large.
-template <int LEVEL, int SRC>
+template <int LEVEL, int SRC, int P>
 __device__ __forceinline__ bool verify_rows(const VerifyBatch &b, int task, int key, int32_t *buf, int32_t *zh,
-                                            uint32_t *hmask, int lane) {
+                                            uint32_t *hmask, int g, int lane) {
     using V = Lv<LEVEL>;
     const uint8_t *sig = b.sig + (size_t)task * V::SIG, *pk = b.pk + (size_t)key * V::PK;
     uint8_t *sq = reinterpret_cast<uint8_t *>(buf);
@@ -218,43 +219,47 @@ __device__ __forceinline__ bool verify_rows(const VerifyBatch &b, int task, int 
     // unpacked polynomial by polynomial between transforms: without this each waits
     // for DRAM in turn (10,000 Dilithium2 tasks 418 -> 406 us, 50,000 1837 -> 1786;
     // A^ as well: no better, Dilithium5 0.4% worse)
-    prefetch_l2(sig, V::SIG, lane);
-    if (SRC != VERIFY_KEYED) prefetch_l2(pk, V::PK, lane);
+    if (g == 0) prefetch_l2(sig, V::SIG, lane);
+    if (SRC != VERIFY_KEYED && g == P - 1) prefetch_l2(pk, V::PK, lane);
     // strict hint decoding into bit masks
-    stage_bytes(sq, sig + V::SIG_H, V::OMEGA + V::K, lane);
-    hmask[lane] = 0;
-    hmask[32 + lane] = 0;
-    __syncwarp();
     bool bad = false;
-    int prev = 0;
+    if (g == 0) {
+        stage_bytes(sq, sig + V::SIG_H, V::OMEGA + V::K, lane);
+        hmask[lane] = 0;
+        hmask[32 + lane] = 0;
+        __syncwarp();
+        int prev = 0;
 #pragma unroll 1
-    for (int i = 0; i < V::K; ++i) {
-        const int end = sq[V::OMEGA + i];
-        if (end < prev || end > V::OMEGA) {
-            bad = true;
-            break;
+        for (int i = 0; i < V::K; ++i) {
+            const int end = sq[V::OMEGA + i];
+            if (end < prev || end > V::OMEGA) {
+                bad = true;
+                break;
+            }
+            for (int j = prev + lane; j < end; j += 32) {
+                const int idx = sq[j];
+                if (j > prev && idx <= sq[j - 1]) bad = true;
+                atomicOr(&hmask[i * 8 + (idx >> 5)], 1u << (idx & 31));
+            }
+            prev = end;
         }
-        for (int j = prev + lane; j < end; j += 32) {
-            const int idx = sq[j];
-            if (j > prev && idx <= sq[j - 1]) bad = true;
-            atomicOr(&hmask[i * 8 + (idx >> 5)], 1u << (idx & 31));
-        }
-        prev = end;
+        if (!bad)
+            for (int j = prev + lane; j < V::OMEGA; j += 32)
+                if (sq[j]) bad = true;
+        bad = __any_sync(FULL, bad);
+        if (P == 1 && bad) return false;
     }
-    if (!bad)
-        for (int j = prev + lane; j < V::OMEGA; j += 32)
-            if (sq[j]) bad = true;
-    if (__any_sync(FULL, bad)) return false;
     // z^ = NTT(z), ||z|| < gamma1 - beta
 #pragma unroll 1
-    for (int j = 0; j < V::L; ++j) {
+    for (int j = g; j < V::L; j += P) {
         unpack_buf_l0<V::ZBITS>(v, sig + V::SIG_Z + j * V::POLYZ, V::GAMMA1, buf, lane);
 #pragma unroll
         for (int m = 0; m < 8; ++m) bad |= iabs(v[m]) >= V::GAMMA1 - V::BETA;
-        if (__any_sync(FULL, bad)) return false;
+        if (P == 1 && __any_sync(FULL, bad)) return false;
         ntt_fwd_global(v, buf);
         store_l2(zh + j * N, v, lane);   // read back by the same lane
     }
+    if (P > 1 && __syncthreads_or(bad)) return false;   // and every warp's z^ and the hints are there
     const int8_t *c = reinterpret_cast<const int8_t *>(b.challenge) + (size_t)task * 256;
 #pragma unroll
     for (int m = 0; m < 8; ++m) ch[m] = c[lane + 32 * m];
@@ -265,7 +270,7 @@ __device__ __forceinline__ bool verify_rows(const VerifyBatch &b, int task, int 
                         : SRC == VERIFY_AHAT ? b.ahat + (size_t)task * V::K * V::L * N
                                              : scr + N;
 #pragma unroll 1
-    for (int i = 0; i < V::K; ++i) {
+    for (int i = g; i < V::K; i += P) {
         int32_t a[V::L][8];   // every load of the row in flight during t1's transform
 #pragma unroll
         for (int j = 0; j < V::L; ++j) {
@@ -308,17 +313,17 @@ __device__ __forceinline__ bool verify_rows(const VerifyBatch &b, int task, int 
 // Dilithium2 tasks with 20, 24, 28, 32 of them: 407, 406, 401, 400 and 1808, 1786,
 // 1760, 1748 us, 5,000 (28, 32) 230, 233; 10,000 Dilithium5 with 16, 20, 24: 1201,
 // 1202, 1212.
-template <int LEVEL, int SRC>
-__global__ void __launch_bounds__(32, LEVEL == 2 ? 28 : 20) k_verify_rows(const VerifyBatch b) {
-    __shared__ __align__(16) int32_t buf[288], zh[Lv<LEVEL>::L * N];
+template <int LEVEL, int SRC, int P>
+__global__ void __launch_bounds__(32 * P, LEVEL != 2 ? 20 / P : P > 1 ? 32 / P : 28) k_verify_rows(const VerifyBatch b) {
+    __shared__ __align__(16) int32_t bufs[P][288], zh[Lv<LEVEL>::L * N];
     __shared__ uint32_t hmask[64];
-    const int task = blockIdx.x, lane = threadIdx.x;
+    const int task = blockIdx.x, g = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int key;
     uint64_t m0;
     size_t mlen;
     const bool r = verify_input<SRC>(b, task, key, m0, mlen) &&
-                   verify_rows<LEVEL, SRC>(b, task, key, buf, zh, hmask, lane);
-    if (lane == 0) b.ok[task] = r;   // 1: c~ decides (k_verify_compare)
+                   verify_rows<LEVEL, SRC, P>(b, task, key, bufs[g], zh, hmask, g, lane);
+    if (threadIdx.x == 0) b.ok[task] = r;   // 1: c~ decides (k_verify_compare)
 }
 
 // c~ = H(mu || w1') of task `pair` against the signature's.
@@ -385,9 +390,20 @@ __global__ void __launch_bounds__(32) k_verify_compare_wide(const VerifyBatch b)
 
 namespace {
 
+// Up to this many tasks everything has a warp (the hashes) or four (the rows) per
+// task.  The rows of so few tasks leave most of the GPU idle: with four warps
+// instead of one 13 tasks of 32 bytes on Dilithium5 keys take 55 us (70), 608 65
+// (77), 13 Dilithium2 verifies 60 (71); 609 and more beside ExpandA gain nothing.  Without sampling (a
+// resident key's or the caller's A^) the line is two hashing warps to a
+// sub-partition: 800 tasks of 4 KB on Dilithium2 keys 155 -> 138 us and 1,216 of 32
+// bytes 64 -> 56 with it at 1,216 instead of 608; at 1,824 1,700 Dilithium3 of 32
+// bytes 73 -> 80.
+constexpr int VERIFY_WIDE_MOST = HASH_WIDE_MOST, VERIFY_WIDE_MOST_RESIDENT = 1216;
+
 template <int LEVEL, int SRC>
 cudaError_t launch_batch(VerifyBatch b, const VerifyFork &f, cudaStream_t s) {
-    const HashSplit split = hash_split(b.n, b.n, SRC == VERIFY_PLAIN ? HASH_LONG_MOST_SAMPLING : HASH_LONG_MOST);
+    const int most = SRC == VERIFY_PLAIN ? VERIFY_WIDE_MOST : VERIFY_WIDE_MOST_RESIDENT;
+    const HashSplit split = hash_split(b.n, b.n, most, SRC == VERIFY_PLAIN ? HASH_LONG_MOST_SAMPLING : HASH_LONG_MOST);
     b.hash_warps = split.warps;
     b.long_bytes = split.long_bytes;
     b.challenge_blocks = (b.n + K16_STATES - 1) / K16_STATES;
@@ -410,7 +426,10 @@ cudaError_t launch_batch(VerifyBatch b, const VerifyFork &f, cudaStream_t s) {
     k_verify_sample<LEVEL><<<b.challenge_blocks + (int)((polys + K16_STATES - 1) / K16_STATES), 32, 0, s>>>(b);
     e = cudaGetLastError();
     if (e == cudaSuccess) {
-        k_verify_rows<LEVEL, SRC><<<b.n, 32, 0, s>>>(b);
+        if (b.n <= most)
+            k_verify_rows<LEVEL, SRC, 4><<<b.n, 128, 0, s>>>(b);
+        else
+            k_verify_rows<LEVEL, SRC, 1><<<b.n, 32, 0, s>>>(b);
         e = cudaGetLastError();
     }
     // the caller's stream waits for the hashes whatever went wrong on it
@@ -420,7 +439,7 @@ cudaError_t launch_batch(VerifyBatch b, const VerifyFork &f, cudaStream_t s) {
     }
     if (e != cudaSuccess) return e;
     const HashGrid h = hash_grid(b.n);
-    if (b.n <= HASH_WIDE_MOST)
+    if (b.n <= most)
         k_verify_compare_wide<LEVEL, SRC><<<b.n, 32, 0, s>>>(b);
     else
         k_verify_compare<LEVEL, SRC><<<h.blocks, h.threads, 0, s>>>(b);

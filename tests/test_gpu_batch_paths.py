@@ -161,3 +161,71 @@ def test_keygen_in_parts(torch_cuda, level, n):
         for part in (slice(0, 2000), slice(2000, 4500), slice(4500, n)):
             for got, want in zip((pk, sk), ctx.keygen(level, dev(seeds[part]))):
                 assert np.array_equal(got[part], host(want))
+
+
+@pytest.mark.parametrize("level", LEVELS)
+@pytest.mark.parametrize("n", [5, 608, 609, 1216, 1217])
+def test_rows_on_four_warps(torch_cuda, orc, level, n):
+    """Signatures spoiled where one warp of a task's four sees it (each z
+    polynomial, the hint, c~) or all do, on both sides of the lines between one and
+    four warps; plain and with resident keys."""
+    from gpu_util import dev, host
+    from paper_2211_12265_gb300 import dil
+    k, l, zbits = {2: (4, 4, 18), 3: (6, 5, 20), 5: (8, 7, 20)}[level]
+    m = l + 4
+    pk, sk, msg, off = _inputs(orc, level, m, 1060, 0, 300)
+    good, _, _ = orc.sign_batch(level, sk, msg, off)
+    bad = good.copy()
+    for j in range(l):                              # z_j's last coefficient out of range
+        bad[j, 32 + 32 * zbits * (j + 1) - 2:32 + 32 * zbits * (j + 1)] = 0
+    bad[l, -1] = 255                                # hint counts
+    bad[l + 1, -k - 1] ^= np.uint8(1)               # unused hint byte, or its order
+    bad[l + 2, 3] ^= np.uint8(64)                   # c~
+    bad[l + 3, 40] ^= np.uint8(1)                   # z within its range
+    assert not orc.verify_batch(level, pk, msg, off, bad).any()
+    pick = np.arange(n) % m
+    spoil = np.arange(n) % 3 != 0
+    sig = np.where(spoil[:, None], bad[pick], good[pick])
+    big = np.concatenate([msg[off[i]:off[i + 1]] for i in pick] + [np.zeros(1, np.uint8)])
+    big_off = np.concatenate([[0], np.cumsum((off[1:] - off[:-1])[pick])]).astype(np.uint64)
+    with dil.Context(0) as ctx:
+        d_msg, d_off, d_sig = dev(big), dev(big_off), dev(sig)
+        ok = host(ctx.verify(level, dev(pk[pick]), d_msg, d_off, d_sig))
+        ks = dil.dil_keystore_create(ctx.handle, level, m, dev(pk))
+        kok = dev(np.full(n, 7, np.uint8))
+        dil.dil_verify_keyed(ctx.handle, ks, n, dev(pick.astype(np.int32)), d_msg, d_off, d_sig, kok)
+        kok = host(kok)
+        dil.dil_keystore_destroy(ks)
+    assert np.array_equal(ok, (~spoil).astype(np.uint8)) and np.array_equal(kok, ok)
+
+
+def test_keyed_verify_of_short_messages_is_no_slower_than_fused(torch_cuda):
+    """A few checks of short messages against resident keys: the fused kernel that
+    two warps per task select bounds the call's time, a twentieth to spare."""
+    from gpu_util import dev
+    from paper_2211_12265_gb300 import dil
+    torch = torch_cuda
+    n = 13
+    took = {}
+    for shape in (None, (8, 2)):
+        with dil.Context(0) as ctx:
+            if shape:
+                ctx.set_tuning(2, shape[0], shape[1], 5)
+            pk, sk = ctx.keygen(5, dev(W.seeds(n, 1070)))
+            msg, off = W.messages(np.full(n, 32), 1070)
+            d_msg, d_off = dev(msg), dev(off.astype(np.uint64))
+            sig, _ = ctx.sign(5, sk, d_msg, d_off)
+            ks = dil.dil_keystore_create(ctx.handle, 5, n, pk)
+            key, ok = dev(np.arange(n, dtype=np.int32)), dev(np.zeros(n, np.uint8))
+            ts = []
+            for _ in range(9):
+                e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+                e0.record()
+                for _ in range(8):
+                    dil.dil_verify_keyed(ctx.handle, ks, n, key, d_msg, d_off, sig, ok)
+                e1.record()
+                torch.cuda.synchronize()
+                ts.append(e0.elapsed_time(e1) / 8)
+            took[shape] = sorted(ts)[4]
+            dil.dil_keystore_destroy(ks)
+    assert took[None] < 1.05 * took[(8, 2)], took
