@@ -1098,7 +1098,7 @@ int dil_verify_host(dil_ctx *c, int level, size_t n, const uint8_t *pk, const ui
     const size_t per = sh.fused ? dil::scratch_polys(dil::OP_VERIFY, level) * POLY_BYTES : batch;
     const size_t tasks = pipe_tasks(c, n, per);
     // one chunk at a time: its hashes run beside the rest, as in dil_verify (1,000
-    // Dilithium3 tasks 250 -> 213 us); of four chunks, each beside the others
+    // Dilithium3 tasks 250 -> 196 us); of four chunks, each beside the others
     dil::VerifyFork fork{};
     if (!sh.fused && pipe_streams(n) == 1) {
         if ((rc = ensure_aux(c))) return rc;

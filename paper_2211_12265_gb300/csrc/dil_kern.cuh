@@ -78,22 +78,61 @@ constexpr int HASH_WIDE_MOST = 608;
 // the same work in a sixth of the issue slots).  1,000 Dilithium2 tasks of 16 KB,
 // Sign 914 us without and 818 with it, Verify 549 and 477; of 256 KB 8200 and
 // 6719, 7460 and 6401.  Messages of 4 KB as well: Verify of 609 Dilithium2 tasks
-// 203 -> 187 us, but Sign of 1,824 Dilithium3 1001 -> 1043.  Verify that samples A^
-// has the higher line, since that slows two threads to a state more: 1,824
-// Dilithium3 of 16 KB 823 -> 634 us, with resident keys 1,800 505 -> 537; Sign of
-// 1,500 Dilithium2 973 -> 936, of 1,800 of 64 KB 2536 -> 2597.
+// 203 -> 187 us, but Sign of 1,824 Dilithium3 1001 -> 1043; Sign of 1,500 Dilithium2
+// of 16 KB 973 -> 936, of 1,800 of 64 KB 2536 -> 2597, Verify with resident keys of
+// 1,800 505 -> 537.
 constexpr size_t HASH_LONG_BYTES = 8192;
-constexpr int HASH_LONG_MOST = 1520, HASH_LONG_MOST_SAMPLING = 1824;
+constexpr int HASH_LONG_MOST = 1520;
+// Beyond that line only where at most HASH_FEW of sixteen tasks in a row have a
+// long message.  Messages of 32 B - 16 KB (a ninth of them long), Verify: 3,000
+// Dilithium3 tasks 863 -> 645 us (708 with four of sixteen, which a group now and
+// then exceeds), 6,000 1034 -> 880, but 10,000 1259 -> 2377; with resident keys
+// 3,000 519 -> 474, 4,000 522 -> 493, 8,191 552 -> 556 and all of 16 KB 574 -> 610.
+constexpr int HASH_FEW = 8, HASH_FEW_MOST = 3072, HASH_FEW_MOST_SAMPLING = 6144;
+static_assert(HASH_FEW_MOST_SAMPLING <= 608 * K16_STATES, "one task to a pair (batch_hash_warps) beside wide warps");
 struct HashSplit {
     int warps, wide;
     size_t long_bytes;
+    int per_group;   // wide warps of sixteen tasks in a row
 };
-// Of n of the on_gpu tasks that run at a time: a warp each up to all_most of
-// these, those with a long message up to long_most.
-inline HashSplit hash_split(int n, int on_gpu, int all_most, int long_most) {
-    if (on_gpu <= all_most) return {0, n, 0};
-    if (on_gpu <= long_most) return {batch_hash_warps(n), n, HASH_LONG_BYTES};
-    return {batch_hash_warps(n), 0, (size_t)-1};
+// The tasks on the GPU up to which every message has a warp, every one of
+// long_bytes or more, few such.
+struct HashLines {
+    int all, every_long, few_long;
+    size_t long_bytes;
+};
+inline HashSplit hash_split(int n, int on_gpu, const HashLines &l) {   // n of the on_gpu tasks that run at a time
+    if (on_gpu <= l.all) return {0, n, 0, 0};
+    const int warps = batch_hash_warps(n);
+    if (on_gpu > l.few_long) return {warps, 0, (size_t)-1, 0};
+    const int groups = (n + K16_STATES - 1) / K16_STATES;
+    if (on_gpu <= l.every_long) return {warps, groups * K16_STATES, l.long_bytes, K16_STATES};
+    return {warps, groups * HASH_FEW, HASH_LONG_BYTES, HASH_FEW};
+}
+
+__device__ __forceinline__ bool is_long(const uint64_t *off, int n, int t, size_t least) {
+    uint64_t m0;
+    size_t mlen;
+    return t < n && message_of(off, t, m0, mlen) && mlen >= least;
+}
+
+// Whether task t (n: none) is a wide warp's.
+__device__ __forceinline__ bool has_wide_warp(const uint64_t *off, int n, int t, size_t least, int per_group) {
+    if (!is_long(off, n, t, least)) return false;
+    if (per_group >= K16_STATES) return true;
+    const int first = t / K16_STATES * K16_STATES;
+    int c = 0;
+    for (int i = 0; i < K16_STATES; ++i) c += is_long(off, n, first + i, least);
+    return c <= per_group;
+}
+
+// The task of wide warp w (all 32 lanes), or -1.
+__device__ __forceinline__ int task_of_wide_warp(const uint64_t *off, int n, int w, size_t least, int per_group,
+                                                 int lane) {
+    const int first = w / per_group * K16_STATES, nth = w % per_group;
+    const unsigned mask = __ballot_sync(FULL, lane < K16_STATES && is_long(off, n, first + lane, least));
+    if (__popc(mask) > per_group || nth >= __popc(mask)) return -1;
+    return first + (int)__fns(mask, 0, nth + 1);
 }
 
 // Launch shape of a kernel that only hashes, one task per pair of threads:

@@ -58,7 +58,9 @@ struct VerifyBatch {
     uint8_t *challenge;      // per task 256 bytes
     int *next;               // counter of the hashing warps
     int hash_warps, challenge_blocks;   // set by the launch
-    size_t long_bytes;                  // messages from here on have a warp each
+    size_t long_bytes;                  // messages from here on may have a warp each
+    int per_group;                      // (hash_split)
+    int pair_ctas;                      // of the kernel with both kinds of hashing warps
 };
 // Per task beside the polynomials: mu (64), tr (32), 32 more, of which the
 // batch's counter takes the first, and the challenge (256).
@@ -95,7 +97,8 @@ struct SignBatch {
     uint32_t *mu, *rhop;
     int *pending, *best, *done, *next, *count;
     int hash_warps, wide_blocks, expand_blocks, fill;
-    size_t long_bytes;       // messages from here on have one of the wide blocks
+    size_t long_bytes;       // messages from here on may have one of the wide blocks
+    int per_group;           // (hash_split)
 };
 int sign_batch_slots(int level, int n, int parts);   // slots worth having beside parts - 1 other batches
 int sign_batch_min_slots(int level, int n);   // slots needed

@@ -143,8 +143,8 @@ struct SignMuJob {
     int task, lane;
     bool first, have_mu;
 
-    __device__ SignMuJob(const SignBatch &b_, int pair, int lane_)
-        : b(b_), task(pair), lane(lane_), first(true), have_mu(false) {}
+    __device__ SignMuJob(const SignBatch &b_, int first_task, int lane_)
+        : b(b_), task(first_task), lane(lane_), first(true), have_mu(false) {}
 
     __device__ __forceinline__ bool next(HashInput &in) {
         using V = Lv<LEVEL>;
@@ -166,9 +166,7 @@ struct SignMuJob {
             }
             first = false;
             if (task >= b.n) return false;
-            const bool valid = sign_input<SRC>(b, task, key, m0, mlen);
-            if (valid && mlen >= b.long_bytes) continue;   // a wide block's
-            const bool stop = pair_bcast(canceled(b), lane);
+            const bool valid = sign_input<SRC>(b, task, key, m0, mlen), stop = pair_bcast(canceled(b), lane);
             if (valid && !stop) break;
             uint8_t *sig = b.sig + (size_t)task * V::SIG;
             for (int i = lane & 1; i < V::SIG; i += 2) sig[i] = 0;
@@ -187,18 +185,17 @@ struct SignMuJob {
     }
 };
 
-// The same for the task of a wide block, a warp on the 25-lane form.  A task is
-// this one's if its message is long; without hashing pairs in the batch, the
-// rejected ones are too.
+// The same for the task of a wide block, a warp on the 25-lane form (hash_split).
 template <int LEVEL, int SRC>
-__device__ __forceinline__ void sign_mu_wide(const SignBatch &b, int task, uint32_t *sm, int lane) {
+__device__ __forceinline__ void sign_mu_wide(const SignBatch &b, int blk, uint32_t *sm, int lane) {
     using V = Lv<LEVEL>;
+    const int task = b.hash_warps ? task_of_wide_warp(b.off, b.n, blk, b.long_bytes, b.per_group, lane) : blk;
+    if (task < 0) return;
     uint8_t *in = reinterpret_cast<uint8_t *>(sm);   // tr, then K || mu
     uint64_t m0 = 0;
     size_t mlen = 0;
     int key;
     const bool valid = sign_input<SRC>(b, task, key, m0, mlen);
-    if (valid ? mlen < b.long_bytes : b.hash_warps > 0) return;
     if (!valid || __shfl_sync(FULL, canceled(b), 0)) {
         sign_zero<LEVEL, 1>(b.sig + (size_t)task * V::SIG, 0, lane);
         if (lane == 0) report(b, task, valid ? DIL_ECANCELED : DIL_EINVAL, 0);
@@ -255,7 +252,9 @@ __global__ void __launch_bounds__(32, 16) k_sign_prepare(const SignBatch b) {
     const int lane = threadIdx.x;
     int blk = blockIdx.x;
     if (blk < b.hash_warps) {
-        SignMuJob<LEVEL, SRC> job(b, blk * K16_STATES + (lane >> 1), lane);
+        int t = blk * K16_STATES + (lane >> 1);   // with WIDE the pair's only task
+        if (WIDE && has_wide_warp(b.off, b.n, t, b.long_bytes, b.per_group)) t = b.n;
+        SignMuJob<LEVEL, SRC> job(b, t, lane);
         hash16_run(job, sm, lane);
         return;
     }
@@ -875,10 +874,11 @@ cudaError_t launch_rounds(SignBatch b, void *ws, cudaStream_t s) {
     if (e != cudaSuccess) return e;
 
     // prepare
-    const HashSplit split = hash_split(b.n, b.on_gpu, HASH_WIDE_MOST, HASH_LONG_MOST);
+    const HashSplit split = hash_split(b.n, b.on_gpu, {HASH_WIDE_MOST, HASH_LONG_MOST, HASH_LONG_MOST, HASH_LONG_BYTES});
     b.hash_warps = split.warps;
     b.wide_blocks = split.wide;
     b.long_bytes = split.long_bytes;
+    b.per_group = split.per_group;
     b.expand_blocks = SRC == SIGN_PLAIN ? blocks_for((long long)b.n * V::K * V::L, K16_STATES) : 0;
     const int secret_blocks = SRC == SIGN_KEYED ? 0 : b.n;
     const size_t prep_smem = 4 * (SRC == SIGN_PLAIN ? EXPAND16_WORDS : HASH16_STAGE_WORDS);

@@ -73,8 +73,8 @@ struct VerifyMuJob {
     int task, lane;
     bool first, have_tr;
 
-    __device__ VerifyMuJob(const VerifyBatch &b_, int pair, int lane_)
-        : b(b_), task(pair), lane(lane_), first(true), have_tr(false) {}
+    __device__ VerifyMuJob(const VerifyBatch &b_, int first_task, int lane_)
+        : b(b_), task(first_task), lane(lane_), first(true), have_tr(false) {}
 
     __device__ __forceinline__ bool next(HashInput &in) {
         using V = Lv<LEVEL>;
@@ -92,7 +92,7 @@ struct VerifyMuJob {
                 }
                 first = false;
                 if (task >= b.n) return false;
-                if (verify_input<SRC>(b, task, key, m0, mlen) && mlen < b.long_bytes) break;
+                if (verify_input<SRC>(b, task, key, m0, mlen)) break;
             }
             if (SRC != VERIFY_KEYED) {
                 in = {nullptr, b.pk + (size_t)task * V::PK, (size_t)V::PK, 0};
@@ -120,15 +120,16 @@ struct VerifyMuJob {
     }
 };
 
-// tr and mu of one task with a long message, a warp on the 25-lane form.
-template <int LEVEL, int SRC>
+// tr and mu of one task, a warp of a CTA of W on the 25-lane form.
+template <int LEVEL, int SRC, int W>
 __device__ __forceinline__ void verify_hash_wide(const VerifyBatch &b, int task, int lane) {
-    __shared__ __align__(16) uint8_t tr[32];
+    __shared__ __align__(16) uint8_t trs[W][32];
+    uint8_t *tr = trs[W > 1 ? threadIdx.x >> 5 : 0];
     using V = Lv<LEVEL>;
     int key;
     uint64_t m0;
     size_t mlen;
-    if (!verify_input<SRC>(b, task, key, m0, mlen) || mlen < b.long_bytes) return;
+    if (!verify_input<SRC>(b, task, key, m0, mlen)) return;
     uint32_t lo = 0, hi = 0;
     if (SRC == VERIFY_KEYED) {
         tr[lane] = b.key_tr[(size_t)key * 32 + lane];
@@ -146,16 +147,32 @@ __device__ __forceinline__ void verify_hash_wide(const VerifyBatch &b, int task,
 // The hashing warps, each a CTA of its own: they are chains (a 16 KB message is
 // 121 blocks, 3.4 us each on a warp of its own), so they get the registers to
 // keep a state and its input (at 64, a block took 4.5 us) and start first.
-// WIDE (hash_split): behind them a block per task, which hashes a long message on
-// the 25-lane form.
-template <int LEVEL, int SRC, bool WIDE>
+template <int LEVEL, int SRC>
 __global__ void __launch_bounds__(32, 16) k_verify_hash(const VerifyBatch b) {
     __shared__ __align__(16) uint32_t stage[HASH16_STAGE_WORDS];
-    if (!WIDE || blockIdx.x < b.hash_warps) {
-        VerifyMuJob<LEVEL, SRC> job(b, blockIdx.x * K16_STATES + (threadIdx.x >> 1), threadIdx.x);
-        hash16_run(job, stage, threadIdx.x);
+    VerifyMuJob<LEVEL, SRC> job(b, blockIdx.x * K16_STATES + (threadIdx.x >> 1), threadIdx.x);
+    hash16_run(job, stage, threadIdx.x);
+}
+
+// With wide warps for long messages (hash_split) behind them, four to a CTA, since
+// the batch's other kernels wait until all these CTAs have started.  The pairs'
+// warps have a CTA each, or (pair_ctas fewer than hash_warps) are four to a CTA,
+// which keeps them off most SMs once ExpandA fills all: 2,400 Dilithium2 tasks of
+// 1,000 bytes 191 -> 165 us, 3,000 of 16 KB 843 -> 658; but 800 of 1,000 bytes 119 ->
+// 128 and, with resident keys, 2,000 of 16 KB 506 -> 531.
+template <int LEVEL, int SRC>
+__global__ void __launch_bounds__(128, 4) k_verify_hash_both(const VerifyBatch b) {
+    __shared__ __align__(16) uint32_t stage[4][HASH16_STAGE_WORDS];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (blockIdx.x < b.pair_ctas) {
+        const int w = b.pair_ctas < b.hash_warps ? blockIdx.x * 4 + warp : warp ? b.hash_warps : blockIdx.x;
+        if (w >= b.hash_warps) return;
+        const int t = w * K16_STATES + (lane >> 1);   // the pair's only task
+        VerifyMuJob<LEVEL, SRC> job(b, has_wide_warp(b.off, b.n, t, b.long_bytes, b.per_group) ? b.n : t, lane);
+        hash16_run(job, stage[warp], lane);
     } else {
-        verify_hash_wide<LEVEL, SRC>(b, blockIdx.x - b.hash_warps, threadIdx.x);
+        const int task = task_of_wide_warp(b.off, b.n, (blockIdx.x - b.pair_ctas) * 4 + warp, b.long_bytes, b.per_group, lane);
+        if (task >= 0) verify_hash_wide<LEVEL, SRC, 4>(b, task, lane);
     }
 }
 
@@ -163,7 +180,7 @@ __global__ void __launch_bounds__(32, 16) k_verify_hash(const VerifyBatch b) {
 // above beside it thirteen Dilithium3 tasks take 92 us instead of 87.
 template <int LEVEL, int SRC>
 __global__ void __launch_bounds__(32) k_verify_hash_wide(const VerifyBatch b) {
-    verify_hash_wide<LEVEL, SRC>(b, blockIdx.x, threadIdx.x);
+    verify_hash_wide<LEVEL, SRC, 1>(b, blockIdx.x, threadIdx.x);
 }
 
 // c = SampleInBall(c~) of the signatures of tasks [first, first + 16), one warp.
@@ -390,22 +407,39 @@ __global__ void __launch_bounds__(32) k_verify_compare_wide(const VerifyBatch b)
 
 namespace {
 
-// Up to this many tasks everything has a warp (the hashes) or four (the rows) per
-// task.  The rows of so few tasks leave most of the GPU idle: with four warps
-// instead of one 13 tasks of 32 bytes on Dilithium5 keys take 55 us (70), 608 65
-// (77), 13 Dilithium2 verifies 60 (71); 609 and more beside ExpandA gain nothing.  Without sampling (a
-// resident key's or the caller's A^) the line is two hashing warps to a
-// sub-partition: 800 tasks of 4 KB on Dilithium2 keys 155 -> 138 us and 1,216 of 32
-// bytes 64 -> 56 with it at 1,216 instead of 608; at 1,824 1,700 Dilithium3 of 32
-// bytes 73 -> 80.
-constexpr int VERIFY_WIDE_MOST = HASH_WIDE_MOST, VERIFY_WIDE_MOST_RESIDENT = 1216;
+// The lines of hash_split.  Up to `all` tasks the rows, too, have four warps a task
+// and the comparison one: the rows of so few leave most of the GPU idle (13 tasks
+// of 32 bytes on Dilithium5 keys 70 us with one warp, 55 with four, 608 77 and 65,
+// 13 Dilithium2 verifies 71 and 60; 609 and more beside ExpandA gain nothing).
+// Without sampling (a resident key's or the caller's A^) that line is two hashing
+// warps to a sub-partition: 800 tasks of 4 KB on Dilithium2 keys 155 -> 138 us and
+// 1,216 of 32 bytes 64 -> 56 with it at 1,216 instead of 608; at 1,824 1,700
+// Dilithium3 of 32 bytes 73 -> 80.
+// Beside sampling warps two threads to a state are slowed more, so shorter
+// messages and larger batches have wide warps: Dilithium3 up to 4 KB 609, 1,000 and
+// 1,824 tasks 244, 262, 364 -> 210, 248, 316 us with the line at 2 KB instead of 8;
+// Dilithium2 of 4 KB 609 203 -> 187, 1,250 215 -> 219, 1,500 217 -> 233.  Once the
+// sampling warps alone fill the GPU the hashing ones start late: 2,400 Dilithium2
+// of 16 KB 824 -> 660 us with a warp each, 2,000 599 -> 643.
+constexpr int FULL_GPU = 152 * 16;   // sampling warps
+template <int LEVEL> bool sampling_fills_gpu(int n) {
+    return (long long)n * Lv<LEVEL>::K * Lv<LEVEL>::L > (FULL_GPU - 152LL) * K16_STATES;
+}
+template <int LEVEL, int SRC>
+HashLines verify_lines(int n) {
+    if (SRC != VERIFY_PLAIN) return {1216, HASH_LONG_MOST, HASH_FEW_MOST, HASH_LONG_BYTES};
+    return {HASH_WIDE_MOST, sampling_fills_gpu<LEVEL>(n) ? FULL_GPU : 1824, HASH_FEW_MOST_SAMPLING,
+            LEVEL == 2 && n > 1250 ? HASH_LONG_BYTES : HASH_LONG_BYTES / 4};
+}
 
 template <int LEVEL, int SRC>
 cudaError_t launch_batch(VerifyBatch b, const VerifyFork &f, cudaStream_t s) {
-    const int most = SRC == VERIFY_PLAIN ? VERIFY_WIDE_MOST : VERIFY_WIDE_MOST_RESIDENT;
-    const HashSplit split = hash_split(b.n, b.n, most, SRC == VERIFY_PLAIN ? HASH_LONG_MOST_SAMPLING : HASH_LONG_MOST);
+    const int most = verify_lines<LEVEL, SRC>(b.n).all;
+    const HashSplit split = hash_split(b.n, b.n, verify_lines<LEVEL, SRC>(b.n));
     b.hash_warps = split.warps;
     b.long_bytes = split.long_bytes;
+    b.per_group = split.per_group;
+    b.pair_ctas = SRC == VERIFY_PLAIN && sampling_fills_gpu<LEVEL>(b.n) ? (split.warps + 3) / 4 : split.warps;
     b.challenge_blocks = (b.n + K16_STATES - 1) / K16_STATES;
     const cudaStream_t hs = f.stream ? f.stream : s;
     cudaError_t e = cudaSuccess;
@@ -418,9 +452,9 @@ cudaError_t launch_batch(VerifyBatch b, const VerifyFork &f, cudaStream_t s) {
     if (!split.warps)
         k_verify_hash_wide<LEVEL, SRC><<<split.wide, 32, 0, hs>>>(b);
     else if (split.wide)
-        k_verify_hash<LEVEL, SRC, true><<<split.warps + split.wide, 32, 0, hs>>>(b);
+        k_verify_hash_both<LEVEL, SRC><<<b.pair_ctas + (split.wide + 3) / 4, 128, 0, hs>>>(b);
     else
-        k_verify_hash<LEVEL, SRC, false><<<split.warps, 32, 0, hs>>>(b);
+        k_verify_hash<LEVEL, SRC><<<split.warps, 32, 0, hs>>>(b);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const long long polys = SRC == VERIFY_PLAIN ? (long long)b.n * Lv<LEVEL>::K * Lv<LEVEL>::L : 0;
     k_verify_sample<LEVEL><<<b.challenge_blocks + (int)((polys + K16_STATES - 1) / K16_STATES), 32, 0, s>>>(b);

@@ -48,6 +48,9 @@ def test_hash_whose_input_is_the_hash_before(torch_cuda, orc, level):
 # at 8,192 bytes and around it), and the two-thread form alone
 SPLITS = [(3, [8191, 70000, 0]), (608, [40, 8192, 300]), (609, [8191, 8192, 8193, 32]), (1520, [0, 9000, 40, 16384]),
           (1521, [8192, 31]), (1824, [32, 12345]), (1825, [8192, 1])]
+# few long messages of sixteen, or too many, around the lines of that rule
+FEW, MANY = [9000] + [40] * 15, [8192] * 9 + [40] * 7
+SPLITS += [(1217, MANY), (1825, FEW), (2400, MANY), (2433, FEW), (3072, MANY + FEW), (3073, FEW), (6144, FEW), (6145, FEW)]
 
 
 @pytest.mark.parametrize("level", LEVELS)
