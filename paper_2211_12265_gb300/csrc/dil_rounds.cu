@@ -30,6 +30,7 @@
 // What bounds the phases at 20,000 Dilithium2 attempts: mask the ALU pipe (87%),
 // prepare and hash the same (75%), front DRAM (69% of the copy rate), back its
 // issue slots (51%, the multiplier 51% of its rate; 20 of 32 warps).
+#include <algorithm>
 #include <climits>
 
 #include "dil_kern.cuh"
@@ -758,12 +759,17 @@ __global__ void __launch_bounds__(128) k_sign_back_wide(const SignBatch b, int r
 // ---------------------------------------------------------------- what is left
 // The plain loop over the tasks still unfinished after round r - 1, from
 // round r's first repetition on, one task per warp; the slots are its scratch.
+// Of valid keys it is a task now and then; a damaged key may hold its task here
+// for thousands of repetitions, and such tasks may be a whole batch, so there are
+// as many warps as tasks, slots and the GPU allow (704 Dilithium2 tasks that hardly
+// ever accept, up to 400 repetitions: 204 ms on 64 warps, 26 with two warps to each,
+// 22 with one; 10,000: 823, 259, 130).
 template <int LEVEL, int SRC>
 __global__ void __launch_bounds__(256, 4) k_sign_rest(const SignBatch b, int r, int workers) {
     extern __shared__ __align__(16) uint8_t smem[];
     using V = Lv<LEVEL>;
+    if (b.count[r] <= 0) return;
     const Round q = round_of(b, r);
-    if (q.p <= 0) return;
     const CtaView v = cta_setup<1>(smem);
     const int w = blockIdx.x * v.groups + v.group;
     if (w >= workers) return;
@@ -907,8 +913,8 @@ cudaError_t launch_rounds(SignBatch b, void *ws, cudaStream_t s) {
             k_sign_back<LEVEL, SRC><<<blocks_for(most, ROUND_WARPS), 32 * ROUND_WARPS, 0, s>>>(b, r);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    const size_t room = (size_t)b.slots * Slot<LEVEL>::POLYS / Scratch<LEVEL>::ITR_POLYS;
-    const int workers = (int)(room < 64 ? room : 64), ctas = blocks_for(workers, 4);
+    const long long room = (long long)b.slots * Slot<LEVEL>::POLYS / Scratch<LEVEL>::ITR_POLYS, gpu = 152 * 16;
+    const int workers = (int)std::min({room, gpu, (long long)b.n}), ctas = blocks_for(workers, 4);
     const size_t rest_smem = cta_bytes(4, 1);
     if ((e = dynamic_smem(k_sign_rest<LEVEL, SRC>, rest_smem)) != cudaSuccess) return e;
     k_sign_rest<LEVEL, SRC><<<ctas, 128, rest_smem, s>>>(b, rounds, workers);

@@ -232,3 +232,73 @@ def test_keyed_verify_of_short_messages_is_no_slower_than_fused(torch_cuda):
             took[shape] = sorted(ts)[4]
             dil.dil_keystore_destroy(ks)
     assert took[None] < 1.05 * took[(8, 2)], took
+
+
+def _stubborn_keys(orc, level, n, seed):
+    """Secret keys whose t0 has only the two extreme values: the hint has too many
+    ones in all but about one repetition of a thousand (Dilithium2)."""
+    pk, sk = orc.keygen_batch(level, W.seeds(n, seed))
+    k = {2: 4, 3: 6, 5: 8}[level]
+    fields = np.random.default_rng(seed).integers(0, 2, (n, 256 * k, 1), dtype=np.uint8)
+    sk[:, -416 * k:] = np.packbits(np.broadcast_to(fields, (n, 256 * k, 13)).reshape(n, -1), axis=1, bitorder="little")
+    return sk
+
+
+def test_many_tasks_that_no_round_settles(torch_cuda, orc):
+    """A batch whose keys (damaged ones) almost never accept is signed by the loop
+    behind the rounds, on as many warps as the GPU holds: eleven times
+    the tasks of a batch that leaves most of it idle take less than four times as
+    long (the rounds before it included)."""
+    import time
+    from gpu_util import dev, host
+    from paper_2211_12265_gb300 import dil
+    torch = torch_cuda
+    m, cap = 8, 400
+    sk = _stubborn_keys(orc, 2, m, 1080)
+    msg, off = W.messages(np.full(m, 32), 1080)
+    osig, ost, oit = orc.sign_batch(2, sk, msg, off.astype(np.uint64), max_iter=cap)
+    assert (ost == dil.EITER).sum() > m // 2
+    took = {}
+    with dil.Context(0) as ctx:
+        ctx.set_max_iter(cap)
+        for n in (64, 704):
+            pick = np.arange(n) % m
+            d_sk, d_off = dev(sk[pick]), dev((np.arange(n + 1) * 32).astype(np.uint64))
+            d_msg = dev(np.concatenate([msg[off[i]:off[i + 1]] for i in pick]))
+            ts = []
+            for _ in range(3):
+                torch.cuda.synchronize()
+                t = time.perf_counter()
+                sig, st, it = ctx.sign(2, d_sk, d_msg, d_off, iterations=True)
+                torch.cuda.synchronize()
+                ts.append(time.perf_counter() - t)
+            took[n] = min(ts)
+            assert np.array_equal(host(st), ost[pick]) and np.array_equal(host(it), oit[pick])
+            assert np.array_equal(host(sig), osig[pick])
+    assert took[704] < 4 * took[64], took
+
+
+@pytest.mark.parametrize("level", LEVELS)
+def test_leftover_tasks_of_a_batch(torch_cuda, orc, level):
+    """The loop behind the rounds on several tasks at a time, resident keys and a
+    workspace of few slots included."""
+    from gpu_util import dev, host
+    from paper_2211_12265_gb300 import dil
+    torch = torch_cuda
+    n, cap = 21, 90
+    sk = _stubborn_keys(orc, level, n, 1090)
+    pk, _ = orc.keygen_batch(level, W.seeds(n, 1090))
+    msg, off = W.messages(np.full(n, 50), 1090)
+    off = off.astype(np.uint64)
+    osig, ost, oit = orc.sign_batch(level, sk, msg, off, max_iter=cap)
+    for budget in (0, 6 << 20):
+        with dil.Context(0, workspace_budget=budget) as ctx:
+            ctx.set_max_iter(cap)
+            sig, st, it = (host(x) for x in ctx.sign(level, dev(sk), dev(msg), dev(off), iterations=True))
+            ks = dil.dil_keystore_create(ctx.handle, level, n, dev(pk), dev(sk))
+            ksig, kst = torch.zeros_like(dev(osig)), dev(np.full(n, 9, np.int32))
+            dil.dil_sign_keyed(ctx.handle, ks, n, dev(np.arange(n, dtype=np.int32)), dev(msg), dev(off), ksig, kst)
+            ksig, kst = host(ksig), host(kst)
+            dil.dil_keystore_destroy(ks)
+        assert np.array_equal(sig, osig) and np.array_equal(st, ost) and np.array_equal(it, oit)
+        assert np.array_equal(ksig, osig) and np.array_equal(kst, ost)
