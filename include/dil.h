@@ -190,8 +190,14 @@ typedef struct {
 } dil_sign_job;
 
 /* Enqueues one persistent Sign launch on `stream` for njobs (1..3) jobs.  The
- * context's repetition cap (dil_set_max_iter) applies.  Uses the context's
- * workspace; calls on one context must not overlap on the GPU.  The launch is
+ * context's repetition cap (dil_set_max_iter) applies.  Calls on one context
+ * must not overlap on the GPU.  The launch has a workspace of its own, up to the
+ * budget and held until a launch needs a larger one or the context is destroyed:
+ * in rounds for four parts of at most 16,384 tasks at a time, about 45, 70 and 110
+ * KB a task by level (3.6 GiB for 40,000 Dilithium5 tasks), on the queue for its
+ * resident warp groups and 32 bytes a task (about 0.2 GiB).  Where the device
+ * refuses a launch in rounds its workspace, the parts get smaller; before they
+ * need less than the queue does, the launch runs on that, if it gets so much.  The launch is
  * asynchronous and reads the jobs' device buffers while it runs: they must
  * stay allocated until the stream has passed the launch (the descriptors are
  * copied, the buffers are not).  A CUDA graph of the launch is cached and
@@ -203,7 +209,7 @@ int dil_sign_persistent(dil_ctx *ctx, int njobs, const dil_sign_job *jobs, void 
  * access (>= 1), helper groups per unfinished task (0 disables speculation).
  * The device queue's shape: with one warp per task group, or without this call,
  * the launch runs in rounds (on the queue, in the shape 8, 2, 0, 1, 4 or the one
- * set, where the workspace budget does not hold a round). */
+ * set, where the workspace budget or the device does not hold them). */
 int dil_set_persistent_tuning(dil_ctx *ctx, int warps_per_cta, int warps_per_task, int ctas_per_sm, int chunk,
                               int speculation);
 
@@ -442,6 +448,10 @@ int dil_test_rounding(dil_ctx *ctx, int level, size_t n, const int32_t *r, const
  * under ordinary contention, so tests can check the per-task DIL_ETIMEOUT
  * path.  DIL_EINVAL outside that range. */
 int dil_test_set_spin_limit(dil_ctx *ctx, int limit);
+
+/* Failure-detection hook: persistent workspaces of more than `bytes` count as
+ * refused by the device from now on (0: none does), as if memory were short. */
+int dil_test_set_alloc_limit(dil_ctx *ctx, size_t bytes);
 
 /* Failure-detection hook: runs the persistent scheduler's bounded device wait
  * (poll until a flag reads 0, at most `limit` polls of ~128 ns) on a flag set

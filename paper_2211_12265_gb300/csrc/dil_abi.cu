@@ -35,11 +35,12 @@ struct dil_ctx {
     cudaGraphExec_t gexec = nullptr;
     dil::PersistJobs gjobs{};
     dil::PersistTuning gtune;
-    bool grounds = false;     // the captured launch runs in rounds
+    bool gwish = false;       // it was to run in rounds
     int gmax_iter = -1;
     int spin_limit = 0;       // polls per bounded device wait (0 = PERSIST_SPIN_LIMIT); tests lower it
     int gspin_limit = -1;
     void *gws = nullptr;
+    size_t alloc_limit = 0;   // larger persistent workspaces count as refused (0: none); a test sets it
     // host-form pipeline: extra streams and the fork / join events
     cudaStream_t aux[3] = {nullptr, nullptr, nullptr};
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -598,12 +599,12 @@ namespace {
 constexpr size_t PART_MOST = 16384;
 struct RoundPlan {
     RoundSize size[dil::PERSIST_MAX_JOBS];
-    size_t region = 0, bytes = 0;   // a stream's workspace, the launch's (0: does not fit the budget)
+    size_t region = 0, bytes = 0;   // a stream's workspace, the launch's (0: does not fit)
 };
 
-RoundPlan round_plan(const dil_ctx *c, const dil::PersistJobs &J) {
+RoundPlan round_plan(const dil::PersistJobs &J, size_t bytes) {
     RoundPlan p;
-    const size_t budget = c->budget > dil::PERSIST_HEADER_BYTES ? (c->budget - dil::PERSIST_HEADER_BYTES) / PIPE_STREAMS : 0;
+    const size_t budget = bytes > dil::PERSIST_HEADER_BYTES ? (bytes - dil::PERSIST_HEADER_BYTES) / PIPE_STREAMS : 0;
     for (int j = 0; j < J.njobs; ++j) {
         const size_t n = J.job[j].n;
         if (n == 0) continue;
@@ -614,6 +615,36 @@ RoundPlan round_plan(const dil_ctx *c, const dil::PersistJobs &J) {
                                                             p.size[j].slots));
     }
     p.bytes = dil::PERSIST_HEADER_BYTES + PIPE_STREAMS * p.region;
+    return p;
+}
+
+// Ensures `bytes` of persistent workspace; DIL_ENOMEM when the device refuses it
+// (the context then holds none).
+int ensure_pws(dil_ctx *c, size_t bytes) {
+    if (bytes <= c->pws_bytes) return DIL_OK;
+    if (c->pws) {
+        cudaDeviceSynchronize();
+        if (c->gexec) cudaGraphExecDestroy(c->gexec);   // of the old address, which a smaller workspace may get
+        c->gexec = nullptr;
+        cudaFree(c->pws);
+        c->pws = nullptr;
+        c->pws_bytes = 0;
+    }
+    if ((c->alloc_limit && bytes > c->alloc_limit) || cudaMalloc(&c->pws, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        c->pws = nullptr;
+        return DIL_ENOMEM;
+    }
+    c->pws_bytes = bytes;
+    return DIL_OK;
+}
+
+// A plan of rounds within `bytes` and its workspace; where the device refuses that
+// much, half as much at a time while that is `least` or more.
+RoundPlan planned_rounds(dil_ctx *c, const dil::PersistJobs &J, size_t bytes, size_t least) {
+    RoundPlan p = round_plan(J, bytes);
+    while (p.bytes && ensure_pws(c, p.bytes) != DIL_OK)
+        p = p.bytes / 2 < least ? RoundPlan{} : round_plan(J, p.bytes / 2);
     return p;
 }
 
@@ -682,59 +713,48 @@ int dil_sign_persistent(dil_ctx *c, int njobs, const dil_sign_job *jobs, void *s
     if (total == 0) return DIL_OK;
     std::lock_guard<std::mutex> lk(c->mu);
     DeviceGuard g(c->device);
+    // SMs per job in proportion to its work (a task's relative cost by level:
+    // persistent Sign rates 3.65 / 2.42 / 1.98 M/s at 10,000 tasks)
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) return DIL_ECUDA;
+    double w[dil::PERSIST_MAX_JOBS], sum = 0;
+    for (int j = 0; j < njobs; ++j) {
+        const int lv = J.job[j].level;
+        w[j] = (double)J.job[j].n * (lv == 2 ? 1.0 : lv == 3 ? 1.51 : 1.84);
+        sum += w[j];
+    }
+    double acc = 0;
+    for (int j = 0; j < njobs; ++j) {
+        acc += w[j];
+        J.sm_end[j] = j + 1 == njobs ? (1 << 30) : (int)(sms * acc / sum + 0.5);
+    }
     // One-warp launches run in rounds; shapes of two or four warps per task, a
-    // budget too small for a round, and the hook that makes bounded waits run out
-    // keep the device queue.
-    RoundPlan plan;
-    if (!(c->ptune_set && c->ptune.p > 1) && c->spin_limit == 0) plan = round_plan(c, J);
-    const bool rounds = plan.bytes != 0;
-    if (!rounds) {   // SMs per job in proportion to its work (a task's relative cost by level:
-                     // persistent Sign rates 3.65 / 2.42 / 1.98 M/s at 10,000 tasks)
-        int sms = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) return DIL_ECUDA;
-        double w[dil::PERSIST_MAX_JOBS], sum = 0;
-        for (int j = 0; j < njobs; ++j) {
-            const int lv = J.job[j].level;
-            w[j] = (double)J.job[j].n * (lv == 2 ? 1.0 : lv == 3 ? 1.51 : 1.84);
-            sum += w[j];
-        }
-        double acc = 0;
-        for (int j = 0; j < njobs; ++j) {
-            acc += w[j];
-            J.sm_end[j] = j + 1 == njobs ? (1 << 30) : (int)(sms * acc / sum + 0.5);
-        }
-    }
-    const size_t need = rounds ? plan.bytes : dil::persist_workspace_bytes(J, c->ptune, c->device);
-    if (need == 0) return DIL_ECUDA;
-    if (need > c->budget) return DIL_ENOMEM;
-    if (rounds) {
-        const int rc = ensure_aux(c);
-        if (rc) return rc;
-    }
-    if (need > c->pws_bytes) {
-        if (c->pws) {
-            cudaDeviceSynchronize();
-            cudaFree(c->pws);
-            c->pws = nullptr;
-            c->pws_bytes = 0;
-        }
-        if (cudaMalloc(&c->pws, need) != cudaSuccess) {
-            cudaGetLastError();
-            return DIL_ENOMEM;
-        }
-        c->pws_bytes = need;
-    }
+    // budget or device memory too small for a round, and the hook that makes
+    // bounded waits run out keep the device queue.
+    const bool wish = !(c->ptune_set && c->ptune.p > 1) && c->spin_limit == 0;
     const int max_iter = c->max_iter;
     if (!c->gexec || !same_jobs(J, c->gjobs) || !same_tune(c->ptune, c->gtune) || max_iter != c->gmax_iter ||
-        c->spin_limit != c->gspin_limit || rounds != c->grounds || c->gws != c->pws) {
+        c->spin_limit != c->gspin_limit || wish != c->gwish || c->gws != c->pws) {
+        // (this also warms the attribute / occupancy queries outside the capture)
+        const size_t queue = dil::persist_workspace_bytes(J, c->ptune, c->device);
+        RoundPlan plan = wish ? planned_rounds(c, J, c->budget, queue) : RoundPlan{};
+        if (plan.bytes == 0) {
+            if (queue == 0) return DIL_ECUDA;
+            const int rc = queue > c->budget ? DIL_ENOMEM : ensure_pws(c, queue);
+            if (rc && wish) plan = planned_rounds(c, J, std::min(queue, c->budget), 0);
+            if (rc && plan.bytes == 0) return rc;
+        }
+        const bool rounds = plan.bytes != 0;
+        if (rounds) {
+            const int rc = ensure_aux(c);
+            if (rc) return rc;
+        }
         if (c->gexec) {
             cudaGraphExecDestroy(c->gexec);
             c->gexec = nullptr;
         }
         if (!c->cap_stream && cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
             return DIL_ECUDA;
-        // warm the attribute / occupancy queries outside the capture
-        if (!rounds && dil::persist_workspace_bytes(J, c->ptune, c->device) == 0) return DIL_ECUDA;
         cudaGraph_t graph = nullptr;
         if (cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) return DIL_ECUDA;
         cudaError_t e = rounds ? launch_rounds(c, J, plan, c->cap_stream)
@@ -756,7 +776,7 @@ int dil_sign_persistent(dil_ctx *c, int njobs, const dil_sign_job *jobs, void *s
         c->gtune = c->ptune;
         c->gmax_iter = max_iter;
         c->gspin_limit = c->spin_limit;
-        c->grounds = rounds;
+        c->gwish = wish;
         c->gws = c->pws;
     }
     return cudaGraphLaunch(c->gexec, (cudaStream_t)stream) == cudaSuccess ? DIL_OK : DIL_ECUDA;
@@ -1247,6 +1267,12 @@ int dil_test_set_spin_limit(dil_ctx *c, int limit) {
     TEST_PROLOGUE(c)
     if (limit < 0 || limit > dil::PERSIST_SPIN_LIMIT) return DIL_EINVAL;
     c->spin_limit = limit;
+    return DIL_OK;
+}
+
+int dil_test_set_alloc_limit(dil_ctx *c, size_t bytes) {
+    TEST_PROLOGUE(c)
+    c->alloc_limit = bytes;
     return DIL_OK;
 }
 

@@ -79,7 +79,7 @@ def load() -> ctypes.CDLL:
                 "dil_test_keccak_rate": [P, I, P],
                 "dil_test_sign_split": [P, I, S, P, P, P, P, P, P, P, P],
                 "dil_test_bounded_wait": [P, I, I, P],
-                "dil_test_set_spin_limit": [P, I],
+                "dil_test_set_spin_limit": [P, I], "dil_test_set_alloc_limit": [P, S],
                 "dil_sign_persistent": [P, I, P, P],
                 "dil_set_persistent_tuning": [P, I, I, I, I, I],
                 "dil_persistent_status": [P, P],
@@ -332,6 +332,11 @@ def dil_test_bounded_wait(ctx, flag_value: int, limit: int) -> int:
 def dil_test_set_spin_limit(ctx, limit: int) -> None:
     """Polls per bounded device wait of later persistent launches (0 = default)."""
     _check(load().dil_test_set_spin_limit(ctx, int(limit)), "dil_test_set_spin_limit")
+
+
+def dil_test_set_alloc_limit(ctx, nbytes: int) -> None:
+    """Persistent workspaces of more than nbytes count as refused by the device (0: none)."""
+    _check(load().dil_test_set_alloc_limit(ctx, int(nbytes)), "dil_test_set_alloc_limit")
 
 
 ISSUE_OPS = {"lop3": 0, "shf": 1, "imul": 2, "imul_hi": 3, "shfl": 4}

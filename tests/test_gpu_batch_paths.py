@@ -302,3 +302,53 @@ def test_leftover_tasks_of_a_batch(torch_cuda, orc, level):
             dil.dil_keystore_destroy(ks)
         assert np.array_equal(sig, osig) and np.array_equal(st, ost) and np.array_equal(it, oit)
         assert np.array_equal(ksig, osig) and np.array_equal(kst, ost)
+
+
+def _persistent(torch, dil, ctx, jobs):
+    """One persistent launch of (level, sk, msg, off) jobs on the device: per job
+    signatures, statuses and repetitions."""
+    outs, descs = [], []
+    for level, sk, msg, off in jobs:
+        n = sk.shape[0]
+        o = (torch.full((n, dil.SIZES[level][2]), 0x5A, dtype=torch.uint8, device="cuda"),
+             torch.full((n,), 9, dtype=torch.int32, device="cuda"), torch.zeros(n, dtype=torch.int32, device="cuda"))
+        outs.append(o)
+        descs.append(dil.sign_job(level, n, sk, msg, off, *o))
+    dil.dil_sign_persistent(ctx.handle, descs)
+    assert dil.dil_persistent_status(ctx.handle) == dil.OK
+    return [tuple(x.cpu().numpy() for x in o) for o in outs]
+
+
+def test_persistent_launch_where_memory_is_short(torch_cuda):
+    """A device that refuses the rounds' workspace: smaller parts, then the device
+    queue, then smaller parts still, and DIL_ENOMEM only where nothing fits; the
+    context is usable throughout and outputs are the same."""
+    from gpu_util import dev
+    from paper_2211_12265_gb300 import dil
+    torch = torch_cuda
+    jobs, want = [], []
+    with dil.Context(0) as ctx:
+        for level, n in ((2, 5000), (5, 3001)):
+            _, sk = ctx.keygen(level, dev(W.seeds(n, 1100 + level)))
+            msg, off = W.messages(np.full(n, 32), 1100 + level)
+            jobs.append((level, sk, dev(msg), dev(off.astype(np.uint64))))
+            want.append([x.cpu().numpy() for x in ctx.sign(*jobs[-1], iterations=True)])
+    mib = 1 << 20
+    # rounds take 388 MiB (both jobs), and 194, 97, 48 ...; the queue in this shape 74
+    for limit in (700 * mib, 250 * mib, 100 * mib, 80 * mib, 60 * mib, 10 * mib):
+        with dil.Context(0) as ctx:
+            dil.dil_set_persistent_tuning(ctx.handle, 4, 1, 1, 1, 4)
+            dil.dil_test_set_alloc_limit(ctx.handle, limit)
+            for part in (jobs[:1], jobs, jobs[:1]):   # a larger workspace, refused; argument sets in turn
+                got = _persistent(torch, dil, ctx, part)
+                for g, w in zip(got, want):
+                    assert all(np.array_equal(a, b) for a, b in zip(g, w)), limit
+    with dil.Context(0) as ctx:
+        dil.dil_test_set_alloc_limit(ctx.handle, 1)
+        with pytest.raises(dil.DilError) as e:
+            _persistent(torch, dil, ctx, jobs)
+        assert str(dil.ENOMEM) in str(e.value)
+        dil.dil_test_set_alloc_limit(ctx.handle, 0)
+        got = _persistent(torch, dil, ctx, jobs)
+        for g, w in zip(got, want):
+            assert all(np.array_equal(a, b) for a, b in zip(g, w))
