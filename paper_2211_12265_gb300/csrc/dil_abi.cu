@@ -595,7 +595,8 @@ bool same_tune(const dil::PersistTuning &a, const dil::PersistTuning &b) {
 namespace {
 // A persistent launch in rounds: each job in parts, the parts dealt over the four
 // streams; a part's workspace serves one after the other.  At most PART_MOST
-// tasks a part: a cancel ends the parts that have not started at once.
+// tasks a part: what is in flight when a cancel arrives runs on, everything behind
+// it leaves its work out.
 constexpr size_t PART_MOST = 16384;
 struct RoundPlan {
     RoundSize size[dil::PERSIST_MAX_JOBS];

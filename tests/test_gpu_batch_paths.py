@@ -352,3 +352,47 @@ def test_persistent_launch_where_memory_is_short(torch_cuda):
         got = _persistent(torch, dil, ctx, jobs)
         for g, w in zip(got, want):
             assert all(np.array_equal(a, b) for a, b in zip(g, w))
+
+
+@pytest.mark.parametrize("delay", [0.0, 0.004])
+def test_cancel_ends_a_launch_in_rounds_at_once(torch_cuda, delay):
+    """Once the cancel word is written, nothing that a later part or round would
+    still sample, transform or check runs: the launch ends in a quarter of its
+    time, and every task is either signed as before or canceled, whatever kernel
+    saw the word first."""
+    import time
+    from gpu_util import dev
+    from paper_2211_12265_gb300 import dil
+    torch = torch_cuda
+    n = 600_000   # about 38 parts of 16,384 tasks
+    with dil.Context(0) as ctx:
+        _, sk = ctx.keygen(2, dev(W.seeds(n, 1110)))
+        msg, off = W.messages(np.full(n, 32), 1110)
+        d_msg, d_off = dev(msg), dev(off.astype(np.uint64))
+        sig = torch.zeros((n, dil.SIZES[2][2]), dtype=torch.uint8, device="cuda")
+        st = torch.zeros(n, dtype=torch.int32, device="cuda")
+        it = torch.zeros(n, dtype=torch.int32, device="cuda")
+        job = [dil.sign_job(2, n, sk, d_msg, d_off, sig, st, it)]
+        dil.dil_sign_persistent(ctx.handle, job)
+        assert dil.dil_persistent_status(ctx.handle) == dil.OK
+        t = time.perf_counter()
+        dil.dil_sign_persistent(ctx.handle, job)
+        assert dil.dil_persistent_status(ctx.handle) == dil.OK
+        whole = time.perf_counter() - t
+        want_sig, want_it = sig.clone(), it.clone()
+        dil.dil_persistent_cancel(ctx.handle)   # its stream exists from here on
+        sig.fill_(0x5A)
+        st.fill_(9)
+        it.fill_(7)
+        torch.cuda.synchronize()
+        dil.dil_sign_persistent(ctx.handle, job)
+        time.sleep(delay)
+        dil.dil_persistent_cancel(ctx.handle)
+        t = time.perf_counter()
+        assert dil.dil_persistent_status(ctx.handle) == dil.ECANCELED
+        rest = time.perf_counter() - t
+        ok, gone = st == dil.OK, st == dil.ECANCELED
+        assert bool((ok | gone).all()) and int(gone.sum()) > n // 2
+        assert torch.equal(sig[ok], want_sig[ok]) and torch.equal(it[ok], want_it[ok])
+        assert not bool(sig[gone].any()) and not bool(it[gone].any())
+    assert rest < whole / 4, (rest, whole)
