@@ -420,6 +420,12 @@ int dil_test_t0_ntt(dil_ctx *ctx, int level, int variant, size_t n, const uint8_
 int dil_test_ntt(dil_ctx *ctx, size_t n, const int32_t *in, int32_t *out, int inverse, void *stream);
 /* ExpandA of n seeds rho (n x 32 bytes) -> n x k x l x 256 int32 in [0, q). */
 int dil_test_expand_a(dil_ctx *ctx, int level, size_t n, const uint8_t *rho, int32_t *ahat, void *stream);
+/* As dil_test_expand_a by the batch's sampler with one squeezed block too few, so
+ * that it samples every polynomial again; lane_order: in the order of the
+ * library's own A^ (words 4 t .. 4 t + 3 hold coefficients 8 t .. 8 t + 3, words
+ * 128 + 4 t .. those four behind). */
+int dil_test_expand_a_refill(dil_ctx *ctx, int level, size_t n, const uint8_t *rho, int lane_order, int32_t *ahat,
+                             void *stream);
 /* ExpandS of n seeds rho' (n x 64 bytes) -> n x (l + k) x 256 int32 (s1 then s2). */
 int dil_test_expand_s(dil_ctx *ctx, int level, size_t n, const uint8_t *rhop, int32_t *s, void *stream);
 /* ExpandMask of n (rho', kappa) pairs -> n x l x 256 int32. */

@@ -1224,6 +1224,13 @@ int dil_test_expand_a(dil_ctx *c, int level, size_t n, const uint8_t *rho, int32
     return status_of(dil::launch_test_expand_a(level, (int)n, rho, ahat, (cudaStream_t)stream));
 }
 
+int dil_test_expand_a_refill(dil_ctx *c, int level, size_t n, const uint8_t *rho, int lane_order, int32_t *ahat,
+                             void *stream) {
+    TEST_PROLOGUE(c)
+    if (!level_ok(level) || n > (size_t)INT32_MAX || (n && (!rho || !ahat))) return DIL_EINVAL;
+    return status_of(dil::launch_test_expand_a_refill(level, (int)n, rho, !lane_order, ahat, (cudaStream_t)stream));
+}
+
 int dil_test_expand_s(dil_ctx *c, int level, size_t n, const uint8_t *rhop, int32_t *s, void *stream) {
     TEST_PROLOGUE(c)
     if (!level_ok(level) || n > (size_t)INT32_MAX || (n && (!rhop || !s))) return DIL_EINVAL;

@@ -11,11 +11,11 @@ namespace dil {
 
 // A^ of task t at ahat + t k l N, polynomial (i, j) at index i l + j,
 // coefficients in index order, each in [0, q).
-template <int LEVEL>
+template <int LEVEL, bool INDEX = true, int BLOCKS = 5>
 __global__ void __launch_bounds__(32, 16) k_expand_a(int n, const uint8_t *rho, size_t rho_stride, int32_t *ahat) {
     __shared__ __align__(16) uint32_t st[EXPAND16_WORDS];
     constexpr int KL = Lv<LEVEL>::K * Lv<LEVEL>::L;
-    expand_a_batch<LEVEL, true>((long long)blockIdx.x * K16_STATES, (long long)n * KL,
+    expand_a_batch<LEVEL, INDEX, BLOCKS>((long long)blockIdx.x * K16_STATES, (long long)n * KL,
                                 [&](int t) { return rho + (size_t)t * rho_stride; },
                                 [&](int t) { return ahat + (size_t)t * KL * N; }, st, threadIdx.x);
 }
@@ -63,11 +63,11 @@ __global__ void __launch_bounds__(256, 4) k_sign_a(int n, const uint8_t *__restr
     }
 }
 
-template <int LEVEL>
+template <int LEVEL, bool INDEX = true, int BLOCKS = 5>
 static cudaError_t launch_expand(int n, const uint8_t *rho, size_t rho_stride, int32_t *ahat, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const long long polys = (long long)n * Lv<LEVEL>::K * Lv<LEVEL>::L;
-    k_expand_a<LEVEL><<<(int)((polys + K16_STATES - 1) / K16_STATES), 32, 0, s>>>(n, rho, rho_stride, ahat);
+    k_expand_a<LEVEL, INDEX, BLOCKS><<<(int)((polys + K16_STATES - 1) / K16_STATES), 32, 0, s>>>(n, rho, rho_stride, ahat);
     return cudaGetLastError();
 }
 
@@ -76,6 +76,15 @@ cudaError_t launch_expand_a(int level, int n, const uint8_t *rho, size_t rho_str
         case 2: return launch_expand<2>(n, rho, rho_stride, ahat, s);
         case 3: return launch_expand<3>(n, rho, rho_stride, ahat, s);
         case 5: return launch_expand<5>(n, rho, rho_stride, ahat, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_test_expand_a_refill(int level, int n, const uint8_t *rho, bool index, int32_t *ahat, cudaStream_t s) {
+    switch (level) {
+        case 2: return index ? launch_expand<2, true, 4>(n, rho, 32, ahat, s) : launch_expand<2, false, 4>(n, rho, 32, ahat, s);
+        case 3: return index ? launch_expand<3, true, 4>(n, rho, 32, ahat, s) : launch_expand<3, false, 4>(n, rho, 32, ahat, s);
+        case 5: return index ? launch_expand<5, true, 4>(n, rho, 32, ahat, s) : launch_expand<5, false, 4>(n, rho, 32, ahat, s);
     }
     return cudaErrorInvalidValue;
 }

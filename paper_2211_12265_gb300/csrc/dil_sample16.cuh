@@ -16,7 +16,8 @@ constexpr int EXPAND16_WORDS = K16_STATES * EXPAND16_STRIDE + 8;
 // ExpandA over a batch: polynomials [first, first + 16) of the `total` = tasks
 // k l polynomials, numbered task by task, one warp.  seed_of(t): the 32 bytes
 // of task t's rho (global memory, any alignment); out_of(t): task t's A^, in
-// index order with INDEX, else in lane order.
+// index order with INDEX, else in lane order.  BLOCKS: squeezed blocks taken at
+// once (a test takes four, which never fill a polynomial).
 // The states stay in registers over the five permutations; the blocks of all
 // go to shared memory, and a lane then takes candidates lane + 32 m of one
 // stream: 24 bits times 32 are whole words, so its shift is fixed and its
@@ -24,7 +25,7 @@ constexpr int EXPAND16_WORDS = K16_STATES * EXPAND16_STRIDE + 8;
 // time, took a quarter of ExpandA's time.)  A stream of 280 candidates leaves
 // fewer than 256 with probability below 1e-30; such a polynomial is sampled
 // again by the form that squeezes until it has enough.
-template <int LEVEL, bool INDEX, class Seed, class Out>
+template <int LEVEL, bool INDEX, int BLOCKS = 5, class Seed, class Out>
 __device__ __forceinline__ void expand_a_batch(long long first, long long total, Seed seed_of, Out out_of,
                                                uint32_t *st, int lane) {
     using V = Lv<LEVEL>;
@@ -42,7 +43,7 @@ __device__ __forceinline__ void expand_a_batch(long long first, long long total,
     if (!p) a[4] = (uint32_t)(ij % V::L) | ((uint32_t)(ij / V::L) << 8) | (0x1Fu << 16);
     if (p) a[20] = 0x80000000u;
 #pragma unroll 1
-    for (int blk = 0; blk < 5; ++blk) {
+    for (int blk = 0; blk < BLOCKS; ++blk) {
         hash16_permute(a, p);
 #pragma unroll
         for (int i = 0; i < 21; ++i) st[s * EXPAND16_STRIDE + 42 * blk + 2 * i + p] = a[i];
@@ -57,7 +58,7 @@ __device__ __forceinline__ void expand_a_batch(long long first, long long total,
         const uint32_t *src = st + u * EXPAND16_STRIDE + w0;
         // the first 256 candidates all below q (0.78 of the polynomials): in place
         uint32_t v[9];
-        bool all = true;
+        bool all = 56 * BLOCKS >= N;
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
             v[m] = __funnelshift_r(src[24 * m], src[24 * m + 1], sh) & 0x7FFFFFu;
@@ -73,7 +74,7 @@ __device__ __forceinline__ void expand_a_batch(long long first, long long total,
         int c = 0;
 #pragma unroll
         for (int m = 0; m < 9; ++m) {
-            const bool acc = v[m] < (uint32_t)Q && (m < 8 || lane < 24);   // 280 candidates
+            const bool acc = v[m] < (uint32_t)Q && (32 * m + 32 <= 56 * BLOCKS || 32 * m + lane < 56 * BLOCKS);
             const uint32_t mask = __ballot_sync(FULL, acc);
             const int to = c + __popc(mask & lanemask_lt(lane));
             if (acc && to < N) dst[INDEX ? to : lane_order(to)] = (int32_t)v[m];

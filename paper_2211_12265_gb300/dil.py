@@ -71,6 +71,7 @@ def load() -> ctypes.CDLL:
                 "dil_test_t0_ntt": [P, I, I, S, P, P, P],
                 "dil_test_sample_in_ball_stream": [P, I, S, P, I, P, P],
                 "dil_test_expand_a": [P, I, S, P, P, P],
+                "dil_test_expand_a_refill": [P, I, S, P, I, P, P],
                 "dil_test_expand_s": [P, I, S, P, P, P],
                 "dil_test_expand_mask": [P, I, S, P, P, P, P],
                 "dil_test_sample_in_ball": [P, I, S, P, P, P],
@@ -277,6 +278,11 @@ def dil_test_ntt(ctx, n, inp, out, inverse, stream=None):
 def dil_test_expand_a(ctx, level, n, rho, ahat, stream=None):
     return _check(load().dil_test_expand_a(ctx, level, n, _ptr(rho), _ptr(ahat), _stream(stream)),
                   "dil_test_expand_a")
+
+
+def dil_test_expand_a_refill(ctx, level, n, rho, lane_order, ahat, stream=None):
+    return _check(load().dil_test_expand_a_refill(ctx, level, n, _ptr(rho), int(lane_order), _ptr(ahat), _stream(stream)),
+                  "dil_test_expand_a_refill")
 
 
 def dil_test_expand_s(ctx, level, n, rhop, s, stream=None):

@@ -396,3 +396,49 @@ def test_cancel_ends_a_launch_in_rounds_at_once(torch_cuda, delay):
         assert torch.equal(sig[ok], want_sig[ok]) and torch.equal(it[ok], want_it[ok])
         assert not bool(sig[gone].any()) and not bool(it[gone].any())
     assert rest < whole / 4, (rest, whole)
+
+
+# Seeds (a number's four bytes eight times) of Dilithium3 keys with a polynomial
+# that ExpandS's first two blocks do not fill: (number, polynomial, coefficients
+# they hold)
+THIRD_BLOCK = [(327, 0, 251), (46958, 1, 255), (54815, 10, 255), (65704, 10, 252)]
+
+
+@pytest.mark.parametrize("n", [4, 17, 40, 700])
+def test_secret_polynomials_that_need_a_third_block(torch_cuda, orc, n):
+    """One key in about ten thousand has such a polynomial; here several of a batch
+    have, first, last and in the middle of the sixteen that a warp samples."""
+    import hashlib
+    from gpu_util import gpu_keygen
+    from paper_2211_12265_gb300 import dil
+    seeds = W.seeds(n, 1120)
+    at = [0, n // 2, n - 2, n - 1]
+    for (number, poly, held), i in zip(THIRD_BLOCK, at):
+        zeta = number.to_bytes(4, "little") * 8
+        blocks = hashlib.shake_256(hashlib.shake_256(zeta).digest(128)[32:96] + bytes([poly, 0])).digest(272)
+        assert sum((b & 15) < 9 for b in blocks) + sum(b >> 4 < 9 for b in blocks) == held < 256
+        seeds[i] = np.frombuffer(zeta, np.uint8)
+    opk, osk = orc.keygen_batch(3, seeds)
+    with dil.Context(0) as ctx:
+        pk, sk = gpu_keygen(ctx, 3, seeds)
+    assert np.array_equal(pk, opk) and np.array_equal(sk, osk)
+
+
+@pytest.mark.parametrize("level", LEVELS)
+@pytest.mark.parametrize("n", [1, 5])
+def test_expand_a_samples_unfilled_polynomials_again(torch_cuda, level, n):
+    """The five blocks that ExpandA takes of a stream fall short with a probability
+    below 1e-30; with four every polynomial does."""
+    from gpu_util import dev, host
+    from paper_2211_12265_gb300 import dil
+    k, l = {2: (4, 4), 3: (6, 5), 5: (8, 7)}[level]
+    rho = dev(W.seeds(n, 1130))
+    c = np.arange(256)
+    word = ((c & 4) << 5) + ((c >> 3) << 2) + (c & 3)   # of coefficient c in lane order
+    with dil.Context(0) as ctx:
+        want, got, lanes = (torch_cuda.zeros((n, k * l, 256), dtype=torch_cuda.int32, device="cuda") for _ in range(3))
+        dil.dil_expand_a(ctx.handle, level, n, rho, 32, want)
+        dil.dil_test_expand_a_refill(ctx.handle, level, n, rho, False, got)
+        dil.dil_test_expand_a_refill(ctx.handle, level, n, rho, True, lanes)
+        want, got, lanes = host(want), host(got), host(lanes)
+    assert np.array_equal(got, want) and np.array_equal(lanes[:, :, word], want)
