@@ -442,3 +442,203 @@ def test_expand_a_samples_unfilled_polynomials_again(torch_cuda, level, n):
         dil.dil_test_expand_a_refill(ctx.handle, level, n, rho, True, lanes)
         want, got, lanes = host(want), host(got), host(lanes)
     assert np.array_equal(got, want) and np.array_equal(lanes[:, :, word], want)
+
+
+def _jobs(torch, dil, spec):
+    """(level, n, lo, hi) jobs on the device and their signatures by dil_sign."""
+    from gpu_util import dev
+    jobs, want = [], []
+    with dil.Context(0) as ctx:
+        for level, n, lo, hi in spec:
+            _, sk = ctx.keygen(level, dev(W.seeds(max(n, 1), 1140 + level)))
+            lens = W.message_lengths(max(n, 1), 1140, "uniform" if hi > lo else "fixed", lo, hi)
+            msg, off = W.messages(lens, 1140 + level)
+            jobs.append((level, sk[:n], dev(msg), dev(off.astype(np.uint64)[:n + 1])))
+            want.append([x.cpu().numpy() for x in ctx.sign(*jobs[-1], iterations=True)] if n else None)
+    return jobs, want
+
+
+@pytest.mark.parametrize("shape", [None, (8, 2, 0, 1, 4), (8, 4, 0, 2, 8), (8, 1, 0, 1, 8)])
+def test_mixed_empty_and_changing_jobs_in_either_form(torch_cuda, shape):
+    """Persistent launches of three levels, with an empty job among others, and of
+    argument sets in turn, in rounds (no shape, or one warp per task) and on the
+    device queue."""
+    from paper_2211_12265_gb300 import dil
+    torch = torch_cuda
+    jobs, want = _jobs(torch, dil, [(2, 300, 0, 1500), (5, 211, 0, 4096), (3, 97, 32, 64), (5, 0, 0, 0)])
+    with dil.Context(0) as ctx:
+        if shape:
+            dil.dil_set_persistent_tuning(ctx.handle, *shape)
+        for pick in ([0, 1, 2], [0, 3, 2], [1], [0, 1, 2], [2, 0]):
+            for g, i in zip(_persistent(torch, dil, ctx, [jobs[i] for i in pick]), pick):
+                if want[i] is not None:
+                    assert all(np.array_equal(a, b) for a, b in zip(g, want[i])), (pick, i)
+
+
+def test_one_warp_queue_on_a_refused_workspace(torch_cuda):
+    """The one-warp queue at its full size, speculation included, where the rounds'
+    workspace is refused: a limit that the queue's fits exactly."""
+    from paper_2211_12265_gb300 import dil
+    torch = torch_cuda
+    jobs, want = _jobs(torch, dil, [(5, 12000, 32, 32)])
+    with dil.Context(0) as ctx:
+        dil.dil_set_persistent_tuning(ctx.handle, 8, 1, 2, 1, 8)
+        # rounds: 4 x 3,000 tasks of 79 KiB and more, halved; queue: 152 x 2 x 8 workers of 124 KiB
+        dil.dil_test_set_alloc_limit(ctx.handle, 310 << 20)
+        (got,) = _persistent(torch, dil, ctx, jobs)
+    assert all(np.array_equal(a, b) for a, b in zip(got, want[0]))
+
+
+def test_cancel_on_the_device_queue(torch_cuda):
+    import time
+    from paper_2211_12265_gb300 import dil
+    torch = torch_cuda
+    n = 200_000
+    jobs, want = _jobs(torch, dil, [(2, n, 32, 32)])
+    level, sk, msg, off = jobs[0]
+    with dil.Context(0) as ctx:
+        dil.dil_set_persistent_tuning(ctx.handle, 8, 2, 0, 1, 4)
+        sig = torch.full((n, dil.SIZES[2][2]), 0x5A, dtype=torch.uint8, device="cuda")
+        st = torch.full((n,), 9, dtype=torch.int32, device="cuda")
+        it = torch.full((n,), 7, dtype=torch.int32, device="cuda")
+        dil.dil_sign_persistent(ctx.handle, [dil.sign_job(2, n, sk, msg, off, sig, st, it)])
+        time.sleep(0.01)
+        dil.dil_persistent_cancel(ctx.handle)
+        assert dil.dil_persistent_status(ctx.handle) == dil.ECANCELED
+        s, g, i = st.cpu().numpy(), sig.cpu().numpy(), it.cpu().numpy()
+        ok, gone = s == dil.OK, s == dil.ECANCELED
+        assert (ok | gone).all() and ok.any() and gone.any()
+        assert not g[gone].any() and not i[gone].any()
+        assert np.array_equal(g[ok], want[0][0][ok]) and np.array_equal(i[ok], want[0][2][ok])
+        (got,) = _persistent(torch, dil, ctx, jobs)   # the next launch starts with the word cleared
+    assert all(np.array_equal(a, b) for a, b in zip(got, want[0]))
+
+
+# Task counts of one stream and of several, with the hashes on a stream of their own
+FORKED = [(2, 40), (2, 5200), (3, 2300), (5, 700)]
+
+
+def _calls(torch, dil, ctx, level, n):
+    """Inputs (their true values, and buffers to fill), outputs and the calls of
+    every device form of one batch."""
+    from gpu_util import dev
+    seeds = dev(W.seeds(n, 1150 + level))
+    msg, off = W.messages(W.message_lengths(n, 1150, "uniform", 0, 300), 1150)
+    msg, off = dev(msg), dev(off.astype(np.uint64))
+    pk, sk = ctx.keygen(level, seeds)
+    sig, st = ctx.sign(level, sk, msg, off)
+    bad = sig.clone()
+    bad[::3, 40] ^= 2
+    key = torch.arange(n, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    true = dict(seeds=seeds, pk=pk, sk=sk, msg=msg, off=off.view(torch.int64), sig=bad, key=key)
+    x = {k: torch.zeros_like(v) for k, v in true.items()}
+    o = dict(pk=torch.zeros_like(pk), sk=torch.zeros_like(sk), sig=torch.zeros_like(sig), st=torch.full_like(st, 9),
+             ok=torch.full((n,), 7, dtype=torch.uint8, device="cuda"), ksig=torch.zeros_like(sig),
+             kst=torch.full_like(st, 9), kok=torch.full((n,), 7, dtype=torch.uint8, device="cuda"))
+    ks = dil.dil_keystore_create(ctx.handle, level, n, pk, sk)
+    want_ok = torch.ones(n, dtype=torch.uint8, device="cuda")
+    want_ok[::3] = 0
+    want = dict(pk=pk, sk=sk, sig=sig, st=st, ok=want_ok, ksig=sig, kst=st, kok=want_ok)
+
+    def run(stream):
+        h = ctx.handle
+        dil.dil_keygen(h, level, n, x["seeds"], o["pk"], o["sk"], stream)
+        dil.dil_sign(h, level, n, x["sk"], x["msg"], x["off"], o["sig"], o["st"], stream)
+        dil.dil_verify(h, level, n, x["pk"], x["msg"], x["off"], x["sig"], o["ok"], stream)
+        dil.dil_sign_keyed(h, ks, n, x["key"], x["msg"], x["off"], o["ksig"], o["kst"], stream)
+        dil.dil_verify_keyed(h, ks, n, x["key"], x["msg"], x["off"], x["sig"], o["kok"], stream)
+    return true, x, o, want, run, ks
+
+
+@pytest.mark.parametrize("level,n", FORKED)
+def test_forked_forms_keep_a_callers_stream_in_order(torch_cuda, level, n):
+    """Inputs that the caller's own stream fills in late, outputs that it copies
+    and overwrites at once: the context's other streams start and end within the
+    caller's."""
+    from paper_2211_12265_gb300 import dil
+    torch = torch_cuda
+    with dil.Context(0) as ctx:
+        true, x, o, want, run, ks = _calls(torch, dil, ctx, level, n)
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            for _ in range(3):
+                for k in x:
+                    x[k].zero_()
+                torch.cuda._sleep(2_000_000)   # about a millisecond
+                for k in x:
+                    x[k].copy_(true[k])
+                run(s)
+                copies = {k: v.clone() for k, v in o.items()}
+                for k in x:
+                    x[k].fill_(1)
+                for v in o.values():
+                    v.fill_(3)
+        s.synchronize()
+        dil.dil_keystore_destroy(ks)
+    for k, v in copies.items():
+        assert torch.equal(v, want[k]), k
+    assert all(bool((v == 3).all()) for v in o.values())
+
+
+@pytest.mark.parametrize("level,n", FORKED)
+def test_forked_forms_under_the_callers_capture(torch_cuda, level, n):
+    """Every device form in a graph of the caller's, replayed on other inputs, with
+    direct calls in between."""
+    from paper_2211_12265_gb300 import dil
+    torch = torch_cuda
+    with dil.Context(0) as ctx:
+        true, x, o, want, run, ks = _calls(torch, dil, ctx, level, n)
+        for k in x:
+            x[k].copy_(true[k])
+        run(torch.cuda.current_stream())   # the workspace is there before the capture
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            run(torch.cuda.current_stream())
+        for k in x:
+            x[k].zero_()
+        for _ in range(2):
+            for v in o.values():
+                v.fill_(3)
+            for k in x:
+                x[k].copy_(true[k])
+            graph.replay()
+            torch.cuda.synchronize()
+            for k, v in o.items():
+                assert torch.equal(v, want[k]), k
+            run(torch.cuda.current_stream())
+        torch.cuda.synchronize()
+        for k, v in o.items():
+            assert torch.equal(v, want[k]), k
+        del graph
+        dil.dil_keystore_destroy(ks)
+
+
+@pytest.mark.parametrize("level", LEVELS)
+def test_keygen_and_verify_in_small_workspaces(torch_cuda, orc, level):
+    """Budgets of one task's scratch and a few tasks' a launch; below one task's
+    the call is refused, whatever the shape."""
+    from gpu_util import dev, host
+    from paper_2211_12265_gb300 import dil
+    k, l = {2: (4, 4), 3: (6, 5), 5: (8, 7)}[level]
+    n = 23
+    pk, sk, msg, off = _inputs(orc, level, n, 1160, 0, 300)
+    sig, _, _ = orc.sign_batch(level, sk, msg, off)
+    gen, ver = 1024 * (l + k * l + l + k), 1024 * (1 + k * l) + 384
+    for budget in (gen, gen + 500, 5 * gen):
+        with dil.Context(0, workspace_budget=budget) as ctx:
+            gpk, gsk = ctx.keygen(level, dev(W.seeds(n, 1160)))
+            assert np.array_equal(host(gpk), pk) and np.array_equal(host(gsk), sk)
+    for budget in (ver, ver + 500, 5 * ver):
+        with dil.Context(0, workspace_budget=budget) as ctx:
+            assert host(ctx.verify(level, dev(pk), dev(msg), dev(off), dev(sig))).all()
+    for shape in (None, (8, 1), (8, 2), (4, 4)):
+        with dil.Context(0, workspace_budget=gen - 1) as c0, dil.Context(0, workspace_budget=ver - 1) as c2:
+            for ctx, op in ((c0, 0), (c2, 2)):
+                if shape:
+                    ctx.set_tuning(op, shape[0], shape[1], level)
+            with pytest.raises(dil.DilError):
+                c0.keygen(level, dev(W.seeds(n, 1160)))
+            with pytest.raises(dil.DilError):
+                c2.verify(level, dev(pk), dev(msg), dev(off), dev(sig))
