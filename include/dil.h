@@ -82,9 +82,10 @@ int dil_set_max_iter(dil_ctx *ctx, int max_iter);
  * whose kernels choose their own shapes: the hashes of independent tasks
  * sixteen to a warp, Sign's rejection loop in rounds over the whole batch.
  * These use streams of the context beside the caller's (which waits for them)
- * for a large batch and for Verify's hashes.  A workspace budget that holds a
- * fused kernel's task but not a batch form's runs the fused kernel with 8
- * warps per CTA and 2 per task.  Outputs do not depend on the shape. */
+ * for a large batch and for Verify's hashes.  Where a workspace budget holds the
+ * scratch of a task of the fused Sign but no round, the fused kernel runs (in the
+ * shape set, or with 8 warps per CTA and 2 per task).  Outputs do not depend on
+ * the shape. */
 int dil_set_tuning(dil_ctx *ctx, int op, int level, int warps_per_cta, int warps_per_task);
 
 /* Alg 1 (Gen): n 32-byte seeds -> n public keys and n secret keys. */
@@ -209,7 +210,7 @@ int dil_sign_persistent(dil_ctx *ctx, int njobs, const dil_sign_job *jobs, void 
  * access (>= 1), helper groups per unfinished task (0 disables speculation).
  * The device queue's shape: with one warp per task group, or without this call,
  * the launch runs in rounds (on the queue, in the shape 8, 2, 0, 1, 4 or the one
- * set, where the workspace budget or the device does not hold them). */
+ * set, where the device refuses their workspace). */
 int dil_set_persistent_tuning(dil_ctx *ctx, int warps_per_cta, int warps_per_task, int ctas_per_sm, int chunk,
                               int speculation);
 

@@ -113,18 +113,16 @@ size_t part_tasks(const dil_ctx *c, size_t n, size_t per, size_t &ns) {
 }
 
 // Launch shape of one call.  The fused forms run when the caller asked for two
-// or four warps per task, and where the budget holds the scratch of a fused
-// task but not that of the batch form (`per` bytes a task).
+// or four warps per task (a task of theirs needs at least the scratch of the batch
+// form's; Sign's rounds need a little more, sign_fused).
 struct Shape {
     bool fused;
     int warps, p;
 };
 
-Shape shape_of(const dil_ctx *c, int op, int level, size_t per) {
+Shape shape_of(const dil_ctx *c, int op, int level) {
     const int w = c->warps[op][lidx(level)], p = c->wpt[op][lidx(level)];
-    if (p > 1) return {true, w, p};
-    if (c->budget < per) return {true, 8, 2};
-    return {false, 0, 0};
+    return {p > 1, w, p};
 }
 
 // The fused kernels' launch shape where a caller set none.
@@ -149,7 +147,8 @@ RoundSize round_size(int level, int src, size_t n, size_t budget, int parts = 1)
     return {0, 0};
 }
 
-// The Sign form of a call: the fused kernel as for the other operations (shape_of).
+// The Sign form of a call: the fused kernel as for the other operations (shape_of),
+// and where the budget holds the scratch of one of its tasks but no round.
 bool sign_fused(const dil_ctx *c, int level, int src) {
     return c->wpt[1][lidx(level)] > 1 || round_size(level, src, 1, c->budget).tasks == 0;
 }
@@ -397,7 +396,7 @@ int dil_keygen(dil_ctx *c, int level, size_t n, const uint8_t *seeds, uint8_t *p
     size_t pkb, skb, sigb;
     sizes_of(level, pkb, skb, sigb);
     const size_t per = dil::scratch_polys(dil::OP_KEYGEN, level) * POLY_BYTES;
-    const Shape sh = shape_of(c, 0, level, per);
+    const Shape sh = shape_of(c, 0, level);
     size_t ns = sh.fused ? 1 : keygen_parts(level, n);
     const size_t tasks = part_tasks(c, n, per, ns);
     return run_streams(c, n, tasks, tasks * per, ns, (cudaStream_t)stream,
@@ -460,8 +459,7 @@ int dil_verify(dil_ctx *c, int level, size_t n, const uint8_t *pk, const uint8_t
     DeviceGuard g(c->device);
     size_t pkb, skb, sigb;
     sizes_of(level, pkb, skb, sigb);
-    const size_t batch = verify_task_bytes(level, dil::VERIFY_PLAIN);
-    const Shape sh = shape_of(c, 2, level, batch);
+    const Shape sh = shape_of(c, 2, level);
     if (!sh.fused) {
         dil::VerifyBatch b{};
         b.pk = pk;
@@ -729,9 +727,9 @@ int dil_sign_persistent(dil_ctx *c, int njobs, const dil_sign_job *jobs, void *s
         acc += w[j];
         J.sm_end[j] = j + 1 == njobs ? (1 << 30) : (int)(sms * acc / sum + 0.5);
     }
-    // One-warp launches run in rounds; shapes of two or four warps per task, a
-    // budget or device memory too small for a round, and the hook that makes
-    // bounded waits run out keep the device queue.
+    // One-warp launches run in rounds; shapes of two or four warps per task, device
+    // memory too short for them, and the hook that makes bounded waits run out keep
+    // the device queue.
     const bool wish = !(c->ptune_set && c->ptune.p > 1) && c->spin_limit == 0;
     const int max_iter = c->max_iter;
     if (!c->gexec || !same_jobs(J, c->gjobs) || !same_tune(c->ptune, c->gtune) || max_iter != c->gmax_iter ||
@@ -907,7 +905,7 @@ int dil_verify_keyed(dil_ctx *c, const dil_keystore *ks, size_t n, const int32_t
     DeviceGuard g(c->device);
     size_t pkb, skb, sigb;
     sizes_of(ks->level, pkb, skb, sigb);
-    const Shape sh = shape_of(c, 2, ks->level, verify_task_bytes(ks->level, dil::VERIFY_KEYED));
+    const Shape sh = shape_of(c, 2, ks->level);
     if (!sh.fused) {
         dil::VerifyBatch b{};
         b.pk = ks->pk;
@@ -1019,7 +1017,7 @@ int dil_keygen_host(dil_ctx *c, int level, size_t n, const uint8_t *seeds, uint8
     if (rc) return rc;
     uint8_t *d_seed = (uint8_t *)c->stage, *d_pk = d_seed + al(32 * n), *d_sk = d_pk + al(pkb * n);
     const size_t per = dil::scratch_polys(dil::OP_KEYGEN, level) * POLY_BYTES;
-    const Shape sh = shape_of(c, 0, level, per);
+    const Shape sh = shape_of(c, 0, level);
     const size_t tasks = pipe_tasks(c, n, per);
     return run_pipeline(c, n, tasks, tasks * per, (cudaStream_t)stream,
                         [&](size_t c0, size_t c1, cudaStream_t s, int32_t *scratch) -> int {
@@ -1115,7 +1113,7 @@ int dil_verify_host(dil_ctx *c, int level, size_t n, const uint8_t *pk, const ui
     uint8_t *d_sig = (uint8_t *)d_off + al(8 * (n + 1));
     uint8_t *d_ok = d_sig + al(sigb * n);
     const size_t batch = verify_task_bytes(level, dil::VERIFY_PLAIN);
-    const Shape sh = shape_of(c, 2, level, pipe_streams(n) * batch);
+    const Shape sh = shape_of(c, 2, level);
     const size_t per = sh.fused ? dil::scratch_polys(dil::OP_VERIFY, level) * POLY_BYTES : batch;
     const size_t tasks = pipe_tasks(c, n, per);
     // one chunk at a time: its hashes run beside the rest, as in dil_verify (1,000

@@ -1,8 +1,9 @@
 // Persistent Sign with a device work queue (section 4.3 of arXiv 2211.12265,
 // dynamic task scheduling, redesigned to run entirely on the device): the form
-// of launches with two or four warps per task, of lowered spin limits, and of
-// workspace budgets that do not hold a round (dil_rounds.cu; one graph of rounds
-// signs 20,000 Dilithium2 + 20,000 Dilithium5 tasks in 14.9 ms, the queue in 22.3).
+// of launches with two or four warps per task, of lowered spin limits, and where the
+// device refuses the workspace of a launch in rounds (dil_rounds.cu; one graph of
+// rounds signs 40,000 Dilithium2 + 40,000 Dilithium5 tasks in 14.9 ms, the queue in
+// 22.3).
 //
 // Workers are groups of P warps that stay resident for the whole launch.  A
 // worker takes a fresh task from the queue (atomic cursor), prepares it into
