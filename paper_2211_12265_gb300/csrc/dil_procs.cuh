@@ -375,8 +375,12 @@ __device__ void mask_stream(const uint8_t *rhop, int kappa, MaskStream &ms, int3
 
 // acc = sum_j A^_ij o v^_j 2^-32, |acc| < q, for one row i of A^ (ahat: the row's
 // l polynomials; read through L2 since another warp or kernel may have written
-// them); v^_j at `vhat`.  The products are summed in
-// 64 bits (|sum| < 7 q 9.1q < 2^31 q) and reduced once.
+// them); v^_j at `vhat`.  The products are summed in 64 bits (|sum| < 7 q 9.1q <
+// 2^31 q) and reduced once.  INDEX: A^ in index order, as the fused Verify and KeyGen
+// sample it: placing its coefficients in lane order one by one cost their samplers
+// more than the loads gain (one Dilithium3 Verify on two warps 131 -> 125 us, one
+// Dilithium5 key 185 -> 174).
+template <bool INDEX = false>
 __device__ __forceinline__ void accumulate_row(int32_t acc[8], const int32_t *ahat, int l, const int32_t *vhat,
                                                int lane) {
     long long sum[8];
@@ -385,7 +389,8 @@ __device__ __forceinline__ void accumulate_row(int32_t acc[8], const int32_t *ah
 #pragma unroll 1
     for (int j = 0; j < l; ++j) {
         int32_t a[8], v[8];
-        load_l2_cg(a, ahat + j * N, lane);
+        if (INDEX) load_seq_cg(a, ahat + j * N, lane);
+        else load_l2_cg(a, ahat + j * N, lane);
         load_l2(v, vhat + j * N, lane);
 #pragma unroll
         for (int m = 0; m < 8; ++m) sum[m] += (long long)a[m] * v[m];
@@ -447,7 +452,7 @@ __device__ void gen_rows(uint8_t *pk, uint8_t *sk, int32_t *scratch, WarpSmem &w
     // t = INTT(A^ o s^1) + s2; (t1, t0) = Power2Round(t), row i into pk and sk
 #pragma unroll 1
     for (int i = g; i < V::K; i += P) {
-        accumulate_row(acc, scratch + (V::L + i * V::L) * N, V::L, scratch, lane);
+        accumulate_row<true>(acc, scratch + (V::L + i * V::L) * N, V::L, scratch, lane);
         ntt_inv(acc, ws.buf, izt, lane);
         load_seq(a, sraw + (V::L + i) * N, lane);
         load_l0(r, sraw + (V::L + i) * N, lane);
@@ -498,7 +503,7 @@ __device__ void gen_task(const uint8_t *__restrict__ seed, uint8_t *pk, uint8_t 
         __syncwarp();
     }
     constexpr int KL = V::K * V::L;
-    expand_a_range<LEVEL>(gs.rho, share_lo<KL, P>(g), share_lo<KL, P>(g + 1), scratch + V::L * N, ws, lane);
+    expand_a_range<LEVEL, true>(gs.rho, share_lo<KL, P>(g), share_lo<KL, P>(g + 1), scratch + V::L * N, ws, lane);
     __threadfence_block();
     group_sync<P>(bar);
     gen_rows<LEVEL, P>(pk, sk, scratch, ws, zt, izt, g, bar, lane);
@@ -910,7 +915,7 @@ __device__ int verify_task(const uint8_t *__restrict__ pk, const uint8_t *__rest
     // A^ = ExpandA(rho) into scratch after z^ (unless resident)
     constexpr int KL = V::K * V::L;
     if constexpr (!KEYED)
-        expand_a_range<LEVEL>(gs.rho, share_lo<KL, P>(g), share_lo<KL, P>(g + 1), scratch + V::L * N, ws, lane);
+        expand_a_range<LEVEL, true>(gs.rho, share_lo<KL, P>(g), share_lo<KL, P>(g + 1), scratch + V::L * N, ws, lane);
     // mu = H(H(rho || t1) || M), on the last warp
     if (g == P - 1) {
         uint32_t lo = 0, hi = 0;
@@ -940,7 +945,7 @@ __device__ int verify_task(const uint8_t *__restrict__ pk, const uint8_t *__rest
     const int32_t *ahat = KEYED ? key + S::AH * N : scratch + V::L * N;
 #pragma unroll 1
     for (int i = g; i < V::K; i += P) {
-        accumulate_row(acc, ahat + i * V::L * N, V::L, scratch, lane);
+        accumulate_row<!KEYED>(acc, ahat + i * V::L * N, V::L, scratch, lane);
         if (KEYED) {
             load_l2_cg(r, key + (S::T1H + i) * N, lane);
         } else {
