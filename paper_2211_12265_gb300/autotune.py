@@ -1,11 +1,11 @@
 """Project autotuner: launch shapes per security level.
 
-For the plain kernels it sweeps, per level and operation, the warps per CTA
-and the warps per task (32 x warps-per-task threads share one task's
-polynomials: the paper's single-warp and four-warp forms, section 3.1); for
-the persistent Sign it also sweeps CTAs per SM, the queue chunk (fresh tasks
-per queue access) and the speculation slots (helper groups per unfinished
-task, section 4.3).  Every candidate is timed with CUDA events on a probe
+For the plain kernels it sweeps, per level and operation, the batch forms (one
+warp per task) and the fused kernels by warps per CTA and warps per task (32 x
+warps-per-task threads share one task's polynomials: the paper's single-warp
+and four-warp forms, section 3.1); for the persistent Sign the graph of rounds
+(one warp per task) and the device queue's shapes by warps per task and
+speculation slots (helper groups per unfinished task, section 4.3).  Every candidate is timed with CUDA events on a probe
 batch (L2 flushed before each timing, median of several) and the fastest is
 kept.  The result is a JSON table keyed by GPU name; ``apply`` installs it on
 a context.  ``tuning_gb300.json`` next to this file is the table measured on
@@ -19,9 +19,10 @@ import os
 HERE = os.path.dirname(os.path.abspath(__file__))
 DEFAULT_TABLE = os.path.join(HERE, "tuning_gb300.json")
 
-PLAIN_SHAPES = [(1, 1), (2, 1), (4, 1), (8, 1), (2, 2), (4, 2), (8, 2), (4, 4), (8, 4)]
-PERSIST_SHAPES = [(4, 1, 0, 1, 4), (8, 1, 0, 1, 0), (8, 1, 0, 1, 4), (8, 1, 0, 1, 8), (8, 1, 0, 1, 16),
-                  (8, 1, 0, 2, 8), (8, 2, 0, 1, 4), (8, 2, 0, 1, 8), (8, 4, 0, 1, 4), (8, 4, 0, 1, 8)]
+# One warp per task is one candidate each: it selects the batch forms and the graph
+# of rounds, whose kernels choose their own shapes.
+PLAIN_SHAPES = [(2, 1), (2, 2), (4, 2), (8, 2), (4, 4), (8, 4)]
+PERSIST_SHAPES = [(8, 1, 0, 1, 8), (8, 2, 0, 1, 4), (8, 2, 0, 1, 8), (8, 4, 0, 1, 4), (8, 4, 0, 1, 8)]
 OPS = {"keygen": 0, "sign": 1, "verify": 2}
 
 
