@@ -174,19 +174,16 @@ size_t verify_task_bytes(int level, int src) {
 constexpr size_t PIPE_MIN_TASKS = 2048;   // smaller batches run as one chunk
 constexpr size_t PIPE_STREAMS = 4;
 
-int ensure_aux(dil_ctx *c) {
-    if (c->aux[0]) return DIL_OK;
-    for (cudaStream_t &a : c->aux)
-        if (cudaStreamCreateWithFlags(&a, cudaStreamNonBlocking) != cudaSuccess) {
-            cudaGetLastError();
-            return DIL_ECUDA;
-        }
-    if (cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess) {
-        cudaGetLastError();
-        return DIL_ECUDA;
-    }
-    return DIL_OK;
+// The context's first `streams` own streams and the fork / join events (made when
+// a call first needs them: a stream costs a context's first Verify 7 us).
+int ensure_aux(dil_ctx *c, size_t streams) {
+    bool ok = true;
+    for (size_t i = 0; i < streams && ok; ++i)
+        if (!c->aux[i]) ok = cudaStreamCreateWithFlags(&c->aux[i], cudaStreamNonBlocking) == cudaSuccess;
+    for (cudaEvent_t *e : {&c->ev_fork, &c->ev_join})
+        if (ok && !*e) ok = cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) cudaGetLastError();
+    return ok ? DIL_OK : DIL_ECUDA;
 }
 
 // Runs chunk(c0, c1, stream, scratch) over n tasks, `per` at a time, on ns streams
@@ -198,7 +195,7 @@ int run_streams(dil_ctx *c, size_t n, size_t per, size_t region, size_t ns, cuda
     const size_t k = (n + per - 1) / per;
     ns = std::min(ns, k);
     int rc = ensure_ws(c, ns * region);
-    if (!rc && ns > 1) rc = ensure_aux(c);
+    if (!rc && ns > 1) rc = ensure_aux(c, ns - 1);
     if (rc) return rc;
     cudaStream_t st[PIPE_STREAMS] = {s0, c->aux[0], c->aux[1], c->aux[2]};
     if (ns > 1) {
@@ -273,7 +270,7 @@ void carve_verify(dil::VerifyBatch &b, void *ws, size_t m, size_t polys) {
 int run_verify_batch(dil_ctx *c, int level, int src, size_t n, const dil::VerifyBatch &all, cudaStream_t s) {
     const size_t polys = dil::verify_batch_polys(level, src), per = verify_task_bytes(level, src);
     const size_t tasks = chunk_tasks(c, per, n);
-    const int rc = ensure_aux(c);
+    const int rc = ensure_aux(c, 1);
     if (rc) return rc;
     size_t pkb, skb, sigb;
     dil_sizes(level, &pkb, &skb, &sigb);
@@ -745,7 +742,7 @@ int dil_sign_persistent(dil_ctx *c, int njobs, const dil_sign_job *jobs, void *s
         }
         const bool rounds = plan.bytes != 0;
         if (rounds) {
-            const int rc = ensure_aux(c);
+            const int rc = ensure_aux(c, PIPE_STREAMS - 1);
             if (rc) return rc;
         }
         if (c->gexec) {
@@ -1120,7 +1117,7 @@ int dil_verify_host(dil_ctx *c, int level, size_t n, const uint8_t *pk, const ui
     // Dilithium3 tasks 250 -> 196 us); of four chunks, each beside the others
     dil::VerifyFork fork{};
     if (!sh.fused && pipe_streams(n) == 1) {
-        if ((rc = ensure_aux(c))) return rc;
+        if ((rc = ensure_aux(c, 1))) return rc;
         fork = {c->aux[0], c->ev_fork, c->ev_join};
     }
     return run_pipeline(c, n, tasks, tasks * per, (cudaStream_t)stream,
