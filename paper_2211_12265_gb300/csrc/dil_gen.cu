@@ -48,6 +48,7 @@ __device__ __forceinline__ void put_words(uint8_t *dst, const uint32_t (&a)[25],
 // scratch, rho' behind it, K to sk.
 template <int LEVEL>
 struct KeygenSeedJob {
+    static constexpr bool CHAINED = false;
     const uint8_t *seed;
     uint8_t *pk, *sk;
     uint32_t *out;
@@ -160,6 +161,7 @@ __global__ void __launch_bounds__(32, LEVEL == 2 ? 28 : 20) k_keygen_rows(uint8_
 // tr = H(pk) of task `pair` into its secret key.
 template <int LEVEL>
 struct KeygenTrJob {
+    static constexpr bool CHAINED = false;
     const uint8_t *pk;
     uint8_t *sk;
     bool todo;

@@ -102,8 +102,8 @@ __device__ __forceinline__ void hash16_permute(uint32_t (&a)[25], bool high) {
 // HASH16_STAGE_WORDS shared words).  Job: `bool next(HashInput &)` gives this
 // thread's pair its next input (both threads of a pair get the same answer),
 // `void done(const uint32_t (&a)[25])` takes the state after the last block
-// (thread p holds words 2 i + p of the output).  What done() writes to global
-// memory may be the next input of the same pair.
+// (thread p holds words 2 i + p of the output).  Job::CHAINED: what done() writes to
+// global memory may be the next input of the same pair.
 template <class Job>
 __device__ __forceinline__ void hash16_run(Job &job, uint32_t *stage_words, int lane) {
     const uint32_t stage = smem_addr(stage_words);
@@ -131,10 +131,10 @@ __device__ __forceinline__ void hash16_run(Job &job, uint32_t *stage_words, int 
 #pragma unroll
             for (int i = 0; i < 25; ++i) a[i] = 0;
             off = 0;
-            // the next input may be what done() wrote: a thread fetches 8-byte
-            // units, of which its partner wrote half
-            __threadfence_block();
-            __syncwarp(3u << (lane & 30));
+            if (Job::CHAINED) {   // a thread fetches 8-byte units, of which its partner wrote half
+                __threadfence_block();
+                __syncwarp(3u << (lane & 30));
+            }
             live = job.next(in);
             if (live) hash16_fetch(in, 0, stage, pair, p);
         }

@@ -145,6 +145,7 @@ __device__ __forceinline__ void enter(const SignBatch &b, int task) {
 // ends), every other one enters round 0.
 template <int LEVEL, int SRC>
 struct SignMuJob {
+    static constexpr bool CHAINED = true;
     const SignBatch &b;
     int task, lane;
     bool first, have_mu;
@@ -410,6 +411,7 @@ __global__ void __launch_bounds__(32, 20) k_sign_front(const SignBatch b, int r)
 // c~ = H(mu || w1) of the attempt in slot `pair`.
 template <int LEVEL>
 struct SignCtJob {
+    static constexpr bool CHAINED = false;
     const SignBatch &b;
     const uint8_t *mu, *w1;
     bool todo;

@@ -69,6 +69,7 @@ __device__ __forceinline__ bool verify_input(const VerifyBatch &b, int t, int &k
 // the first by the pair's index, the next ones from the batch's counter.
 template <int LEVEL, int SRC>
 struct VerifyMuJob {
+    static constexpr bool CHAINED = true;
     const VerifyBatch &b;
     int task, lane;
     bool first, have_tr;
@@ -346,6 +347,7 @@ __global__ void __launch_bounds__(32 * P, LEVEL != 2 ? 20 / P : P > 1 ? 32 / P :
 // c~ = H(mu || w1') of task `pair` against the signature's.
 template <int LEVEL, int SRC>
 struct VerifyCompareJob {
+    static constexpr bool CHAINED = false;
     const VerifyBatch &b;
     int task, lane;
     bool todo;
