@@ -223,8 +223,8 @@ int dil_persistent_status(dil_ctx *ctx, void *stream);
 /* Cancels the persistent launch of this context that is running: sets its
  * cancel word through a copy on a stream of its own (the launch keeps
  * the SMs, so no kernel is involved) and returns once the word is written.
- * The launch then claims no more repetitions (in rounds: kernels that are still
- * to run leave their work out; those in flight end as they are): tasks that already hold an
+ * The launch then claims no more repetitions (in rounds: parts in flight end with
+ * the round they are in, later ones do not start): tasks that already hold an
  * accepting repetition finish as DIL_OK with their normal signature, every
  * other task ends with status DIL_ECANCELED, 0 iterations and an all-zero
  * signature, and the grid exits.  A launch that has not started yet resets

@@ -590,8 +590,8 @@ bool same_tune(const dil::PersistTuning &a, const dil::PersistTuning &b) {
 namespace {
 // A persistent launch in rounds: each job in parts, the parts dealt over the four
 // streams; a part's workspace serves one after the other.  At most PART_MOST
-// tasks a part: what is in flight when a cancel arrives runs on, everything behind
-// it leaves its work out.
+// tasks a part: a cancel ends those in flight with their round, and the ones behind
+// them leave their work out.
 constexpr size_t PART_MOST = 16384;
 struct RoundPlan {
     RoundSize size[dil::PERSIST_MAX_JOBS];
@@ -668,8 +668,9 @@ cudaError_t launch_rounds(dil_ctx *c, const dil::PersistJobs &J, const RoundPlan
             b.status = x.status ? x.status + c0 : nullptr;
             b.iters = x.iters ? x.iters + c0 : nullptr;
             b.max_iter = sign_cap(c, x.level);
-            b.cancel = dil::persist_cancel_word(c->pws);
             const size_t k = turn % PIPE_STREAMS;
+            b.cancel = dil::persist_cancel_word(c->pws);
+            b.stop = dil::persist_stop_word(c->pws, k);
             e = dil::launch_sign_batch(x.level, dil::SIGN_PLAIN, b,
                                        static_cast<uint8_t *>(c->pws) + dil::PERSIST_HEADER_BYTES + k * p.region, st[k]);
         }

@@ -89,6 +89,10 @@ struct SignBatch {
     int n_keys;
     int max_iter;
     const int *cancel;       // nullable: tasks without an accepted repetition end once it is set
+    int *stop;               // nullable, with cancel: set by the batch before on the same stream where that saw
+                             // the cancel.  It does not change while this batch runs, so all of its blocks agree
+                             // on it: one that leaves its work out on the cancel word itself could leave a task
+                             // with a part of its repetitions looked at
     int slots;               // attempts of a round, at least sign_batch_min_slots
     int parts;               // batches that share the GPU
     int on_gpu;              // tasks of them all that run at a time
@@ -195,7 +199,8 @@ struct PersistQueue {
     int error;        // DIL_ETIMEOUT when a bounded wait ran out
     int cancel;       // set by the host (dil_persistent_cancel) while the launch runs
     int next_job[PERSIST_MAX_JOBS];   // per job: next fresh task (job-local index)
-    int pad[26];
+    int stop[4];      // of a launch in rounds, per stream: SignBatch::stop
+    int pad[22];
 };
 struct PersistTuning {
     int warps = 8;        // warps per CTA
@@ -205,10 +210,11 @@ struct PersistTuning {
     int spec = 4;         // helper groups per unfinished task (0 = no speculation)
 };
 // Header bytes of a persistent launch's workspace (the queue, which a launch in
-// rounds shares for its error and cancel words), and the latter's address.
+// rounds shares for its error, cancel and stop words), and these words' addresses.
 constexpr size_t PERSIST_HEADER_BYTES = 256;
 static_assert(sizeof(PersistQueue) <= PERSIST_HEADER_BYTES, "queue header");
 inline const int *persist_cancel_word(const void *ws) { return &static_cast<const PersistQueue *>(ws)->cancel; }
+inline int *persist_stop_word(void *ws, size_t stream) { return &static_cast<PersistQueue *>(ws)->stop[stream]; }
 // Device bytes a persistent launch needs for `total` tasks of the given levels.
 size_t persist_workspace_bytes(const PersistJobs &J, const PersistTuning &t, int device);
 // Polls of a bounded device wait before it gives up (the default of a launch).

@@ -109,11 +109,6 @@ __device__ __forceinline__ const int32_t *pre_of(const SignBatch &b, int t) {
 // A host cancel of the batch (seen through L2; any lane).
 __device__ __forceinline__ bool canceled(const SignBatch &b) { return b.cancel && __ldcg(b.cancel) != 0; }
 
-// The same for a warp (all 32 lanes).  The word stays set until the launch has
-// ended, so a kernel that sees it may leave its work out: the checks behind it see
-// it, too, and accept nothing.
-__device__ __forceinline__ bool stopped(const SignBatch &b) { return b.cancel && __shfl_sync(FULL, canceled(b), 0); }
-
 // Status and repetitions of a task without a signature.
 __device__ __forceinline__ void report(const SignBatch &b, int task, int status, int iters) {
     if (b.status) b.status[task] = status;
@@ -273,7 +268,8 @@ __global__ void __launch_bounds__(32, 16) k_sign_prepare(const SignBatch b) {
         }
         blk -= b.wide_blocks;
     }
-    if (stopped(b)) return;
+    // canceled before this batch began: the hashing blocks reject every task
+    if (b.stop && *b.stop) return;
     if constexpr (SRC != SIGN_KEYED) {
         if (blk < b.expand_blocks) {
             expand_a_batch<LEVEL, false>(
@@ -302,7 +298,7 @@ __global__ void __launch_bounds__(32, 16) k_sign_mask(const SignBatch b, int r) 
     const Round q = round_of(b, r);
     // a state per polynomial: polynomial j of the attempt in slot i is the round's i l + j-th
     const int polys = q.p * q.m * V::L, first = blockIdx.x * K16_STATES;
-    if (first >= polys || stopped(b)) return;
+    if (first >= polys) return;
     const int s = lane >> 1, p = lane & 1;
     const int mine = min(first + s, polys - 1), slot = mine / V::L, i = slot / q.m;
     const int rep = q.base + slot - i * q.m;
@@ -683,10 +679,9 @@ __global__ void __launch_bounds__(32 * ROUND_WARPS, 8) k_sign_back(const SignBat
     int32_t *buf = bufs[warp], *zt = tables, *izt = tables + NTT_TABLE_WORDS;
     const int i = s / q.m, task = pending_list(b, r)[i], rep = q.base + s - i * q.m;
     int32_t *slot = slot_of<LEVEL>(b, s);
-    // a repetition past the cap, past one that has been accepted, or behind a cancel is
-    // not looked at
+    // a repetition past the cap, or past one that has been accepted, is not looked at
     int skip = 0;
-    if (lane == 0) skip = rep >= b.max_iter || canceled(b) || (q.m > 1 && atomicOr(&b.best[task], 0) < rep);
+    if (lane == 0) skip = rep >= b.max_iter || (q.m > 1 && atomicOr(&b.best[task], 0) < rep);
     bool accepted = false;
     if (!__shfl_sync(FULL, skip, 0)) {
         int32_t ch[8];
@@ -721,7 +716,7 @@ __global__ void __launch_bounds__(128) k_sign_back_wide(const SignBatch b, int r
     const int i = s / q.m, task = pending_list(b, r)[i], rep = q.base + s - i * q.m;
     int32_t *slot = slot_of<LEVEL>(b, s);
     const int32_t *pre = pre_of<LEVEL, SRC>(b, task);
-    bool bad = threadIdx.x == 0 && (rep >= b.max_iter || canceled(b) || (q.m > 1 && atomicOr(&b.best[task], 0) < rep));
+    bool bad = threadIdx.x == 0 && (rep >= b.max_iter || (q.m > 1 && atomicOr(&b.best[task], 0) < rep));
     bool accepted = !__syncthreads_or(bad);
     if (accepted) {
         int32_t ch[8];
@@ -777,6 +772,7 @@ template <int LEVEL, int SRC>
 __global__ void __launch_bounds__(256, 4) k_sign_rest(const SignBatch b, int r, int workers) {
     extern __shared__ __align__(16) uint8_t smem[];
     using V = Lv<LEVEL>;
+    if (b.stop && blockIdx.x == 0 && threadIdx.x == 0 && canceled(b)) *b.stop = 1;   // for the next batch in line
     if (b.count[r] <= 0) return;
     const Round q = round_of(b, r);
     const CtaView v = cta_setup<1>(smem);
@@ -794,7 +790,7 @@ __global__ void __launch_bounds__(256, 4) k_sign_rest(const SignBatch b, int r, 
         int it = q.base;
         bool ok = false, stop = false;
         MaskStream ms{0, 0};
-        while (it < b.max_iter && !(stop = stopped(b))) {
+        while (it < b.max_iter && !(stop = __shfl_sync(FULL, canceled(b), 0))) {
             ok = sign_attempt<LEVEL, 1>(it * V::L, pre, itr, ms, *v.gs, *v.ws, v.zt, v.izt, 0, v.bar, v.lane);
             ++it;
             if (ok) break;
