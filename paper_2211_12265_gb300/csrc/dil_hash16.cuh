@@ -4,10 +4,12 @@
 // of independent tasks (H(pk), mu, rho', c~) share the permutation's
 // instructions instead of running one per warp.
 //
-// A lone chain is no slower this way (250 SM clocks per round for a warp on
-// its own, 224 for the 25-lane form) and a loaded SM spends 3.2 clocks per
-// state and round on it where the 25-lane form spends 18.7: the bound is the
-// ALU pipe, which the logic and funnel shifts of a round occupy for 2.8.
+// A lone chain takes 250 SM clocks per round for a warp on its own and about a
+// thousand a block for absorbing, 224 and 150 in the 25-lane form (a 136-byte block
+// 3.8 to 4.0 us against 2.7), so long messages of small batches go there
+// (hash_split).  A loaded SM spends 3.2 clocks per state and round on this one, 18.7
+// on that: the bound is the ALU pipe, which the logic and funnel shifts of a round
+// occupy for 2.8.
 #pragma once
 #include "dil_keccak16.cuh"
 #include "dil_sample.cuh"

@@ -154,13 +154,14 @@ __device__ __forceinline__ uint64_t rider_word(const uint8_t *src, size_t len, i
 }
 
 // A SHAKE256 hash of `len` bytes of global memory (any alignment) that
-// rides in the last instance (15) of the sixteen-state batches of a sampler:
-// before each of the batch's permutations one 136-byte rate block of the
+// rides in the last instance (15) of sixteen-state batches.  No sampler of the
+// library carries one (the batch forms hash sixteen tasks to a warp): it and
+// K16ChainRider are the sixteen-state primitive's tests.  Before each of the batch's permutations one 136-byte rate block of the
 // input (the last one padded) is absorbed into instance 15, so the hash
 // needs no permutation of its own.  Once the permutation after the final
 // block has run, the first 32 output bytes go to `out` (8-byte aligned
 // shared memory).  A hash longer than the batches' permutations is finished
-// on the 25-lane form (finish).  The samplers that carry it use instances
+// on the 25-lane form (finish).  A batch that carries it uses instances
 // 0..14 only.  Block counts are 32-bit: an input of 2^31 blocks (292 GB)
 // would not fit in device memory.
 struct K16Rider {
@@ -234,7 +235,7 @@ struct K16Rider {
 };
 
 // A SHAKE256 hash that rides like K16Rider over an input that is still being
-// written (KeyGen's H(pk) while the rows of t are packed): a permutation
+// written: a permutation
 // advances it only when the next block's bytes exist (set_ready), and between
 // such permutations its state lives in shared memory (`save`, 25 x 8 bytes,
 // 8-byte aligned), so instance 15 may be overwritten in between (the other

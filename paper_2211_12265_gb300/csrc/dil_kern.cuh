@@ -65,7 +65,7 @@ inline int batch_hash_warps(int n) {
 }
 
 // Up to this many hashes a warp each, on the 25-lane form: while every warp has a
-// sub-partition to itself a block takes 2.7 us that way and 3.4 two threads to a
+// sub-partition to itself a block takes 2.7 us that way and 3.8 two threads to a
 // state (224 and 250 clocks a round; absorbing costs 150 and 1,000), and the
 // chain of a hash's blocks is what a small batch waits for.
 constexpr int HASH_WIDE_MOST = 608;

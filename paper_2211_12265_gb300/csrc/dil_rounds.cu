@@ -13,23 +13,23 @@
 //          smallest accepting repetition, or keeps the task for the next round
 // m grows as tasks finish (round_reps), so the long tail of the rejection loop
 // is evaluated in parallel and a round keeps filling the GPU.
-// The host launches as many rounds as leave no task over in all but a
-// vanishing share of batches, and then a kernel that runs the plain loop on
-// whatever is left.
+// The host launches as many rounds as leave at most 0.02 tasks over in
+// expectation (a launch of valid keys in fifty keeps one, and each of a batch's
+// parts counts), and then a kernel that runs the plain loop on whatever is left.
 //
 // Against one fused kernel with a task per warp (dil_sign.cu): every hash runs
 // at 3.2 SM clocks per round and state instead of 18.7 (c~) or with a third of
 // its output unused (masks sampled sixteen nonces ahead), each kernel's code
 // fits the instruction cache (the fused kernel's first stall is instruction
 // fetch), and no SM idles while a few tasks run 20 to 30 repetitions one after
-// the other.  Fused -> rounds: 10,000 Dilithium2 tasks 3396 -> 1521 us, 10,000
-// Dilithium3 (32 B - 4 KB) 5350 -> 2345 us, 150 Dilithium5 1580 -> 347 us, one
+// the other.  Fused -> rounds: 10,000 Dilithium2 tasks 3396 -> 1525 us, 10,000
+// Dilithium3 (32 B - 4 KB) 5350 -> 2340 us, 150 Dilithium5 1580 -> 340 to 375, one
 // Dilithium2 task 176 -> 101 us (of 256 KB 5568 -> 5431; 7862 with two threads to
 // its hash's state).
 //
-// What bounds the phases at 20,000 Dilithium2 attempts: mask the ALU pipe (87%),
-// prepare and hash the same (75%), front DRAM (69% of the copy rate), back its
-// issue slots (51%, the multiplier 51% of its rate; 20 of 32 warps).
+// What bounds the phases at 10,000 Dilithium2 tasks and 20,000 attempts: mask and
+// prepare the ALU pipe (82 and 71%), hash its few warps' chains (57% of that pipe),
+// front DRAM (59% of its peak), back its loads and issue slots (47%; 18 of 32 warps).
 #include <algorithm>
 #include <climits>
 

@@ -323,7 +323,9 @@ __device__ __forceinline__ void expand_s_pair(const uint8_t *rhop, int nonce0, i
 // Sixteen-instance ExpandS: polynomials with nonces 0 .. count - 1 (count <=
 // 16; s1 then s2), coefficient c of polynomial s to out[s N + c] (coefficient
 // order, global memory).  The candidates of two instances are voted on at
-// once, one per half-warp: 9 rounds of 16 bytes cover a block's 136.
+// once, one per half-warp: 9 rounds of 16 bytes cover a block's 136.  (KeyGen
+// samples with expand_s_batch; this one is the primitive that the tests hold
+// against the oracle.)
 template <int ETA>
 __device__ __forceinline__ void expand_s_16(const uint8_t *rhop, int count, int32_t *out, uint32_t *kst,
                                             int lane) {

@@ -146,7 +146,7 @@ __device__ __forceinline__ void verify_hash_wide(const VerifyBatch &b, int task,
 }
 
 // The hashing warps, each a CTA of its own: they are chains (a 16 KB message is
-// 121 blocks, 3.4 us each on a warp of its own), so they get the registers to
+// 121 blocks, 3.8 us each on a warp of its own), so they get the registers to
 // keep a state and its input (at 64, a block took 4.5 us) and start first.
 template <int LEVEL, int SRC>
 __global__ void __launch_bounds__(32, 16) k_verify_hash(const VerifyBatch b) {
