@@ -364,7 +364,7 @@ def test_cancel_ends_a_launch_in_rounds_soon(torch_cuda):
     from paper_2211_12265_gb300 import dil
     torch = torch_cuda
     n = 600_000   # about 38 parts of 16,384 tasks
-    whole, rest = [], []
+    whole, rest, hits = [], [], 0
     with dil.Context(0) as ctx:
         _, sk = ctx.keygen(2, dev(W.seeds(n, 1110)))
         msg, off = W.messages(np.full(n, 32), 1110)
@@ -386,17 +386,21 @@ def test_cancel_ends_a_launch_in_rounds_soon(torch_cuda):
             it.fill_(7)
             torch.cuda.synchronize()
             dil.dil_sign_persistent(ctx.handle, job)
-            time.sleep(0.001 * (2 + k))
+            time.sleep(0.001 * (3 + k))
             dil.dil_persistent_cancel(ctx.handle)
             t = time.perf_counter()
-            assert dil.dil_persistent_status(ctx.handle) == dil.ECANCELED
-            if k < 8:
-                rest.append(time.perf_counter() - t)
+            status = dil.dil_persistent_status(ctx.handle)
+            t = time.perf_counter() - t
             ok, gone = st == dil.OK, st == dil.ECANCELED
-            assert bool((ok | gone).all()) and bool(gone.any())
+            assert bool((ok | gone).all())
+            assert status == dil.ECANCELED or not bool(gone.any())
+            if bool(gone.any()):   # not where the host came before the launch, or after it
+                hits += 1
+                if k < 8:
+                    rest.append(t)
             assert torch.equal(sig[ok], want_sig[ok]) and torch.equal(it[ok], want_it[ok])
             assert not bool(sig[gone].any()) and not bool(it[gone].any())
-    assert min(rest) < min(whole) / 4, (rest, whole)
+    assert hits > 10 and min(rest) < min(whole) / 4, (hits, rest, whole)
 
 
 # Seeds (a number's four bytes eight times) of Dilithium3 keys with a polynomial
