@@ -80,11 +80,15 @@ cudaError_t launch_expand_a(int level, int n, const uint8_t *rho, size_t rho_str
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_test_expand_a_refill(int level, int n, const uint8_t *rho, bool index, int32_t *ahat, cudaStream_t s) {
-    switch (level) {
-        case 2: return index ? launch_expand<2, true, 4>(n, rho, 32, ahat, s) : launch_expand<2, false, 4>(n, rho, 32, ahat, s);
-        case 3: return index ? launch_expand<3, true, 4>(n, rho, 32, ahat, s) : launch_expand<3, false, 4>(n, rho, 32, ahat, s);
-        case 5: return index ? launch_expand<5, true, 4>(n, rho, 32, ahat, s) : launch_expand<5, false, 4>(n, rho, 32, ahat, s);
+cudaError_t launch_test_expand_a_refill(int level, int n, const uint8_t *rho, bool index, int32_t *ahat,
+                                        cudaStream_t s) {
+    switch (2 * level + index) {
+        case 4: return launch_expand<2, false, 4>(n, rho, 32, ahat, s);
+        case 5: return launch_expand<2, true, 4>(n, rho, 32, ahat, s);
+        case 6: return launch_expand<3, false, 4>(n, rho, 32, ahat, s);
+        case 7: return launch_expand<3, true, 4>(n, rho, 32, ahat, s);
+        case 10: return launch_expand<5, false, 4>(n, rho, 32, ahat, s);
+        case 11: return launch_expand<5, true, 4>(n, rho, 32, ahat, s);
     }
     return cudaErrorInvalidValue;
 }

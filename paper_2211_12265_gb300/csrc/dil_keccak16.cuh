@@ -156,11 +156,11 @@ __device__ __forceinline__ uint64_t rider_word(const uint8_t *src, size_t len, i
 // A SHAKE256 hash of `len` bytes of global memory (any alignment) that
 // rides in the last instance (15) of sixteen-state batches.  No sampler of the
 // library carries one (the batch forms hash sixteen tasks to a warp): it and
-// K16ChainRider are the sixteen-state primitive's tests.  Before each of the batch's permutations one 136-byte rate block of the
-// input (the last one padded) is absorbed into instance 15, so the hash
-// needs no permutation of its own.  Once the permutation after the final
-// block has run, the first 32 output bytes go to `out` (8-byte aligned
-// shared memory).  A hash longer than the batches' permutations is finished
+// K16ChainRider are the sixteen-state primitive's tests.  Before each of the
+// batch's permutations one 136-byte rate block of the input (the last one padded)
+// is absorbed into instance 15, so the hash needs no permutation of its own.  Once
+// the permutation after the final block has run, the first 32 output bytes go to
+// `out` (8-byte aligned shared memory).  A hash longer than the batches' permutations is finished
 // on the 25-lane form (finish).  A batch that carries it uses instances
 // 0..14 only.  Block counts are 32-bit: an input of 2^31 blocks (292 GB)
 // would not fit in device memory.

@@ -150,7 +150,8 @@ cudaError_t launch_test_k16_chain_rider(int n, const uint8_t *in, const uint64_t
 cudaError_t launch_test_t0_ntt(int level, int variant, int n, const uint8_t *sk, int32_t *tmp, int32_t *out,
                                cudaStream_t s);
 cudaError_t launch_test_expand_a(int level, int n, const uint8_t *rho, int32_t *out, cudaStream_t s);
-cudaError_t launch_test_expand_a_refill(int level, int n, const uint8_t *rho, bool index, int32_t *ahat, cudaStream_t s);
+cudaError_t launch_test_expand_a_refill(int level, int n, const uint8_t *rho, bool index, int32_t *ahat,
+                                        cudaStream_t s);
 cudaError_t launch_test_expand_s(int level, int n, const uint8_t *rhop, int32_t *out, cudaStream_t s);
 cudaError_t launch_test_expand_mask(int level, int n, const uint8_t *rhop, const int32_t *kappa, int32_t *out,
                                     cudaStream_t s);

@@ -1,8 +1,8 @@
 // Verify of a batch (Alg 3).
 //
 // Batch form.  One kernel hashes tr = H(pk) and mu = H(tr || M), sixteen tasks
-// to a warp (in small batches, and for their long messages, a warp each).  Beside it, on a stream of their own where the caller has one to
-// spare, run SampleInBall(c~), sixteen tasks to a warp, with ExpandA, sixteen
+// to a warp (in small batches, and for their long messages, a warp each).  Beside
+// it, on a stream of their own where the caller has one to spare, run SampleInBall(c~), sixteen tasks to a warp, with ExpandA, sixteen
 // polynomials to a warp whatever tasks they belong to (dil_sample16.cuh; not
 // with a resident key's or the caller's A^), and then the arithmetic up to the
 // packed w1', one task per warp.  The last kernel recomputes c~ = H(mu || w1'),
@@ -172,7 +172,8 @@ __global__ void __launch_bounds__(128, 4) k_verify_hash_both(const VerifyBatch b
         VerifyMuJob<LEVEL, SRC> job(b, has_wide_warp(b.off, b.n, t, b.long_bytes, b.per_group) ? b.n : t, lane);
         hash16_run(job, stage[warp], lane);
     } else {
-        const int task = task_of_wide_warp(b.off, b.n, (blockIdx.x - b.pair_ctas) * 4 + warp, b.long_bytes, b.per_group, lane);
+        const int w = (blockIdx.x - b.pair_ctas) * 4 + warp;
+        const int task = task_of_wide_warp(b.off, b.n, w, b.long_bytes, b.per_group, lane);
         if (task >= 0) verify_hash_wide<LEVEL, SRC, 4>(b, task, lane);
     }
 }
